@@ -53,6 +53,28 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// ---------------------------------------------------------------- warp roles
+// The warp's index in the block, the same register value in every lane (a
+// plain threadIdx.x >> 5 is not known to be uniform).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// True in one lane of the (converged) warp.  The thread that issues MMAs and
+// TMA copies is chosen with it and not by `lane == 0`: their operands sit in
+// warp-uniform registers, and only under elect.sync does the compiler know
+// that a single lane is active and move the operands there directly.  Under
+// `lane == 0` every tcgen05.mma took 154 cycles to issue whatever its shape,
+// every TMA copy 58; under elect.sync 128 x N x 16 MMAs follow one another
+// every 48 (N 64), 64 (N 128) and 128 (N 256) cycles, which is the tensor
+// pipe's and the operand reads' own rate, and a TMA copy takes 15.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

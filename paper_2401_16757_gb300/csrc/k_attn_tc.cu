@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 9);
   const uint32_t done_bar = smem_u32(bars + 10);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int t0 = blockIdx.x * kAQ, h = blockIdx.y;
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
   const int col0 = h * kAD;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- TMA producer
       mbar_arrive_expect_tx(q_full, kTile);
       tma_load_2d(smem_u32(smem + kOffQ), &tmQ, q_full, col0, t0);
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
         mbar_wait_bounded(kv_full(j & 1), (j >> 1) & 1, &no_abort, nullptr);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- MMA issuer
       constexpr int bf = std::is_same<T, __nv_bfloat16>::value ? 1 : 0;
       constexpr uint32_t idesc_s = idesc_f16(bf, kAQ, kAK);

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   auto full_bar = [&](int s) { return full0 + 8u * s; };
   auto empty_bar = [&](int s) { return empty0 + 8u * s; };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int m0 = TAP ? 0 : blockIdx.x * kBM, n0 = blockIdx.y * BN;
   // tap mode: this CTA's patch (image, patch row th, patch column tw)
   int pimg = 0, pth = 0, ptw = 0;
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (csplit) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");  // peers started (waited before DSMEM use)
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- TMA producer: weight tiles of the first stages go
       // out before waiting for the previous kernel (they do not depend on it)
       const int early = min(nk, kStages);
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     pdl_wait();
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- MMA issuer
       constexpr uint32_t idesc = idesc_f16(std::is_same<T, __nv_bfloat16>::value ? 1 : 0, kBM, BN);
       for (int i = 0; i < nk; ++i) {

@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
   auto full_bar = [&](int s) { return full0 + 8u * s; };
   auto empty_bar = [&](int s) { return empty0 + 8u * s; };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   // m-tiles: 128-row blocks of the output matrix, or pixel patches (kATap)
   const int hw = p.Ho * p.Wo;
   const int patches = p.tiles_w * p.tiles_h;
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
   pdl_launch_dependents();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- TMA producer.  The weight tiles of the first stages
       // go out before waiting for the previous kernel (they do not depend on it).
       auto coords = [&](int g, int* kx, int* m0, int* n0) {
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
     }
   } else if (warp == 1) {
     pdl_wait();
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- MMA issuer
       constexpr uint32_t idesc = idesc_f16(std::is_same<T, __nv_bfloat16>::value ? 1 : 0, kPBM, BN);
       int g = 0;

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) tc_conv_small_kernel(const Smal
   // per k: element offset inside the receptive window and the tap (dy, dx);
   // k >= K gets dy = kInvalidTap, which fails the bounds test
   int2* tab = reinterpret_cast<int2*>(reinterpret_cast<uint8_t*>(bars) + 64);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = warp_index();
   const int n0 = blockIdx.y * kSmBN;
   const uint32_t bar0 = smem_u32(bars);
 
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) tc_conv_small_kernel(const Smal
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)(buf * kSmBN);
       for (int kb = 0; kb < nkb; ++kb) {
