@@ -13,8 +13,9 @@
 // streaming the weight matrix):
 //   warp 0      TMA producer (one elected lane)
 //   warp 1      TMEM allocation and MMA issue (one elected lane)
-//   warps 2..5  im2col gather (conv) and the epilogue (TMEM -> registers ->
-//               global), warp w reading TMEM lanes 32*(w % 4) .. +31.
+//   warps 2..5  im2col gather (conv)
+//   warps 2..9  epilogue: TMEM -> registers -> shared memory -> global, warp w
+//               reading TMEM lanes 32*(w % 4) .. +31 of one half of the columns.
 // Every wait is bounded; on timeout the kernel records kDevErrTimeout in
 // the error word, drains what it started, frees TMEM and returns.
 #include <cudaTypedefs.h>
@@ -37,7 +38,8 @@ namespace {
 
 constexpr int kBM = 128;
 constexpr int kBK = 64;  // 64 x 2 bytes = one 128-byte swizzle row
-constexpr int kThreads = 192;
+constexpr int kEpiThreads = 256;
+constexpr int kThreads = 64 + kEpiThreads;
 constexpr int kABytes = kBM * kBK * 2;
 
 // N tile 256 serves GEMMs of at most kFewRows rows (one partly filled M
@@ -52,7 +54,7 @@ template <int BN> struct Cfg {
   static constexpr int kStageBytes = kStages * (kABytes + kBBytes);
   // cluster split-K receive buffer.  BN 64/128 (row owners): up to 16 splits
   // x ceil(128/splits) rows.  BN 256 (column owners): splits x kFewRows rows
-  // x (columns per owner + 4), at most kFewRows x (256 + 8 x 8) floats.
+  // x (columns per owner + 4), at most kFewRows x 6 x 52 floats (2 to 8 splits).
   static constexpr int kRecvBytes = BN == 256 ? kFewRows * (BN + 64) * 4 : (kBM + 15) * (BN + 4) * 4;
   static constexpr int kBiasBytes = BN * 4;
   static constexpr int kSmem = kStageBytes + kRecvBytes + kBiasBytes + 256 + 1024;
@@ -147,7 +149,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // bias of this tile to shared memory (weights: ready before the kernel)
   if (threadIdx.x >= 64) {
     const T* bias = static_cast<const T*>(p.e.bias);
-    for (int j = threadIdx.x - 64; j < BN; j += 128) sbias[j] = (bias && n0 + j < p.N) ? to_f<T>(bias[n0 + j]) : 0.f;
+    for (int j = threadIdx.x - 64; j < BN; j += kEpiThreads) sbias[j] = (bias && n0 + j < p.N) ? to_f<T>(bias[n0 + j]) : 0.f;
   }
   tc_fence_before();
   __syncthreads();
@@ -155,6 +157,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = *tmem_slot;
   pdl_launch_dependents();
   if (csplit) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");  // peers started (waited before DSMEM use)
+
+  const bool vec = epi_vec_ok(p);
+  const int rmode = res_mode(p.e);
+  // cluster split-K: what epilogue thread t sums after the exchange, and its
+  // residual, requested while the MMAs run.  BN 64/128: 8 columns of up to
+  // kRedN rows of this CTA's share of the rows; BN 256: 8 columns of one row
+  // of this CTA's share of the columns
+  constexpr int kColGroups = BN / 8, kRedRows = kEpiThreads / kColGroups, kRedN = BN == 256 ? 1 : 64 / kRedRows;
+  const int t = (int)threadIdx.x - 64;
+  int red_m[kRedN];
+  uint4 red_res[kRedN];
 
   if (warp == 0) {
     if (elect_one()) {
@@ -203,9 +216,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_commit(accum_bar);  // fires once every MMA issued above has completed
     }
   } else {
-    const int t = threadIdx.x - 64;  // 0..127
     pdl_wait();
-    if (GATHER) {
+    if (GATHER && t < 128) {
       // ---------------- implicit im2col gather of A (row t of the tile)
       const int m = m0 + t;
       const bool mvalid = m < p.M;
@@ -275,87 +287,82 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3;
     const int row = q * 32 + lane;
     const int m = row_m(row);  // -1: this row has no output
-    const bool vec_ok = ((p.ldy | n0) % 8 == 0) && (!p.e.res || ((p.e.ldr | n0) % 8 == 0));
-    // without a split, the residual of the first 32 columns is requested
-    // while the MMAs run, each later chunk's one chunk ahead of its use (zeros
-    // for layers without one: one loop for both measured faster than two)
-    const bool has_res = splits == 1;
+    const bool any_row = __any_sync(0xffffffffu, m >= 0);
+    const int c_lo = (warp - 2) / 4 * (BN / 2), c_hi = c_lo + BN / 2;  // this warp's columns
+    const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
     uint4 rnext[4];
-    if (has_res) res_prefetch32<T>(rnext, p, m, n0, vec_ok);
+    if (splits == 1) {
+      epi_res_load<T>(rnext, p, m, n0 + c_lo, vec);
+    } else if (csplit && BN == 256) {
+      const int cpo = (((BN + splits - 1) / splits) + 7) & ~7;
+      const int w8 = (min(BN, ((int)blockIdx.z + 1) * cpo) - (int)blockIdx.z * cpo) / 8;
+      const int rr = w8 > 0 ? t / w8 : kFewRows;
+      red_m[0] = rr < kFewRows ? row_m(rr) : -1;
+      if (red_m[0] >= 0) red_res[0] = res8<T>(p, red_m[0], n0 + (int)blockIdx.z * cpo + 8 * (t - rr * w8), vec);
+    } else if (csplit) {
+      const int rpo = (kBM + splits - 1) / splits;
+#pragma unroll
+      for (int j = 0; j < kRedN; ++j) {
+        const int rr = j * kRedRows + t / kColGroups;
+        red_m[j] = rr < rpo && (int)blockIdx.z * rpo + rr < kBM ? row_m((int)blockIdx.z * rpo + rr) : -1;
+        red_res[j] = res8<T>(p, red_m[j], n0 + 8 * (t % kColGroups), vec);
+      }
+    }
     const bool ok = mbar_wait_bounded(accum_bar, 0, abort_flag, p.err);
     tc_fence_after();
-    if (ok && splits == 1) {
+    const bool all_ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
+    if (splits == 1) {
+      // the stage ring is idle now (every load was consumed by an MMA that
+      // has completed): its first 16 KB stage the warps' pieces
+      const uint32_t stage = smem_u32(sA) + (uint32_t)((warp - 2) * kEpiStage);
+      if (all_ok && any_row) {
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        uint4 rcur[4];
-        if (has_res) {
+        for (int c0 = c_lo; c0 < c_hi && n0 + c0 < p.N; c0 += 32) {
+          uint4 rcur[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) rcur[i] = rnext[i];
-          if (c0 + 32 < BN) res_prefetch32<T>(rnext, p, m, n0 + c0 + 32, vec_ok);
-        }
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-        tmem_ld_wait();
-        if (m >= 0 && n0 + c0 < p.N) {
-          float v[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-          if (has_res) finish32r<T>(v, sbias + c0, p, m, n0 + c0, vec_ok, rcur);
-          else finish32<T>(v, sbias + c0, p, m, n0 + c0, vec_ok);
-        }
-      }
-    } else if (csplit && BN == 256) {
-      // cluster split-K over columns (at most kFewRows rows): columns
-      // [o * cpo, (o + 1) * cpo) of the tile belong to CTA o of the cluster;
-      // this split's partial goes to slot blockIdx.z of each owner
-      const int cpo = (((BN + splits - 1) / splits) + 3) & ~3;
-      const int rs = cpo + 4;  // row stride of a slot, floats
-      const bool mine = ok && m >= 0 && row < kFewRows;
-      asm volatile("barrier.cluster.wait;" ::: "memory");  // every peer is running
-#pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-        tmem_ld_wait();
-        if (mine) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int c = c0 + 4 * j;
-            const uint32_t owner = (uint32_t)(c / cpo);
-            const int cl = c - (int)owner * cpo;
-            const uint32_t la = smem_u32(recv) + (uint32_t)((((int)blockIdx.z * kFewRows + row) * rs + cl) * 4);
-            uint32_t ra;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(owner));
-            asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(ra), "f"(__uint_as_float(r[4 * j])),
-                         "f"(__uint_as_float(r[4 * j + 1])), "f"(__uint_as_float(r[4 * j + 2])),
-                         "f"(__uint_as_float(r[4 * j + 3]))
-                         : "memory");
-          }
+          if (c0 + 32 < c_hi) epi_res_load<T>(rnext, p, m, n0 + c0 + 32, vec);
+          epi_piece<T>(lanes + (uint32_t)c0, sbias + c0, stage, p, m, n0 + c0, vec, rmode, rcur);
         }
       }
     } else if (csplit) {
-      // cluster split-K: push this split's rows to the CTA that owns them
-      // (owner of row w = w / rows_per_owner), slot = this split's index
-      const int rpo = (kBM + splits - 1) / splits;
-      const uint32_t owner = (uint32_t)(row / rpo);
-      const int rr = row - (int)owner * rpo;
-      const uint32_t base = smem_u32(recv) + (uint32_t)(((blockIdx.z * rpo + rr) * (BN + 4)) * 4);
       asm volatile("barrier.cluster.wait;" ::: "memory");  // every peer is running
+      // push this split's partial rows to their owners, slot = this split's index
+      const bool mine = BN == 256 ? m >= 0 && row < kFewRows : m >= 0;
+      if (all_ok && __any_sync(0xffffffffu, mine)) {
+        // BN 64/128: owner of row w = w / rows_per_owner.  BN 256 (at most
+        // kFewRows rows): columns [o * cpo, (o + 1) * cpo) belong to CTA o
+        const int rpo = (kBM + splits - 1) / splits;
+        const int cpo = (((BN + splits - 1) / splits) + 7) & ~7;
+        const uint32_t owner = (uint32_t)(row / rpo);
+        uint32_t base = 0;
+        if (BN != 256) {
+          const uint32_t la = smem_u32(recv) + (uint32_t)((((int)blockIdx.z * rpo + row - (int)owner * rpo) * (BN + 4)) * 4);
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base) : "r"(la), "r"(owner));
+        }
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-        tmem_ld_wait();
-        if (ok && m >= 0) {
+        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+          uint32_t r[16];
+          tmem_ld_32x32b_x16(lanes + (uint32_t)c0, r);
+          tmem_ld_wait();
+          if (mine) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            uint32_t ra;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(base + (uint32_t)((c0 + 4 * j) * 4)), "r"(owner));
-            asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(ra), "f"(__uint_as_float(r[4 * j])),
-                         "f"(__uint_as_float(r[4 * j + 1])), "f"(__uint_as_float(r[4 * j + 2])),
-                         "f"(__uint_as_float(r[4 * j + 3]))
-                         : "memory");
+            for (int j = 0; j < 4; ++j) {
+              const int c = c0 + 4 * j;
+              uint32_t ra = base + (uint32_t)c * 4;
+              if (BN == 256) {
+                const uint32_t o = (uint32_t)(c / cpo);
+                const uint32_t la =
+                    smem_u32(recv) + (uint32_t)((((int)blockIdx.z * kFewRows + row) * (cpo + 4) + c - (int)o * cpo) * 4);
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(o));
+              }
+              asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(ra), "f"(__uint_as_float(r[4 * j])),
+                           "f"(__uint_as_float(r[4 * j + 1])), "f"(__uint_as_float(r[4 * j + 2])),
+                           "f"(__uint_as_float(r[4 * j + 3]))
+                           : "memory");
+            }
           }
+          __syncwarp();
         }
       }
     } else if (ok) {
@@ -364,21 +371,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       float* part = p.partial + ((int64_t)blockIdx.z * p.M) * p.N;
       const bool pvec = (p.N % 4 == 0);
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
+      for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+        uint32_t r[16];
+        tmem_ld_32x32b_x16(lanes + (uint32_t)c0, r);
         tmem_ld_wait();
         const int n = n0 + c0;
         if (m >= 0 && n < p.N) {
           float* dst = part + (int64_t)m * p.N + n;
-          if (pvec && n + 32 <= p.N) {
+          if (pvec && n + 16 <= p.N) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 4)
+            for (int j = 0; j < 16; j += 4)
               __stcg(reinterpret_cast<float4*>(dst + j), make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
                                                                        __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])));
           } else {
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
+            for (int j = 0; j < 16; ++j)
               if (n + j < p.N) __stcg(dst + j, __uint_as_float(r[j]));
           }
         }
@@ -396,73 +403,59 @@ __global__ void __launch_bounds__(kThreads, 1)
       epi_bar();
       if (*last_flag) {
         __threadfence();
+        const int n = n0 + 8 * (t % kColGroups);
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 32) {
-          const int n = n0 + c0;
-          if (m < 0 || n >= p.N) continue;
-          float v[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = 0.f;
+        for (int rr = t / kColGroups; rr < kBM; rr += kRedRows) {
+          const int mm = row_m(rr);
+          if (mm < 0 || n >= p.N) continue;
+          float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
           for (int z = 0; z < splits; ++z) {
-            const float* src = p.partial + ((int64_t)z * p.M + m) * p.N + n;
-            if (pvec && n + 32 <= p.N) {
-#pragma unroll
-              for (int j = 0; j < 32; j += 4) {
-                const float4 f = __ldcg(reinterpret_cast<const float4*>(src + j));
-                v[j] += f.x; v[j + 1] += f.y; v[j + 2] += f.z; v[j + 3] += f.w;
-              }
+            const float* src = p.partial + ((int64_t)z * p.M + mm) * p.N + n;
+            if (pvec && n + 8 <= p.N) {
+              const float4 f = __ldcg(reinterpret_cast<const float4*>(src));
+              const float4 g = __ldcg(reinterpret_cast<const float4*>(src + 4));
+              v[0] += f.x; v[1] += f.y; v[2] += f.z; v[3] += f.w;
+              v[4] += g.x; v[5] += g.y; v[6] += g.z; v[7] += g.w;
             } else {
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
+              for (int j = 0; j < 8; ++j)
                 if (n + j < p.N) v[j] += __ldcg(src + j);
             }
           }
-          finish32<T>(v, sbias + c0, p, m, n, vec_ok);
+          finish8<T>(v, sbias + 8 * (t % kColGroups), p, mm, n, vec, rmode, res8<T>(p, mm, n, vec));
         }
       }
     }
   }
   if (csplit) {
     if (threadIdx.x < 64) asm volatile("barrier.cluster.wait;" ::: "memory");  // pairs the early arrive
-    // all pushes are visible after this barrier; each CTA reduces the rows
-    // it owns from its own receive buffer, in split order 0..S-1
+    // all pushes are visible after this barrier; each CTA reduces its share
+    // from its own receive buffer, in split order 0..S-1
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-    if constexpr (BN == 256) {
-      // this CTA owns columns [c_lo, c_hi) of the tile, every row
-      const int cpo = (((BN + splits - 1) / splits) + 3) & ~3;
-      const int rs = cpo + 4;
-      const int c_lo = (int)blockIdx.z * cpo, c_hi = min(BN, c_lo + cpo);
-      const int rows = max(0, min(kFewRows, p.M - m0));
-      const int w4 = max(0, c_hi - c_lo) / 4;
-      const int groups = rows * w4;
-      for (int g = threadIdx.x; g < groups; g += kThreads) {
-        const int rr = g / w4, c4 = g % w4;
-        const int n = n0 + c_lo + 4 * c4;
-        const float* src = recv + rr * rs + 4 * c4;
-        float4 acc = *reinterpret_cast<const float4*>(src);
-        for (int z = 1; z < splits; ++z) {
-          const float4 v = *reinterpret_cast<const float4*>(src + z * kFewRows * rs);
-          acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-        }
-        if (n < p.N) finish4<T>(acc, sbias + c_lo + 4 * c4, p, m0 + rr, n);
-      }
-    } else {
+    if (t >= 0) {
       const int rpo = (kBM + splits - 1) / splits;
-      const int r0 = (int)blockIdx.z * rpo;
-      const int rows = TAP ? max(0, min(rpo, kBM - r0)) : max(0, min(min(rpo, kBM - r0), p.M - m0 - r0));
-      const int groups = rows * (BN / 4);
-      for (int g = threadIdx.x; g < groups; g += kThreads) {
-        const int rr = g / (BN / 4), c4 = g % (BN / 4);
-        const int n = n0 + 4 * c4;
-        const int mm = row_m(r0 + rr);
-        if (mm < 0) continue;
-        const float* src = recv + rr * (BN + 4) + 4 * c4;
-        float4 acc = *reinterpret_cast<const float4*>(src);
+      const int cpo = (((BN + splits - 1) / splits) + 7) & ~7;
+      const int c_own = BN == 256 ? (int)blockIdx.z * cpo : 0;  // this CTA's first column
+      const int w8 = BN == 256 ? max(1, (min(BN, c_own + cpo) - c_own) / 8) : kColGroups;
+      const int rs = BN == 256 ? cpo + 4 : BN + 4;                      // floats per receive row
+      const int zs = (BN == 256 ? kFewRows : rpo) * rs;                 // floats per split
+      const int c8 = t % w8 * 8;
+#pragma unroll
+      for (int j = 0; j < kRedN; ++j) {
+        const int rr = j * kRedRows + t / w8, n = n0 + c_own + c8;
+        if (red_m[j] < 0 || n >= p.N) continue;
+        const float* src = recv + rr * rs + c8;
+        float4 a0 = *reinterpret_cast<const float4*>(src), a1 = *reinterpret_cast<const float4*>(src + 4);
+#pragma unroll 4
         for (int z = 1; z < splits; ++z) {
-          const float4 v = *reinterpret_cast<const float4*>(src + z * rpo * (BN + 4));
-          acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+          const float4 f = *reinterpret_cast<const float4*>(src + z * zs);
+          const float4 g = *reinterpret_cast<const float4*>(src + z * zs + 4);
+          a0.x += f.x; a0.y += f.y; a0.z += f.z; a0.w += f.w;
+          a1.x += g.x; a1.y += g.y; a1.z += g.z; a1.w += g.w;
         }
-        if (n < p.N) finish4<T>(acc, sbias + 4 * c4, p, mm, n);
+        const float v[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        finish8<T>(v, sbias + c_own + c8, p, red_m[j], n, vec, rmode, red_res[j]);
       }
     }
   }

@@ -9,9 +9,11 @@
 //   warp 0       TMA producer: the weight tile B of every k-block, and A too
 //                for plain GEMMs (linear layers, 1x1 stride-1 convs)
 //   warp 1       TMEM owner and MMA issuer (one elected lane)
-//   warps 2..5   epilogue: TMEM -> registers -> bias / residual / activation
-//                -> global, warp w reading TMEM lanes 32 * (w % 4) .. + 31
-//   warps 6..9   (convolutions without whole-tap TMA) implicit im2col gather of
+//   warps 2..9   epilogue: TMEM -> registers -> bias / residual / activation
+//                -> shared memory -> global, warp w reading TMEM lanes
+//                32 * (w % 4) .. + 31 of one half of the tile's columns (four
+//                warps and all columns where the stages leave no room for eight)
+//   then 4 warps (convolutions without whole-tap TMA) implicit im2col gather of
 //                A with cp.async
 // A-operand modes: kAT2d (row-major A by 2-D TMA), kAGather (cp.async im2col
 // gather), kATap (convolution A by one 4-D TMA per k-block: the 64 channels
@@ -53,18 +55,23 @@ template <int BN, int MS> struct PCfg {
   static constexpr int kB = BN * kPBK * 2;
   static constexpr int kSA = MS * kPA;      // A bytes per stage
   static constexpr int kStageBytes = kStages * (kSA + kB);
-  static constexpr int kBias = 2 * 4 * BN * 4;  // [buffer][epilogue warp][BN] fp32
-  static constexpr int kSmem = kStageBytes + kBias + 256 + 1024;
+  static constexpr int kEpiWarps = MS == 4 ? 4 : 8;
+  static constexpr int kCols = BN / (kEpiWarps / 4);      // columns per epilogue warp
+  static constexpr int kBias = kEpiWarps * kCols * 4;     // [epilogue warp][its columns] fp32
+  static constexpr int kStaging = kEpiWarps * kEpiStage;  // a 32 x 32 output piece per warp
+  static constexpr int kSmem = kStageBytes + kBias + kStaging + 256 + 1024;
   static_assert(kSmem <= 232448, "dynamic shared memory above the 227 KB per-CTA limit");
   static_assert(2 * MS * BN <= 512, "TMEM holds 512 fp32 columns");
 };
 
 constexpr int kAT2d = 0, kAGather = 1, kATap = 2;
 
-template <int AMODE> constexpr int persist_threads() { return AMODE == kAGather ? 320 : 192; }
+template <int BN, int AMODE, int MS> constexpr int persist_threads() {
+  return 64 + 32 * PCfg<BN, MS>::kEpiWarps + (AMODE == kAGather ? 128 : 0);
+}
 
 template <typename T, int BN, int AMODE, int MS>
-__global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
+__global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
     tc_persist_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const TcArgs p) {
   constexpr bool GATHER = AMODE == kAGather;
@@ -75,8 +82,9 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
   uint8_t* sB = smem + kStages * Cfg::kSA;
-  float* sbias = reinterpret_cast<float*>(smem + Cfg::kStageBytes);  // [2][4][BN]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kStageBytes + Cfg::kBias);
+  uint8_t* staging = smem + Cfg::kStageBytes;
+  float* sbias = reinterpret_cast<float*>(staging + Cfg::kStaging);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(staging + Cfg::kStaging + Cfg::kBias);
   // bars: full[kStages], empty[kStages], tfull[2], tempty[2], drain
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -107,7 +115,7 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull0 + 8u * b, 1);
-      mbar_init(tempty0 + 8u * b, 4);  // one arrival per epilogue warp
+      mbar_init(tempty0 + 8u * b, Cfg::kEpiWarps);  // one arrival per epilogue warp
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -272,19 +280,22 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
       volatile int no_abort = 0;
       mbar_wait_bounded(drain_bar, 0, &no_abort, p.err);
     }
-  } else if (warp < 6) {
+  } else if (warp < 2 + Cfg::kEpiWarps) {
     // ---------------- epilogue
     pdl_wait();
     const int q = warp & 3;
     const int row = q * 32 + lane;
+    const int c_lo = (warp - 2) / 4 * Cfg::kCols;  // this warp's columns
+    float* sb = sbias + (warp - 2) * Cfg::kCols;   // its own copy of their bias: no cross-warp barrier
+    const uint32_t stage = smem_u32(staging) + (uint32_t)((warp - 2) * kEpiStage);
+    const bool vec = epi_vec_ok(p);
+    const int rmode = res_mode(p.e);
     for (int lt = 0; lt < my_tiles; ++lt) {
       const int buf = lt & 1, use = lt >> 1;
       const int tile = tile_of(lt);
-      const int n0 = (tile / mtp) * BN;
-      // each warp stages its own copy of the tile's bias: no cross-warp barrier
-      float* sb = sbias + (buf * 4 + q) * BN;
+      const int n0 = (tile / mtp) * BN + c_lo;
       const T* bias = static_cast<const T*>(p.e.bias);
-      for (int j = lane; j < BN; j += 32) sb[j] = (bias && n0 + j < p.N) ? to_f<T>(bias[n0 + j]) : 0.f;
+      for (int j = lane; j < Cfg::kCols; j += 32) sb[j] = (bias && n0 + j < p.N) ? to_f<T>(bias[n0 + j]) : 0.f;
       __syncwarp();
       // output row of this thread's TMEM lane in sub-tile sub, -1 when unused
       auto row_of = [&](int sub) {
@@ -305,41 +316,29 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
         }
         return m;
       };
-      const bool vec_ok = ((p.ldy | n0) % 8 == 0) && (!p.e.res || ((p.e.ldr | n0) % 8 == 0));
       // the residual of the first 32 columns is requested while the
-      // accumulator is still being computed, each later chunk's one chunk
-      // ahead of its use.  The same loop serves layers without a residual
-      // (zeros): skipping it for them measured slower on whole networks
-      // (YOLOv3 resident 0.742 -> 0.788 ms, ResNet-50 0.330 -> 0.345 ms)
-      const bool has_res = true;
+      // accumulator is still being computed, each later piece's one ahead
+      int m = row_of(0);
       uint4 rnext[4];
-      if (has_res) res_prefetch32<T>(rnext, p, row_of(0), n0, vec_ok);
+      epi_res_load<T>(rnext, p, m, n0, vec);
       const bool got = mbar_wait_bounded(tfull0 + 8u * buf, use & 1, abort_flag, p.err);
       if (!__all_sync(0xffffffffu, got)) break;  // tcgen05.ld is warp-collective
       tc_fence_after();
 #pragma unroll 1
       for (int sub = 0; sub < MS; ++sub) {
-        const int m = row_of(sub);
+        const int m_next = sub + 1 < MS ? row_of(sub + 1) : -1;
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 32) {
+        for (int c0 = 0; c0 < Cfg::kCols; c0 += 32) {
           uint4 rcur[4];
-          if (has_res) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) rcur[i] = rnext[i];
-            if (c0 + 32 < BN) res_prefetch32<T>(rnext, p, m, n0 + c0 + 32, vec_ok);
-            else if (sub + 1 < MS) res_prefetch32<T>(rnext, p, row_of(sub + 1), n0, vec_ok);
-          }
-          uint32_t r[32];
-          tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((buf * MS + sub) * BN + c0), r);
-          tmem_ld_wait();
-          if (m >= 0 && n0 + c0 < p.N) {
-            float v[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-            if (has_res) finish32r<T>(v, sb + c0, p, m, n0 + c0, vec_ok, rcur);
-            else finish32<T>(v, sb + c0, p, m, n0 + c0, vec_ok);
-          }
+          for (int i = 0; i < 4; ++i) rcur[i] = rnext[i];
+          if (c0 + 32 < Cfg::kCols) epi_res_load<T>(rnext, p, m, n0 + c0 + 32, vec);
+          else if (sub + 1 < MS) epi_res_load<T>(rnext, p, m_next, n0, vec);
+          if (n0 + c0 < p.N)
+            epi_piece<T>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((buf * MS + sub) * BN + c_lo + c0), sb + c0, stage,
+                         p, m, n0 + c0, vec, rmode, rcur);
         }
+        m = m_next;
       }
       tc_fence_before();
       __syncwarp();
@@ -348,7 +347,7 @@ __global__ void __launch_bounds__(persist_threads<AMODE>(), 1)
   } else if (GATHER) {
     // ---------------- implicit im2col gather of A (row t of every tile)
     pdl_wait();
-    const int t = threadIdx.x - 192;  // 0..127
+    const int t = threadIdx.x - (64 + 32 * Cfg::kEpiWarps);  // 0..127
     const uint32_t row_off = (uint32_t)((t >> 3) * 1024 + (t & 7) * 128);
     const uint32_t sw = (uint32_t)(t & 7);
     const bool whole_tap = (p.C % kPBK) == 0;  // a 64-wide k-block never straddles taps
@@ -449,7 +448,7 @@ int launch_persist_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)std::min<int64_t>(tiles, sms));
-  cfg.blockDim = dim3(persist_threads<AMODE>());
+  cfg.blockDim = dim3(persist_threads<BN, AMODE, MS>());
   cfg.dynamicSmemBytes = PCfg<BN, MS>::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

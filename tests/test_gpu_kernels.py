@@ -1,0 +1,54 @@
+"""Kernel branches at the sizes where they can go wrong (tile edges, ragged
+columns, smallest and largest of a branch's range), against the CPU oracle."""
+import pytest
+
+from paper_2401_16757_gb300 import capi
+import synth
+from helpers import Runner, check_close, oracle_outputs
+from oracle import plan as OP
+
+pytestmark = pytest.mark.gpu
+
+
+def _linear(src, k, n, act="none", res=None, res_post=False, bias=True):
+    return dict(op="linear", src=[src], k=k, n=n, act=act, res=res, res_post=res_post, bias=bias)
+
+
+def _check(layers, inp, dtype, budget=None):
+    """The resident engine against the oracle, and a swapped one (where the
+    model has layers enough to swap) bit-equal to it."""
+    m = dict(name="yolov3", model_id=43, dtype=dtype, input=inp, layers=layers, outputs=[len(layers) - 1])
+    w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
+    host = capi.HostWeights(w)
+    rs = Runner(m, w, capi.Plan.resident(d), host)
+    got = rs.run(x)
+    check_close(m, rs.decode(got), oracle_outputs(m, w, x))
+    biggest = max(sum(OP.align(b) for b in OP.layer_tensor_bytes(m, i)) for i in range(len(layers)))
+    sw = Runner(m, w, capi.Plan.partition(d, 2 * biggest + 512, capi.options(swap_variant=capi.SWAP_ZEROCOPY)), host)
+    assert all(a.tobytes() == b.tobytes() for a, b in zip(sw.run(x), got)), "swapped and resident differ"
+    return rs
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("act,res_post", [("relu", False), ("leaky", True), ("swiglu", False)])
+@pytest.mark.parametrize("rows,k,n", [
+    (200, 256, 40),     # one tile per CTA, one 32-column piece and a quarter
+    (200, 256, 255),    # odd width: 2-byte moves
+    (40, 2048, 130),    # K split over a cluster, rows shared out, odd multiple of 2
+    (129, 1024, 264),   # the same, second M tile of one row
+    (12, 2048, 520),    # few rows: columns shared out
+    (16, 2048, 333),
+    (2600, 128, 264),   # persistent
+    (2600, 128, 255),
+    (5000, 64, 48),
+])
+def test_tile_epilogue(dtype, act, res_post, rows, k, n):
+    _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
+
+
+@pytest.mark.parametrize("hw", [160, 220])
+def test_sub_tiles_with_a_residual(hw):
+    """Two and four 128-row sub-tiles per tile, the residual of the next
+    sub-tile requested during the one before."""
+    conv = dict(op="conv", src=[-1], cin=64, cout=48, kh=1, kw=1, stride=1, pad=0, act="none", res=None, res_post=False)
+    _check([conv, dict(conv, act="leaky", res=0, res_post=True)], (2, hw, hw, 64), "f16")
