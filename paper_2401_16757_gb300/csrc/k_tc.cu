@@ -682,6 +682,35 @@ int active_clusters(int dtype, int c) {
   return dtype == SWAPNET_BF16 ? active_clusters_inst<__nv_bfloat16>(c) : active_clusters_inst<__half>(c);
 }
 
+// Time of a persistent kernel in SM cycles, from rates measured on the GB300:
+// an SM loads up to ~130 bytes per clock from L2, all SMs together ~12900; a
+// CTA's 128 x N x 16 MMA takes N/2 cycles (not below 48: the operand reads);
+// a warp's 32 x 32 epilogue piece takes about 1400.  bytes: loaded per CTA
+// and k-block; mma: cycles per k-block; pieces: epilogue pieces per warp and
+// tile.  The epilogue of a tile overlaps the MMAs of the next.
+double persist_cycles(int64_t tiles, int64_t slots, int ctas_per_slot, int KB, double bytes, double mma, int pieces) {
+  const double active = (double)std::min(tiles, slots) * ctas_per_slot;
+  const double stage = std::max(mma, bytes / std::min(130.0, 12900.0 / active));
+  const double epi = 1400.0 * pieces, waves = (double)((tiles + slots - 1) / slots);
+  return waves * std::max(KB * stage + 300.0, epi) + epi;
+}
+
+// N tile of the paired kernel with the least persist_cycles (ties: the
+// widest) for mt 128-row blocks; sets *cycles.
+int pair_tile(int64_t mt, int64_t N, int KB, int sms, double* cycles) {
+  int best_bn = 0;
+  *cycles = 0.0;
+  for (int bn = 256; bn >= 64; bn -= 32) {
+    const int64_t tiles = (mt + 1) / 2 * ((N + bn - 1) / bn);
+    const double c = persist_cycles(tiles, sms / 2, 2, KB, kABytes + 64.0 * bn, 2.0 * std::max(bn, 64), (bn / 32 + 1) / 2);
+    if (!best_bn || c < *cycles) {
+      best_bn = bn;
+      *cycles = c;
+    }
+  }
+  return best_bn;
+}
+
 int max_cluster(int dtype, int bn, bool gather) {
   const bool bf = dtype == SWAPNET_BF16;
   if (bn == 256) return bf ? max_cluster_inst<__nv_bfloat16, 256, kA2d>() : max_cluster_inst<__half, 256, kA2d>();
@@ -744,8 +773,22 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
         if ((sp_tiles + 3) / 4 * nt64 >= sms) p->msub = 4;
         else if ((sp_tiles + 1) / 2 * nt64 >= sms) p->msub = 2;
       }
-      p->tiles = (sp_tiles + p->msub - 1) / p->msub * ((g.N + pbn - 1) / pbn);
-      int rc = make_tmap(&p->tmB, g.dtype, g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2, (uint32_t)pbn);
+      // pairs of SMs on 256-row tiles where the model of both kernels says so
+      if (p->msub == 1 && sp_tiles > 1 && (!g.conv || tmac)) {
+        const int KB = p->kb_per_split;
+        const double one = persist_cycles(sp_tiles * ((Nd + pbn - 1) / pbn), sms, 1, KB, kABytes + 128.0 * pbn,
+                                          2.0 * std::max(pbn, 96), std::max(1, pbn / 64));
+        double two = 0.0;
+        const int bn2 = pair_tile(sp_tiles, Nd, KB, sms, &two);
+        if (two < one) {
+          p->pair = 1;
+          p->bn = bn2;
+        }
+      }
+      const int mtile = p->pair ? 2 : p->msub;
+      p->tiles = (sp_tiles + mtile - 1) / mtile * ((g.N + p->bn - 1) / p->bn);
+      int rc = make_tmap(&p->tmB, g.dtype, g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2,
+                         (uint32_t)(p->pair ? p->bn / 2 : p->bn));
       if (rc) return rc;
       if (!g.conv && g.A) {
         rc = make_tmap(&p->tmA, g.dtype, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, (uint32_t)kBM);
@@ -867,6 +910,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
 
 int launch_tc_gemm(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   if (!pl.ready) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "tcgen05 GEMM not prepared");
+  if (pl.pair) return launch_tc_pair(g, pl, err, s);
   if (pl.persist) return launch_tc_persist(g, pl, err, s);
   const bool bf = g.dtype == SWAPNET_BF16;
   if (g.conv && pl.tma_conv) {

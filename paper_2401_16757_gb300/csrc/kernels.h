@@ -161,6 +161,7 @@ struct TcPlan {
   uint64_t scratch_bytes;  // fp32 partials of all splits
   int persist;      // persistent kernel (one CTA per SM looping over tiles)
   int tma_conv;     // convolution A by 4-D TMA per filter tap (tmA is then 4-D)
+  int pair;         // persistent on pairs of SMs: tiles of 256 x bn, bn any multiple of 32 up to 256
   int msub;         // persistent: 128-row sub-tiles per tile (2 for N tiles of 64 with A by TMA)
   int wt, ht, tiles_w, tiles_h;  // its output patch and patch counts per image
   int ready;
@@ -168,6 +169,7 @@ struct TcPlan {
 int tc_prepare(const TcGemm& g, TcPlan* p);
 int launch_tc_gemm(const TcGemm& g, const TcPlan& p, int* dev_err, cudaStream_t s);
 int launch_tc_persist(const TcGemm& g, const TcPlan& p, int* dev_err, cudaStream_t s);
+int launch_tc_pair(const TcGemm& g, const TcPlan& p, int* dev_err, cudaStream_t s);
 
 // tcgen05 convolution for channel counts the gather cannot fetch in 16-byte
 // pieces (C % 8 != 0), K = kh*kw*C <= 192: weights built in shared memory,

@@ -52,3 +52,23 @@ def test_sub_tiles_with_a_residual(hw):
     sub-tile requested during the one before."""
     conv = dict(op="conv", src=[-1], cin=64, cout=48, kh=1, kw=1, stride=1, pad=0, act="none", res=None, res_post=False)
     _check([conv, dict(conv, act="leaky", res=0, res_post=True)], (2, hw, hw, 64), "f16")
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("act,res_post", [("none", False), ("swiglu", False)])
+@pytest.mark.parametrize("rows,k,n", [
+    (1000, 200, 1000),   # 4 x 256-row tiles, last one half empty; ragged k-block, ragged last columns
+    (897, 64, 1501),     # one k-block, odd width, an odd number of 128-row blocks
+    (385, 1088, 4160),   # several tiles per pair
+    (2049, 576, 288),    # one row in the last tile
+])
+def test_paired_gemm(dtype, act, res_post, rows, k, n):
+    _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
+
+
+@pytest.mark.parametrize("stride,cin,cout,hw,batch", [(1, 64, 256, 52, 3), (2, 128, 160, 75, 5), (1, 64, 96, 57, 4)])
+def test_paired_conv(stride, cin, cout, hw, batch):
+    """Convolutions by 4-D TMA on pairs of SMs: patches past the last one, strides, ragged patch edges."""
+    conv = dict(op="conv", src=[-1], cin=cin, cout=cout, kh=3, kw=3, stride=stride, pad=1, act="leaky", res=None,
+                res_post=False)
+    _check([conv, dict(conv, res=0, res_post=True)], (batch, hw, hw, cin), "f16")
