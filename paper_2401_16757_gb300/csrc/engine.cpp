@@ -1124,8 +1124,8 @@ static int run_unit(swapnet_engine* e, int u, const void* din, void* dout, cudaS
         if (skinny_ok(m, L))
           return launch_linear_skinny(m.dtype, x, L.n, L.d.cin, X.w, U.rows, ep, y + (int64_t)U.row0 * es,
                                       L.d.cout, s, X.in_place ? 0 : 1, e->num_sms, e->err_word);
-        return launch_linear_tiled(m.dtype, x, L.n, L.d.cin, X.w, U.rows, ep, y + (int64_t)U.row0 * es, L.d.cout,
-                                   s);
+        return launch_linear_tiled(m.dtype, x, L.n, L.d.cin, X.w, U.rows, L.d.cout, ep, y + (int64_t)U.row0 * es,
+                                   L.d.cout, s);
       }
       ep.res = r;
       if (small_conv_ok(m, L)) {

@@ -411,55 +411,188 @@ template <typename T> int skinny_dispatch(const SkJob& j, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------ tiled linear
-// General fallback for any M, K, N and dtype: 64 x 64 output tile per CTA,
-// 16 x 16 threads with 4 x 4 outputs each, K staged through shared memory
-// in steps of 16, fp32 accumulation in a fixed order.
+// General fallback for any M, K, N and dtype (fp32 rows beyond the skinny
+// kernel's 16, 16-bit layers whose K the other kernels do not take): one
+// TM x TN output tile per CTA, fp32 FMAs.  K is walked in chunks of BK that
+// cp.async brings into a ring of kTlStages stages (the weights' first stages
+// before the programmatic wait), rows as they lie in memory, padded by four
+// floats so that eight rows' 16-byte pieces fall on different banks.  A
+// chunk's k are shared out to KG groups of threads; each thread keeps RM x RN
+// outputs of its group's sum, two partial sums (even and odd k) per output in
+// one packed fma.rn.f32x2.  At the end the groups' sums are added in group
+// order through shared memory, so a result does not depend on scheduling.
+//
+// What bounds it: for the batches it serves (17 to a few hundred rows) the
+// parallelism, hence two tiles: 32 x 32 with K split 8 ways inside the CTA
+// while 64 x 64 tiles would not fill the SMs, 64 x 64 (K split in two) from
+// there on.  100 x 1000 x 1000 fp32:
+// 91 us with 64 x 64 tiles of 16 k per step, loaded and waited for element by
+// element; 13.9 us now.
+constexpr int kTlStages = 4;
+constexpr int kTlThreads = 256;
+constexpr int kTlWideTiles = 128;  // 64 x 64 tiles from which they are taken
+
+template <int TM, int TN, int RM, int RN, int BK> struct TlCfg {
+  static constexpr int kCols = TM / RM;                     // threads along M in a group
+  static constexpr int kGroup = kCols * (TN / RN);          // threads per k group
+  static constexpr int KG = kTlThreads / kGroup;
+  static constexpr int kRow = BK + 4;                       // floats per staged row
+  static constexpr int kStage = (TM + TN) * kRow;           // floats per stage
+  static constexpr int kPartRow = TN + 4;
+  static constexpr int kSmem = 4 * (kTlStages * kStage > KG * TM * kPartRow ? kTlStages * kStage : KG * TM * kPartRow);
+  static_assert(BK % (4 * KG) == 0 && TM * (BK / 4) % kTlThreads == 0 && TN * (BK / 4) % kTlThreads == 0, "shares");
+};
+
+__device__ __forceinline__ void cp_async_4(uint32_t dst, const void* src, bool valid) {
+  const int n = valid ? 4 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+
+// acc.xy += a.xy * b.xy, both halves rounded as a scalar FMA would.
+__device__ __forceinline__ void fma2(uint64_t& acc, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// Four consecutive k of row r (of `rows`) of a row-major matrix into shared
+// memory; zeros past the matrix.  vec: rows are 16-byte aligned (fp32).
 template <typename T>
-__global__ void __launch_bounds__(256) linear_tiled_kernel(const T* __restrict__ x, int M, int K,
-                                                           const T* __restrict__ W, int N, Epi e,
-                                                           T* __restrict__ y, int64_t ldy) {
-  __shared__ float xs[16][64 + 1];
-  __shared__ float ws[16][64 + 1];
+__device__ __forceinline__ void tl_load4(uint32_t dst, const T* base, int r, int rows, int k, int K, bool vec) {
+  const T* src = base + (int64_t)r * K + k;
+  if constexpr (sizeof(T) == 4) {
+    if (vec) {
+      const bool ok = r < rows && k < K;
+      cp_async_16(dst, ok ? src : base, ok);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool ok = r < rows && k + j < K;
+        cp_async_4(dst + 4 * j, ok ? src + j : base, ok);
+      }
+    }
+  } else {
+    float f[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) f[j] = r < rows && k + j < K ? to_f<T>(src[j]) : 0.f;
+    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3])
+                 : "memory");
+  }
+}
+
+template <typename T, int TM, int TN, int RM, int RN, int BK>
+__global__ void __launch_bounds__(kTlThreads, 2) linear_tiled_kernel(const T* __restrict__ x, int M, int K,
+                                                                     const T* __restrict__ W, int N, Epi e,
+                                                                     T* __restrict__ y, int64_t ldy, int vec) {
+  using C = TlCfg<TM, TN, RM, RN, BK>;
+  extern __shared__ __align__(16) float tl_smem[];
+  const int tid = threadIdx.x;
+  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+  const int chunks = (K + BK - 1) / BK;
+  const uint32_t base = smem_u32(tl_smem);
+  auto load_x = [&](int c) {
+    const uint32_t st = base + (uint32_t)((c % kTlStages) * C::kStage * 4);
+#pragma unroll
+    for (int i = tid; i < TM * (BK / 4); i += kTlThreads) {
+      const int r = i / (BK / 4), q = i % (BK / 4);
+      tl_load4<T>(st + (uint32_t)(r * C::kRow + 4 * q) * 4, x, m0 + r, M, c * BK + 4 * q, K, vec);
+    }
+  };
+  auto load_w = [&](int c) {
+    const uint32_t st = base + (uint32_t)((c % kTlStages) * C::kStage * 4);
+#pragma unroll
+    for (int i = tid; i < TN * (BK / 4); i += kTlThreads) {
+      const int r = i / (BK / 4), q = i % (BK / 4);
+      tl_load4<T>(st + (uint32_t)((TM + r) * C::kRow + 4 * q) * 4, W, n0 + r, N, c * BK + 4 * q, K, vec);
+    }
+  };
+  // the weights do not depend on the kernel before
+  for (int c = 0; c < kTlStages - 1 && c < chunks; ++c) load_w(c);
   pdl_wait();
   pdl_launch_dependents();
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int i = threadIdx.x; i < 16 * 64; i += 256) {
-      const int kk = i % 16, r = i / 16;
-      const int m = m0 + r, n = n0 + r, k = k0 + kk;
-      xs[kk][r] = (m < M && k < K) ? to_f<T>(x[(int64_t)m * K + k]) : 0.f;
-      ws[kk][r] = (n < N && k < K) ? to_f<T>(W[(int64_t)n * K + k]) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = xs[kk][ty + 16 * i]; b[i] = ws[kk][tx + 16 * i]; }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
+  for (int c = 0; c < kTlStages - 1; ++c) {
+    if (c < chunks) load_x(c);
+    cp_async_commit();
   }
-  const T* bias = reinterpret_cast<const T*>(e.bias);
-  const T* res = reinterpret_cast<const T*>(e.res);
+  const int g = tid / C::kGroup, tg = tid % C::kGroup;
+  const int tm = tg % C::kCols, tn = tg / C::kCols;
+  uint64_t acc[RM][RN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 16 * i;
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j) acc[i][j] = 0ull;
+  for (int c = 0; c < chunks; ++c) {
+    cp_async_wait<kTlStages - 2>();
+    __syncthreads();  // chunk c has landed for every thread; the stage refilled below is no longer read
+    const int cn = c + kTlStages - 1;
+    if (cn < chunks) {
+      load_w(cn);
+      load_x(cn);
+    }
+    cp_async_commit();
+    const float* st = tl_smem + (c % kTlStages) * C::kStage + g * (BK / C::KG);
+#pragma unroll
+    for (int kk = 0; kk < BK / C::KG; kk += 4) {
+      ulonglong2 a[RM];
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+        a[i] = *reinterpret_cast<const ulonglong2*>(st + (tm + i * C::kCols) * C::kRow + kk);
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(st + (TM + tn + j * (TN / RN)) * C::kRow + kk);
+#pragma unroll
+        for (int i = 0; i < RM; ++i) {
+          fma2(acc[i][j], a[i].x, b.x);
+          fma2(acc[i][j], a[i].y, b.y);
+        }
+      }
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  // the groups' sums, added in group order
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j)
+      tl_smem[(g * TM + tm + i * C::kCols) * C::kPartRow + tn + j * (TN / RN)] =
+          __uint_as_float((uint32_t)acc[i][j]) + __uint_as_float((uint32_t)(acc[i][j] >> 32));
+  __syncthreads();
+  const T* bias = static_cast<const T*>(e.bias);
+  const T* res = static_cast<const T*>(e.res);
+#pragma unroll 1
+  for (int i = tid; i < TM * (TN / 4); i += kTlThreads) {
+    const int r = i / (TN / 4), q = i % (TN / 4);
+    const int m = m0 + r, n = n0 + 4 * q;
     if (m >= M) continue;
+    float4 s = *reinterpret_cast<const float4*>(tl_smem + r * C::kPartRow + 4 * q);
+#pragma unroll
+    for (int h = 1; h < C::KG; ++h) {
+      const float4 v = *reinterpret_cast<const float4*>(tl_smem + (h * TM + r) * C::kPartRow + 4 * q);
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    const float v[4] = {s.x, s.y, s.z, s.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
-      if (n >= N) continue;
-      const float rv = res ? to_f<T>(res[(int64_t)m * e.ldr + n]) : 0.f;
-      y[(int64_t)m * ldy + n] =
-          from_f<T>(epilogue(acc[i][j], bias ? to_f<T>(bias[n]) : 0.f, rv, res != nullptr, e.act, e.res_post));
+      if (n + j >= N) continue;
+      const float rv = res ? to_f<T>(res[(int64_t)m * e.ldr + n + j]) : 0.f;
+      y[(int64_t)m * ldy + n + j] =
+          from_f<T>(epilogue(v[j], bias ? to_f<T>(bias[n + j]) : 0.f, rv, res != nullptr, e.act, e.res_post));
     }
   }
+}
+
+template <typename T, int TM, int TN, int RM, int RN, int BK>
+int tiled_launch(const T* x, int M, int K, const T* W, int N, const Epi& e, T* y, int64_t ldy, int vec, cudaStream_t s) {
+  using C = TlCfg<TM, TN, RM, RN, BK>;
+  static std::atomic<uint64_t> attr_done{0};  // per instantiation, one bit per device
+  auto kern = linear_tiled_kernel<T, TM, TN, RM, RN, BK>;
+  if (attr_needed(attr_done)) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem) != cudaSuccess)
+      SN_FAIL(SWAPNET_ERR_CUDA, "cudaFuncSetAttribute failed");
+    attr_set(attr_done);
+  }
+  launch_pdl(kern, dim3((N + TN - 1) / TN, (M + TM - 1) / TM), dim3(kTlThreads), (size_t)C::kSmem, s, x, M, K, W, N, e, y,
+             ldy, vec);
+  return SWAPNET_OK;
 }
 
 // ------------------------------------------------------------ direct conv
@@ -711,13 +844,23 @@ int launch_linear_skinny(int dtype, const void* x, int M, int K, const void* W, 
   return launch_linear_skinny_job(dtype, j, s);
 }
 
-int launch_linear_tiled(int dtype, const void* x, int M, int K, const void* W, int N, const Epi& e, void* y,
+int launch_linear_tiled(int dtype, const void* x, int M, int K, const void* W, int N, int N_layer, const Epi& e, void* y,
                         int64_t ldy, cudaStream_t s) {
   if (M < 1 || K < 1 || N < 1) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "tiled linear: empty shape");
-  const dim3 grid((N + 63) / 64, (M + 63) / 64);
-  SN_DISPATCH(dtype, T,
-              launch_pdl(linear_tiled_kernel<T>, grid, dim3(256), 0, s, static_cast<const T*>(x), M, K,
-                         static_cast<const T*>(W), N, e, static_cast<T*>(y), ldy));
+  // 16-byte copies need 16-byte aligned fp32 rows
+  const int vec = dtype == SWAPNET_F32 && K % 4 == 0 && (((uintptr_t)x | (uintptr_t)W) & 15) == 0;
+  // 64 x 64 tiles once they give every SM one.  The two tiles share K out
+  // differently, so the choice follows the whole layer's width: a column
+  // piece of a layer sums each output as the whole layer would
+  const int64_t tiles = (int64_t)((M + 63) / 64) * ((N_layer + 63) / 64);
+  int rc = SWAPNET_OK;
+  SN_DISPATCH(dtype, T, {
+    const T* xt = static_cast<const T*>(x);
+    const T* wt = static_cast<const T*>(W);
+    if (tiles >= kTlWideTiles) rc = tiled_launch<T, 64, 64, 8, 4, 32>(xt, M, K, wt, N, e, static_cast<T*>(y), ldy, vec, s);
+    else rc = tiled_launch<T, 32, 32, 4, 8, 64>(xt, M, K, wt, N, e, static_cast<T*>(y), ldy, vec, s);
+  });
+  if (rc) return rc;
   return last_launch();
 }
 

@@ -81,8 +81,9 @@ struct SkJob {
 int launch_linear_skinny_job(int dtype, const SkJob& j, cudaStream_t s);
 
 // General tiled SIMT linear (any M, K, N): the fallback when neither the
-// tensor-core nor the skinny kernel applies.
-int launch_linear_tiled(int dtype, const void* x, int M, int K, const void* W, int N, const Epi& e, void* y,
+// tensor-core nor the skinny kernel applies.  N_layer: N of the whole layer
+// this is a column piece of (the tile size follows it).
+int launch_linear_tiled(int dtype, const void* x, int M, int K, const void* W, int N, int N_layer, const Epi& e, void* y,
                         int64_t ldy, cudaStream_t s);
 
 // Direct convolution (SIMT) for any channel count; NHWC in, NHWC out.

@@ -72,3 +72,32 @@ def test_paired_conv(stride, cin, cout, hw, batch):
     conv = dict(op="conv", src=[-1], cin=cin, cout=cout, kh=3, kw=3, stride=stride, pad=1, act="leaky", res=None,
                 res_post=False)
     _check([conv, dict(conv, res=0, res_post=True)], (batch, hw, hw, cin), "f16")
+
+
+@pytest.mark.parametrize("dtype,rows,k,n", [
+    ("f32", 17, 64, 33),        # one chunk, 16-byte copies
+    ("f32", 33, 1001, 129),     # rows of odd length: 4-byte copies, ragged last chunk
+    ("f32", 100, 1000, 1000),
+    ("f32", 65, 7, 31),         # K below one 4-wide step of every k group
+    ("f32", 512, 260, 1029),    # 64 x 64 tiles, all edges ragged
+    ("f32", 700, 1023, 768),
+    ("f16", 20, 1001, 70),      # 16-bit rows that neither TMA nor 16-byte loads take
+    ("bf16", 600, 333, 1100),
+])
+def test_tiled_linear(dtype, rows, k, n):
+    rs = _check([_linear(-1, k, n, "relu"), _linear(-1, k, n, "leaky", res=0, res_post=True)], (rows, 1, 1, k), dtype)
+    assert set(rs.engine.unit_kernels()) == {"tiled_linear"}
+
+
+def test_tiled_linear_pieces_sum_as_the_whole_layer():
+    """A fp32 layer split into column pieces by a small budget: same bits as the whole layer."""
+    m = dict(name="yolov3", model_id=44, dtype="f32", input=(130, 1, 1, 900), outputs=[1],
+             layers=[_linear(-1, 900, 3000, "relu"), _linear(0, 3000, 40)])
+    w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
+    host = capi.HostWeights(w)
+    sw = Runner(m, w, capi.Plan.partition(d, 4_000_000, capi.options(swap_variant=capi.SWAP_ZEROCOPY)), host)
+    rs = Runner(m, w, capi.Plan.resident(d), host)
+    assert len(sw.plan.units()) > 2
+    got = rs.run(x)
+    assert all(a.tobytes() == b.tobytes() for a, b in zip(sw.run(x), got))
+    check_close(m, rs.decode(got), oracle_outputs(m, w, x))
