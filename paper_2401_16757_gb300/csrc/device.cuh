@@ -103,28 +103,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Wait for the phase with the given parity to complete.  Polls without
-// suspending for the first iterations (short, latency-critical waits), then
-// with the suspending try_wait.  Gives up after kWaitLimitNs (or at once
-// when *abort is set by another thread), setting *abort and the global
+// Wait for the phase with the given parity to complete.  The first
+// (suspending) try_wait is the whole cost when the phase is complete or
+// about to be: 56 cycles.  (A polling loop of test_wait before it, which the
+// compiler unrolled, cost 206 cycles on a phase already complete, more than
+// a k-block's MMAs of a 64-wide tile.)  Gives up after kWaitLimitNs (or at
+// once when *abort is set by another thread), setting *abort and the global
 // error word; returns false then.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, volatile int* abort,
                                                   int* err) {
-  for (int it = 0; it < 16; ++it)
-    if (mbar_test_wait(bar, parity)) return true;
+  if (mbar_try_wait(bar, parity)) return true;
   uint64_t t0 = 0;
+#pragma unroll 1
   for (uint32_t it = 0;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 63) == 63) {

@@ -111,16 +111,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     return m0 + r < p.M ? m0 + r : -1;
   };
-  // A tile of k-block kb into stage buffer dst (TMA modes)
-  auto load_a = [&](uint32_t dst, uint32_t bar, int kb) {
-    if (TAP) {
-      const int k0 = kb * kBK, tap = k0 / p.C, c0 = k0 - tap * p.C;
-      const int ry = tap / p.kw, rx = tap - ry * p.kw;
-      tma_load_4d(dst, &tmA, bar, c0, ptw * p.wt * p.stride - p.pad + rx, pth * p.ht * p.stride - p.pad + ry, pimg);
-    } else {
-      tma_load_2d(dst, &tmA, bar, kb * kBK, m0);
-    }
-  };
   const int KB = (p.K + kBK - 1) / kBK;
   const int kb0 = blockIdx.z * p.kb_per_split;
   const int nk = min(KB, kb0 + p.kb_per_split) - kb0;  // >= 1 by construction
@@ -173,21 +163,54 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (elect_one()) {
       // ---------------- TMA producer: weight tiles of the first stages go
       // out before waiting for the previous kernel (they do not depend on it)
+      // The loop runs on one thread, whose every dependent instruction takes
+      // 4-5 cycles: with the stage and filter tap found by divisions an
+      // iteration took 300 cycles and set the pace of the whole kernel (a
+      // k-block's MMAs take 192), so everything advances by increments.
       const int early = min(nk, kStages);
+      const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
+      const uint32_t tx = kBBytes + a_bytes;
       for (int i = 0; i < early; ++i) {
-        mbar_arrive_expect_tx(full_bar(i), kBBytes + a_bytes);
-        tma_load_2d(smem_u32(sB + i * kBBytes), &tmB, full_bar(i), (kb0 + i) * kBK, n0);
+        mbar_arrive_expect_tx(full_bar(i), tx);
+        tma_load_2d(b0 + i * kBBytes, &tmB, full_bar(i), (kb0 + i) * kBK, n0);
       }
+      // the next A k-block: channel c0 of filter tap (rx, ry), whose patch
+      // starts at pixel (px + rx, py + ry)
+      int c0 = 0, rx = 0, ry = 0, px = 0, py = 0;
+      if (TAP) {
+        const int k0 = kb0 * kBK, tap = k0 / p.C;
+        c0 = k0 - tap * p.C;
+        ry = tap / p.kw;
+        rx = tap - ry * p.kw;
+        px = ptw * p.wt * p.stride - p.pad;
+        py = pth * p.ht * p.stride - p.pad;
+      }
+      auto load_a = [&](int s, int i) {
+        if (TAP) {
+          tma_load_4d(a0 + s * kABytes, &tmA, full_bar(s), c0, px + rx, py + ry, pimg);
+          c0 += kBK;
+          if (c0 == p.C) {
+            c0 = 0;
+            if (++rx == p.kw) { rx = 0; ++ry; }
+          }
+        } else {
+          tma_load_2d(a0 + s * kABytes, &tmA, full_bar(s), (kb0 + i) * kBK, m0);
+        }
+      };
       pdl_wait();
       if (!GATHER)
-        for (int i = 0; i < early; ++i) load_a(smem_u32(sA + i * kABytes), full_bar(i), kb0 + i);
-      int i = early;
+        for (int i = 0; i < early; ++i) load_a(i, i);
+      int i = early, s = 0;
+      uint32_t par = 0;
       for (; i < nk; ++i) {
-        const int s = i % kStages, r = i / kStages, kb = kb0 + i;
-        if (!mbar_wait_bounded(empty_bar(s), (r & 1) ^ 1, abort_flag, p.err)) break;
-        mbar_arrive_expect_tx(full_bar(s), kBBytes + a_bytes);
-        tma_load_2d(smem_u32(sB + s * kBBytes), &tmB, full_bar(s), kb * kBK, n0);
-        if (!GATHER) load_a(smem_u32(sA + s * kABytes), full_bar(s), kb);
+        if (!mbar_wait_bounded(empty_bar(s), par, abort_flag, p.err)) break;
+        mbar_arrive_expect_tx(full_bar(s), tx);
+        tma_load_2d(b0 + s * kBBytes, &tmB, full_bar(s), (kb0 + i) * kBK, n0);
+        if (!GATHER) load_a(s, i);
+        if (++s == kStages) {
+          s = 0;
+          par ^= 1;
+        }
       }
       if (i < nk) {
         // aborted: let the loads already issued land before the CTA exits
@@ -203,15 +226,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (elect_one()) {
       // ---------------- MMA issuer
       constexpr uint32_t idesc = idesc_f16(std::is_same<T, __nv_bfloat16>::value ? 1 : 0, kBM, BN);
+      const uint64_t ad0 = smem_desc_sw128(smem_u32(sA)), bd0 = smem_desc_sw128(smem_u32(sB));
+      uint32_t s = 0, par = 0;
       for (int i = 0; i < nk; ++i) {
-        const int s = i % kStages, r = i / kStages;
-        if (!mbar_wait_bounded(full_bar(s), r & 1, abort_flag, p.err)) break;
+        if (!mbar_wait_bounded(full_bar(s), par, abort_flag, p.err)) break;
         tc_fence_after();
-        const uint64_t ad = smem_desc_sw128(smem_u32(sA + s * kABytes));
-        const uint64_t bd = smem_desc_sw128(smem_u32(sB + s * kBBytes));
+        // the descriptors' address field counts 16 bytes
+        const uint64_t ad = ad0 + s * (uint32_t)(kABytes >> 4), bd = bd0 + s * (uint32_t)(kBBytes >> 4);
 #pragma unroll
         for (int k = 0; k < kBK / 16; ++k) tc_mma_f16(tmem, ad + 2ull * k, bd + 2ull * k, idesc, (i | k) != 0);
         tc_commit(empty_bar(s));
+        if (++s == kStages) {
+          s = 0;
+          par ^= 1;
+        }
       }
       tc_commit(accum_bar);  // fires once every MMA issued above has completed
     }

@@ -253,8 +253,9 @@ __global__ void __launch_bounds__(kQThreads, 1)
       if (elect_one()) {
         // ---------------- MMA issuer (for both CTAs)
         const uint32_t idesc = idesc_f16(std::is_same<T, __nv_bfloat16>::value ? 1 : 0, 2 * kQBM, bn);
-        int s = 0;
-        uint32_t par = 0;
+        const uint64_t ad0 = smem_desc_sw128(smem_u32(smem)), bd0 = smem_desc_sw128(smem_u32(smem) + kQA);
+        const uint32_t dstep = (uint32_t)stage_bytes >> 4;  // the descriptors' address field counts 16 bytes
+        uint32_t s = 0, par = 0;
         bool ok = true;
         for (int lt = 0; lt < my_tiles && ok; ++lt) {
           const int buf = lt & 1, use = lt >> 1;
@@ -267,12 +268,14 @@ __global__ void __launch_bounds__(kQThreads, 1)
               break;
             }
             tc_fence_after();
-            const uint64_t ad = smem_desc_sw128(smem_u32(smem) + (uint32_t)(s * stage_bytes));
-            const uint64_t bd = smem_desc_sw128(smem_u32(smem) + (uint32_t)(s * stage_bytes + kQA));
+            const uint64_t ad = ad0 + s * dstep, bd = bd0 + s * dstep;
 #pragma unroll
             for (int k = 0; k < kQBK / 16; ++k) tc2_mma_f16(d, ad + 2ull * k, bd + 2ull * k, idesc, (kb | k) != 0);
             tc2_commit(empty0 + 8u * s, 3);
-            if (++s == stages) { s = 0; par ^= 1; }
+            if (++s == (uint32_t)stages) {
+              s = 0;
+              par ^= 1;
+            }
           }
           if (ok) tc2_commit(tfull0 + 8u * buf, 3);
         }

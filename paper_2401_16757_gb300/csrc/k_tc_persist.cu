@@ -249,29 +249,34 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
     if (elect_one()) {
       // ---------------- MMA issuer
       constexpr uint32_t idesc = idesc_f16(std::is_same<T, __nv_bfloat16>::value ? 1 : 0, kPBM, BN);
-      int g = 0;
+      const uint64_t ad0 = smem_desc_sw128(smem_u32(sA)), bd0 = smem_desc_sw128(smem_u32(sB));
+      uint32_t s = 0, par = 0;
       bool ok = true;
       for (int lt = 0; lt < my_tiles && ok; ++lt) {
         const int buf = lt & 1, use = lt >> 1;
         if (!mbar_wait_bounded(tempty0 + 8u * buf, (use & 1) ^ 1, abort_flag, p.err)) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(buf * MS * BN);
-        for (int kb = 0; kb < KB; ++kb, ++g) {
-          const int s = g % kStages, r = g / kStages;
-          if (!mbar_wait_bounded(full_bar(s), r & 1, abort_flag, p.err)) {
+        for (int kb = 0; kb < KB; ++kb) {
+          if (!mbar_wait_bounded(full_bar(s), par, abort_flag, p.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint64_t bd = smem_desc_sw128(smem_u32(sB + s * Cfg::kB));
+          // the descriptors' address field counts 16 bytes
+          const uint64_t ad = ad0 + s * (uint32_t)(Cfg::kSA >> 4), bd = bd0 + s * (uint32_t)(Cfg::kB >> 4);
 #pragma unroll
           for (int sub = 0; sub < MS; ++sub) {
-            const uint64_t ad = smem_desc_sw128(smem_u32(sA + s * Cfg::kSA + sub * kPA));
 #pragma unroll
             for (int k = 0; k < kPBK / 16; ++k)
-              tc_mma_f16(d + (uint32_t)(sub * BN), ad + 2ull * k, bd + 2ull * k, idesc, (kb | k) != 0);
+              tc_mma_f16(d + (uint32_t)(sub * BN), ad + (uint64_t)(sub * (kPA >> 4)) + 2ull * k, bd + 2ull * k, idesc,
+                         (kb | k) != 0);
           }
           tc_commit(empty_bar(s));
+          if (++s == kStages) {
+            s = 0;
+            par ^= 1;
+          }
         }
         if (ok) tc_commit(tfull0 + 8u * buf);
       }
