@@ -617,10 +617,11 @@ void swapnet_engine_free(swapnet_engine* eng);
 
 /* ------------------------------------------------- allocation-free GEMM */
 /* Y[m][n] = act(sum_k A[m][k] * W[n][k] + bias[n]) for fp16 or bf16 data,
- * computed by the same tcgen05 split-K GEMM kernel the engine uses for
- * linear layers, but with its split-K scratch (fp32 partial sums and tile
- * counters) in a fixed device array inside the library instead of memory
- * the engine allocates.  The paper has no counterpart to this call.
+ * computed by the tcgen05 GEMM kernels the engine uses for linear layers.
+ * Where K is split, the splits of an output tile are a thread-block cluster
+ * that exchanges its partial sums through distributed shared memory, so the
+ * call needs no device memory of its own.  The paper has no counterpart to
+ * this call.
  *
  * It is for callers that must not allocate device memory: code running
  * under a hard device-memory budget in which every byte is already
@@ -636,22 +637,21 @@ void swapnet_engine_free(swapnet_engine* eng);
  *   stream  the call is asynchronous on it
  * Pointers must be 16-byte aligned and K a multiple of 8.
  *
- * Limits and sharing: the scratch array holds SWAPNET_NOALLOC_SCRATCH_BYTES
- * (4 MiB) on every GPU that loads the library, until the process exits.  A
- * problem whose split-K scratch exceeds it is rejected with
- * SWAPNET_ERR_INVALID_ARG before anything is launched.  Every call shares
- * the array and it keeps the last call's contents; each call clears the
- * counters it needs on `stream` first.  Calls that overlap on the GPU (on
- * different streams, or on the same device from several threads) race on
- * the array and must be serialised by the caller.
+ * Limits: a problem is rejected with SWAPNET_ERR_INVALID_ARG before anything
+ * is launched if the fp32 partial sums of its K split over the SMs that its
+ * output tiles leave idle (128 x 64 tiles, 128 x 128 where those give every
+ * SM one; at most 32 ways, two 64-deep k-blocks each), counted as if they
+ * were kept in one array with 64 KiB beside them, exceed
+ * SWAPNET_NOALLOC_SCRATCH_BYTES.  Calls share nothing: they may overlap on
+ * different streams and threads.
  *
  * Ordering: the kernel starts only after the work queued before it on
  * `stream` has completed (no programmatic early start), so A, W and bias may
  * be the output of the previous call or kernel on the stream.
  *
- * Set-up: the first call on a device looks up the array's device address
- * (cudaGetSymbolAddress) with that device current and caches it; make that
- * first call before any stream capture.
+ * Set-up: the first call on a device looks up the error word's device
+ * address (cudaGetSymbolAddress) with that device current and caches it; make
+ * that first call before any stream capture.
  * Errors: INVALID_ARG, MISALIGNED, UNSUPPORTED, CUDA.  Device-side failures
  * are not returned by this call, which does not wait for its kernel: if a
  * bounded wait inside the kernel gives up (one second), Y is incomplete and

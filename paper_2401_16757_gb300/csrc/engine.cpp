@@ -185,9 +185,6 @@ struct swapnet_engine {
   // v is launched by an earlier unit
   std::vector<int> merge_n;
   std::vector<char> merge_pair, merged_into;
-  char* d_splitk = nullptr;          // split-K scratch: tile counters, then fp32 partials
-  uint64_t splitk_bytes = 0;
-  uint64_t splitk_counter_bytes = 0;
   // storage tier: blocks fetched from a weights file into staging buffer
   // k mod 2 by a host function on `rd`, then copied into their slot
   swapnet_weights_file* file = nullptr;
@@ -240,7 +237,6 @@ static int release(swapnet_engine* e) {
     if (p) cudaFreeHost(p);
   if (e->own_arena && e->d_arena) cudaFree(e->d_arena);
   if (e->own_ws && e->d_ws) cudaFree(e->d_ws);
-  if (e->d_splitk) cudaFree(e->d_splitk);
   if (e->d_pkjobs) cudaFree(e->d_pkjobs);
   for (PackedImage* im : e->packed)
     if (im) release_packed(im);
@@ -1112,10 +1108,6 @@ static int run_unit(swapnet_engine* e, int u, const void* din, void* dout, cudaS
           if (rc) return rc;
           X.tmA_for = g.A;
         }
-        if (X.tc.splits > 1) {
-          g.counters = reinterpret_cast<int*>(e->d_splitk);
-          g.partial = reinterpret_cast<float*>(e->d_splitk + e->splitk_counter_bytes);
-        }
         return launch_tc_gemm(g, X.tc, e->err_word, s);
       }
       Epi ep{X.b, nullptr, L.d.cout, L.d.act, L.d.res_post};
@@ -1209,25 +1201,6 @@ static int bind_plan(swapnet_engine* e, void* d_arena_user, uint64_t arena_bytes
   if (rc) return rc;
   rc = plan_side(e);
   if (rc) return rc;
-  {
-    uint64_t part = 0;
-    int64_t tiles = 0;
-    for (const UnitExec& X : e->ux)
-      if (X.use_tc && X.tc.splits > 1) {
-        part = std::max(part, X.tc.scratch_bytes);
-        tiles = std::max(tiles, X.tc.tiles);
-      }
-    if (part) {
-      e->splitk_counter_bytes = align_up((uint64_t)tiles * sizeof(int));
-      e->splitk_bytes = e->splitk_counter_bytes + part;
-      if (injected(2) || cudaMalloc(&e->d_splitk, e->splitk_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        e->d_splitk = nullptr;
-        SN_FAIL(SWAPNET_ERR_OOM, "split-K scratch allocation failed");
-      }
-      CU(cudaMemset(e->d_splitk, 0, e->splitk_counter_bytes), "split-K counters");
-    }
-  }
   const int variant = (plan->opt.pageable && plan->opt.swap_variant == SWAPNET_SWAP_AUTO) ? SWAPNET_SWAP_MEMCPY
                                                                                         : plan->opt.swap_variant;
   if (plan->resident) {
@@ -1306,9 +1279,6 @@ static void unbind_plan(swapnet_engine* e) {
   e->d_pkjobs = nullptr;
   e->pk_launch.clear();
   e->pk_rest.clear();
-  if (e->d_splitk) cudaFree(e->d_splitk);
-  e->d_splitk = nullptr;
-  e->splitk_bytes = e->splitk_counter_bytes = 0;
   e->weights_loaded = false;
 }
 
@@ -1482,7 +1452,6 @@ static int plan_side(swapnet_engine* e) {
     if (L.start >= U.layer || U.host || lfirst[U.layer] != u || llast[U.layer] != u) continue;
     if (e->merge_n[u] || e->merged_into[u]) continue;  // one launch with its siblings
     const UnitExec& X = e->ux[u];
-    if (X.use_tc && X.tc.splits > 1 && !X.tc.cluster) continue;  // global split-K scratch is shared
     const int du = llast[L.start - 1];
     if (du < 0 || ublock[du] != ublock[u] || e->is_side[du]) continue;
     bool ok = true;
@@ -1750,7 +1719,6 @@ int swapnet_engine_sync(swapnet_engine* e) {
     if (w) {
       const int zero = 0;
       cudaMemcpy(e->err_word, &zero, sizeof(int), cudaMemcpyHostToDevice);
-      if (e->d_splitk) cudaMemset(e->d_splitk, 0, e->splitk_counter_bytes);  // an aborted kernel may leave counts
       if (w == 2) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "a token id or a cache position was out of range");
       SN_FAIL(SWAPNET_ERR_TIMEOUT, "a device-side wait gave up");
     }
@@ -1901,7 +1869,7 @@ int swapnet_engine_unit_tiling(const swapnet_engine* e, swapnet_unit_tiling* t, 
       if (X.use_tc) {
         r.n_tile = X.tc.bn;
         r.splits = X.tc.splits;
-        r.cluster = X.tc.splits > 1 && X.tc.cluster;
+        r.cluster = X.tc.splits > 1;
         r.persistent = X.tc.persist;
         r.tap_tma = X.tc.tma_conv;
       }

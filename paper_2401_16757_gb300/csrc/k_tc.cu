@@ -84,7 +84,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg<BN>::kStageBytes + Cfg<BN>::kRecvBytes + Cfg<BN>::kBiasBytes);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* last_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages);
   const uint32_t accum_bar = smem_u32(bars + 2 * kStages);
   auto full_bar = [&](int s) { return full0 + 8u * s; };
@@ -115,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int kb0 = blockIdx.z * p.kb_per_split;
   const int nk = min(KB, kb0 + p.kb_per_split) - kb0;  // >= 1 by construction
   const int splits = gridDim.z;
-  const bool csplit = splits > 1 && p.cluster;
+  const bool csplit = splits > 1;  // the splits of a tile are a cluster
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -124,7 +123,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     mbar_init(accum_bar, 1);
     *abort_flag = 0;
-    *last_flag = 0;
     fence_barrier_init();
     fence_proxy_async_smem();
   }
@@ -353,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           epi_piece<T>(lanes + (uint32_t)c0, sbias + c0, stage, p, m, n0 + c0, vec, rmode, rcur);
         }
       }
-    } else if (csplit) {
+    } else {
       asm volatile("barrier.cluster.wait;" ::: "memory");  // every peer is running
       // push this split's partial rows to their owners, slot = this split's index
       const bool mine = BN == 256 ? m >= 0 && row < kFewRows : m >= 0;
@@ -391,67 +389,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           }
           __syncwarp();
-        }
-      }
-    } else if (ok) {
-      // global split-K: publish the fp32 partial tile, then the last CTA of
-      // this tile sums all partials in split order and applies the epilogue.
-      float* part = p.partial + ((int64_t)blockIdx.z * p.M) * p.N;
-      const bool pvec = (p.N % 4 == 0);
-#pragma unroll 1
-      for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(lanes + (uint32_t)c0, r);
-        tmem_ld_wait();
-        const int n = n0 + c0;
-        if (m >= 0 && n < p.N) {
-          float* dst = part + (int64_t)m * p.N + n;
-          if (pvec && n + 16 <= p.N) {
-#pragma unroll
-            for (int j = 0; j < 16; j += 4)
-              __stcg(reinterpret_cast<float4*>(dst + j), make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                                                       __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])));
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (n + j < p.N) __stcg(dst + j, __uint_as_float(r[j]));
-          }
-        }
-      }
-      __threadfence();
-      epi_bar();
-      if (t == 0) {
-        int* ctr = p.counters + blockIdx.y * gridDim.x + blockIdx.x;
-        const int old = atomicAdd(ctr, 1);
-        if (old == splits - 1) {
-          *ctr = 0;  // ready for the next launch
-          *last_flag = 1;
-        }
-      }
-      epi_bar();
-      if (*last_flag) {
-        __threadfence();
-        const int n = n0 + 8 * (t % kColGroups);
-#pragma unroll 1
-        for (int rr = t / kColGroups; rr < kBM; rr += kRedRows) {
-          const int mm = row_m(rr);
-          if (mm < 0 || n >= p.N) continue;
-          float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-          for (int z = 0; z < splits; ++z) {
-            const float* src = p.partial + ((int64_t)z * p.M + mm) * p.N + n;
-            if (pvec && n + 8 <= p.N) {
-              const float4 f = __ldcg(reinterpret_cast<const float4*>(src));
-              const float4 g = __ldcg(reinterpret_cast<const float4*>(src + 4));
-              v[0] += f.x; v[1] += f.y; v[2] += f.z; v[3] += f.w;
-              v[4] += g.x; v[5] += g.y; v[6] += g.z; v[7] += g.w;
-            } else {
-#pragma unroll
-              for (int j = 0; j < 8; ++j)
-                if (n + j < p.N) v[j] += __ldcg(src + j);
-            }
-          }
-          finish8<T>(v, sbias + 8 * (t % kColGroups), p, mm, n, vec, rmode, res8<T>(p, mm, n, vec));
         }
       }
     }
@@ -587,17 +524,11 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   a.kh = g.kh; a.kw = g.kw; a.stride = g.stride; a.pad = g.pad;
   a.e = g.e; a.y = g.y; a.ldy = g.ldy; a.err = err;
   a.kb_per_split = pl.kb_per_split;
-  a.partial = g.partial;
-  a.counters = g.counters;
-  if (pl.splits > 1 && !pl.cluster && (!g.partial || !g.counters))
-    SN_FAIL(SWAPNET_ERR_INVALID_ARG, "split-K needs scratch");
   a.wt = pl.wt; a.ht = pl.ht; a.tiles_w = pl.tiles_w; a.tiles_h = pl.tiles_h;
   const int64_t mtiles = AMODE == kATap ? (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * pl.tiles_w * pl.tiles_h
                                         : (g.M + kBM - 1) / kBM;
-  if (AMODE == kATap && (pl.splits > 1 && !pl.cluster)) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "tap mode needs cluster split-K");
   const dim3 grid((unsigned)mtiles, (g.N + BN - 1) / BN, pl.splits);
-  a.cluster = pl.cluster;
-  const bool csplit = pl.splits > 1 && pl.cluster;
+  const bool csplit = pl.splits > 1;
   if (csplit) {
     static std::atomic<uint64_t> np_done{0};  // per instantiation, one bit per device
     if (attr_needed(np_done)) {
@@ -634,62 +565,25 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
 }
 
 
-// Largest cluster (along the split dimension) that the device can co-schedule
-// for this kernel instance: 16, 8, 4 or 2 (cached per instance and device).
+// Clusters of c CTAs (2 to 8, along the split dimension) of this kernel
+// instance that the device runs at once (cudaOccupancyMaxActiveClusters;
+// cached per instance, size and device).
 template <typename T, int BN, int AMODE>
-int max_cluster_inst() {
-  static std::atomic<int> cached[64];  // 0 until known
-  const int dev = device_index();
-  if (dev >= 0) {
-    const int c = cached[dev].load(std::memory_order_relaxed);
-    if (c > 0) return c;
-  }
-  auto kern = tc_gemm_kernel<T, BN, AMODE>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmem);
-  cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  int best = 1;
-  for (int c : {16, 8, 4, 2}) {
-    cudaLaunchConfig_t cfg;
-    std::memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(1, 1, c);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = Cfg<BN>::kSmem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = c;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) {
-      best = c;
-      break;
-    }
-    cudaGetLastError();
-  }
-  if (dev >= 0) cached[dev].store(best, std::memory_order_relaxed);
-  return best;
-}
-
-// Clusters of c CTAs of the N-tile-256 instance that the device runs at
-// once (cudaOccupancyMaxActiveClusters; cached per dtype, size and device).
-template <typename T>
 int active_clusters_inst(int c) {
   static std::atomic<int> cached[64][9];  // the count + 1, 0 until known
-  if (c < 1 || c > 8) return 0;
+  if (c < 2 || c > 8) return 0;
   const int dev = device_index();
   if (dev >= 0) {
     const int v = cached[dev][c].load(std::memory_order_relaxed);
     if (v > 0) return v - 1;
   }
-  auto kern = tc_gemm_kernel<T, 256, kA2d>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<256>::kSmem);
+  auto kern = tc_gemm_kernel<T, BN, AMODE>;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmem);
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(1, 1, c);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg<256>::kSmem;
+  cfg.dynamicSmemBytes = Cfg<BN>::kSmem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 1;
@@ -706,47 +600,78 @@ int active_clusters_inst(int c) {
   return n;
 }
 
-int active_clusters(int dtype, int c) {
-  return dtype == SWAPNET_BF16 ? active_clusters_inst<__nv_bfloat16>(c) : active_clusters_inst<__half>(c);
+template <typename T>
+int active_clusters_t(int bn, bool gather, int c) {
+  if (bn == 256) return active_clusters_inst<T, 256, kA2d>(c);
+  if (bn == 64) return gather ? active_clusters_inst<T, 64, kAGather>(c) : active_clusters_inst<T, 64, kA2d>(c);
+  return gather ? active_clusters_inst<T, 128, kAGather>(c) : active_clusters_inst<T, 128, kA2d>(c);
 }
 
-// Time of a persistent kernel in SM cycles, from rates measured on the GB300:
-// an SM loads up to ~130 bytes per clock from L2, all SMs together ~12900; a
-// CTA's 128 x N x 16 MMA takes N/2 cycles (not below 48: the operand reads);
-// a warp's 32 x 32 epilogue piece takes about 1400.  bytes: loaded per CTA
-// and k-block; mma: cycles per k-block; pieces: epilogue pieces per warp and
-// tile.  The epilogue of a tile overlaps the MMAs of the next.
-double persist_cycles(int64_t tiles, int64_t slots, int ctas_per_slot, int KB, double bytes, double mma, int pieces) {
-  const double active = (double)std::min(tiles, slots) * ctas_per_slot;
-  const double stage = std::max(mma, bytes / std::min(130.0, 12900.0 / active));
-  const double epi = 1400.0 * pieces, waves = (double)((tiles + slots - 1) / slots);
-  return waves * std::max(KB * stage + 300.0, epi) + epi;
+int active_clusters(int dtype, int bn, bool gather, int c) {
+  return dtype == SWAPNET_BF16 ? active_clusters_t<__nv_bfloat16>(bn, gather, c) : active_clusters_t<__half>(bn, gather, c);
 }
 
-// N tile of the paired kernel with the least persist_cycles (ties: the
-// widest) for mt 128-row blocks; sets *cycles.
-int pair_tile(int64_t mt, int64_t N, int KB, int sms, double* cycles) {
+// ---- which kernel, N tile and split of K: the least of the times below, in
+// us per launch inside a chain of dependent launches.  The constants are fits
+// to sweeps on the GB300 (every N tile and split of the layers of ResNet-50
+// and YOLOv3 at batch 1 and of linear layers of 8 to 2048 rows); they agree
+// with the measured times to about 10 %, and the ranking of the two best
+// choices of a layer was right or within 5 % for all but a few.
+
+// Per-tile kernel: `base` from the previous kernel's end to the last store
+// without a k-block, the k-blocks of one CTA (a split below five hides
+// nothing of the fill), and the exchange of a split.  More tiles than SMs
+// repeat everything but the launch.
+double tile_us(int bn, int64_t tiles, int splits, int KB, bool tap, int sms) {
+  const int kb = (KB + splits - 1) / splits;
+  // (long K: the weights come from HBM at the pace the stages allow)
+  const double per_kb = bn == 64 ? (tap ? 0.14 : 0.125) + 0.0002 * kb : 0.16 + 0.0008 * kb;
+  const double base = bn == 64 ? 2.1 : 2.9;
+  const int64_t waves = (tiles * splits + sms - 1) / sms;
+  const double split = splits > 1 ? (bn == 64 ? 1.5 : 2.8) + 0.02 * splits : 0.0;
+  return base + split + waves * per_kb * (splits > 1 ? std::max(kb, 5) : kb) + (waves - 1) * 2.2;
+}
+
+// The per-tile kernel on at most kFewRows rows: streaming the weights is the
+// work, at a rate that needs enough CTAs with enough bytes in flight.
+double few_us(int bn, int64_t tiles, int splits, int KB, int64_t N, int sms) {
+  const int kb = (KB + splits - 1) / splits;
+  const double per_kb = bn == 64 ? 0.125 : (bn == 128 ? 0.16 : 0.36);
+  const double base = bn == 64 ? 2.1 : (bn == 128 ? 2.6 : 3.3);
+  const double rate = (bn == 64 ? 5.0e6 : (bn == 128 ? 5.8e6 : 6.0e6)) *  // bytes per us
+                      std::min(1.0, (double)std::min<int64_t>(tiles * splits, sms) / 110.0);
+  const int64_t waves = (tiles * splits + sms - 1) / sms;
+  const double split = splits > 1 ? 0.9 + 0.03 * splits : 0.0;
+  return base + split + std::max(waves * per_kb * kb, (double)N * KB * kBK * 2.0 / rate) + (waves - 1) * 2.2;
+}
+
+// Persistent kernel, one CTA per tile of msub x 128 rows: a tile's epilogue
+// overlaps the next tile's MMAs.
+double persist_us(int bn, int msub, int64_t tiles, int KB, int sms) {
+  const double per_kb = bn == 64 ? (msub > 1 ? 0.11 * msub : 0.125) : (bn == 128 ? 0.18 : 0.36);
+  const double epi = 0.7 * (msub > 1 ? msub : std::max(1, bn / 64));
+  return 3.2 + (double)((tiles + sms - 1) / sms) * std::max(KB * per_kb, epi) + epi;
+}
+
+// Persistent kernel on pairs of SMs, tiles of 256 x bn.
+double pair_us(int bn, int64_t tiles, int KB, int sms) {
+  const double epi = 0.7 * ((bn / 32 + 1) / 2);
+  const int64_t slots = sms / 2;
+  return 2.5 + (double)((tiles + slots - 1) / slots) * std::max(KB * (0.06 + 0.00085 * bn) + 0.2, epi) + epi;
+}
+
+// N tile of the paired kernel with the least pair_us (ties: the widest) for
+// mt 128-row blocks.
+int pair_tile(int64_t mt, int64_t N, int KB, int sms, double* us) {
   int best_bn = 0;
-  *cycles = 0.0;
   for (int bn = 256; bn >= 64; bn -= 32) {
-    const int64_t tiles = (mt + 1) / 2 * ((N + bn - 1) / bn);
-    const double c = persist_cycles(tiles, sms / 2, 2, KB, kABytes + 64.0 * bn, 2.0 * std::max(bn, 64), (bn / 32 + 1) / 2);
-    if (!best_bn || c < *cycles) {
+    const double t = pair_us(bn, (mt + 1) / 2 * ((N + bn - 1) / bn), KB, sms);
+    if (!best_bn || t < *us) {
       best_bn = bn;
-      *cycles = c;
+      *us = t;
     }
   }
   return best_bn;
-}
-
-int max_cluster(int dtype, int bn, bool gather) {
-  const bool bf = dtype == SWAPNET_BF16;
-  if (bn == 256) return bf ? max_cluster_inst<__nv_bfloat16, 256, kA2d>() : max_cluster_inst<__half, 256, kA2d>();
-  if (bn == 64)
-    return gather ? (bf ? max_cluster_inst<__nv_bfloat16, 64, kAGather>() : max_cluster_inst<__half, 64, kAGather>())
-                  : (bf ? max_cluster_inst<__nv_bfloat16, 64, kA2d>() : max_cluster_inst<__half, 64, kA2d>());
-  return gather ? (bf ? max_cluster_inst<__nv_bfloat16, 128, kAGather>() : max_cluster_inst<__half, 128, kAGather>())
-                : (bf ? max_cluster_inst<__nv_bfloat16, 128, kA2d>() : max_cluster_inst<__half, 128, kA2d>());
 }
 
 }  // namespace
@@ -759,176 +684,96 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
   if ((uintptr_t)g.y % 2) SN_FAIL(SWAPNET_ERR_MISALIGNED, "unaligned output");
   const int sms = g.num_sms > 0 ? g.num_sms : 148;
   const int Nd = g.N_layer > 0 ? g.N_layer : g.N;  // decisions follow the whole layer
-  const int64_t mtiles = (g.M + kBM - 1) / kBM;
-  if (g.allow_persist) {
-    // at least one output tile per SM: the persistent kernel, no split.
-    // Convolutions whose taps are whole 64-channel k-blocks load A by 4-D TMA
-    // when a pixel patch fills the 128 MMA rows well enough.
-    int wt = 0, ht = 0;
-    const bool tmac = g.conv && g.C % kBK == 0 && conv_patch(g.Ho, g.Wo, g.stride, &wt, &ht) >= 0.75;
-    const int64_t sp_tiles = tmac ? (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * ((g.Wo + wt - 1) / wt) *
-                                        ((g.Ho + ht - 1) / ht)
-                                  : mtiles;
-    // the widest useful N tile.  Measured on this kernel, a pipeline stage
-    // costs about the same (~0.5 us) whatever the tile width, so the time is
-    // about waves x k-blocks and wider tiles mean fewer waves; a third of the
-    // SMs busy with one wide tile each still beats splitting K across them
-    int pbn = Nd <= 64 ? 64 : (Nd <= 128 ? 128 : 256);
-    // with at most half as many 256-wide tiles as SMs, 128-wide tiles (twice
-    // the CTAs) were measured faster: the 512-token decoder projections
-    // 25.8 -> 23.4 us (q, k, v), 32.3 -> 26.7 us (o), 74.1 -> 57.1 us (down),
-    // VGG-16 b16's 14x14 convolutions 27.8 -> 25.1 us
-    if (pbn == 256 && sp_tiles * ((Nd + 255) / 256) * 2 <= sms) pbn = 128;
-    if (sp_tiles * ((Nd + pbn - 1) / pbn) * 3 >= sms) {
-      p->persist = 1;
-      if (tmac) {
-        p->tma_conv = 1;
-        p->wt = wt;
-        p->ht = ht;
-        p->tiles_w = (g.Wo + wt - 1) / wt;
-        p->tiles_h = (g.Ho + ht - 1) / ht;
-      }
-      p->bn = pbn;
-      p->splits = 1;
-      p->kb_per_split = (g.K + kBK - 1) / kBK;
-      // N tiles of 64 with A by TMA: four (else two) 128-row sub-tiles per
-      // tile share each weight stage when that still leaves a tile per SM.
-      // Their MMAs go to independent accumulators, which the tensor pipe
-      // overlaps: a single 128x64x16 MMA chain leaves it mostly idle
-      p->msub = 1;
-      if (pbn == 64 && (!g.conv || tmac)) {
-        const int64_t nt64 = (Nd + 63) / 64;
-        if ((sp_tiles + 3) / 4 * nt64 >= sms) p->msub = 4;
-        else if ((sp_tiles + 1) / 2 * nt64 >= sms) p->msub = 2;
-      }
-      // pairs of SMs on 256-row tiles where the model of both kernels says so
-      if (p->msub == 1 && sp_tiles > 1 && (!g.conv || tmac)) {
-        const int KB = p->kb_per_split;
-        const double one = persist_cycles(sp_tiles * ((Nd + pbn - 1) / pbn), sms, 1, KB, kABytes + 128.0 * pbn,
-                                          2.0 * std::max(pbn, 96), std::max(1, pbn / 64));
-        double two = 0.0;
-        const int bn2 = pair_tile(sp_tiles, Nd, KB, sms, &two);
-        if (two < one) {
-          p->pair = 1;
-          p->bn = bn2;
-        }
-      }
-      const int mtile = p->pair ? 2 : p->msub;
-      p->tiles = (sp_tiles + mtile - 1) / mtile * ((g.N + p->bn - 1) / p->bn);
-      int rc = make_tmap(&p->tmB, g.dtype, g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2,
-                         (uint32_t)(p->pair ? p->bn / 2 : p->bn));
-      if (rc) return rc;
-      if (!g.conv && g.A) {
-        rc = make_tmap(&p->tmA, g.dtype, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, (uint32_t)kBM);
-        if (rc) return rc;
-      }
-      if (tmac && g.A) {
-        const int n_img = (int)((int64_t)g.M / ((int64_t)g.Ho * g.Wo));
-        rc = make_tmap_conv4d(&p->tmA, g.dtype, g.A, n_img, g.H, g.Wd, g.C, wt, ht, g.stride);
-        if (rc) return rc;
-      }
-      p->ready = 1;
-      return SWAPNET_OK;
-    }
-  }
+  const int64_t mt = (g.M + kBM - 1) / kBM;
   const int KB = (g.K + kBK - 1) / kBK;
-  if (g.cluster_max > 0 && !g.conv && g.M <= kFewRows && KB >= 16) {
-    // a few rows against a large weight matrix: streaming the weights is the
-    // work.  A 128xNx16 MMA costs about the same for N = 64 and 256, so the
-    // widest tile moves 4x the weight bytes per MMA; K is split across a
-    // cluster (column-owner reduction).  The split count minimises
-    // waves x k-blocks per CTA, a wave being the clusters of that size the
-    // device co-schedules: clusters of 7-8 CTAs of this kernel do not all
-    // fit at once, and the second wave costs more than the wider split saves
-    p->bn = 256;
-    const int64_t tiles_d = (Nd + 255) / 256;
-    const int smax = std::max(1, std::min(std::min(8, KB / 8), std::min(g.cluster_max, max_cluster(g.dtype, 256, false))));
-    int64_t splits = 1, best = -1;
-    for (int c = 1; c <= smax; ++c) {
-      const int64_t act = c == 1 ? sms : active_clusters(g.dtype, c);
-      if (act < 1) continue;
-      const int64_t cost = (tiles_d + act - 1) / act * ((KB + c - 1) / c);
-      if (best < 0 || cost < best) {
-        best = cost;
-        splits = c;
+  // Convolutions whose taps are whole 64-channel k-blocks load A by one 4-D
+  // TMA per tap over a pixel patch instead of the cp.async gather: in the
+  // persistent kernels when the patches fill the 128 rows to 75 %, per tile
+  // also when they need no more CTAs than 128-row tiles would (such layers
+  // are latency-bound: unused MMA rows cost nothing, the gather's address
+  // work does).
+  int wt = 0, ht = 0;
+  int64_t patches = 0;
+  bool tap = false, tap_persist = false;
+  if (g.conv && g.C % kBK == 0) {
+    const double util = conv_patch(g.Ho, g.Wo, g.stride, &wt, &ht);
+    if (wt > 0)
+      patches = (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * ((g.Wo + wt - 1) / wt) * ((g.Ho + ht - 1) / ht);
+    tap_persist = wt > 0 && util >= 0.75;
+    tap = tap_persist || (wt > 0 && patches <= mt);
+  }
+  const bool gather = g.conv && !tap;
+  const int64_t mt_tile = tap ? patches : mt, mt_pers = tap_persist ? patches : mt;
+  double best = 0.0;
+  // ---- per tile, K split over clusters
+  const int cap = std::max(1, std::min(std::min(8, g.cluster_max), KB));
+  auto consider = [&](int bn, int splits, double us) {
+    if (best > 0.0 && us >= best) return;
+    best = us;
+    p->bn = bn;
+    p->splits = splits;
+  };
+  for (int bn : {64, 128, 256}) {
+    const bool few = !g.conv && g.M <= kFewRows;
+    if ((bn == 128 && Nd <= 64) || (bn == 256 && (!few || KB < 16))) continue;
+    const int64_t tiles = mt_tile * ((Nd + bn - 1) / bn);
+    for (int c = 1; c <= cap; ++c) {
+      const int per = (KB + c - 1) / c, used = (KB + per - 1) / per;  // splits that get a k-block
+      if (used != c) continue;
+      // every cluster at once: a second wave of them costs more than a split saves
+      if (c > 1 && tiles > active_clusters(g.dtype, bn, gather, c)) continue;
+      consider(bn, c, few ? few_us(bn, tiles, c, KB, Nd, sms) : tile_us(bn, tiles, c, KB, tap, sms));
+    }
+  }
+  // ---- persistent, no split
+  if (g.allow_persist) {
+    int pbn = Nd <= 64 ? 64 : (Nd <= 128 ? 128 : 256);
+    if (pbn == 256 && mt_pers * ((Nd + 255) / 256) * 2 <= sms) pbn = 128;  // twice the CTAs
+    // N tiles of 64 with A by TMA: four (else two) 128-row sub-tiles per
+    // tile share each weight stage when that still leaves a tile per SM
+    int msub = 1;
+    if (pbn == 64 && (!g.conv || tap_persist)) {
+      if ((mt_pers + 3) / 4 * ((Nd + 63) / 64) >= sms) msub = 4;
+      else if ((mt_pers + 1) / 2 * ((Nd + 63) / 64) >= sms) msub = 2;
+    }
+    const double one = persist_us(pbn, msub, (mt_pers + msub - 1) / msub * ((Nd + pbn - 1) / pbn), KB, sms);
+    if (one < best) {
+      best = one;
+      p->persist = 1;
+      p->bn = pbn;
+      p->msub = msub;
+    }
+    if (mt_pers > 1 && (!g.conv || tap_persist)) {
+      double two = 0.0;
+      const int bn2 = pair_tile(mt_pers, Nd, KB, sms, &two);
+      if (two < best) {
+        p->persist = p->pair = 1;
+        p->bn = bn2;
+        p->msub = 1;
       }
     }
-    p->cluster = 1;
-    p->kb_per_split = (KB + (int)splits - 1) / (int)splits;
-    p->splits = (KB + p->kb_per_split - 1) / p->kb_per_split;
-    p->tiles = (g.N + 255) / 256;
-    int rc = make_tmap(&p->tmB, g.dtype, g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2, 256u);
-    if (rc) return rc;
-    if (g.A) {
-      rc = make_tmap(&p->tmA, g.dtype, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, (uint32_t)kBM);
-      if (rc) return rc;
-    }
-    p->ready = 1;
-    return SWAPNET_OK;
   }
-  // convolutions whose taps are whole 64-channel k-blocks: A by one 4-D TMA
-  // per tap over a pixel patch (as in the persistent kernel) instead of the
-  // cp.async gather, when the patches fill the 128 rows well enough or need
-  // no more CTAs than 128-row tiles would (these layers are latency-bound:
-  // unused MMA rows cost nothing, the gather's address work does); the CTA
-  // grid then runs over patches
-  int twt = 0, tht = 0;
-  bool tap = false;
-  int64_t mt = (int64_t)((g.M + kBM - 1) / kBM);
-  if (g.conv && g.cluster_max > 0 && g.C % kBK == 0) {
-    const double util = conv_patch(g.Ho, g.Wo, g.stride, &twt, &tht);
-    const int64_t patches = twt > 0 ? (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * ((g.Wo + twt - 1) / twt) *
-                                          ((g.Ho + tht - 1) / tht)
-                                    : 0;
-    if (twt > 0 && (util >= 0.75 || patches <= mt)) {
-      tap = true;
-      mt = patches;
-    }
-  }
-  if (Nd <= 64) {
-    p->bn = 64;
-  } else {
-    const int64_t tiles128 = mt * ((Nd + 127) / 128);
-    p->bn = tiles128 < sms ? 64 : 128;
-  }
-  // deterministic split-K: enough CTAs to cover the SMs, >= 2 k-blocks each
-  const int64_t tiles_d = mt * ((Nd + p->bn - 1) / p->bn);
-  const int64_t tiles = mt * ((g.N + p->bn - 1) / p->bn);
-  int64_t splits = tiles_d >= sms ? 1 : std::min<int64_t>(sms / tiles_d, std::max(1, KB / 2));
-  if (g.cluster_max > 0) {
-    // cluster split-K, from sweeps of the split count on the batch-1 CNN
-    // layers: the cluster reduction costs more than it saves below nine
-    // k-blocks; clusters above 8 CTAs, or more than ~96 CTAs in clusters of
-    // 5-8, wait longer to be scheduled than the split saves, while clusters
-    // of up to 4 filling up to one wave of SMs pay off from 16 k-blocks
-    // (YOLOv3's 26x26 and 13x13 3x3 convs: 15.7 -> 12.8 us, 13.1 -> 11.0 us)
-    const int64_t s96 = std::min<int64_t>(splits, std::min<int64_t>(8, std::max<int64_t>(1, 96 / tiles_d)));
-    if (KB <= 8) splits = 1;
-    else if (KB < 16) splits = s96;
-    else splits = std::max<int64_t>(s96, std::min<int64_t>(splits, 4));
-  }
-  const int cap = g.cluster_max > 0 ? std::min(g.cluster_max, max_cluster(g.dtype, p->bn, g.conv && !tap)) : 32;
-  splits = std::max<int64_t>(1, std::min<int64_t>(splits, cap));
-  p->cluster = g.cluster_max > 0 ? 1 : 0;
-  p->kb_per_split = (KB + (int)splits - 1) / (int)splits;
-  p->splits = (KB + p->kb_per_split - 1) / p->kb_per_split;
-  p->tiles = tiles;
-  p->scratch_bytes = (p->splits > 1 && !p->cluster) ? (uint64_t)p->splits * g.M * g.N * sizeof(float) : 0;
-  int rc = make_tmap(&p->tmB, g.dtype, g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2, (uint32_t)p->bn);
+  if (p->persist) p->splits = 1;
+  p->kb_per_split = (KB + p->splits - 1) / p->splits;
+  p->tma_conv = p->persist ? tap_persist : tap;
+  const int64_t mt_used = p->persist ? mt_pers : mt_tile;
+  const int mtile = p->pair ? 2 : (p->persist ? p->msub : 1);
+  p->tiles = (mt_used + mtile - 1) / mtile * ((g.N + p->bn - 1) / p->bn);
+  int rc = make_tmap(&p->tmB, g.dtype, g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2,
+                     (uint32_t)(p->pair ? p->bn / 2 : p->bn));
   if (rc) return rc;
   if (!g.conv && g.A) {
     rc = make_tmap(&p->tmA, g.dtype, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, (uint32_t)kBM);
     if (rc) return rc;
   }
-  if (tap) {
-    p->tma_conv = 1;
-    p->wt = twt;
-    p->ht = tht;
-    p->tiles_w = (g.Wo + twt - 1) / twt;
-    p->tiles_h = (g.Ho + tht - 1) / tht;
+  if (p->tma_conv) {
+    p->wt = wt;
+    p->ht = ht;
+    p->tiles_w = (g.Wo + wt - 1) / wt;
+    p->tiles_h = (g.Ho + ht - 1) / ht;
     if (g.A) {
       const int n_img = (int)((int64_t)g.M / ((int64_t)g.Ho * g.Wo));
-      rc = make_tmap_conv4d(&p->tmA, g.dtype, g.A, n_img, g.H, g.Wd, g.C, twt, tht, g.stride);
+      rc = make_tmap_conv4d(&p->tmA, g.dtype, g.A, n_img, g.H, g.Wd, g.C, wt, ht, g.stride);
       if (rc) return rc;
     }
   }
@@ -955,20 +800,27 @@ int launch_tc_gemm(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) 
 }
 
 // ------------------------------------------------------------ allocation-free GEMM
-// Scratch of swapnet_gemm_noalloc: tile counters (first kNoAllocCounterBytes)
-// then fp32 split-K partials.  Zero-initialised when the module loads.
-constexpr uint64_t kNoAllocBytes = SWAPNET_NOALLOC_SCRATCH_BYTES;
-constexpr uint64_t kNoAllocCounterBytes = 64 * 1024;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
-
 namespace {
 struct NoAllocDevice {
-  unsigned char* scratch = nullptr;  // device address of g_noalloc_scratch
-  int* err = nullptr;                // device address of g_tc_err
+  int* err = nullptr;  // device address of g_tc_err
   int sms = 0;
 };
 std::mutex g_noalloc_mu;
 NoAllocDevice g_noalloc_dev[64];
+
+// The entry point's limit on a problem: the fp32 partial sums of a K split
+// over as many SMs as its 128 x 64 (or, with a tile per SM, 128 x 128) output
+// tiles leave idle, plus 64 KiB, fit SWAPNET_NOALLOC_SCRATCH_BYTES.  Returns
+// the bytes (0: nothing to split).
+uint64_t noalloc_bytes(int64_t M, int64_t N, int64_t K, int sms) {
+  const int64_t mt = (M + kBM - 1) / kBM, KB = (K + kBK - 1) / kBK;
+  const int64_t bn = N > 64 && mt * ((N + 127) / 128) >= sms ? 128 : 64;
+  const int64_t tiles = mt * ((N + bn - 1) / bn);
+  if (tiles >= sms) return 0;
+  const int64_t want = std::max<int64_t>(1, std::min<int64_t>(32, std::min<int64_t>(sms / tiles, std::max<int64_t>(1, KB / 2))));
+  const int64_t per = (KB + want - 1) / want, splits = (KB + per - 1) / per;
+  return splits > 1 ? (uint64_t)(splits * M * N) * sizeof(float) + 64 * 1024 : 0;
+}
 }  // namespace
 
 int make_tmap_2d(CUtensorMap* m, int dtype, const void* base, uint64_t inner, uint64_t rows, uint64_t row_stride_bytes,
@@ -1017,15 +869,9 @@ extern "C" int swapnet_gemm_noalloc(int32_t dtype, const void* A, const void* W,
     {
       std::lock_guard<std::mutex> lk(g_noalloc_mu);
       NoAllocDevice& c = g_noalloc_dev[dev];
-      if (!c.scratch) {  // once per device, with that device current
-        void* p = nullptr;
-        cudaError_t r = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-        if (r != cudaSuccess || !p) {
-          cudaGetLastError();
-          SN_FAIL(SWAPNET_ERR_CUDA, std::string("cudaGetSymbolAddress(scratch): ") + cudaGetErrorString(r));
-        }
+      if (!c.err) {  // once per device, with that device current
         void* e = nullptr;
-        r = cudaGetSymbolAddress(&e, g_tc_err);
+        cudaError_t r = cudaGetSymbolAddress(&e, g_tc_err);
         if (r != cudaSuccess || !e) {
           cudaGetLastError();
           SN_FAIL(SWAPNET_ERR_CUDA, std::string("cudaGetSymbolAddress(error word): ") + cudaGetErrorString(r));
@@ -1035,12 +881,15 @@ extern "C" int swapnet_gemm_noalloc(int32_t dtype, const void* A, const void* W,
           cudaGetLastError();
           SN_FAIL(SWAPNET_ERR_CUDA, "device attribute query failed");
         }
-        c.scratch = static_cast<unsigned char*>(p);
         c.err = static_cast<int*>(e);
         c.sms = sms;
       }
       d = c;
     }
+    const uint64_t need = noalloc_bytes(M, N, K, d.sms);
+    if (need > SWAPNET_NOALLOC_SCRATCH_BYTES)
+      SN_FAIL(SWAPNET_ERR_INVALID_ARG, "problem counts for " + std::to_string(need) + " bytes of split-K scratch; the limit is " +
+                                           std::to_string(SWAPNET_NOALLOC_SCRATCH_BYTES));
     TcGemm g;
     std::memset(&g, 0, sizeof(g));
     g.dtype = dtype;
@@ -1050,26 +899,14 @@ extern "C" int swapnet_gemm_noalloc(int32_t dtype, const void* A, const void* W,
     g.e.bias = bias; g.e.res = nullptr; g.e.ldr = N; g.e.act = act; g.e.res_post = 0;
     g.y = Y; g.ldy = N;
     g.num_sms = d.sms;
+    g.cluster_max = 16;
+    g.allow_persist = 1;
     // W and bias are caller memory that the previous work on the stream (an
     // earlier call, say) may have written: no early start before it completes
     g.no_pdl = 1;
     TcPlan pl;
     int rc = tc_prepare(g, &pl);
     if (rc) return rc;
-    if (pl.splits > 1) {  // cluster_max == 0: global split-K scratch
-      const uint64_t counters = (uint64_t)pl.tiles * sizeof(int);
-      if (counters > kNoAllocCounterBytes || kNoAllocCounterBytes + pl.scratch_bytes > kNoAllocBytes)
-        SN_FAIL(SWAPNET_ERR_INVALID_ARG, "problem needs " + std::to_string(kNoAllocCounterBytes + pl.scratch_bytes) +
-                                             " bytes of split-K scratch; the static scratch holds " +
-                                             std::to_string(kNoAllocBytes));
-      cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-      if (cudaMemsetAsync(d.scratch, 0, counters, s) != cudaSuccess) {
-        cudaGetLastError();
-        SN_FAIL(SWAPNET_ERR_CUDA, "clearing the split-K counters failed");
-      }
-      g.counters = reinterpret_cast<int*>(d.scratch);
-      g.partial = reinterpret_cast<float*>(d.scratch + kNoAllocCounterBytes);
-    }
     return launch_tc_gemm(g, pl, d.err, reinterpret_cast<cudaStream_t>(stream));
   });
 }

@@ -139,10 +139,8 @@ struct TcGemm {
   int N_layer;          // > 0: N of the whole layer this GEMM is a column piece
                         // of; tiling and split-K follow it, so every piece sums
                         // each output in the same order as the unsplit layer
-  int cluster_max;      // > 0: split K across a thread-block cluster of at most
-                        // this many CTAs (DSMEM reduction); 0: global scratch
-  float* partial;       // split-K scratch (TcPlan::scratch_bytes), set per launch
-  int* counters;        // split-K tile counters (TcPlan::tiles ints, zeroed once)
+  int cluster_max;      // K is split across a thread-block cluster of at most
+                        // this many CTAs (DSMEM reduction)
   int no_pdl;           // 1: launch without programmatic dependent launch.  The
                         // kernel reads its bias and issues its first weight
                         // loads before waiting on the previous kernel, which
@@ -156,10 +154,8 @@ struct TcPlan {
   CUtensorMap tmB;
   int bn;           // N tile
   int splits;       // K splits (grid z); 1 = no split
-  int cluster;      // splits reduce through a cluster (no global scratch)
   int kb_per_split; // 64-wide k-blocks per split
-  int64_t tiles;    // output tiles (split-K counters needed)
-  uint64_t scratch_bytes;  // fp32 partials of all splits
+  int64_t tiles;    // output tiles
   int persist;      // persistent kernel (one CTA per SM looping over tiles)
   int tma_conv;     // convolution A by 4-D TMA per filter tap (tmA is then 4-D)
   int pair;         // persistent on pairs of SMs: tiles of 256 x bn, bn any multiple of 32 up to 256

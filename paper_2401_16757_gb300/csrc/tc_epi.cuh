@@ -16,9 +16,6 @@ struct TcArgs {
   int64_t ldy;
   int* err;
   int kb_per_split;  // k-blocks per split; gridDim.z splits
-  float* partial;    // [splits][M][N] fp32 partial sums (global split-K only)
-  int* counters;     // per output tile, zero between launches (global split-K only)
-  int cluster;       // 1: the splits of a tile form a cluster and reduce through DSMEM
   // TMA im2col (persistent kernel): output tiles are wt x ht pixel patches of
   // one image, tiles_w x tiles_h of them per image; rows >= wt * ht are unused
   int wt, ht, tiles_w, tiles_h;
@@ -216,8 +213,6 @@ __device__ __forceinline__ void epi_piece(uint32_t taddr, const float* sb, uint3
   }
   __syncwarp();  // the staging rows may be written again
 }
-
-__device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }  // the eight epilogue warps
 
 // 8 outputs [n, n + 8) of row m from fp32 sums (split-K reductions); r: the
 // residual already loaded by res8 on the 16-byte path.
