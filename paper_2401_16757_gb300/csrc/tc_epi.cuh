@@ -54,10 +54,27 @@ __device__ __forceinline__ int res_mode(const Epi& e) {
   return !e.res ? kResNone : (e.res_post ? kResPost : kResPre);
 }
 
+// r / d for d = 1 + e^-r >= 1: an approximate quotient and one Newton
+// (Markstein) correction by its remainder, within an ulp of the correctly
+// rounded one that the compiler's division gives but without its test and
+// branch per element, which kept the elements of a thread from overlapping
+// (a 32 x 32 SwiGLU piece took 5.8 us of a warp, and a 79 x 2752 x 1024 SwiGLU layer 9.9 us, 5.0 with
+// this; 4.0 without an activation).
+// The quotient is left uncorrected where it is infinite (r is) and from d =
+// 1e36 on, where r / d is below 1e-34: the remainder of infinite operands is
+// not a number.
+__device__ __forceinline__ float gate_quotient(float r, float d) {
+  float rc;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(rc) : "f"(d));
+  const float q = r * rc;
+  const float c = fmaf(fmaf(-q, d, r), rc, q);
+  return d < 1e36f && q < INFINITY ? c : q;
+}
+
 // One output element; the arithmetic of epilogue() in device.cuh.
 template <int RES>
 __device__ __forceinline__ float epi1(float acc, float bias, float r, int act) {
-  if (RES == kResGate) return r / (1.0f + expf(-r)) * (acc + bias);
+  if (RES == kResGate) return gate_quotient(r, 1.0f + expf(-r)) * (acc + bias);
   float v = acc + bias;
   if (RES == kResPre) v += r;
   const float neg = act == SWAPNET_ACT_RELU ? 0.f : (act == SWAPNET_ACT_LEAKY ? 0.1f * v : v);

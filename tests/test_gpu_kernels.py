@@ -101,3 +101,25 @@ def test_tiled_linear_pieces_sum_as_the_whole_layer():
     got = rs.run(x)
     assert all(a.tobytes() == b.tobytes() for a, b in zip(sw.run(x), got))
     check_close(m, rs.decode(got), oracle_outputs(m, w, x))
+
+
+@pytest.mark.parametrize("rows", [70, 16])
+def test_swiglu_extreme_gates(rows):
+    """Gates far out on both sides (e^-gate overflows to infinity, vanishes, stays normal) and zeros, through the
+    tensor-core epilogues: the float64 definition, to the rounding of the stored type."""
+    import numpy as np
+    import torch
+    k = 1024
+    m = dict(name="yolov3", model_id=45, dtype="bf16", input=(rows, 1, 1, k), outputs=[0, 1],
+             layers=[_linear(-1, k, k, bias=False), _linear(-1, k, k, "swiglu", res=0, bias=False)])
+    eye = torch.eye(k, dtype=torch.bfloat16).view(torch.uint16).numpy()
+    gates = torch.tensor([0.0, -0.0, 1e-30, -1e-30, 1.0, -1.0, 20.0, -20.0, 80.0, -80.0, -87.0, -88.5, -89.0, -100.0, 100.0,
+                          -300.0, 3e4, -3e4], dtype=torch.bfloat16)
+    x = gates.repeat(rows * k // gates.numel() + 1)[:rows * k].view(rows, k)
+    r = Runner(m, [[eye], [eye]], capi.Plan.resident(capi.Desc(m)))
+    gate, out = (torch.from_numpy(t.copy()).view(torch.bfloat16).double().reshape(rows, k) for t in r.run(x.view(torch.uint16).numpy()))
+    g = x.double()
+    assert torch.equal(gate, g)
+    ref = g * torch.sigmoid(g) * g
+    # one rounding to bf16 and two fp32 roundings (2^-8 + 2^-22); below 1e-33 fp32's own range ends
+    assert torch.all((out - ref).abs() <= ref.abs() * 2.0 ** -8 * 1.01 + 1e-33)
