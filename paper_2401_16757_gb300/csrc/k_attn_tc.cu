@@ -9,22 +9,30 @@
 // One CTA owns 128 queries of one head.  For each tile of 128 keys:
 //   S = Q K^T   tcgen05.mma kind::f16, M 128 (queries) x N 128 (keys) x K 128
 //               (head dims); Q and the key tile by TMA (128-byte swizzle,
-//               K-major), S in TMEM columns [0, 128)
-//   P           warps 2..5, one query row per thread: the row of S from TMEM,
-//               causal mask, running max m and denominator l, p = e^(s - m)
-//               written to shared memory as two bf16/fp16 parts p_hi + p_lo
-//               (p_lo = round(p - p_hi)), so the product with V keeps about
-//               16 significant bits of p instead of 8
+//               K-major); S in one of two TMEM buffers, so the next tile's S
+//               is computed during this tile's softmax
+//   P           warps 2..9, two threads per query row (64 keys each): the
+//               scores from TMEM into registers, causal mask (only in tiles
+//               that the diagonal or the end of the run crosses), running max
+//               m (the halves exchange theirs through shared memory) and
+//               denominator l, p = e^(s - m) written to shared memory as two
+//               bf16/fp16 parts p_hi + p_lo (p_lo = round(p - p_hi)), so the
+//               product with V keeps about 16 significant bits of p, not 8
 //   O_t = P V   tcgen05.mma, M 128 x N 128 x K 16 steps for each part; V
 //               is the value tile as loaded by TMA (two 64-dim boxes),
 //               [keys][dims] with the dims contiguous, i.e. the B operand in
-//               MN-major layout; O_t in TMEM columns [128, 256)
-//   O           the softmax warps keep the row's 128 outputs in registers:
-//               O = O * e^(m_old - m_new) + O_t
-// and at the end write O / l.  Warp 0 issues the TMA loads (key and value
-// tiles double-buffered), warp 1 owns TMEM and issues the MMAs.  Every wait
-// is bounded: on timeout the kernel records kDevErrTimeout, drains the loads
-// and MMAs it started, frees TMEM and returns.
+//               MN-major layout
+//   O           each softmax thread keeps 64 of its row's outputs in
+//               registers: O = O * e^(m_old - m_new) + O_t, added while the
+//               next tile's scores are already there
+// and at the end writes O / l.  Warp 0 issues the TMA loads (key and value
+// tiles double-buffered), warp 1 owns TMEM and issues the MMAs.  What bounds
+// it is the softmax's instruction stream, about 9 per score on eight warps;
+// 512 queries of 32 heads 24.0 us with one thread per query, the scores read
+// twice and every phase waiting for the one before, 14.5 us now; 79 queries
+// on a cache of 100, 8 heads, 14.2 -> 9.3 us (both alone, launch included).
+// Every wait is bounded: on timeout the kernel records kDevErrTimeout, drains
+// the loads and MMAs it started, frees TMEM and returns.
 #include <cudaTypedefs.h>
 
 #include <cstring>
@@ -41,19 +49,21 @@ namespace {
 constexpr int kAQ = 128;        // queries per CTA (MMA M)
 constexpr int kAK = 128;        // keys per tile
 constexpr int kAD = 128;        // head width
-constexpr int kAThreads = 192;  // warp 0 TMA, warp 1 MMA, warps 2..5 softmax
+constexpr int kASoft = 256;      // softmax threads: two per query
+constexpr int kAThreads = 64 + kASoft;  // warp 0 TMA, warp 1 MMA, warps 2..9 softmax
 constexpr int kHalf = 128 * 64 * 2;  // one 128-row x 64-column swizzled half tile (16 KB)
 constexpr int kTile = 2 * kHalf;     // 128 x 128 elements
-// shared memory: Q | K stage 0, 1 | V stage 0, 1 | P_hi | P_lo | barriers
+// shared memory: Q | K stage 0, 1 | V stage 0, 1 | P_hi | P_lo | exchange | barriers
 constexpr int kOffQ = 0;
 constexpr int kOffK = kOffQ + kTile;
 constexpr int kOffV = kOffK + 2 * kTile;
 constexpr int kOffPh = kOffV + 2 * kTile;
 constexpr int kOffPl = kOffPh + kTile;
-constexpr int kOffBar = kOffPl + kTile;
+constexpr int kOffX = kOffPl + kTile;  // [half][query] floats
+constexpr int kOffBar = kOffX + 2 * kAQ * 4;
 constexpr int kASmem = kOffBar + 128 + 1024;  // + barriers, TMEM slot, flags; + alignment slack
 static_assert(kASmem <= 232448, "attention tile set exceeds the shared memory of a CTA");
-constexpr uint32_t kTmemCols = 256;  // S: [0, 128), O_t: [128, 256)
+constexpr uint32_t kTmemCols = 512;  // S: [0, 128) and [128, 256), O_t: [256, 384)
 
 // Shared-memory descriptor of a B operand stored MN-major with the 128-byte
 // swizzle (the layout TMA gives a [K rows][64 N] box): 8-row K groups are
@@ -78,11 +88,24 @@ struct AttnArgs {
   int* err;
 };
 
-template <typename T>
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-  const T x = from_f<T>(a), y = from_f<T>(b);
-  return (uint32_t)(*reinterpret_cast<const uint16_t*>(&x)) |
-         ((uint32_t)(*reinterpret_cast<const uint16_t*>(&y)) << 16);
+template <typename T> __device__ __forceinline__ uint32_t pack2(float lo, float hi);
+template <> __device__ __forceinline__ uint32_t pack2<__half>(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+template <> __device__ __forceinline__ uint32_t pack2<__nv_bfloat16>(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+template <typename T> __device__ __forceinline__ float2 unpack2(uint32_t u);
+template <> __device__ __forceinline__ float2 unpack2<__half>(uint32_t u) {
+  return make_float2(__half2float(__ushort_as_half((unsigned short)(u & 0xffffu))),
+                     __half2float(__ushort_as_half((unsigned short)(u >> 16))));
+}
+template <> __device__ __forceinline__ float2 unpack2<__nv_bfloat16>(uint32_t u) {
+  return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
 }
 
 template <typename T>
@@ -95,12 +118,12 @@ __global__ void __launch_bounds__(kAThreads, 1)
   const uint32_t q_full = smem_u32(bars + 0);
   auto kv_full = [&](int s) { return smem_u32(bars + 1 + s); };
   auto kv_empty = [&](int s) { return smem_u32(bars + 3 + s); };
-  const uint32_t s_full = smem_u32(bars + 5);
-  const uint32_t p_full = smem_u32(bars + 6);
-  const uint32_t o_full = smem_u32(bars + 7);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 9);
-  const uint32_t done_bar = smem_u32(bars + 10);
+  auto s_full = [&](int b) { return smem_u32(bars + 5 + b); };
+  const uint32_t p_full = smem_u32(bars + 7);
+  const uint32_t o_full = smem_u32(bars + 8);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 9);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 10);
+  const uint32_t done_bar = smem_u32(bars + 11);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int t0 = blockIdx.x * kAQ, h = blockIdx.y;
@@ -110,8 +133,9 @@ __global__ void __launch_bounds__(kAThreads, 1)
       mbar_init(kv_full(s), 1);
       mbar_init(kv_empty(s), 1);
     }
-    mbar_init(s_full, 1);
-    mbar_init(p_full, 128);
+    mbar_init(s_full(0), 1);
+    mbar_init(s_full(1), 1);
+    mbar_init(p_full, kASoft);
     mbar_init(o_full, 1);
     mbar_init(done_bar, 1);
     *abort_flag = 0;
@@ -128,7 +152,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t tS = tmem, tO = tmem + 128;
+  const uint32_t tO = tmem + 256;
   // q, the caches and the position are written by the kernel before
   pdl_wait();
   pdl_launch_dependents();
@@ -167,32 +191,40 @@ __global__ void __launch_bounds__(kAThreads, 1)
       constexpr int bf = std::is_same<T, __nv_bfloat16>::value ? 1 : 0;
       constexpr uint32_t idesc_s = idesc_f16(bf, kAQ, kAK);
       constexpr uint32_t idesc_pv = idesc_f16(bf, kAQ, kAD) | (1u << 16);  // B (values) MN-major, N = 128
-      bool ok = mbar_wait_bounded(q_full, 0, abort_flag, p.err);
-      for (int kt = 0; ok && kt < nkt; ++kt) {
-        const int s = kt & 1;
-        if (!mbar_wait_bounded(kv_full(s), (kt >> 1) & 1, abort_flag, p.err)) break;
+      const uint64_t qd = smem_desc_sw128(smem_u32(smem + kOffQ)), kd = smem_desc_sw128(smem_u32(smem + kOffK));
+      const uint64_t pd[2] = {smem_desc_sw128(smem_u32(smem + kOffPh)), smem_desc_sw128(smem_u32(smem + kOffPl))};
+      const uint64_t vd = smem_desc_sw128_mn(smem_u32(smem + kOffV));
+      // scores of tile kt into TMEM buffer kt % 2 (read by the softmax of
+      // tile kt - 2, which has handed its P over by now)
+      auto scores = [&](int kt) -> bool {
+        const uint32_t b = (uint32_t)(kt & 1);
+        if (!mbar_wait_bounded(kv_full(b), (kt >> 1) & 1, abort_flag, p.err)) return false;
         tc_fence_after();
-        const uint32_t qa = smem_u32(smem + kOffQ), ka = smem_u32(smem + kOffK + s * kTile);
+        const uint64_t kb_d = kd + b * (uint32_t)(kTile >> 4);  // the descriptors' address field counts 16 bytes
 #pragma unroll
         for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            tc_mma_f16(tS, smem_desc_sw128(qa + kb * kHalf) + 2ull * k, smem_desc_sw128(ka + kb * kHalf) + 2ull * k,
+            tc_mma_f16(tmem + b * 128u, qd + (uint64_t)(kb * (kHalf >> 4) + 2 * k), kb_d + (uint64_t)(kb * (kHalf >> 4) + 2 * k),
                        idesc_s, (kb | k) != 0);
-        tc_commit(s_full);
+        tc_commit(s_full(b));
+        return true;
+      };
+      bool ok = mbar_wait_bounded(q_full, 0, abort_flag, p.err) && nkt > 0 && scores(0);
+      for (int kt = 0; ok && kt < nkt; ++kt) {
+        if (kt + 1 < nkt && !scores(kt + 1)) break;
         if (!mbar_wait_bounded(p_full, kt & 1, abort_flag, p.err)) break;
         tc_fence_after();
-        const uint32_t va = smem_u32(smem + kOffV + s * kTile);
+        const uint64_t vt = vd + (uint32_t)(kt & 1) * (uint32_t)(kTile >> 4);
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
-          const uint32_t pa = smem_u32(smem + (part ? kOffPl : kOffPh));
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)  // 16 keys per step, all 128 head dims (both 64-wide halves)
-            tc_mma_f16(tO, smem_desc_sw128(pa + (ks >> 2) * kHalf) + 2ull * (ks & 3),
-                       smem_desc_sw128_mn(va + ks * 2048), idesc_pv, (part | ks) != 0);
+            tc_mma_f16(tO, pd[part] + (uint64_t)((ks >> 2) * (kHalf >> 4) + 2 * (ks & 3)), vt + (uint64_t)(ks * (2048 >> 4)),
+                       idesc_pv, (part | ks) != 0);
         }
         tc_commit(o_full);
-        tc_commit(kv_empty(s));
+        tc_commit(kv_empty(kt & 1));
       }
       // every MMA issued must have finished before TMEM is freed (on the
       // normal path the softmax warps have already waited for the last one)
@@ -201,108 +233,121 @@ __global__ void __launch_bounds__(kAThreads, 1)
       mbar_wait_bounded(done_bar, 0, &no_abort, nullptr);
     }
   } else {
-    // ---------------- softmax and output: warps 2..5, query row per thread
-    const int q4 = warp & 3;
+    // ---------------- softmax and output: warps 2..9, half a query row per thread
+    const int q4 = warp & 3, half = (warp - 2) >> 2;
     const int row = q4 * 32 + lane;
     const int tq = t0 + row;
     // last visible key: padding rows reuse the last query's horizon; never
     // past the cache (a position beyond it is reported by the RoPE kernel)
     const int qpos = min(pos0 + min(tq, p.tokens - 1), p.max_seq - 1);
+    // horizon of the warp's first row: keys up to it are visible to all 32
+    const int qpos_min = min(pos0 + min(t0 + q4 * 32, p.tokens - 1), p.max_seq - 1);
     const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-    const uint32_t prow = (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
+    const uint32_t prow = (uint32_t)half * kHalf + (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
     const uint32_t psw = (uint32_t)(row & 7);
-    float m = -INFINITY, l = 0.f;
-    float o[kAD];
+    float* xch = reinterpret_cast<float*>(smem + kOffX);
+    // the two warps of a row quarter meet here; both take part in every
+    // tile's exchange, also after a timeout
+    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + q4) : "memory"); };
+    float m = -INFINITY, l = 0.f, alpha = 0.f;
+    float o[64];
 #pragma unroll
-    for (int d = 0; d < kAD; ++d) o[d] = 0.f;
+    for (int d = 0; d < 64; ++d) o[d] = 0.f;
     bool ok = true;
+    // O = O * alpha + O_t of tile kt (alpha: that tile's rescaling)
+    auto add_tile = [&](int kt) {
+      ok = ok && mbar_wait_bounded(o_full, kt & 1, abort_flag, p.err);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) return;
+      tc_fence_after();
+#pragma unroll
+      for (int c0 = 0; c0 < 64; c0 += 16) {
+        uint32_t r[16];
+        tmem_ld_32x32b_x16(tO + lane_off + (uint32_t)(half * 64 + c0), r);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[c0 + i] = fmaf(o[c0 + i], alpha, __uint_as_float(r[i]));
+      }
+    };
     for (int kt = 0; kt < nkt; ++kt) {
-      if (!mbar_wait_bounded(s_full, kt & 1, abort_flag, p.err)) {
-        ok = false;
-        break;
-      }
+      const int b = kt & 1, k0 = kt * kAK + half * 64;  // this thread's first key
+      ok = ok && mbar_wait_bounded(s_full(b), (kt >> 1) & 1, abort_flag, p.err);
+      ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
-      const int kbase = kt * kAK;
-      // pass 1: the row maximum over this tile's visible keys
-      float mx = m;
-#pragma unroll 1
-      for (int c0 = 0; c0 < kAK; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(tS + lane_off + (uint32_t)c0, r);
-        tmem_ld_wait();
+      uint32_t s[64];
+      float mx = -INFINITY;
+      if (ok) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (kbase + c0 + i <= qpos) mx = fmaxf(mx, __uint_as_float(r[i]));
-      }
-      const float alpha = exp2f((m - mx) * p.scale_log2);  // 0 on the first tile (m = -inf)
-      // pass 2: p = e^(s - mx), split into two parts, to shared memory
-      float lt = 0.f;
-#pragma unroll 1
-      for (int c0 = 0; c0 < kAK; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(tS + lane_off + (uint32_t)c0, r);
-        tmem_ld_wait();
-        uint32_t hi[16], lo[16];
-#pragma unroll
-        for (int i = 0; i < 32; i += 2) {
-          float pv[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const bool vis = kbase + c0 + i + u <= qpos;
-            pv[u] = vis ? exp2f((__uint_as_float(r[i + u]) - mx) * p.scale_log2) : 0.f;
-            lt += pv[u];
-          }
-          const T h0 = from_f<T>(pv[0]), h1 = from_f<T>(pv[1]);
-          hi[i / 2] = (uint32_t)(*reinterpret_cast<const uint16_t*>(&h0)) |
-                      ((uint32_t)(*reinterpret_cast<const uint16_t*>(&h1)) << 16);
-          lo[i / 2] = pack2<T>(pv[0] - to_f<T>(h0), pv[1] - to_f<T>(h1));
+        for (int c0 = 0; c0 < 64; c0 += 32) {
+          uint32_t (&r)[32] = *reinterpret_cast<uint32_t (*)[32]>(s + c0);
+          tmem_ld_32x32b_x32(tmem + (uint32_t)b * 128u + lane_off + (uint32_t)(half * 64 + c0), r);
         }
-        // keys c0..c0+31 of the row: k-block c0 / 64, 16-byte chunks (c0 % 64) / 8 + 0..3
-        const uint32_t kb = (uint32_t)(c0 >> 6), ch0 = (uint32_t)((c0 & 63) >> 3);
+        tmem_ld_wait();
+        if (k0 + 63 > qpos_min) {  // the diagonal or the run's end crosses these keys
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const uint32_t off = kb * kHalf + prow + (((ch0 + c) ^ psw) << 4);
-          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(smem_u32(smem + kOffPh) + off), "r"(hi[4 * c]),
-                       "r"(hi[4 * c + 1]), "r"(hi[4 * c + 2]), "r"(hi[4 * c + 3])
-                       : "memory");
-          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(smem_u32(smem + kOffPl) + off), "r"(lo[4 * c]),
-                       "r"(lo[4 * c + 1]), "r"(lo[4 * c + 2]), "r"(lo[4 * c + 3])
-                       : "memory");
+          for (int i = 0; i < 64; ++i)
+            if (k0 + i > qpos) s[i] = 0xff800000u;  // -inf
         }
+#pragma unroll
+        for (int i = 0; i < 64; ++i) mx = fmaxf(mx, __uint_as_float(s[i]));
       }
-      l = l * alpha + lt;
+      xch[half * kAQ + row] = mx;
+      pair_sync();
+      // key 0 is visible to every query: the maximum is finite from tile 0 on
+      mx = fmaxf(m, fmaxf(mx, xch[(half ^ 1) * kAQ + row]));
+      pair_sync();  // read by both before either writes again
+      if (kt > 0) add_tile(kt - 1);  // and P may be written again
+      alpha = exp2f((m - mx) * p.scale_log2);  // 0 on the first tile (m = -inf)
       m = mx;
-      fence_proxy_async_smem();  // P is read by the tensor cores (async proxy)
-      tc_fence_before();
-      mbar_arrive(p_full);
-      if (!mbar_wait_bounded(o_full, kt & 1, abort_flag, p.err)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
+      if (ok) {
+        float lt = 0.f;
 #pragma unroll
-      for (int c0 = 0; c0 < kAD; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(tO + lane_off + (uint32_t)c0, r);
-        tmem_ld_wait();
+        for (int c = 0; c < 8; ++c) {  // 8 keys: one 16-byte chunk of each part
+          uint32_t hi[4], lo[4];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) o[c0 + i] = fmaf(o[c0 + i], alpha, __uint_as_float(r[i]));
-      }
-      tc_fence_before();
-    }
-    if (ok && tq < p.tokens && nkt > 0) {
-      const float inv = 1.0f / l;
-      uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + (int64_t)tq * p.width + col0);
-#pragma unroll
-      for (int c = 0; c < kAD / 8; ++c) {
-        uint4 v;
-        v.x = pack2<T>(o[8 * c] * inv, o[8 * c + 1] * inv);
-        v.y = pack2<T>(o[8 * c + 2] * inv, o[8 * c + 3] * inv);
-        v.z = pack2<T>(o[8 * c + 4] * inv, o[8 * c + 5] * inv);
-        v.w = pack2<T>(o[8 * c + 6] * inv, o[8 * c + 7] * inv);
-        dst[c] = v;
+          for (int i = 0; i < 4; ++i) {
+            const float p0 = exp2f((__uint_as_float(s[8 * c + 2 * i]) - mx) * p.scale_log2);
+            const float p1 = exp2f((__uint_as_float(s[8 * c + 2 * i + 1]) - mx) * p.scale_log2);
+            lt += p0;
+            lt += p1;
+            hi[i] = pack2<T>(p0, p1);
+            const float2 h = unpack2<T>(hi[i]);
+            lo[i] = pack2<T>(p0 - h.x, p1 - h.y);
+          }
+          const uint32_t off = prow + (((uint32_t)c ^ psw) << 4);
+          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(smem_u32(smem + kOffPh) + off), "r"(hi[0]), "r"(hi[1]),
+                       "r"(hi[2]), "r"(hi[3])
+                       : "memory");
+          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(smem_u32(smem + kOffPl) + off), "r"(lo[0]), "r"(lo[1]),
+                       "r"(lo[2]), "r"(lo[3])
+                       : "memory");
+        }
+        l = l * alpha + lt;
+        fence_proxy_async_smem();  // P is read by the tensor cores (async proxy)
+        tc_fence_before();
+        mbar_arrive(p_full);
       }
     }
+    if (nkt > 0) {
+      add_tile(nkt - 1);
+      xch[half * kAQ + row] = l;
+      pair_sync();
+      const float other = xch[(half ^ 1) * kAQ + row];
+      if (ok && tq < p.tokens) {
+        const float inv = 1.0f / (half ? other + l : l + other);
+        uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + (int64_t)tq * p.width + col0 + half * 64);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          uint4 v;
+          v.x = pack2<T>(o[8 * c] * inv, o[8 * c + 1] * inv);
+          v.y = pack2<T>(o[8 * c + 2] * inv, o[8 * c + 3] * inv);
+          v.z = pack2<T>(o[8 * c + 4] * inv, o[8 * c + 5] * inv);
+          v.w = pack2<T>(o[8 * c + 6] * inv, o[8 * c + 7] * inv);
+          dst[c] = v;
+        }
+      }
+    }
+    tc_fence_before();
   }
   tc_fence_before();
   __syncthreads();
