@@ -1,4 +1,4 @@
-// Causal attention of a long query run (the decoder prefill) on the tcgen05
+// Causal attention of a run of queries (the decoder prefill) on the tcgen05
 // tensor cores, for head width 128 (fp16 / bf16 storage, fp32 arithmetic).
 //
 // Per head h, query t (position pos0 + t) attends to cache positions
@@ -405,14 +405,23 @@ int launch_t(const void* q, const void* kc, const void* vc, const int* pos_ptr, 
 
 }  // namespace
 
-bool attention_tc_supported(int dtype, int tokens, int heads, int width) {
-  return (dtype == SWAPNET_F16 || dtype == SWAPNET_BF16) && heads > 0 && width == heads * kAD && tokens >= 64;
+// Where this kernel takes over from the split-key one (a cluster of CTAs per
+// query and head), whose time grows with queries x heads x keys while this
+// one's is about 6 us and 1.5 us per 128 keys of the cache's filled part
+// (which only the device knows).  Measured, split-key against this, RoPE
+// included: 128 (query, head) pairs on a cache of 100 keys 6.2-10.7 against
+// 6.6 us, of 900 keys 24 against 18.8 us; 1024 pairs 52 against 8.8 and 339
+// against 19 us; caches of at most 128 keys 6.3 against 6.7 us at 256 pairs,
+// 9.9 against 6.8 us at 512.
+bool attention_tc_supported(int dtype, int tokens, int heads, int width, int max_seq) {
+  return (dtype == SWAPNET_F16 || dtype == SWAPNET_BF16) && heads > 0 && width == heads * kAD &&
+         (int64_t)tokens * heads >= (max_seq > kAK ? 128 : 512);
 }
 
 int launch_attention_tc(int dtype, const void* q, const void* kc, const void* vc, const int* pos_ptr, int tokens,
                         int heads, int width, int max_seq, void* out, int* err, cudaStream_t s) {
-  if (!attention_tc_supported(dtype, tokens, heads, width))
-    SN_FAIL(SWAPNET_ERR_UNSUPPORTED, "tensor-core attention: fp16/bf16, head width 128, at least 64 queries");
+  if ((dtype != SWAPNET_F16 && dtype != SWAPNET_BF16) || heads < 1 || width != heads * kAD)
+    SN_FAIL(SWAPNET_ERR_UNSUPPORTED, "tensor-core attention: fp16/bf16, head width 128");
   if (((uintptr_t)q | (uintptr_t)kc | (uintptr_t)vc | (uintptr_t)out) & 15)
     SN_FAIL(SWAPNET_ERR_MISALIGNED, "tensor-core attention: operands must be 16-byte aligned");
   if (dtype == SWAPNET_BF16)

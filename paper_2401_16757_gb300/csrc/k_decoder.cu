@@ -1,8 +1,7 @@
 // Decoder-layer kernels: embedding gather (zero-copy from the host-resident
 // table), RMSNorm, RoPE + KV-cache append, causal attention for short query
-// runs (the decode step: keys split over a thread-block cluster) and for
-// long runs the tensor cores do not take (warp per query, online softmax),
-// row argmax, and the device-side advance of the cache position.
+// runs (the decode step: keys split over a thread-block cluster), row argmax,
+// and the device-side advance of the cache position.
 // bf16 / fp16 storage, fp32 arithmetic, fixed reduction orders.
 #include <cooperative_groups.h>
 
@@ -221,10 +220,8 @@ __global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, con
 }
 
 // ------------------------------------------------------------ attention
-// Runs of at least 64 queries (the prefill) take the tcgen05 kernel
-// (k_attn_tc.cu).  Shorter runs take one of two SIMT kernels with the same
-// arithmetic definition: fewer than kRowsMinWarps (query, head) pairs (a
-// decode step) the CTA kernel, more the warp kernel.
+// Runs of many queries (the prefill) take the tcgen05 kernel (k_attn_tc.cu,
+// attention_tc_supported).
 //
 // Short query runs (a decode step): the visible keys of one (query t,
 // head h) are split into S consecutive chunks of `chunk` keys, one CTA per
@@ -251,7 +248,6 @@ constexpr int kSpThreads = 256;
 constexpr int kSpMaxSplit = 8;      // portable cluster size
 constexpr int kSpKeysPerPass = kSpThreads / 16;
 constexpr int kSpVPre = 8;          // value rows per thread requested with the keys
-constexpr int kRowsMinWarps = 1024;
 constexpr int kRopeManyHeads = 4096;  // (token, head) pairs from which a RoPE thread takes four heads
 
 struct SplitPlan {
@@ -428,59 +424,6 @@ __global__ void __launch_bounds__(kSpThreads) attention_split_kernel(const T* __
   cluster.sync();  // the first CTA has read every chunk before any CTA exits
 }
 
-// Long query runs (prefill): warp = one (query, head), each lane holding 4
-// of the 128 head dimensions; keys are visited in position order with an
-// online softmax in fp32 (m running max, l running denominator, acc running
-// numerator).  With hundreds of queries per head there are enough warps to
-// hide each warp's chain of one memory round trip per key.
-template <typename T>
-__device__ __forceinline__ void load4(const T* p, float* f) {
-  const uint2 u = *reinterpret_cast<const uint2*>(p);
-  const T* e = reinterpret_cast<const T*>(&u);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) f[j] = to_f<T>(e[j]);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) attention_rows_kernel(const T* __restrict__ q, const T* __restrict__ kc,
-                                                             const T* __restrict__ vc,
-                                                             const int* __restrict__ pos_ptr, int T_, int heads,
-                                                             int width, int max_seq, T* __restrict__ out) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= T_ * heads) return;
-  const int t = warp / heads, h = warp % heads;
-  const int n = min(*pos_ptr + t + 1, max_seq);
-  const int c0 = h * kDh + lane * 4;
-  float qv[4];
-  load4<T>(q + (int64_t)t * width + c0, qv);
-  const float scale = rsqrtf((float)kDh);
-  float m = -INFINITY, l = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int j = 0; j < n; ++j) {
-    float kv[4];
-    load4<T>(kc + (int64_t)j * width + c0, kv);
-    float s = qv[0] * kv[0] + qv[1] * kv[1] + qv[2] * kv[2] + qv[3] * kv[3];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    s *= scale;
-    const float mn = fmaxf(m, s);
-    const float a = expf(m - mn);   // 0 on the first key (m = -inf)
-    const float p = expf(s - mn);
-    float vv[4];
-    load4<T>(vc + (int64_t)j * width + c0, vv);
-    l = l * a + p;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) acc[d] = acc[d] * a + p * vv[d];
-    m = mn;
-  }
-  const float inv = 1.0f / l;
-  T* o = out + (int64_t)t * width + c0;
-#pragma unroll
-  for (int d = 0; d < 4; ++d) o[d] = from_f<T>(acc[d] * inv);
-}
-
 size_t attention_split_smem_bytes(int chunk) {
   return sizeof(float) * (16 * kDh + kDh + 2 + kSpThreads / 32 + (size_t)chunk);
 }
@@ -613,15 +556,8 @@ int launch_attention(int dtype, void* q, const void* k, const void* v, void* kc,
                              static_cast<T*>(kc), static_cast<T*>(vc), pos_ptr, heads, kDh, theta, max_seq, err),
                   "rope launch");
     if (rc) return rc;
-    if (attention_tc_supported(dtype, tokens, heads, width))  // prefill: both contractions on the tensor cores
+    if (attention_tc_supported(dtype, tokens, heads, width, max_seq))  // both contractions on the tensor cores
       return launch_attention_tc(dtype, q, kc, vc, pos_ptr, tokens, heads, width, max_seq, out, err, s);
-    if (tokens * heads >= kRowsMinWarps) {
-      const int warps = tokens * heads;
-      return done(launch_pdl(attention_rows_kernel<T>, dim3((warps * 32 + 255) / 256), dim3(256), 0, s,
-                             static_cast<const T*>(q), static_cast<const T*>(kc), static_cast<const T*>(vc),
-                             pos_ptr, tokens, heads, width, max_seq, static_cast<T*>(out)),
-                  "attention launch");
-    }
     // decode: the visible keys split over a cluster of CTAs per (query, head)
     const SplitPlan sp = split_plan(max_seq);
     const size_t smem = attention_split_smem_bytes(sp.chunk);

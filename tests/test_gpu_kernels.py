@@ -123,3 +123,48 @@ def test_swiglu_extreme_gates(rows):
     ref = g * torch.sigmoid(g) * g
     # one rounding to bf16 and two fp32 roundings (2^-8 + 2^-22); below 1e-33 fp32's own range ends
     assert torch.all((out - ref).abs() <= ref.abs() * 2.0 ** -8 * 1.01 + 1e-33)
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("tokens,heads,pos,max_seq", [
+    (1, 8, 0, 40), (1, 8, 299, 300),                    # one query: the split-key kernel, first and last position
+    (15, 8, 200, 400), (16, 8, 200, 400),               # either side of 128 (query, head) pairs
+    (63, 8, 20, 128), (64, 8, 64, 128),                 # a cache of one key tile: either side of 512 pairs
+    (128, 1, 0, 129), (129, 1, 127, 256), (130, 2, 126, 1000),  # query and key tiles full, one over
+])
+def test_attention_against_float64(dtype, tokens, heads, pos, max_seq):
+    """The attention kernels on the engine's own stored (rotated) queries and cache, against float64; and the
+    appended cache rows, the positions around them untouched."""
+    import numpy as np
+    import torch
+    td, d = (torch.float16 if dtype == "f16" else torch.bfloat16), heads * 128
+    m = dict(name="llm", model_id=46, dtype=dtype, input=(tokens, 1, 1, d), outputs=[0, 1, 2, 3],
+             layers=[_linear(-1, d, d, bias=False), _linear(-1, d, d, bias=False), _linear(-1, d, d, bias=False),
+                     dict(op="attention", src=[0, 1, 2], heads=heads, max_seq=max_seq, theta=10000.0)])
+    g = torch.Generator().manual_seed(7)
+    host = lambda t: t.view(torch.uint16).numpy() if dtype == "bf16" else t.numpy()
+    w = [[host((torch.randn((d, d), generator=g) * d ** -0.5 * s).to(td))] for s in (2.0, 2.0, 1.0)]
+    cache = torch.randn((2, max_seq, d), generator=g).to(td)
+    r = Runner(m, w, capi.Plan.resident(capi.Desc(m)))
+    state = torch.zeros(r.info["state_bytes"], dtype=torch.uint8, device="cuda")
+    state[:4].view(torch.int32).fill_(pos)
+    state[256:].view(td).view(2, max_seq, d).copy_(cache)
+    r.engine.bind_state(state.data_ptr(), r.info["state_bytes"])
+    x = torch.randn((tokens, d), generator=g).to(td)
+    q, k, v, out = (torch.from_numpy(t.copy().view(np.int16)).view(td).double().reshape(tokens, d) for t in r.run(host(x)))
+    after = state[256:].view(td).view(2, max_seq, d).cpu()
+    n = pos + tokens
+    assert torch.equal(after[:, :pos], cache[:, :pos]) and torch.equal(after[:, n:], cache[:, n:])
+    assert torch.equal(after[1, pos:n].double(), v)
+    i = torch.arange(64, dtype=torch.float64)
+    ang = torch.arange(pos, n, dtype=torch.float64)[:, None, None] * 10000.0 ** (-2.0 * i / 128)
+    a, b = k.view(tokens, heads, 64, 2).unbind(-1)
+    rot = torch.stack((a * ang.cos() - b * ang.sin(), a * ang.sin() + b * ang.cos()), -1).reshape(tokens, d)
+    # angles are fp32: their error is up to |angle| 2^-23, a few 1e-5 here, below the rounding of the stored type
+    assert torch.linalg.norm(after[0, pos:n].double() - rot) <= 2e-3 * torch.linalg.norm(rot) * (1 if dtype == "f16" else 2)
+    kk, vv = (after[j, :n].double().view(n, heads, 128).permute(1, 0, 2) for j in (0, 1))
+    s = q.view(tokens, heads, 128).permute(1, 0, 2) @ kk.transpose(1, 2) / 128 ** 0.5
+    s = s.masked_fill(torch.arange(n)[None, :] > torch.arange(pos, n)[:, None], -torch.inf)
+    ref = (torch.softmax(s, -1) @ vv).permute(1, 0, 2).reshape(tokens, d)
+    # one rounding to the stored type (relative 2^-12 and 2^-9 rms) and fp32 sums
+    assert torch.linalg.norm(out - ref) <= (4e-4 if dtype == "f16" else 2.5e-3) * torch.linalg.norm(ref)
