@@ -73,6 +73,8 @@ struct UnitExec {
   TcGemm g{};
   TcPlan tc{};
   const void* tmA_for = nullptr;  // A pointer the TMA map was encoded for
+  TcPlan tc_group{};              // first unit of a tensor-core group: the shared launch's plan
+  const void* group_for = nullptr;
   bool in_place = false;          // parameters read in mapped host memory
 };
 
@@ -939,13 +941,24 @@ static bool whole_skinny(const swapnet_engine* e, int u) {
          U.rows == e->plan.model.L[U.layer].d.cout;
 }
 
-// Merged GEMV launches (option merge): inside one block, consecutive whole
+// A whole linear layer on the tensor-core kernels, without residual and
+// without a split of K (its sums are then the same in a shared launch).
+static bool whole_tc(const swapnet_engine* e, int u) {
+  const Unit& U = e->plan.units[u];
+  const Layer& L = e->plan.model.L[U.layer];
+  const UnitExec& X = e->ux[u];
+  return e->unit_kind[u] == SWAPNET_KERNEL_TC_GEMM && L.d.op == SWAPNET_OP_LINEAR && X.use_tc && X.tc.ready &&
+         X.tc.splits == 1 && !U.host && U.row0 == 0 && U.rows == L.d.cout && L.d.res == SWAPNET_SRC_NONE;
+}
+
+// Merged launches (option merge): inside one block, consecutive whole
 // GEMV layers that read the same input with the same K and rows run as one
 // launch: up to kSkMaxSeg siblings none of which reads another's output
 // (e.g. the q, k, v projections), or a pair whose second layer takes the
 // first's output as its residual and nothing else of it (e.g. gate and up
-// of a SwiGLU feed-forward).  Results are bit-identical to separate
-// launches.
+// of a SwiGLU feed-forward).  Siblings of equal width and activation on the
+// tensor-core kernels (the q, k, v projections of a prompt) share a launch in
+// the same way.  Results are bit-identical to separate launches.
 static void plan_merges(swapnet_engine* e) {
   const swapnet_plan& p = e->plan;
   const Model& m = p.model;
@@ -956,8 +969,21 @@ static void plan_merges(swapnet_engine* e) {
   if (!p.opt.merge) return;
   for (const Block& B : p.blocks) {
     for (int u = B.u0; u < B.u1; ++u) {
-      if (!whole_skinny(e, u)) continue;
       const Layer& L0 = m.L[p.units[u].layer];
+      if (whole_tc(e, u)) {
+        int k = 1;
+        for (; k < kTcMaxSeg && u + k < B.u1 && whole_tc(e, u + k); ++k) {
+          const Layer& L = m.L[p.units[u + k].layer];
+          if (L.d.src0 != L0.d.src0 || L.d.cin != L0.d.cin || L.n != L0.n || L.d.cout != L0.d.cout || L.d.act != L0.d.act)
+            break;
+        }
+        if (k == 1) continue;
+        e->merge_n[u] = k - 1;
+        for (int i = 1; i < k; ++i) e->merged_into[u + i] = 1;
+        u += k - 1;
+        continue;
+      }
+      if (!whole_skinny(e, u)) continue;
       auto same_input = [&](int v) {
         const Layer& L = m.L[p.units[v].layer];
         return v < B.u1 && whole_skinny(e, v) && L.d.src0 == L0.d.src0 && L.d.cin == L0.d.cin && L.n == L0.n;
@@ -990,11 +1016,28 @@ static void plan_merges(swapnet_engine* e) {
   }
 }
 
-// Launch unit u with the merge_n[u] units after it as one GEMV launch.
+// Launch unit u with the merge_n[u] units after it as one launch.
 static int run_group(swapnet_engine* e, int u, const void* din, void* dout, cudaStream_t s) {
   const swapnet_plan& p = e->plan;
   const Model& m = p.model;
   const Layer& L0 = m.L[p.units[u].layer];
+  if (e->unit_kind[u] == SWAPNET_KERNEL_TC_GEMM) {
+    UnitExec& X = e->ux[u];
+    TcGemm g;
+    unit_gemm(e, p.units[u], X, act_ptr(e, L0.d.src0, din, dout), nullptr, out_ptr(e, p.units[u].layer, dout), &g);
+    g.nseg = 1 + e->merge_n[u];
+    for (int i = 1; i < g.nseg; ++i) {
+      g.Wx[i - 1] = e->ux[u + i].w;
+      g.bx[i - 1] = e->ux[u + i].b;
+      g.yx[i - 1] = out_ptr(e, p.units[u + i].layer, dout);
+    }
+    if (!X.tc_group.ready || X.group_for != g.A) {
+      const int rc = tc_prepare(g, &X.tc_group);
+      if (rc) return rc;
+      X.group_for = g.A;
+    }
+    return launch_tc_gemm(g, X.tc_group, e->err_word, s);
+  }
   SkJob j{};
   j.x = act_ptr(e, L0.d.src0, din, dout);
   j.M = L0.n;

@@ -67,9 +67,10 @@ template <int BN> struct Cfg {
 // for the padding; the CTA's 128 rows are that patch, rows >= wt * ht unused)
 constexpr int kA2d = 0, kAGather = 1, kATap = 2;
 
-template <typename T, int BN, int AMODE>
+// NS: layers that a launch may hold (1, or kTcMaxSeg siblings)
+template <typename T, int BN, int AMODE, int NS>
 __global__ void __launch_bounds__(kThreads, 1)
-    tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs p) {
+    tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ TcSegs<NS> sg, const TcArgs p) {
   constexpr bool GATHER = AMODE == kAGather;
   constexpr bool TAP = AMODE == kATap;
   constexpr int kStages = Cfg<BN>::kStages;
@@ -90,7 +91,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   auto empty_bar = [&](int s) { return empty0 + 8u * s; };
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int m0 = TAP ? 0 : blockIdx.x * kBM, n0 = blockIdx.y * BN;
+  const int m0 = TAP ? 0 : blockIdx.x * kBM;
+  int seg = 0, n0 = (int)blockIdx.y * BN;
+  if constexpr (NS > 1) {
+    const int nt = (p.N + BN - 1) / BN;
+    seg = (int)blockIdx.y / nt;
+    n0 -= seg * nt * BN;
+  }
+  const CUtensorMap* tmB = &sg.m[seg];
   // tap mode: this CTA's patch (image, patch row th, patch column tw)
   int pimg = 0, pth = 0, ptw = 0;
   if (TAP) {
@@ -131,12 +139,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish();
   }
   if (threadIdx.x == 0) {
-    prefetch_tmap(&tmB);
+    prefetch_tmap(tmB);
     if (!GATHER) prefetch_tmap(&tmA);
   }
   // bias of this tile to shared memory (weights: ready before the kernel)
   if (threadIdx.x >= 64) {
-    const T* bias = static_cast<const T*>(p.e.bias);
+    const T* bias = seg_bias<T>(p, sg, seg);
     for (int j = threadIdx.x - 64; j < BN; j += kEpiThreads) sbias[j] = (bias && n0 + j < p.N) ? to_f<T>(bias[n0 + j]) : 0.f;
   }
   tc_fence_before();
@@ -146,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_launch_dependents();
   if (csplit) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");  // peers started (waited before DSMEM use)
 
-  const bool vec = epi_vec_ok(p);
+  const bool vec = epi_vec_ok(p, seg_y<T>(p, sg, seg));
   const int rmode = res_mode(p.e);
   // cluster split-K: what epilogue thread t sums after the exchange, and its
   // residual, requested while the MMAs run.  BN 64/128: 8 columns of up to
@@ -170,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t tx = kBBytes + a_bytes;
       for (int i = 0; i < early; ++i) {
         mbar_arrive_expect_tx(full_bar(i), tx);
-        tma_load_2d(b0 + i * kBBytes, &tmB, full_bar(i), (kb0 + i) * kBK, n0);
+        tma_load_2d(b0 + i * kBBytes, tmB, full_bar(i), (kb0 + i) * kBK, n0);
       }
       // the next A k-block: channel c0 of filter tap (rx, ry), whose patch
       // starts at pixel (px + rx, py + ry)
@@ -203,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (; i < nk; ++i) {
         if (!mbar_wait_bounded(empty_bar(s), par, abort_flag, p.err)) break;
         mbar_arrive_expect_tx(full_bar(s), tx);
-        tma_load_2d(b0 + s * kBBytes, &tmB, full_bar(s), (kb0 + i) * kBK, n0);
+        tma_load_2d(b0 + s * kBBytes, tmB, full_bar(s), (kb0 + i) * kBK, n0);
         if (!GATHER) load_a(s, i);
         if (++s == kStages) {
           s = 0;
@@ -348,7 +356,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int i = 0; i < 4; ++i) rcur[i] = rnext[i];
           if (c0 + 32 < c_hi) epi_res_load<T>(rnext, p, m, n0 + c0 + 32, vec);
-          epi_piece<T>(lanes + (uint32_t)c0, sbias + c0, stage, p, m, n0 + c0, vec, rmode, rcur);
+          epi_piece<T>(lanes + (uint32_t)c0, sbias + c0, stage, p, seg_y<T>(p, sg, seg), m, n0 + c0, vec, rmode,
+                       rcur);
         }
       }
     } else {
@@ -420,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           a1.x += g.x; a1.y += g.y; a1.z += g.z; a1.w += g.w;
         }
         const float v[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        finish8<T>(v, sbias + c_own + c8, p, red_m[j], n, vec, rmode, red_res[j]);
+        finish8<T>(v, sbias + c_own + c8, p, seg_y<T>(p, sg, seg), red_m[j], n, vec, rmode, red_res[j]);
       }
     }
   }
@@ -507,10 +516,10 @@ double conv_patch(int ho, int wo, int stride, int* wt, int* ht) {
   return best;
 }
 
-template <typename T, int BN, int AMODE>
+template <typename T, int BN, int AMODE, int NS = 1>
 int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   static std::atomic<uint64_t> attr_done{0};  // per instantiation, one bit per device
-  auto kern = tc_gemm_kernel<T, BN, AMODE>;
+  auto kern = tc_gemm_kernel<T, BN, AMODE, NS>;
   if (attr_needed(attr_done)) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmem) != cudaSuccess)
       SN_FAIL(SWAPNET_ERR_CUDA, "cudaFuncSetAttribute failed");
@@ -527,7 +536,7 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   a.wt = pl.wt; a.ht = pl.ht; a.tiles_w = pl.tiles_w; a.tiles_h = pl.tiles_h;
   const int64_t mtiles = AMODE == kATap ? (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * pl.tiles_w * pl.tiles_h
                                         : (g.M + kBM - 1) / kBM;
-  const dim3 grid((unsigned)mtiles, (g.N + BN - 1) / BN, pl.splits);
+  const dim3 grid((unsigned)mtiles, (g.N + BN - 1) / BN * std::max(1, g.nseg), pl.splits);
   const bool csplit = pl.splits > 1;
   if (csplit) {
     static std::atomic<uint64_t> np_done{0};  // per instantiation, one bit per device
@@ -559,7 +568,7 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, pl.tmA, pl.tmB, a);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, pl.tmA, make_segs<NS>(g, pl), a);
   if (le != cudaSuccess) SN_FAIL(SWAPNET_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(le));
   return SWAPNET_OK;
 }
@@ -577,7 +586,7 @@ int active_clusters_inst(int c) {
     const int v = cached[dev][c].load(std::memory_order_relaxed);
     if (v > 0) return v - 1;
   }
-  auto kern = tc_gemm_kernel<T, BN, AMODE>;
+  auto kern = tc_gemm_kernel<T, BN, AMODE, 1>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmem);
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
@@ -661,11 +670,11 @@ double pair_us(int bn, int64_t tiles, int KB, int sms) {
 }
 
 // N tile of the paired kernel with the least pair_us (ties: the widest) for
-// mt 128-row blocks.
-int pair_tile(int64_t mt, int64_t N, int KB, int sms, double* us) {
+// mt 128-row blocks and nseg segments of N columns.
+int pair_tile(int64_t mt, int64_t N, int nseg, int KB, int sms, double* us) {
   int best_bn = 0;
   for (int bn = 256; bn >= 64; bn -= 32) {
-    const double t = pair_us(bn, (mt + 1) / 2 * ((N + bn - 1) / bn), KB, sms);
+    const double t = pair_us(bn, (mt + 1) / 2 * ((N + bn - 1) / bn) * nseg, KB, sms);
     if (!best_bn || t < *us) {
       best_bn = bn;
       *us = t;
@@ -703,6 +712,8 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
     tap = tap_persist || (wt > 0 && patches <= mt);
   }
   const bool gather = g.conv && !tap;
+  const int nseg = std::max(1, g.nseg);
+  if (nseg > kTcMaxSeg || (nseg > 1 && (g.conv || g.e.res))) SN_FAIL(SWAPNET_ERR_UNSUPPORTED, "segments: linear layers without residual");
   const int64_t mt_tile = tap ? patches : mt, mt_pers = tap_persist ? patches : mt;
   double best = 0.0;
   // ---- per tile, K split over clusters
@@ -715,9 +726,10 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
   };
   for (int bn : {64, 128, 256}) {
     const bool few = !g.conv && g.M <= kFewRows;
-    if ((bn == 128 && Nd <= 64) || (bn == 256 && (!few || KB < 16))) continue;
-    const int64_t tiles = mt_tile * ((Nd + bn - 1) / bn);
-    for (int c = 1; c <= cap; ++c) {
+    if ((bn == 128 && Nd <= 64) || (bn == 256 && (!few || KB < 16 || nseg > 1))) continue;
+    const int64_t tiles = mt_tile * ((Nd + bn - 1) / bn) * nseg;
+    // segments: an unsplit sum, as each layer's own launch makes it
+    for (int c = 1; c <= (nseg > 1 ? 1 : cap); ++c) {
       const int per = (KB + c - 1) / c, used = (KB + per - 1) / per;  // splits that get a k-block
       if (used != c) continue;
       // every cluster at once: a second wave of them costs more than a split saves
@@ -737,7 +749,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
       else if ((mt_pers + 1) / 2 * ((Nd + 63) / 64) >= sms) msub = 2;
     }
     const double one = persist_us(pbn, msub, (mt_pers + msub - 1) / msub * ((Nd + pbn - 1) / pbn), KB, sms);
-    if (one < best) {
+    if (one < best && nseg == 1) {
       best = one;
       p->persist = 1;
       p->bn = pbn;
@@ -745,7 +757,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
     }
     if (mt_pers > 1 && (!g.conv || tap_persist)) {
       double two = 0.0;
-      const int bn2 = pair_tile(mt_pers, Nd, KB, sms, &two);
+      const int bn2 = pair_tile(mt_pers, Nd, nseg, KB, sms, &two);
       if (two < best) {
         p->persist = p->pair = 1;
         p->bn = bn2;
@@ -758,9 +770,11 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
   p->tma_conv = p->persist ? tap_persist : tap;
   const int64_t mt_used = p->persist ? mt_pers : mt_tile;
   const int mtile = p->pair ? 2 : (p->persist ? p->msub : 1);
-  p->tiles = (mt_used + mtile - 1) / mtile * ((g.N + p->bn - 1) / p->bn);
-  int rc = make_tmap(&p->tmB, g.dtype, g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2,
-                     (uint32_t)(p->pair ? p->bn / 2 : p->bn));
+  p->tiles = (mt_used + mtile - 1) / mtile * ((g.N + p->bn - 1) / p->bn) * nseg;
+  int rc = SWAPNET_OK;
+  for (int i = 0; i < nseg && !rc; ++i)
+    rc = make_tmap(&p->tmB[i], g.dtype, i ? g.Wx[i - 1] : g.W, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.K * 2,
+                   (uint32_t)(p->pair ? p->bn / 2 : p->bn));
   if (rc) return rc;
   if (!g.conv && g.A) {
     rc = make_tmap(&p->tmA, g.dtype, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, (uint32_t)kBM);
@@ -786,6 +800,11 @@ int launch_tc_gemm(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) 
   if (pl.pair) return launch_tc_pair(g, pl, err, s);
   if (pl.persist) return launch_tc_persist(g, pl, err, s);
   const bool bf = g.dtype == SWAPNET_BF16;
+  if (g.nseg > 1) {
+    if (pl.bn == 64)
+      return bf ? launch_inst<__nv_bfloat16, 64, kA2d, kTcMaxSeg>(g, pl, err, s) : launch_inst<__half, 64, kA2d, kTcMaxSeg>(g, pl, err, s);
+    return bf ? launch_inst<__nv_bfloat16, 128, kA2d, kTcMaxSeg>(g, pl, err, s) : launch_inst<__half, 128, kA2d, kTcMaxSeg>(g, pl, err, s);
+  }
   if (g.conv && pl.tma_conv) {
     if (pl.bn == 64) return bf ? launch_inst<__nv_bfloat16, 64, kATap>(g, pl, err, s) : launch_inst<__half, 64, kATap>(g, pl, err, s);
     return bf ? launch_inst<__nv_bfloat16, 128, kATap>(g, pl, err, s) : launch_inst<__half, 128, kATap>(g, pl, err, s);

@@ -107,9 +107,11 @@ __device__ __forceinline__ void tc2_commit(uint32_t bar, uint16_t mask) {
       : "memory");
 }
 
-template <typename T, int AMODE>  // AMODE: kPair2d or kPairTap
+// AMODE: 0 (row-major A) or 1 (convolution, A by filter tap); NS: layers that a
+// launch may hold (1, or kTcMaxSeg siblings)
+template <typename T, int AMODE, int NS>
 __global__ void __launch_bounds__(kQThreads, 1)
-    tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs p,
+    tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ TcSegs<NS> sg, const TcArgs p,
                    const int bn, const int stages) {
   constexpr bool TAP = AMODE == 1;
   extern __shared__ uint8_t smem_raw[];
@@ -131,9 +133,11 @@ __global__ void __launch_bounds__(kQThreads, 1)
   const int patches = p.tiles_w * p.tiles_h;
   // 128-row blocks of the output matrix, or pixel patches
   const int mt = TAP ? (p.M / (p.Ho * p.Wo)) * patches : (p.M + kQBM - 1) / kQBM;
-  const int nt = (p.N + bn - 1) / bn;
+  const int nt = (p.N + bn - 1) / bn;  // n-tiles per segment
   const int mtp = (mt + 1) / 2;
-  const int tiles = mtp * nt;
+  int nseg = 1;
+  if constexpr (NS > 1) nseg = sg.nseg;
+  const int tiles = mtp * nt * nseg;
   const int KB = (p.K + kQBK - 1) / kQBK;
   const int my_tiles = pair < tiles ? (tiles - 1 - pair) / pairs + 1 : 0;
   const int work = my_tiles * KB;
@@ -153,7 +157,7 @@ __global__ void __launch_bounds__(kQThreads, 1)
     *abort_flag = 0;
     fence_barrier_init();
     fence_proxy_async_smem();
-    prefetch_tmap(&tmB);
+    for (int i = 0; i < nseg; ++i) prefetch_tmap(&sg.m[i]);
     prefetch_tmap(&tmA);
   }
   if (warp == 1) {
@@ -177,9 +181,12 @@ __global__ void __launch_bounds__(kQThreads, 1)
       const uint32_t lfull0 = map_rank(full0, 0);
       const uint32_t tx = 2 * (a_bytes + (uint32_t)b_bytes);  // both CTAs' bytes of a stage
       int n0 = 0, ay = 0, az = 0, aw = 0;
+      const CUtensorMap* tmB = &sg.m[0];
       auto start_tile = [&](int lt) {
         const int tile = tile_of(lt);
-        n0 = (tile / mtp) * bn + rank * (bn / 2);
+        const int ntile = tile / mtp, seg = NS > 1 ? ntile / nt : 0;
+        tmB = &sg.m[seg];
+        n0 = (ntile - seg * nt) * bn + rank * (bn / 2);
         const int idx = (tile % mtp) * 2 + rank;  // past the last one: only out-of-range coordinates (zero fill)
         if (TAP) {
           const int img = idx / patches, rem = idx - img * patches;
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(kQThreads, 1)
       };
       auto load_b = [&](int s) {
         if (rank == 0) mbar_arrive_expect_tx(full0 + 8u * s, tx);
-        tma2_load_2d(smem_u32(smem) + (uint32_t)(s * stage_bytes + kQA), &tmB, lfull0 + 8u * s, kb * kQBK, n0);
+        tma2_load_2d(smem_u32(smem) + (uint32_t)(s * stage_bytes + kQA), tmB, lfull0 + 8u * s, kb * kQBK, n0);
       };
       auto load_a = [&](int s) {
         const uint32_t dst = smem_u32(smem) + (uint32_t)(s * stage_bytes);
@@ -295,13 +302,15 @@ __global__ void __launch_bounds__(kQThreads, 1)
     float* sb = sbias + (warp - 2) * 128;                    // its own copy of their bias: no cross-warp barrier
     const uint32_t stage = smem_u32(staging) + (uint32_t)((warp - 2) * kEpiStage);
     const uint32_t ltempty0 = map_rank(tempty0, 0);
-    const bool vec = epi_vec_ok(p);
     const int rmode = res_mode(p.e);
     for (int lt = 0; lt < my_tiles; ++lt) {
       const int buf = lt & 1, use = lt >> 1;
       const int tile = tile_of(lt);
-      const int n0 = (tile / mtp) * bn + c_lo;
-      const T* bias = static_cast<const T*>(p.e.bias);
+      const int ntile = tile / mtp, seg = NS > 1 ? ntile / nt : 0;
+      const int n0 = (ntile - seg * nt) * bn + c_lo;
+      T* const y = seg_y<T>(p, sg, seg);
+      const bool vec = epi_vec_ok(p, y);
+      const T* bias = seg_bias<T>(p, sg, seg);
       for (int j = lane; j < cols; j += 32) sb[j] = (bias && n0 + j < p.N) ? to_f<T>(bias[n0 + j]) : 0.f;
       __syncwarp();
       const int idx = (tile % mtp) * 2 + rank;
@@ -330,7 +339,7 @@ __global__ void __launch_bounds__(kQThreads, 1)
 #pragma unroll
         for (int i = 0; i < 4; ++i) rcur[i] = rnext[i];
         if (c + 32 < cols) epi_res_load<T>(rnext, p, m, n0 + c + 32, vec);
-        epi_piece<T>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + c_lo + c), sb + c, stage, p, m, n0 + c,
+        epi_piece<T>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + c_lo + c), sb + c, stage, p, y, m, n0 + c,
                      vec, rmode, rcur);
       }
       tc_fence_before();
@@ -348,10 +357,10 @@ __global__ void __launch_bounds__(kQThreads, 1)
   }
 }
 
-template <typename T, int AMODE>
+template <typename T, int AMODE, int NS = 1>
 int launch_pair_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   static std::atomic<uint64_t> attr_done{0};  // per instantiation, one bit per device
-  auto kern = tc_pair_kernel<T, AMODE>;
+  auto kern = tc_pair_kernel<T, AMODE, NS>;
   if (attr_needed(attr_done)) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kQSmem) != cudaSuccess)
       SN_FAIL(SWAPNET_ERR_CUDA, "cudaFuncSetAttribute failed");
@@ -381,7 +390,7 @@ int launch_pair_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = g.no_pdl ? 1 : 2;
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, pl.tmA, pl.tmB, a, (int)pl.bn, stages);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, pl.tmA, make_segs<NS>(g, pl), a, (int)pl.bn, stages);
   if (le != cudaSuccess) SN_FAIL(SWAPNET_ERR_CUDA, std::string("paired GEMM launch: ") + cudaGetErrorString(le));
   return SWAPNET_OK;
 }
@@ -391,6 +400,9 @@ int launch_pair_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s
 int launch_tc_pair(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   if (pl.bn < 32 || pl.bn > 256 || pl.bn % 32 || (g.conv && !pl.tma_conv))
     SN_FAIL(SWAPNET_ERR_INVALID_ARG, "paired GEMM: bad tile");
+  if (g.nseg > 1)
+    return g.dtype == SWAPNET_BF16 ? launch_pair_inst<__nv_bfloat16, 0, kTcMaxSeg>(g, pl, err, s)
+                                   : launch_pair_inst<__half, 0, kTcMaxSeg>(g, pl, err, s);
   if (g.dtype == SWAPNET_BF16)
     return g.conv ? launch_pair_inst<__nv_bfloat16, 1>(g, pl, err, s) : launch_pair_inst<__nv_bfloat16, 0>(g, pl, err, s);
   return g.conv ? launch_pair_inst<__half, 1>(g, pl, err, s) : launch_pair_inst<__half, 0>(g, pl, err, s);

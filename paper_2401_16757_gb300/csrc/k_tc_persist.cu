@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
     const int c_lo = (warp - 2) / 4 * Cfg::kCols;  // this warp's columns
     float* sb = sbias + (warp - 2) * Cfg::kCols;   // its own copy of their bias: no cross-warp barrier
     const uint32_t stage = smem_u32(staging) + (uint32_t)((warp - 2) * kEpiStage);
-    const bool vec = epi_vec_ok(p);
+    const bool vec = epi_vec_ok(p, p.y);
     const int rmode = res_mode(p.e);
     for (int lt = 0; lt < my_tiles; ++lt) {
       const int buf = lt & 1, use = lt >> 1;
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
           else if (sub + 1 < MS) epi_res_load<T>(rnext, p, m_next, n0, vec);
           if (n0 + c0 < p.N)
             epi_piece<T>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((buf * MS + sub) * BN + c_lo + c0), sb + c0, stage,
-                         p, m, n0 + c0, vec, rmode, rcur);
+                         p, static_cast<T*>(p.y), m, n0 + c0, vec, rmode, rcur);
         }
         m = m_next;
       }
@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
 
 template <typename T, int BN, int AMODE, int MS>
 int launch_persist_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
+  if (g.nseg > 1) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "persistent GEMM: one layer per launch");
   static std::atomic<uint64_t> attr_done{0};  // per instantiation, one bit per device
   auto kern = tc_persist_kernel<T, BN, AMODE, MS>;
   if (attr_needed(attr_done)) {
@@ -461,7 +462,7 @@ int launch_persist_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = g.no_pdl ? 0 : 1;
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, pl.tmA, pl.tmB, a);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, pl.tmA, pl.tmB[0], a);
   if (le != cudaSuccess) SN_FAIL(SWAPNET_ERR_CUDA, std::string("persistent GEMM launch: ") + cudaGetErrorString(le));
   return SWAPNET_OK;
 }

@@ -120,7 +120,16 @@ struct ZcSeg {
 int launch_zerocopy(const ZcSeg* segs, int nseg, int ctas, cudaStream_t s);
 
 // tcgen05 GEMM / implicit-GEMM convolution (fp16 or bf16, fp32 accumulate).
+//
+// Sibling linear layers that read the same A with the same K, N, activation
+// and no residual (e.g. the q, k, v projections) may share a launch: nseg of
+// them, segment i > 0 with weights, bias and output in Wx / bx / yx[i - 1].
+constexpr int kTcMaxSeg = 3;
 struct TcGemm {
+  int nseg;           // 0 or 1: one layer
+  const void* Wx[kTcMaxSeg - 1];
+  const void* bx[kTcMaxSeg - 1];
+  void* yx[kTcMaxSeg - 1];
   int dtype;          // SWAPNET_F16 or SWAPNET_BF16
   int M, N, K;
   // B operand: weights [N][K] row-major (K contiguous)
@@ -151,7 +160,7 @@ struct TcGemm {
 // Pre-encoded descriptors of one GEMM (built once per layer at load time).
 struct TcPlan {
   CUtensorMap tmA;  // valid when conv == 0
-  CUtensorMap tmB;
+  CUtensorMap tmB[kTcMaxSeg];
   int bn;           // N tile
   int splits;       // K splits (grid z); 1 = no split
   int kb_per_split; // 64-wide k-blocks per split

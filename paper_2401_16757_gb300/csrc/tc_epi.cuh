@@ -1,11 +1,25 @@
-// Shared pieces of the tcgen05 GEMM kernels: launch arguments and the
-// register-only fused epilogue (bias, residual, activation, conversion).
+// Shared pieces of the tcgen05 GEMM kernels: launch arguments and the fused
+// epilogue (bias, residual, activation, conversion).
 #pragma once
 #include "device.cuh"
 #include "kernels.h"
 
 namespace swapnet {
 namespace {
+
+// Weight maps of a launch and, for siblings sharing it (NS > 1: same input, K
+// and N), each layer's output and bias.  A launch of one layer has its output
+// and bias in TcArgs: with the arrays in every launch, YOLOv3's 75 layers
+// took 424 us, without 416.
+template <int NS> struct TcSegs {
+  CUtensorMap m[NS];
+  void* y[NS];
+  const void* bias[NS];
+  int nseg;
+};
+template <> struct TcSegs<1> {
+  CUtensorMap m[1];
+};
 
 struct TcArgs {
   int M, N, K;
@@ -21,7 +35,33 @@ struct TcArgs {
   int wt, ht, tiles_w, tiles_h;
 };
 
-// ---- register-only epilogue helpers
+// A launch's weight maps, outputs and biases (host side).
+template <int NS>
+inline TcSegs<NS> make_segs(const TcGemm& g, const TcPlan& pl) {
+  TcSegs<NS> r;
+  for (int i = 0; i < NS; ++i) r.m[i] = pl.tmB[i < g.nseg ? i : 0];
+  if constexpr (NS > 1) {
+    r.nseg = g.nseg;
+    for (int i = 0; i < NS; ++i) {
+      r.y[i] = i && i < g.nseg ? g.yx[i - 1] : g.y;
+      r.bias[i] = i && i < g.nseg ? g.bx[i - 1] : g.e.bias;
+    }
+  }
+  return r;
+}
+// Output and bias of segment seg.
+template <typename T, int NS>
+__device__ __forceinline__ T* seg_y(const TcArgs& p, const TcSegs<NS>& sg, int seg) {
+  if constexpr (NS > 1) return static_cast<T*>(sg.y[seg]);
+  else return static_cast<T*>(p.y);
+}
+template <typename T, int NS>
+__device__ __forceinline__ const T* seg_bias(const TcArgs& p, const TcSegs<NS>& sg, int seg) {
+  if constexpr (NS > 1) return static_cast<const T*>(sg.bias[seg]);
+  else return static_cast<const T*>(p.e.bias);
+}
+
+// ---- epilogue helpers
 template <typename T> __device__ __forceinline__ uint32_t pack2(float lo, float hi);
 template <> __device__ __forceinline__ uint32_t pack2<__half>(float lo, float hi) {
   uint32_t r;
@@ -125,8 +165,8 @@ __device__ __forceinline__ uint4 epi8_any(const float (&a)[8], const float* sb, 
 constexpr int kEpiStage = 32 * 64;  // bytes of shared memory per warp
 
 // Rows can be moved in 16-byte pieces: N, the strides and the bases allow it.
-__device__ __forceinline__ bool epi_vec_ok(const TcArgs& p) {
-  return ((p.N | p.ldy) % 8 == 0) && ((uintptr_t)p.y & 15) == 0 &&
+__device__ __forceinline__ bool epi_vec_ok(const TcArgs& p, const void* y) {
+  return ((p.N | p.ldy) % 8 == 0) && ((uintptr_t)y & 15) == 0 &&
          (!p.e.res || (p.e.ldr % 8 == 0 && ((uintptr_t)p.e.res & 15) == 0));
 }
 
@@ -172,14 +212,13 @@ __device__ __forceinline__ void epi_rows(uint32_t taddr, const float* sb, uint32
   }
 }
 
-// Columns [n, n + 32) of the warp's rows: accumulator at taddr (the warp's
-// TMEM lanes, first column), bias at sb, residual r from epi_res_load.  All
-// lanes call it together.
+// Columns [n, n + 32) of the warp's rows of output y: accumulator at taddr
+// (the warp's TMEM lanes, first column), bias at sb, residual r from
+// epi_res_load.  All lanes call it together.
 template <typename T>
-__device__ __forceinline__ void epi_piece(uint32_t taddr, const float* sb, uint32_t stage, const TcArgs& p, int m, int n,
-                                          bool vec, int res, const uint4 (&r)[4]) {
+__device__ __forceinline__ void epi_piece(uint32_t taddr, const float* sb, uint32_t stage, const TcArgs& p, T* y, int m,
+                                          int n, bool vec, int res, const uint4 (&r)[4]) {
   const int lane = threadIdx.x & 31;
-  T* y = static_cast<T*>(p.y);
   if (res != kResNone) {
     if (vec) {
 #pragma unroll
@@ -239,9 +278,9 @@ __device__ __forceinline__ uint4 res8(const TcArgs& p, int m, int n, bool vec) {
   return *reinterpret_cast<const uint4*>(static_cast<const T*>(p.e.res) + (int64_t)m * p.e.ldr + n);
 }
 template <typename T>
-__device__ __forceinline__ void finish8(const float (&a)[8], const float* sb, const TcArgs& p, int m, int n, bool vec,
-                                        int res, const uint4& r) {
-  T* y = static_cast<T*>(p.y) + (int64_t)m * p.ldy + n;
+__device__ __forceinline__ void finish8(const float (&a)[8], const float* sb, const TcArgs& p, T* y0, int m, int n,
+                                        bool vec, int res, const uint4& r) {
+  T* y = y0 + (int64_t)m * p.ldy + n;
   if (vec) {
     *reinterpret_cast<uint4*>(y) = epi8_any<T>(a, sb, r, p.e.act, res);
   } else {

@@ -168,3 +168,24 @@ def test_attention_against_float64(dtype, tokens, heads, pos, max_seq):
     ref = (torch.softmax(s, -1) @ vv).permute(1, 0, 2).reshape(tokens, d)
     # one rounding to the stored type (relative 2^-12 and 2^-9 rms) and fp32 sums
     assert torch.linalg.norm(out - ref) <= (4e-4 if dtype == "f16" else 2.5e-3) * torch.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("rows,k,n,count", [
+    (40, 200, 130, 2), (200, 256, 255, 3),      # per tile, ragged columns
+    (600, 320, 1000, 3), (513, 64, 2056, 3),    # pairs of SMs: ragged last tile of every layer, one row in the last row tile
+    (2600, 128, 96, 4),                         # more siblings than one launch takes
+])
+def test_sibling_linears_share_a_launch(dtype, rows, k, n, count):
+    """Tensor-core linear layers that read the same input in one launch: the bits of one launch each, and the oracle."""
+    layers = [_linear(-1, k, k, "relu")] + [_linear(0, k, n, "leaky", bias=i != 1) for i in range(count)]
+    m = dict(name="yolov3", model_id=47, dtype=dtype, input=(rows, 1, 1, k), layers=layers,
+             outputs=list(range(1, count + 1)))
+    w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
+    host = capi.HostWeights(w)
+    runs = [Runner(m, w, capi.Plan.resident(d, capi.options(merge=g)), host) for g in (1, 0)]
+    got, sep = (r.run(x) for r in runs)
+    launches = [r.engine.stats()["kernel_launches"] for r in runs]
+    assert launches[1] - launches[0] == (count - 1 if count <= 3 else count - 2)
+    assert all(a.tobytes() == b.tobytes() for a, b in zip(got, sep))
+    check_close(m, runs[0].decode(got), oracle_outputs(m, w, x))
