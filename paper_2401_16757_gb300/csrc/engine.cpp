@@ -937,8 +937,9 @@ static int plan_side(swapnet_engine* e);
 // or read in place.
 static bool whole_skinny(const swapnet_engine* e, int u) {
   const Unit& U = e->plan.units[u];
-  return e->unit_kind[u] == SWAPNET_KERNEL_SKINNY && !U.host && U.row0 == 0 &&
-         U.rows == e->plan.model.L[U.layer].d.cout;
+  const Layer& L = e->plan.model.L[U.layer];
+  return e->unit_kind[u] == SWAPNET_KERNEL_SKINNY && !skinny_rows_kernel(e->plan.model.dtype, L.n) && !U.host &&
+         U.row0 == 0 && U.rows == L.d.cout;
 }
 
 // A whole linear layer on the tensor-core kernels, without residual and
@@ -1052,11 +1053,6 @@ static int run_group(swapnet_engine* e, int u, const void* din, void* dout, cuda
     j.seg[i] = SkSeg{X.w, Epi{X.b, r, L.d.cout, L.d.act, L.d.res_post}, L.d.cout,
                      out_ptr(e, p.units[v].layer, dout), L.d.cout};
   }
-  j.device_weights = 1;
-  for (int i = 0; i < j.nseg; ++i)
-    if (e->ux[u + i].in_place) j.device_weights = 0;
-  j.num_sms = e->num_sms;
-  j.err = e->err_word;
   return launch_linear_skinny_job(m.dtype, j, s);
 }
 
@@ -1158,7 +1154,7 @@ static int run_unit(swapnet_engine* e, int u, const void* din, void* dout, cudaS
         ep.res = r ? r + (int64_t)U.row0 * es : nullptr;
         if (skinny_ok(m, L))
           return launch_linear_skinny(m.dtype, x, L.n, L.d.cin, X.w, U.rows, ep, y + (int64_t)U.row0 * es,
-                                      L.d.cout, s, X.in_place ? 0 : 1, e->num_sms, e->err_word);
+                                      L.d.cout, s);
         return launch_linear_tiled(m.dtype, x, L.n, L.d.cin, X.w, U.rows, L.d.cout, ep, y + (int64_t)U.row0 * es,
                                    L.d.cout, s);
       }

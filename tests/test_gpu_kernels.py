@@ -189,3 +189,11 @@ def test_sibling_linears_share_a_launch(dtype, rows, k, n, count):
     assert launches[1] - launches[0] == (count - 1 if count <= 3 else count - 2)
     assert all(a.tobytes() == b.tobytes() for a, b in zip(got, sep))
     check_close(m, runs[0].decode(got), oracle_outputs(m, w, x))
+
+
+@pytest.mark.parametrize("rows", [2, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("k,n", [(4, 1), (128, 9), (1020, 40), (1024, 64), (1028, 7), (3000, 130)])
+def test_few_row_fp32_linear(rows, k, n):
+    """The few-row kernel at the edges of its k chunks (1024), features per CTA and rows; with a residual."""
+    rs = _check([_linear(-1, k, n, "leaky"), _linear(-1, k, n, "relu", res=0)], (rows, 1, 1, k), "f32")
+    assert set(rs.engine.unit_kernels()) == {"skinny_linear"}
