@@ -1053,6 +1053,7 @@ static int run_group(swapnet_engine* e, int u, const void* din, void* dout, cuda
     j.seg[i] = SkSeg{X.w, Epi{X.b, r, L.d.cout, L.d.act, L.d.res_post}, L.d.cout,
                      out_ptr(e, p.units[v].layer, dout), L.d.cout};
   }
+  j.num_sms = e->num_sms;
   return launch_linear_skinny_job(m.dtype, j, s);
 }
 
@@ -1154,7 +1155,7 @@ static int run_unit(swapnet_engine* e, int u, const void* din, void* dout, cudaS
         ep.res = r ? r + (int64_t)U.row0 * es : nullptr;
         if (skinny_ok(m, L))
           return launch_linear_skinny(m.dtype, x, L.n, L.d.cin, X.w, U.rows, ep, y + (int64_t)U.row0 * es,
-                                      L.d.cout, s);
+                                      L.d.cout, e->num_sms, s);
         return launch_linear_tiled(m.dtype, x, L.n, L.d.cin, X.w, U.rows, L.d.cout, ep, y + (int64_t)U.row0 * es,
                                    L.d.cout, s);
       }

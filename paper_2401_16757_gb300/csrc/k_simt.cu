@@ -58,120 +58,215 @@ template <typename T> __device__ __forceinline__ uint4 pack16(const float* f) {
   return v;
 }
 
-// ------------------------------------------------------------ skinny linear
-// One warp per output feature, for all M rows: lane l reads the 16-byte
-// chunks l, l+32, ... of the feature's weight row, kSkBatch loads in flight
-// per lane, and keeps one fp32 partial sum per row in chunk order; a
-// butterfly combines the lanes, so the result does not depend on
-// scheduling.  The weights do not depend on the kernel before (they are in
-// place before this kernel is launched), so the first batch is requested
-// before the programmatic wait and overlaps that kernel's drain.
+// ------------------------------------------------------------ GEMV
+// Linear layers of 1 to 4 rows of 16-bit values, or one row of fp32: the time
+// is streaming the weights.  Persistent CTAs (two per SM) take groups of eight
+// weight rows; K is walked in passes, of which a lane takes one 16-byte chunk
+// of every row (chunk 32 w + l of the pass for lane l of warp w), so a loaded
+// chunk of x meets eight rows.  The loads of two passes are in flight ahead of
+// the one being summed, across groups, so that a group's reductions and
+// stores never leave HBM idle; the first two passes' weights are requested
+// before the programmatic wait (they do not depend on the kernel before).  A
+// lane's sums are halved across the lanes, the warps' added in warp order
+// through shared memory: a fixed order for every output.
 //
 // One launch may serve several layers that read the same input (SkJob
-// segments, e.g. the q, k, v projections): the warps are dealt to the
-// segments' features in order.  In pair mode (a gate and the layer whose
-// epilogue takes the gate's output as its residual, e.g. SwiGLU) one warp
-// computes feature o of both: it stores the gate's rounded output and uses
-// that same rounded value as the second layer's residual.  Every feature is
-// computed by the same per-row routine as in a one-layer launch, so the
-// results are bit-identical to launching the layers one by one.
-constexpr int kSkWarps = 8;
-constexpr int kSkBatch = 8;
+// segments, e.g. the q, k, v projections): the groups are dealt to the
+// segments in order.  In pair mode (a gate and the layer whose epilogue takes
+// the gate's output as its residual, e.g. SwiGLU) a group is four features of
+// both: the gate's rounded output is stored and that same rounded value is
+// the second layer's residual.  Every output is summed as in a one-layer
+// launch, so the results are bit-identical to launching the layers one by
+// one.
+// Bound by HBM: against one warp per feature with eight loads in flight and
+// none while it sums, whose last wave of CTAs leaves the chip part empty:
+// 11008 x 4096 bf16 19.0 -> 13.7 us (6.6 TB/s, launch included), 4096 x 11008
+// 19.1 -> 15.0, 4096 x 4096 (from L2) 6.1 -> 4.4, 32000 x 4096 40.2 -> 36.7.
+constexpr int kGvWarps = 8;
+constexpr int kGvRows = 8;  // weight rows per group
 
 template <typename T, int MT>
-__device__ __forceinline__ void sk_row(const T* __restrict__ x, int M, int K, const T* __restrict__ wrow, int lane,
-                                       uint4 (&wv)[kSkBatch], bool preloaded, float (&acc)[MT]) {
+__global__ void __launch_bounds__(kGvWarps * 32, MT <= 2 ? 2 : 1) gemv_kernel(const SkJob j, const int groups) {
   constexpr int V = Vec16<T>::N;
-  const int kchunks = K / V;  // K % V == 0 (checked on the host)
-  auto load_batch = [&](int c0) {
+  constexpr int NV = MT * kGvRows;
+  constexpr int kPass = kGvWarps * 32 * V;  // k per pass
+  __shared__ float red[2][kGvWarps][NV];
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const int K = j.K, k0 = (warp * 32 + lane) * V;
+  const int passes = (K + kPass - 1) / kPass;
+  const int G = gridDim.x;
+  const int items = (int)blockIdx.x < groups ? (groups - 1 - (int)blockIdx.x) / G + 1 : 0;
+  const T* x = static_cast<const T*>(j.x);
+  const int per = j.pair ? kGvRows / 2 : kGvRows;  // features per group
+  // segment and first feature of a group
+  auto locate = [&](int g, int* o) {
+    int si = 0;
+    if (!j.pair)
+      while (si + 1 < j.nseg) {
+        const int n = (j.seg[si].N + per - 1) / per;
+        if (g < n) break;
+        g -= n;
+        ++si;
+      }
+    *o = g * per;
+    return si;
+  };
+  // load cursor: rows 0..3 of its group start at pa, rows 4..7 at pb; of each
+  // four, va and vb exist
+  int lg = blockIdx.x, lp = 0, va = 0, vb = 0;
+  const T *pa = nullptr, *pb = nullptr;
+  auto open_group = [&]() {
+    if (lg >= groups) {
+      va = vb = 0;
+      return;
+    }
+    int o;
+    const int si = locate(lg, &o);
+    const T* W = static_cast<const T*>(j.seg[0].W);
+    int N = j.seg[0].N;
 #pragma unroll
-    for (int u = 0; u < kSkBatch; ++u) {
-      const int ch = c0 + u * 32;
-      wv[u] = ch < kchunks ? ld_stream16(wrow + (int64_t)ch * V) : make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 1; i < kSkMaxSeg; ++i)
+      if (i == si) {
+        W = static_cast<const T*>(j.seg[i].W);
+        N = j.seg[i].N;
+      }
+    pa = W + (int64_t)o * K + k0;
+    va = min(4, N - o);
+    if (j.pair) {
+      pb = static_cast<const T*>(j.seg[1].W) + (int64_t)o * K + k0;
+      vb = va;
+    } else {
+      pb = pa + (int64_t)4 * K;
+      vb = max(0, min(4, N - o - 4));
     }
   };
+  struct Buf {
+    uint4 w[kGvRows];
+    uint4 x[MT];
+  };
+  auto load_w = [&](Buf& b) {
+    const bool in = k0 + lp * kPass < K;
 #pragma unroll
-  for (int m = 0; m < MT; ++m) acc[m] = 0.f;
-  for (int c0 = lane; c0 < kchunks; c0 += 32 * kSkBatch) {
-    if (c0 != lane || !preloaded) load_batch(c0);
-#pragma unroll
-    for (int u = 0; u < kSkBatch; ++u) {
-      const int ch = c0 + u * 32;
-      if (ch < kchunks) {
-        float wf[V];
-        unpack16<T>(wv[u], wf);
-#pragma unroll
-        for (int m = 0; m < MT; ++m) {
-          if (m < M) {
-            float xv[V];
-            unpack16<T>(__ldg(reinterpret_cast<const uint4*>(x + (int64_t)m * K + (int64_t)ch * V)), xv);
-#pragma unroll
-            for (int i = 0; i < V; ++i) acc[m] = fmaf(wf[i], xv[i], acc[m]);
-          }
-        }
-      }
+    for (int f = 0; f < kGvRows; ++f) {
+      b.w[f] = make_uint4(0u, 0u, 0u, 0u);
+      const bool ok = in && (f < 4 ? f < va : f - 4 < vb);
+      if (ok) b.w[f] = ld_stream16((f < 4 ? pa : pb) + (int64_t)(f & 3) * K + (int64_t)lp * kPass);
     }
-  }
+  };
+  auto load_x = [&](Buf& b, int p) {
+    const int k = k0 + p * kPass;
 #pragma unroll
-  for (int m = 0; m < MT; ++m) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], off);
-  }
-}
-
-template <typename T, int MT>
-__global__ void __launch_bounds__(kSkWarps * 32) linear_skinny_kernel(const SkJob j) {
-  constexpr int V = Vec16<T>::N;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int o = blockIdx.x * kSkWarps + warp;
-  // this warp's segment (pair mode: both segments, feature o)
-  int si = 0;
-  if (!j.pair)
-    for (int i = 0; i + 1 < j.nseg && o >= j.seg[i].N; ++i) {
-      o -= j.seg[i].N;
-      si = i + 1;
+    for (int m = 0; m < MT; ++m)
+      b.x[m] = m < j.M && k < K ? __ldg(reinterpret_cast<const uint4*>(x + (int64_t)m * K + k)) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  auto next_load = [&]() {
+    if (++lp == passes) {
+      lp = 0;
+      lg += G;
+      open_group();
     }
-  SkSeg S = j.seg[0];
-#pragma unroll
-  for (int i = 1; i < kSkMaxSeg; ++i)
-    if (i == si) S = j.seg[i];
-  const bool active = o < S.N;
-  const T* x = static_cast<const T*>(j.x);
-  uint4 wv[kSkBatch];
-  if (active) {
-    const T* wrow = static_cast<const T*>(S.W) + (int64_t)o * j.K;
-#pragma unroll
-    for (int u = 0; u < kSkBatch; ++u) {
-      const int ch = lane + u * 32;
-      wv[u] = ch < j.K / V ? ld_stream16(wrow + (int64_t)ch * V) : make_uint4(0u, 0u, 0u, 0u);
-    }
-  }
+  };
+  Buf A, B;
+  open_group();
+  load_w(A);
+  const int pA = lp;
+  next_load();
+  load_w(B);
+  const int pB = lp;
+  next_load();
   pdl_wait();
   pdl_launch_dependents();
-  if (!active) return;
-  float acc[MT];
-  float gate[MT];
-  const int passes = j.pair ? 2 : 1;
-  for (int p = 0; p < passes; ++p) {
-    if (p == 1) S = j.seg[1];
-    sk_row<T, MT>(x, j.M, j.K, static_cast<const T*>(S.W) + (int64_t)o * j.K, lane, wv, p == 0, acc);
-    const float b = S.e.bias ? to_f<T>(static_cast<const T*>(S.e.bias)[o]) : 0.f;
+  load_x(A, pA);
+  load_x(B, pB);
+  float acc[NV];  // [row of x][weight row]
+#pragma unroll
+  for (int i = 0; i < NV; ++i) acc[i] = 0.f;
+  auto sum = [&](const Buf& b) {
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
-      if (m < j.M) {
-        float r = 0.f;
-        bool has_r = S.e.res != nullptr;
-        if (p == 1) {
-          r = gate[m];
-          has_r = true;
-        } else if (has_r) {
-          r = to_f<T>(static_cast<const T*>(S.e.res)[(int64_t)m * S.e.ldr + o]);
-        }
-        const T out = from_f<T>(epilogue(acc[m], b, r, has_r, S.e.act, S.e.res_post));
-        gate[m] = to_f<T>(out);  // the stored value, as the paired layer would read it
-        if (lane == m) static_cast<T*>(S.y)[(int64_t)m * S.ldy + o] = out;
+      float xf[V];
+      unpack16<T>(b.x[m], xf);
+#pragma unroll
+      for (int f = 0; f < kGvRows; ++f) {
+        float wf[V];
+        unpack16<T>(b.w[f], wf);
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[m * kGvRows + f] = fmaf(wf[i], xf[i], acc[m * kGvRows + f]);
       }
     }
+  };
+  // a group's sums across lanes and warps, its outputs
+  auto finish = [&](int g, int par) {
+    // halve the sums a lane holds while there are several, then add across
+    // the lanes that hold the same one; the highest lane bits say which
+#pragma unroll
+    for (int off = 16, n = NV / 2; off > 0; off >>= 1, n >>= 1) {
+      if (n > 0) {
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+          const bool up = lane & off;
+          const float send = up ? acc[i] : acc[i + n], keep = up ? acc[i + n] : acc[i];
+          acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+      } else {
+        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], off);
+      }
+    }
+    if (NV >= 32) {
+#pragma unroll
+      for (int i = 0; i < (NV + 31) / 32; ++i) red[par][warp][lane * (NV / 32) + i] = acc[i];
+    } else if (lane % (32 / (NV < 32 ? NV : 32)) == 0) {
+      red[par][warp][lane / (32 / (NV < 32 ? NV : 32))] = acc[0];
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) acc[i] = 0.f;
+    __syncthreads();
+    const int f = threadIdx.x % per, m = threadIdx.x / per;
+    if (m >= j.M) return;
+    int o;
+    const int si = locate(g, &o);
+    o += f;
+    SkSeg S = j.seg[0];
+#pragma unroll
+    for (int i = 1; i < kSkMaxSeg; ++i)
+      if (i == si) S = j.seg[i];
+    if (o >= S.N) return;
+    auto total = [&](int i) {
+      float t = red[par][0][i];
+#pragma unroll
+      for (int h = 1; h < kGvWarps; ++h) t += red[par][h][i];
+      return t;
+    };
+    auto emit = [&](const SkSeg& q, float t, float r, bool has_r) {
+      const float bias = q.e.bias ? to_f<T>(static_cast<const T*>(q.e.bias)[o]) : 0.f;
+      const T out = from_f<T>(epilogue(t, bias, r, has_r, q.e.act, q.e.res_post));
+      static_cast<T*>(q.y)[(int64_t)m * q.ldy + o] = out;
+      return to_f<T>(out);  // the stored value, as a paired layer reads it
+    };
+    const bool has_r = S.e.res != nullptr;
+    const float r = has_r ? to_f<T>(static_cast<const T*>(S.e.res)[(int64_t)m * S.e.ldr + o]) : 0.f;
+    const float gate = emit(S, total(m * kGvRows + f), r, has_r);
+    if (j.pair) emit(j.seg[1], total(m * kGvRows + f + 4), gate, true);
+  };
+  int cp = 0, cg = blockIdx.x, par = 0;  // pass and group being summed
+  const int total = items * passes;
+  auto step = [&](Buf& b, int it) {
+    sum(b);
+    if (it + 2 < total) {
+      load_w(b);
+      load_x(b, lp);
+      next_load();
+    }
+    if (++cp == passes) {
+      cp = 0;
+      finish(cg, par);
+      cg += G;
+      par ^= 1;
+    }
+  };
+  for (int it = 0; it < total; it += 2) {
+    step(A, it);
+    if (it + 1 < total) step(B, it + 1);
   }
 }
 
@@ -279,14 +374,15 @@ template <typename T> int skinny_dispatch(const SkJob& j, cudaStream_t s) {
       return e == cudaSuccess ? SWAPNET_OK : SWAPNET_ERR_CUDA;
     }
   }
-  int rows = j.seg[0].N;
+  const int per = j.pair ? kGvRows / 2 : kGvRows;
+  int groups = (j.seg[0].N + per - 1) / per;
   if (!j.pair)
-    for (int i = 1; i < j.nseg; ++i) rows += j.seg[i].N;
-  const dim3 grid((rows + kSkWarps - 1) / kSkWarps), block(kSkWarps * 32);
+    for (int i = 1; i < j.nseg; ++i) groups += (j.seg[i].N + per - 1) / per;
+  const dim3 grid(std::max(1, std::min(groups, 2 * std::max(1, j.num_sms)))), block(kGvWarps * 32);
   cudaError_t e;
-  if (j.M <= 1) e = launch_pdl(linear_skinny_kernel<T, 1>, grid, block, 0, s, j);
-  else if (j.M <= 2) e = launch_pdl(linear_skinny_kernel<T, 2>, grid, block, 0, s, j);
-  else if (j.M <= 4) e = launch_pdl(linear_skinny_kernel<T, 4>, grid, block, 0, s, j);
+  if (j.M <= 1) e = launch_pdl(gemv_kernel<T, 1>, grid, block, 0, s, j, groups);
+  else if (j.M <= 2) e = launch_pdl(gemv_kernel<T, 2>, grid, block, 0, s, j, groups);
+  else if (j.M <= 4) e = launch_pdl(gemv_kernel<T, 4>, grid, block, 0, s, j, groups);
   else SN_FAIL(SWAPNET_ERR_UNSUPPORTED, "skinny linear: more rows than the GEMV takes");  // 16-bit layers of 5 rows and
                                                                                           // more run on the tensor cores
   return e == cudaSuccess ? SWAPNET_OK : SWAPNET_ERR_CUDA;
@@ -715,13 +811,14 @@ int launch_linear_skinny_job(int dtype, const SkJob& j, cudaStream_t s) {
 }
 
 int launch_linear_skinny(int dtype, const void* x, int M, int K, const void* W, int N, const Epi& e, void* y,
-                         int64_t ldy, cudaStream_t s) {
+                         int64_t ldy, int num_sms, cudaStream_t s) {
   SkJob j{};
   j.x = x;
   j.M = M;
   j.K = K;
   j.nseg = 1;
   j.seg[0] = SkSeg{W, e, N, y, ldy};
+  j.num_sms = num_sms;
   return launch_linear_skinny_job(dtype, j, s);
 }
 

@@ -50,7 +50,7 @@ struct Epi {
 // y[m, col0 + o] (row stride ldy) = epi(sum_k x[m,k] W[o,k]) for o < N,
 // M <= 16.  fp32 / fp16 / bf16; fixed-order reduction (deterministic).
 int launch_linear_skinny(int dtype, const void* x, int M, int K, const void* W, int N, const Epi& e, void* y,
-                         int64_t ldy, cudaStream_t s);
+                         int64_t ldy, int num_sms, cudaStream_t s);
 // fp32 layers of this many rows run the few-row kernel, one layer per launch.
 constexpr int kRowsMin = 2;
 bool skinny_rows_kernel(int dtype, int M);
@@ -73,6 +73,7 @@ struct SkJob {
   int M, K;
   int nseg, pair;
   SkSeg seg[kSkMaxSeg];
+  int num_sms;
 };
 int launch_linear_skinny_job(int dtype, const SkJob& j, cudaStream_t s);
 

@@ -197,3 +197,26 @@ def test_few_row_fp32_linear(rows, k, n):
     """The few-row kernel at the edges of its k chunks (1024), features per CTA and rows; with a residual."""
     rs = _check([_linear(-1, k, n, "leaky"), _linear(-1, k, n, "relu", res=0)], (rows, 1, 1, k), "f32")
     assert set(rs.engine.unit_kernels()) == {"skinny_linear"}
+
+
+@pytest.mark.parametrize("dtype,rows", [("f16", 1), ("bf16", 1), ("f16", 2), ("bf16", 3), ("f16", 4), ("f32", 1)])
+@pytest.mark.parametrize("k,n", [(8, 1), (2048, 9), (2056, 40), (4104, 300), (11008, 21), (1024, 5000)])
+def test_gemv(dtype, rows, k, n):
+    """The GEMV at the edges of its passes (2048 or 1024 k), weight-row groups (8) and one group per CTA; a residual,
+    and a gate with its SwiGLU layer in one launch."""
+    rs = _check([_linear(-1, k, n), _linear(-1, k, n, "swiglu", res=0, bias=False), _linear(1, n, 24, "relu")] if n % 8 == 0
+                else [_linear(-1, k, n), _linear(-1, k, n, "leaky", res=0, res_post=True)], (rows, 1, 1, k), dtype)
+    assert set(rs.engine.unit_kernels()) == {"skinny_linear"}
+
+
+def test_gemv_segments_of_ragged_widths():
+    """Three siblings of widths that are no multiple of a group in one launch: the bits of one launch each."""
+    layers = [_linear(-1, 520, 13), _linear(-1, 520, 700, "relu"), _linear(-1, 520, 8)]
+    m = dict(name="yolov3", model_id=48, dtype="bf16", input=(1, 1, 1, 520), layers=layers, outputs=[0, 1, 2])
+    w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
+    host = capi.HostWeights(w)
+    a, b = (Runner(m, w, capi.Plan.resident(d, capi.options(merge=g)), host) for g in (1, 0))
+    got = a.run(x)
+    assert all(p.tobytes() == q.tobytes() for p, q in zip(got, b.run(x)))
+    assert a.engine.stats()["kernel_launches"] == 1 and b.engine.stats()["kernel_launches"] == 3
+    check_close(m, a.decode(got), oracle_outputs(m, w, x))
