@@ -9,8 +9,7 @@
 // also staged by TMA, or the implicit im2col of an NHWC input for general
 // convolutions, gathered by four warps with cp.async (zero fill for padding)
 // into the same swizzled layout.  One CTA computes one 128 x BN tile (BN 64
-// or 128; 256 for linear layers of at most kFewRows rows, whose work is
-// streaming the weight matrix):
+// or 128; 256 for linear layers of at most kFewRows rows):
 //   warp 0      TMA producer (one elected lane)
 //   warp 1      TMEM allocation and MMA issue (one elected lane)
 //   warps 2..5  im2col gather (conv)
@@ -42,30 +41,39 @@ constexpr int kEpiThreads = 256;
 constexpr int kThreads = 64 + kEpiThreads;
 constexpr int kABytes = kBM * kBK * 2;
 
-// N tile 256 serves GEMMs of at most kFewRows rows (one partly filled M
-// tile) that stream a large weight matrix: their cluster split-K partials
-// are distributed by column, so the receive buffer holds kFewRows rows.
-constexpr int kFewRows = 16;
-
-template <int BN> struct Cfg {
-  static constexpr int kStages = BN == 64 ? 6 : 4;
-  static constexpr int kLag = kStages - 2;  // gather: cp.async groups in flight per thread
-  static constexpr int kBBytes = BN * kBK * 2;
-  static constexpr int kStageBytes = kStages * (kABytes + kBBytes);
-  // cluster split-K receive buffer.  BN 64/128 (row owners): up to 16 splits
-  // x ceil(128/splits) rows.  BN 256 (column owners): splits x kFewRows rows
-  // x (columns per owner + 4), at most kFewRows x 6 x 52 floats (2 to 8 splits).
-  static constexpr int kRecvBytes = BN == 256 ? kFewRows * (BN + 64) * 4 : (kBM + 15) * (BN + 4) * 4;
-  static constexpr int kBiasBytes = BN * 4;
-  static constexpr int kSmem = kStageBytes + kRecvBytes + kBiasBytes + 256 + 1024;
-};
-
 // A operand: kA2d (2-D TMA of a row-major matrix: linear layers, 1x1
 // stride-1 convs), kAGather (cp.async im2col gather by warps 2..5), kATap
 // (convs whose taps are whole 64-channel k-blocks: one 4-D TMA per k-block
 // of the tap's 64 channels over a wt x ht patch of output pixels, zero fill
-// for the padding; the CTA's 128 rows are that patch, rows >= wt * ht unused)
-constexpr int kA2d = 0, kAGather = 1, kATap = 2;
+// for the padding; the CTA's 128 rows are that patch, rows >= wt * ht unused),
+// kAFew (2-D TMA of at most kFewRows rows, whose work is streaming the weight
+// matrix: only those rows are loaded and the other MMA rows read whatever
+// lies behind them, results nobody uses, so a stage is 2 KB of A and the
+// weight tile and the stages hold 128-170 KB of weights in flight; an N tile
+// of 256 exists for it alone; the splits' partials are shared out by column).
+// Measured inside chains of such layers, weights from HBM, 16 rows, with
+// 16 KB of A per stage and 4-6 stages before: 1024 -> 1024 4.2 to 3.4 us, 1024 <-> 2752 5.8
+// to 3.9, 2048 <-> 8192 12.9 to 8.4, 4096 -> 4096 9.4 to 8.7, 8192 -> 8192
+// 26.2 to 24.3 (5.5 TB/s); 25088 -> 4096 alone 37.9 to 33.2.
+constexpr int kA2d = 0, kAGather = 1, kATap = 2, kAFew = 3;
+constexpr int kFewRows = 16;
+
+template <int BN, int AMODE> struct Cfg {
+  static constexpr bool kFew = AMODE == kAFew;
+  static constexpr int kStages = kFew ? (BN == 64 ? 16 : (BN == 128 ? 10 : 5)) : (BN == 64 ? 6 : 4);
+  static constexpr int kLag = kStages - 2;  // gather: cp.async groups in flight per thread
+  static constexpr int kAStage = kFew ? kFewRows * kBK * 2 : kABytes;
+  static constexpr int kARegion = kStages * kAStage + kABytes - kAStage;  // the last stage's MMA reads 128 rows too
+  static constexpr int kBBytes = BN * kBK * 2;
+  static constexpr int kStageBytes = kARegion + kStages * kBBytes;
+  // cluster split-K receive buffer.  Row owners: up to 16 splits x
+  // ceil(128/splits) rows.  Few rows (column owners): splits x kFewRows rows x
+  // (columns per owner, a multiple of 8, + 4): 2 to 8 splits of up to BN + 76 floats.
+  static constexpr int kRecvBytes = kFew ? kFewRows * (BN + 76) * 4 : (kBM + 15) * (BN + 4) * 4;
+  static constexpr int kBiasBytes = BN * 4;
+  static constexpr int kSmem = kStageBytes + kRecvBytes + kBiasBytes + 512 + 1024;
+  static_assert(kSmem <= 232448, "dynamic shared memory above the 227 KB per-CTA limit");
+};
 
 // NS: layers that a launch may hold (1, or kTcMaxSeg siblings)
 template <typename T, int BN, int AMODE, int NS>
@@ -73,16 +81,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ TcSegs<NS> sg, const TcArgs p) {
   constexpr bool GATHER = AMODE == kAGather;
   constexpr bool TAP = AMODE == kATap;
-  constexpr int kStages = Cfg<BN>::kStages;
-  constexpr int kLag = Cfg<BN>::kLag;
-  constexpr int kBBytes = Cfg<BN>::kBBytes;
+  constexpr bool FEW = AMODE == kAFew;
+  using C = Cfg<BN, AMODE>;
+  constexpr int kStages = C::kStages;
+  constexpr int kLag = C::kLag;
+  constexpr int kAStage = C::kAStage;
+  constexpr int kBBytes = C::kBBytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
-  uint8_t* sB = smem + kStages * kABytes;
-  float* recv = reinterpret_cast<float*>(smem + Cfg<BN>::kStageBytes);
-  float* sbias = reinterpret_cast<float*>(smem + Cfg<BN>::kStageBytes + Cfg<BN>::kRecvBytes);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg<BN>::kStageBytes + Cfg<BN>::kRecvBytes + Cfg<BN>::kBiasBytes);
+  uint8_t* sB = smem + C::kARegion;
+  float* recv = reinterpret_cast<float*>(smem + C::kStageBytes);
+  float* sbias = reinterpret_cast<float*>(smem + C::kStageBytes + C::kRecvBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStageBytes + C::kRecvBytes + C::kBiasBytes);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages);
@@ -108,7 +119,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     pth = rem / p.tiles_w;
     ptw = rem - pth * p.tiles_w;
   }
-  const uint32_t a_bytes = TAP ? (uint32_t)(p.wt * p.ht * 128) : (GATHER ? 0u : (uint32_t)kABytes);
+  const uint32_t a_bytes = TAP ? (uint32_t)(p.wt * p.ht * 128) : (GATHER ? 0u : (uint32_t)kAStage);
   // output row of tile row r (-1: no output)
   auto row_m = [&](int r) -> int {
     if (TAP) {
@@ -157,10 +168,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const bool vec = epi_vec_ok(p, seg_y<T>(p, sg, seg));
   const int rmode = res_mode(p.e);
   // cluster split-K: what epilogue thread t sums after the exchange, and its
-  // residual, requested while the MMAs run.  BN 64/128: 8 columns of up to
-  // kRedN rows of this CTA's share of the rows; BN 256: 8 columns of one row
+  // residual, requested while the MMAs run.  row owners: 8 columns of up to
+  // kRedN rows of this CTA's share of the rows; few rows: 8 columns of one row
   // of this CTA's share of the columns
-  constexpr int kColGroups = BN / 8, kRedRows = kEpiThreads / kColGroups, kRedN = BN == 256 ? 1 : 64 / kRedRows;
+  constexpr int kColGroups = BN / 8, kRedRows = kEpiThreads / kColGroups, kRedN = FEW ? 1 : 64 / kRedRows;
   const int t = (int)threadIdx.x - 64;
   int red_m[kRedN];
   uint4 red_res[kRedN];
@@ -193,14 +204,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       auto load_a = [&](int s, int i) {
         if (TAP) {
-          tma_load_4d(a0 + s * kABytes, &tmA, full_bar(s), c0, px + rx, py + ry, pimg);
+          tma_load_4d(a0 + s * kAStage, &tmA, full_bar(s), c0, px + rx, py + ry, pimg);
           c0 += kBK;
           if (c0 == p.C) {
             c0 = 0;
             if (++rx == p.kw) { rx = 0; ++ry; }
           }
         } else {
-          tma_load_2d(a0 + s * kABytes, &tmA, full_bar(s), (kb0 + i) * kBK, m0);
+          tma_load_2d(a0 + s * kAStage, &tmA, full_bar(s), (kb0 + i) * kBK, m0);
         }
       };
       pdl_wait();
@@ -238,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!mbar_wait_bounded(full_bar(s), par, abort_flag, p.err)) break;
         tc_fence_after();
         // the descriptors' address field counts 16 bytes
-        const uint64_t ad = ad0 + s * (uint32_t)(kABytes >> 4), bd = bd0 + s * (uint32_t)(kBBytes >> 4);
+        const uint64_t ad = ad0 + s * (uint32_t)(kAStage >> 4), bd = bd0 + s * (uint32_t)(kBBytes >> 4);
 #pragma unroll
         for (int k = 0; k < kBK / 16; ++k) tc_mma_f16(tmem, ad + 2ull * k, bd + 2ull * k, idesc, (i | k) != 0);
         tc_commit(empty_bar(s));
@@ -277,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (; i < nk; ++i) {
         const int s = i % kStages, r = i / kStages;
         if (!mbar_wait_bounded(empty_bar(s), (r & 1) ^ 1, abort_flag, p.err)) break;
-        const uint32_t dst_row = smem_u32(sA + s * kABytes) + row_off;
+        const uint32_t dst_row = smem_u32(sA + s * kAStage) + row_off;
         if (whole_tap) {
           const int iy = iy0 + ry, ix = ix0 + rx;
           const bool valid = mvalid && k < p.K && (unsigned)iy < (unsigned)p.H && (unsigned)ix < (unsigned)p.Wd;
@@ -327,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint4 rnext[4];
     if (splits == 1) {
       epi_res_load<T>(rnext, p, m, n0 + c_lo, vec);
-    } else if (csplit && BN == 256) {
+    } else if (csplit && FEW) {
       const int cpo = (((BN + splits - 1) / splits) + 7) & ~7;
       const int w8 = (min(BN, ((int)blockIdx.z + 1) * cpo) - (int)blockIdx.z * cpo) / 8;
       const int rr = w8 > 0 ? t / w8 : kFewRows;
@@ -363,15 +374,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
       asm volatile("barrier.cluster.wait;" ::: "memory");  // every peer is running
       // push this split's partial rows to their owners, slot = this split's index
-      const bool mine = BN == 256 ? m >= 0 && row < kFewRows : m >= 0;
+      const bool mine = FEW ? m >= 0 && row < kFewRows : m >= 0;
       if (all_ok && __any_sync(0xffffffffu, mine)) {
-        // BN 64/128: owner of row w = w / rows_per_owner.  BN 256 (at most
-        // kFewRows rows): columns [o * cpo, (o + 1) * cpo) belong to CTA o
+        // owner of row w = w / rows_per_owner; few rows: columns [o * cpo, (o + 1) * cpo) belong to CTA o
         const int rpo = (kBM + splits - 1) / splits;
         const int cpo = (((BN + splits - 1) / splits) + 7) & ~7;
         const uint32_t owner = (uint32_t)(row / rpo);
         uint32_t base = 0;
-        if (BN != 256) {
+        if (!FEW) {
           const uint32_t la = smem_u32(recv) + (uint32_t)((((int)blockIdx.z * rpo + row - (int)owner * rpo) * (BN + 4)) * 4);
           asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base) : "r"(la), "r"(owner));
         }
@@ -385,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int j = 0; j < 4; ++j) {
               const int c = c0 + 4 * j;
               uint32_t ra = base + (uint32_t)c * 4;
-              if (BN == 256) {
+              if (FEW) {
                 const uint32_t o = (uint32_t)(c / cpo);
                 const uint32_t la =
                     smem_u32(recv) + (uint32_t)((((int)blockIdx.z * kFewRows + row) * (cpo + 4) + c - (int)o * cpo) * 4);
@@ -410,10 +420,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (t >= 0) {
       const int rpo = (kBM + splits - 1) / splits;
       const int cpo = (((BN + splits - 1) / splits) + 7) & ~7;
-      const int c_own = BN == 256 ? (int)blockIdx.z * cpo : 0;  // this CTA's first column
-      const int w8 = BN == 256 ? max(1, (min(BN, c_own + cpo) - c_own) / 8) : kColGroups;
-      const int rs = BN == 256 ? cpo + 4 : BN + 4;                      // floats per receive row
-      const int zs = (BN == 256 ? kFewRows : rpo) * rs;                 // floats per split
+      const int c_own = FEW ? (int)blockIdx.z * cpo : 0;  // this CTA's first column
+      const int w8 = FEW ? max(1, (min(BN, c_own + cpo) - c_own) / 8) : kColGroups;
+      const int rs = FEW ? cpo + 4 : BN + 4;                      // floats per receive row
+      const int zs = (FEW ? kFewRows : rpo) * rs;                 // floats per split
       const int c8 = t % w8 * 8;
 #pragma unroll
       for (int j = 0; j < kRedN; ++j) {
@@ -521,7 +531,7 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   static std::atomic<uint64_t> attr_done{0};  // per instantiation, one bit per device
   auto kern = tc_gemm_kernel<T, BN, AMODE, NS>;
   if (attr_needed(attr_done)) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (Cfg<BN, AMODE>::kSmem)) != cudaSuccess)
       SN_FAIL(SWAPNET_ERR_CUDA, "cudaFuncSetAttribute failed");
     attr_set(attr_done);
   }
@@ -550,7 +560,7 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   std::memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = grid;
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg<BN>::kSmem;
+  cfg.dynamicSmemBytes = (Cfg<BN, AMODE>::kSmem);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   int na = 0;
@@ -587,12 +597,12 @@ int active_clusters_inst(int c) {
     if (v > 0) return v - 1;
   }
   auto kern = tc_gemm_kernel<T, BN, AMODE, 1>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmem);
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (Cfg<BN, AMODE>::kSmem));
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(1, 1, c);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg<BN>::kSmem;
+  cfg.dynamicSmemBytes = (Cfg<BN, AMODE>::kSmem);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 1;
@@ -610,14 +620,17 @@ int active_clusters_inst(int c) {
 }
 
 template <typename T>
-int active_clusters_t(int bn, bool gather, int c) {
-  if (bn == 256) return active_clusters_inst<T, 256, kA2d>(c);
+int active_clusters_t(int bn, bool gather, bool few, int c) {
+  if (few)
+    return bn == 256 ? active_clusters_inst<T, 256, kAFew>(c)
+                     : (bn == 64 ? active_clusters_inst<T, 64, kAFew>(c) : active_clusters_inst<T, 128, kAFew>(c));
   if (bn == 64) return gather ? active_clusters_inst<T, 64, kAGather>(c) : active_clusters_inst<T, 64, kA2d>(c);
   return gather ? active_clusters_inst<T, 128, kAGather>(c) : active_clusters_inst<T, 128, kA2d>(c);
 }
 
-int active_clusters(int dtype, int bn, bool gather, int c) {
-  return dtype == SWAPNET_BF16 ? active_clusters_t<__nv_bfloat16>(bn, gather, c) : active_clusters_t<__half>(bn, gather, c);
+int active_clusters(int dtype, int bn, bool gather, bool few, int c) {
+  return dtype == SWAPNET_BF16 ? active_clusters_t<__nv_bfloat16>(bn, gather, few, c)
+                               : active_clusters_t<__half>(bn, gather, few, c);
 }
 
 // ---- which kernel, N tile and split of K: the least of the times below, in
@@ -642,16 +655,21 @@ double tile_us(int bn, int64_t tiles, int splits, int KB, bool tap, int sms) {
 }
 
 // The per-tile kernel on at most kFewRows rows: streaming the weights is the
-// work, at a rate that needs enough CTAs with enough bytes in flight.
+// work.  A k-block slows down as more CTAs share the L2 (from 64 of them on),
+// and the whole matrix may have to come from HBM, at a rate that needs a CTA
+// on most SMs.  More CTAs than SMs cost a
+// whole CTA's fill again.
 double few_us(int bn, int64_t tiles, int splits, int KB, int64_t N, int sms) {
   const int kb = (KB + splits - 1) / splits;
-  const double per_kb = bn == 64 ? 0.125 : (bn == 128 ? 0.16 : 0.36);
-  const double base = bn == 64 ? 2.1 : (bn == 128 ? 2.6 : 3.3);
-  const double rate = (bn == 64 ? 5.0e6 : (bn == 128 ? 5.8e6 : 6.0e6)) *  // bytes per us
-                      std::min(1.0, (double)std::min<int64_t>(tiles * splits, sms) / 110.0);
-  const int64_t waves = (tiles * splits + sms - 1) / sms;
-  const double split = splits > 1 ? 0.9 + 0.03 * splits : 0.0;
-  return base + split + std::max(waves * per_kb * kb, (double)N * KB * kBK * 2.0 / rate) + (waves - 1) * 2.2;
+  const double alone = bn == 64 ? 0.118 : (bn == 128 ? 0.133 : 0.27);
+  const double shared = bn == 64 ? 0.082 : (bn == 128 ? 0.057 : 0.04);
+  const double base = bn == 64 ? 1.95 : (bn == 128 ? 2.5 : 3.6);
+  const int64_t ctas = tiles * splits, waves = (ctas + sms - 1) / sms;
+  const double busy = std::min(1.0, std::max(0.0, (ctas - 64) / 88.0));
+  const double hbm = 6.9e6 * (0.6 + 0.4 * std::min(1.0, ctas / 128.0));  // bytes per us
+  const double split = splits > 1 ? 1.0 + 0.08 * splits : 0.0;
+  return base + split + std::max(waves * (alone + shared * busy) * kb, (double)N * KB * kBK * 2.0 / hbm) +
+         (waves - 1) * 2.5;
 }
 
 // Persistent kernel, one CTA per tile of msub x 128 rows: a tile's epilogue
@@ -724,21 +742,21 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
     p->bn = bn;
     p->splits = splits;
   };
+  const bool few = !g.conv && g.M <= kFewRows && nseg == 1;
   for (int bn : {64, 128, 256}) {
-    const bool few = !g.conv && g.M <= kFewRows;
-    if ((bn == 128 && Nd <= 64) || (bn == 256 && (!few || KB < 16 || nseg > 1))) continue;
+    if ((bn == 128 && Nd <= 64) || (bn == 256 && (!few || KB < 16))) continue;
     const int64_t tiles = mt_tile * ((Nd + bn - 1) / bn) * nseg;
     // segments: an unsplit sum, as each layer's own launch makes it
     for (int c = 1; c <= (nseg > 1 ? 1 : cap); ++c) {
       const int per = (KB + c - 1) / c, used = (KB + per - 1) / per;  // splits that get a k-block
       if (used != c) continue;
       // every cluster at once: a second wave of them costs more than a split saves
-      if (c > 1 && tiles > active_clusters(g.dtype, bn, gather, c)) continue;
+      if (c > 1 && tiles > active_clusters(g.dtype, bn, gather, few, c)) continue;
       consider(bn, c, few ? few_us(bn, tiles, c, KB, Nd, sms) : tile_us(bn, tiles, c, KB, tap, sms));
     }
   }
   // ---- persistent, no split
-  if (g.allow_persist) {
+  if (g.allow_persist && !few) {
     int pbn = Nd <= 64 ? 64 : (Nd <= 128 ? 128 : 256);
     if (pbn == 256 && mt_pers * ((Nd + 255) / 256) * 2 <= sms) pbn = 128;  // twice the CTAs
     // N tiles of 64 with A by TMA: four (else two) 128-row sub-tiles per
@@ -766,6 +784,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
     }
   }
   if (p->persist) p->splits = 1;
+  p->few = few && !p->persist;
   p->kb_per_split = (KB + p->splits - 1) / p->splits;
   p->tma_conv = p->persist ? tap_persist : tap;
   const int64_t mt_used = p->persist ? mt_pers : mt_tile;
@@ -777,7 +796,8 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
                    (uint32_t)(p->pair ? p->bn / 2 : p->bn));
   if (rc) return rc;
   if (!g.conv && g.A) {
-    rc = make_tmap(&p->tmA, g.dtype, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, (uint32_t)kBM);
+    rc = make_tmap(&p->tmA, g.dtype, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2,
+                   (uint32_t)(p->few ? kFewRows : kBM));
     if (rc) return rc;
   }
   if (p->tma_conv) {
@@ -800,6 +820,11 @@ int launch_tc_gemm(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) 
   if (pl.pair) return launch_tc_pair(g, pl, err, s);
   if (pl.persist) return launch_tc_persist(g, pl, err, s);
   const bool bf = g.dtype == SWAPNET_BF16;
+  if (pl.few) {
+    if (pl.bn == 64) return bf ? launch_inst<__nv_bfloat16, 64, kAFew>(g, pl, err, s) : launch_inst<__half, 64, kAFew>(g, pl, err, s);
+    if (pl.bn == 128) return bf ? launch_inst<__nv_bfloat16, 128, kAFew>(g, pl, err, s) : launch_inst<__half, 128, kAFew>(g, pl, err, s);
+    return bf ? launch_inst<__nv_bfloat16, 256, kAFew>(g, pl, err, s) : launch_inst<__half, 256, kAFew>(g, pl, err, s);
+  }
   if (g.nseg > 1) {
     if (pl.bn == 64)
       return bf ? launch_inst<__nv_bfloat16, 64, kA2d, kTcMaxSeg>(g, pl, err, s) : launch_inst<__half, 64, kA2d, kTcMaxSeg>(g, pl, err, s);
@@ -814,7 +839,6 @@ int launch_tc_gemm(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) 
     return bf ? launch_inst<__nv_bfloat16, 128, kAGather>(g, pl, err, s) : launch_inst<__half, 128, kAGather>(g, pl, err, s);
   }
   if (pl.bn == 64) return bf ? launch_inst<__nv_bfloat16, 64, kA2d>(g, pl, err, s) : launch_inst<__half, 64, kA2d>(g, pl, err, s);
-  if (pl.bn == 256) return bf ? launch_inst<__nv_bfloat16, 256, kA2d>(g, pl, err, s) : launch_inst<__half, 256, kA2d>(g, pl, err, s);
   return bf ? launch_inst<__nv_bfloat16, 128, kA2d>(g, pl, err, s) : launch_inst<__half, 128, kA2d>(g, pl, err, s);
 }
 

@@ -164,6 +164,7 @@ struct TcPlan {
   int64_t tiles;    // output tiles
   int persist;      // persistent kernel (one CTA per SM looping over tiles)
   int tma_conv;     // convolution A by 4-D TMA per filter tap (tmA is then 4-D)
+  int few;          // per-tile kernel on at most 16 rows (A boxes of 16 rows)
   int pair;         // persistent on pairs of SMs: tiles of 256 x bn, bn any multiple of 32 up to 256
   int msub;         // persistent: 128-row sub-tiles per tile (2 for N tiles of 64 with A by TMA)
   int wt, ht, tiles_w, tiles_h;  // its output patch and patch counts per image

@@ -46,6 +46,23 @@ def test_tile_epilogue(dtype, act, res_post, rows, k, n):
     _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
 
 
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("rows,k,n,n_tile,splits", [
+    (5, 8, 8, 64, 1),          # one ragged k-block, one piece of 8 columns
+    (16, 72, 1001, 64, 1),     # odd width
+    (15, 1336, 77, 64, 7),     # column shares of 16: the last splits own none
+    (9, 1992, 130, 64, 8),
+    (8, 3264, 3778, 128, 4),
+    (13, 64, 9793, 128, 1),    # one k-block
+    (7, 1032, 19551, 256, 1),
+    (16, 4872, 10561, 256, 3),  # shares of 88 columns, the last of 80
+])
+def test_few_row_gemm(dtype, rows, k, n, n_tile, splits):
+    rs = _check([_linear(-1, k, n, "relu")], (rows, 1, 1, k), dtype)
+    t = rs.engine.unit_tiling()[0]
+    assert (t["n_tile"], t["splits"], t["persistent"]) == (n_tile, splits, 0)
+
+
 @pytest.mark.parametrize("hw", [160, 220])
 def test_sub_tiles_with_a_residual(hw):
     """Two and four 128-row sub-tiles per tile, the residual of the next
