@@ -167,12 +167,15 @@ __global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, con
                                                           T* __restrict__ vc, const int* __restrict__ pos_ptr,
                                                           int heads, int dh, float theta, int max_seq, int* err) {
   using Vec = typename RopeVec<NP>::type;
-  pdl_wait();
-  pdl_launch_dependents();
   const int t = blockIdx.y;
   const int chunks = dh / (2 * NP);  // chunks of NP pairs in a head
   const int id = blockIdx.x * blockDim.x + threadIdx.x;
   const int ch = id % chunks, h0 = id / chunks * HPT;
+  float inv[NP];
+#pragma unroll
+  for (int u = 0; u < NP; ++u) inv[u] = powf(theta, -2.0f * (float)(ch * NP + u) / (float)dh);
+  pdl_wait();
+  pdl_launch_dependents();  // after the wait: attention_split_kernel reads older cache rows before its own
   if (h0 >= heads) return;
   const int pos = *pos_ptr + t;
   if (pos >= max_seq) {
@@ -192,10 +195,7 @@ __global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, con
   }
   float sn[NP], cs[NP];
 #pragma unroll
-  for (int u = 0; u < NP; ++u) {
-    const float inv = powf(theta, -2.0f * (float)(ch * NP + u) / (float)dh);
-    sincosf((float)pos * inv, &sn[u], &cs[u]);
-  }
+  for (int u = 0; u < NP; ++u) sincosf((float)pos * inv[u], &sn[u], &cs[u]);
   auto rotate = [&](const Vec& x) {
     Vec y;
     const T* e = reinterpret_cast<const T*>(&x);
@@ -236,13 +236,22 @@ __global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, con
 //   phase 3: a_c[d] = sum_j p_j v_j[d]: thread (key group g, 8-dim slice)
 //            over keys g, g + 16, ... with 16-byte loads (the first eight of
 //            them issued before phase 1, so that they arrive during it),
-//            then the 16 groups added in index order.
-// After a cluster barrier the cluster's first CTA reads every chunk's
-// (m_c, l_c, a_c) through distributed shared memory and combines them in
-// chunk order: M = max m_c, L = sum l_c e^(m_c - M),
-// out[d] = sum a_c[d] e^(m_c - M) / L  (chunks past the visible keys hold
-// l_c = 0 and are skipped).  The result is that of one exact softmax over
-// all visible keys, with every sum in a fixed order.
+//            then the two groups of each warp and the warps in index order.
+// Every CTA leaves (m_c, l_c, a_c) in the shared memory of the cluster's
+// first CTA, which after a cluster barrier combines them in chunk order:
+// M = max m_c, L = sum l_c e^(m_c - M), out[d] = sum a_c[d] e^(m_c - M) / L
+// (chunks past the visible keys hold l_c = 0 and are skipped).  The result is
+// that of one exact softmax over all visible keys, with every sum in a fixed
+// order.
+// A decode step is bound by this chain of latencies (at 32 heads and 540
+// keys its 8.9 MB would take 1.3 us).  The cache rows of earlier runs are
+// requested while rope_append_kernel still runs: it lets this kernel start
+// only after every launch before it has completed.  With the rotation, 32
+// heads of 540 keys: 7.35 us with all loads after the wait and the results
+// read by the first CTA one after the other, 6.7 with the results pushed,
+// 5.75 with the early loads.  (The rotation within this launch: 6.9, and
+// 4.5 us more inside a decode step, where its clusters can only be placed
+// once the projections have left; the small rotation grid hides that.)
 constexpr int kDh = 128;
 constexpr int kSpThreads = 256;
 constexpr int kSpMaxSplit = 8;      // portable cluster size
@@ -276,42 +285,60 @@ __device__ __forceinline__ float sp_block_reduce(float v, float* red, bool is_ma
   return r;
 }
 
+// Shared memory, in floats: one partial sum per warp, the cluster's a_c and
+// (m_c, l_c) (used in the first CTA), the reductions' partials, the chunk's
+// scores.
+constexpr int kSpWarps = kSpThreads / 32;
+constexpr int kSpPart = kSpWarps * kDh, kSpAcc = kSpMaxSplit * kDh;
+constexpr int kSpFixed = kSpPart + kSpAcc + 2 * kSpMaxSplit + kSpWarps;
+
+size_t attention_split_smem_bytes(int chunk) { return sizeof(float) * (kSpFixed + (size_t)chunk); }
+
+// (kc and vc are written by the launch that this one overlaps: no read-only loads)
 template <typename T>
-__global__ void __launch_bounds__(kSpThreads) attention_split_kernel(const T* __restrict__ q,
-                                                                     const T* __restrict__ kc,
-                                                                     const T* __restrict__ vc,
-                                                                     const int* __restrict__ pos_ptr, int width,
-                                                                     int max_seq, int chunk, T* __restrict__ out) {
-  extern __shared__ float sp_smem[];
-  float* part = sp_smem;                         // 16 groups x kDh partial sums
-  float* acc = part + 16 * kDh;                  // kDh: this chunk's a_c
-  float* ml = acc + kDh;                         // m_c, l_c
-  float* red = ml + 2;                           // kSpThreads / 32 partials
-  float* sc = red + kSpThreads / 32;             // chunk scores
+__global__ void __launch_bounds__(kSpThreads, 2)
+    attention_split_kernel(const T* q, const T* kc, const T* vc, const int* pos_ptr, int width, int max_seq, int chunk,
+                           T* out) {
+  extern __shared__ __align__(16) float sp_smem[];
+  float* part = sp_smem;
+  float* acc = part + kSpPart;
+  float* ml = acc + kSpAcc;
+  float* red = ml + 2 * kSpMaxSplit;
+  float* sc = red + kSpWarps;
   cg::cluster_group cluster = cg::this_cluster();
-  pdl_wait();
-  pdl_launch_dependents();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // started: its shared memory may be written
+  const int tid = threadIdx.x;
   const int c = (int)cluster.block_rank();
   const int split = (int)cluster.num_blocks();
   const int h = blockIdx.y, t = blockIdx.z;
-  const int tid = threadIdx.x;
-  const int n = min(*pos_ptr + t + 1, max_seq);
+  const int pos0 = *pos_ptr;
+  const int n = min(pos0 + t + 1, max_seq);
   const int j0 = c * chunk, j1 = min(j0 + chunk, n);
+  const int jo = min(j1, pos0);  // keys from pos0 on belong to this run
   const int64_t col = (int64_t)h * kDh;
+  const int sl = tid & 15, kq = tid >> 4;
+  const T* kcol = kc + col + sl * 8;
+  const T* vcol = vc + col + sl * 8;
   const float scale = rsqrtf((float)kDh);
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  auto row = [&](const T* p, int j) { return *reinterpret_cast<const uint4*>(p + (int64_t)j * width); };
+  // the first four passes of keys and the first kSpVPre value rows this
+  // thread sums in phase 3 (keys kq, kq + 16, ... of the chunk both)
+  uint4 ku[4], vpre[kSpVPre];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int j = j0 + kq + r * kSpKeysPerPass;
+    ku[r] = j < jo ? row(kcol, j) : zero;
+  }
+#pragma unroll
+  for (int r = 0; r < kSpVPre; ++r) {
+    const int j = j0 + kq + r * 16;
+    vpre[r] = j < jo ? row(vcol, j) : zero;
+  }
+  pdl_wait();
+  pdl_launch_dependents();
   float m_c = -INFINITY, l_c = 0.f;
   if (j0 < j1) {
-    const int sl = tid & 15, kq = tid >> 4;
-    // the first kSpVPre value rows this thread sums in phase 3 (keys
-    // kq, kq + 16, ... of the chunk), requested now so that they arrive
-    // while the scores and the softmax are computed
-    uint4 vpre[kSpVPre];
-#pragma unroll
-    for (int r = 0; r < kSpVPre; ++r) {
-      const int j = j0 + kq + r * 16;
-      vpre[r] = j < j1 ? *reinterpret_cast<const uint4*>(vc + (int64_t)j * width + col + sl * 8)
-                       : make_uint4(0u, 0u, 0u, 0u);
-    }
     // phase 1: lane group of 16 per key, 8 dims per thread
     float qv[8];
     {
@@ -320,14 +347,26 @@ __global__ void __launch_bounds__(kSpThreads) attention_split_kernel(const T* __
 #pragma unroll
       for (int i = 0; i < 8; ++i) qv[i] = to_f<T>(e[i]);
     }
-    float mx = -INFINITY;
-    for (int jb = j0; jb < j1; jb += 4 * kSpKeysPerPass) {
-      uint4 ku[4];
+    if (jo < j1) {
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        const int j = jb + r * kSpKeysPerPass + kq;
-        ku[r] = j < j1 ? *reinterpret_cast<const uint4*>(kc + (int64_t)j * width + col + sl * 8)
-                       : make_uint4(0u, 0u, 0u, 0u);
+        const int j = j0 + kq + r * kSpKeysPerPass;
+        if (j >= jo && j < j1) ku[r] = row(kcol, j);
+      }
+#pragma unroll
+      for (int r = 0; r < kSpVPre; ++r) {
+        const int j = j0 + kq + r * 16;
+        if (j >= jo && j < j1) vpre[r] = row(vcol, j);
+      }
+    }
+    float mx = -INFINITY;
+    for (int jb = j0; jb < j1; jb += 4 * kSpKeysPerPass) {
+      if (jb > j0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int j = jb + r * kSpKeysPerPass + kq;
+          ku[r] = j < j1 ? row(kcol, j) : zero;
+        }
       }
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
@@ -354,78 +393,66 @@ __global__ void __launch_bounds__(kSpThreads) attention_split_kernel(const T* __
       l += pj;
     }
     l_c = sp_block_reduce(l, red, false);  // the barriers inside also publish sc[]
-    // phase 3: key group g = tid / 16, dims 8 * (tid % 16) .. + 7
-    const int g = tid >> 4;
+    // phase 3: key group kq, dims 8 * sl .. + 7
     float a[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) a[i] = 0.f;
-    const T* vcol = vc + col + sl * 8;
-#pragma unroll
-    for (int r = 0; r < kSpVPre; ++r) {
-      const int j = j0 + g + r * 16;
+    auto add = [&](const uint4& vv, int j) {
       if (j < j1) {
         const float pj = sc[j - j0];
-        const T* e = reinterpret_cast<const T*>(&vpre[r]);
+        const T* e = reinterpret_cast<const T*>(&vv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) a[i] = fmaf(pj, to_f<T>(e[i]), a[i]);
       }
-    }
-    for (int jb = j0 + g + kSpVPre * 16; jb < j1; jb += 4 * 16) {
+    };
+#pragma unroll
+    for (int r = 0; r < kSpVPre; ++r) add(vpre[r], j0 + kq + r * 16);
+    for (int jb = j0 + kq + kSpVPre * 16; jb < j1; jb += 4 * 16) {
       uint4 vu[4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int j = jb + r * 16;
-        vu[r] = j < j1 ? *reinterpret_cast<const uint4*>(vcol + (int64_t)j * width) : make_uint4(0u, 0u, 0u, 0u);
-      }
+      for (int r = 0; r < 4; ++r) vu[r] = jb + r * 16 < j1 ? row(vcol, jb + r * 16) : zero;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int j = jb + r * 16;
-        if (j < j1) {
-          const float pj = sc[j - j0];
-          const T* e = reinterpret_cast<const T*>(&vu[r]);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) a[i] = fmaf(pj, to_f<T>(e[i]), a[i]);
-        }
-      }
+      for (int r = 0; r < 4; ++r) add(vu[r], jb + r * 16);
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) part[g * kDh + sl * 8 + i] = a[i];
+    for (int i = 0; i < 8; ++i) a[i] += __shfl_xor_sync(0xffffffffu, a[i], 16);
+    if (tid % 32 < 16) {
+      float4* pw = reinterpret_cast<float4*>(part + (tid >> 5) * kDh + sl * 8);
+      pw[0] = make_float4(a[0], a[1], a[2], a[3]);
+      pw[1] = make_float4(a[4], a[5], a[6], a[7]);
+    }
     __syncthreads();
-    if (tid < kDh) {
-      float sum = 0.f;
-      for (int gg = 0; gg < 16; ++gg) sum += part[gg * kDh + tid];
-      acc[tid] = sum;
-    }
-  } else if (tid < kDh) {
-    acc[tid] = 0.f;
+  }
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (j0 < j1 && tid < kDh) {
+    float sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < kSpWarps; ++w) sum += part[w * kDh + tid];
+    cluster.map_shared_rank(acc, 0)[c * kDh + tid] = sum;
   }
   if (tid == 0) {
-    ml[0] = m_c;
-    ml[1] = l_c;
+    float* rml = cluster.map_shared_rank(ml, 0) + 2 * c;
+    rml[0] = m_c;
+    rml[1] = l_c;
   }
-  cluster.sync();  // every chunk's (m_c, l_c, a_c) is visible to the cluster
-  if (c == 0 && tid < kDh) {
+  cluster.sync();  // every chunk's (m_c, l_c, a_c) is visible to the first CTA
+  if (c != 0) return;
+  if (tid < kDh) {
     float M = -INFINITY;
-    for (int r = 0; r < split; ++r) {
-      const float* rml = cluster.map_shared_rank(ml, r);
-      if (rml[1] > 0.f) M = fmaxf(M, rml[0]);
-    }
+#pragma unroll
+    for (int r = 0; r < kSpMaxSplit; ++r)
+      if (r < split && ml[2 * r + 1] > 0.f) M = fmaxf(M, ml[2 * r]);
     float L = 0.f, o = 0.f;
-    for (int r = 0; r < split; ++r) {
-      const float* rml = cluster.map_shared_rank(ml, r);
-      if (rml[1] > 0.f) {
-        const float w = expf(rml[0] - M);
-        L += rml[1] * w;
-        o += cluster.map_shared_rank(acc, r)[tid] * w;
+#pragma unroll
+    for (int r = 0; r < kSpMaxSplit; ++r) {
+      if (r < split && ml[2 * r + 1] > 0.f) {
+        const float w = expf(ml[2 * r] - M);
+        L += ml[2 * r + 1] * w;
+        o += acc[r * kDh + tid] * w;
       }
     }
     out[(int64_t)t * width + col + tid] = from_f<T>(o / L);
   }
-  cluster.sync();  // the first CTA has read every chunk before any CTA exits
-}
-
-size_t attention_split_smem_bytes(int chunk) {
-  return sizeof(float) * (16 * kDh + kDh + 2 + kSpThreads / 32 + (size_t)chunk);
 }
 
 // ------------------------------------------------------------ argmax

@@ -145,6 +145,7 @@ def test_swiglu_extreme_gates(rows):
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("tokens,heads,pos,max_seq", [
     (1, 8, 0, 40), (1, 8, 299, 300),                    # one query: the split-key kernel, first and last position
+    (3, 4, 62, 200), (5, 2, 510, 4096), (127, 1, 130, 1030),  # the run's own keys across chunks and load passes
     (15, 8, 200, 400), (16, 8, 200, 400),               # either side of 128 (query, head) pairs
     (63, 8, 20, 128), (64, 8, 64, 128),                 # a cache of one key tile: either side of 512 pairs
     (128, 1, 0, 129), (129, 1, 127, 256), (130, 2, 126, 1000),  # query and key tiles full, one over
