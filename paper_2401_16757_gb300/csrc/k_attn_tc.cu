@@ -153,14 +153,28 @@ __global__ void __launch_bounds__(kAThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t tO = tmem + 256;
-  // q, the caches and the position are written by the kernel before
-  pdl_wait();
-  pdl_launch_dependents();
+  // The launch before rotates q and appends the run's own cache rows; it let
+  // this one start only after every launch before it had completed, so the
+  // position and the key and value tiles of earlier runs are read already.
   const int pos0 = *p.pos_ptr;
   const int last_q = min(t0 + kAQ, p.tokens) - 1;
   const int n_keys = max(0, min(pos0 + last_q + 1, p.max_seq));
   const int nkt = (n_keys + kAK - 1) / kAK;
   const int col0 = h * kAD;
+  auto load_kv = [&](int kt) {
+    const int s = kt & 1;
+    mbar_arrive_expect_tx(kv_full(s), 2 * kTile);
+    const uint32_t ks = smem_u32(smem + kOffK + s * kTile), vs = smem_u32(smem + kOffV + s * kTile);
+    tma_load_2d(ks, &tmK, kv_full(s), col0, kt * kAK);
+    tma_load_2d(ks + kHalf, &tmK, kv_full(s), col0 + 64, kt * kAK);
+    tma_load_2d(vs, &tmV, kv_full(s), col0, kt * kAK);
+    tma_load_2d(vs + kHalf, &tmV, kv_full(s), col0 + 64, kt * kAK);
+  };
+  const int early = max(0, min(min(2, nkt), pos0 / kAK));  // whole tiles of older rows, one per buffer
+  if (warp == 0 && elect_one())
+    for (int kt = 0; kt < early; ++kt) load_kv(kt);
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp == 0) {
     if (elect_one()) {
@@ -168,16 +182,10 @@ __global__ void __launch_bounds__(kAThreads, 1)
       mbar_arrive_expect_tx(q_full, kTile);
       tma_load_2d(smem_u32(smem + kOffQ), &tmQ, q_full, col0, t0);
       tma_load_2d(smem_u32(smem + kOffQ + kHalf), &tmQ, q_full, col0 + 64, t0);
-      int kt = 0;
+      int kt = early;
       for (; kt < nkt; ++kt) {
-        const int s = kt & 1;
-        if (kt >= 2 && !mbar_wait_bounded(kv_empty(s), ((kt >> 1) - 1) & 1, abort_flag, p.err)) break;
-        mbar_arrive_expect_tx(kv_full(s), 2 * kTile);
-        const uint32_t ks = smem_u32(smem + kOffK + s * kTile), vs = smem_u32(smem + kOffV + s * kTile);
-        tma_load_2d(ks, &tmK, kv_full(s), col0, kt * kAK);
-        tma_load_2d(ks + kHalf, &tmK, kv_full(s), col0 + 64, kt * kAK);
-        tma_load_2d(vs, &tmV, kv_full(s), col0, kt * kAK);
-        tma_load_2d(vs + kHalf, &tmV, kv_full(s), col0 + 64, kt * kAK);
+        if (kt >= 2 && !mbar_wait_bounded(kv_empty(kt & 1), ((kt >> 1) - 1) & 1, abort_flag, p.err)) break;
+        load_kv(kt);
       }
       // let every load issued land before the CTA can exit
       volatile int no_abort = 0;
