@@ -31,10 +31,20 @@
 // 512 queries of 32 heads 24.0 us with one thread per query, the scores read
 // twice and every phase waiting for the one before, 14.5 us now; 79 queries
 // on a cache of 100, 8 heads, 14.2 -> 9.3 us (both alone, launch included).
+// Few queries on a long cache leave most SMs idle and the key tiles one
+// after the other: then a cluster of 3 to 8 CTAs shares a (query tile,
+// head)'s key tiles (SPLIT; tile kt to CTA kt mod parts, parts known once the
+// position is), and the CTAs' (m, l, O) are combined in CTA order through
+// distributed shared memory, M = max m, O = sum O e^(m - M) / sum l e^(m - M).
+// On 900 earlier keys: 64 queries of 8 heads 18.9 -> 9.7 us, 512 of 8 heads
+// 27.1 -> 15.2, 128 of 32 heads 21.9 -> 16.2; a nearly empty cache of 1500
+// keys pays 0.4-0.8 us for the possibility.
 // Every wait is bounded: on timeout the kernel records kDevErrTimeout, drains
 // the loads and MMAs it started, frees TMEM and returns.
+#include <cooperative_groups.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 #include <type_traits>
 
@@ -63,6 +73,10 @@ constexpr int kOffX = kOffPl + kTile;  // [half][query] floats
 constexpr int kOffBar = kOffX + 2 * kAQ * 4;
 constexpr int kASmem = kOffBar + 128 + 1024;  // + barriers, TMEM slot, flags; + alignment slack
 static_assert(kASmem <= 232448, "attention tile set exceeds the shared memory of a CTA");
+constexpr int kAMaxSplit = 8;   // portable cluster size
+constexpr int kORow = kAD + 4;  // floats of an output row handed to the cluster (over the key and value tiles)
+static_assert(kAQ * kORow * 4 <= 4 * kTile, "the output rows overlay the key and value tiles");
+
 constexpr uint32_t kTmemCols = 512;  // S: [0, 128) and [128, 256), O_t: [256, 384)
 
 // Shared-memory descriptor of a B operand stored MN-major with the 128-byte
@@ -80,11 +94,16 @@ __device__ __forceinline__ uint64_t smem_desc_sw128_mn(uint32_t addr) {
   return d;
 }
 
+// Sharing a query tile's keys out costs about 2 us (the cluster's barriers,
+// the outputs through distributed shared memory), a key tile 1.6 us.
+__host__ __device__ inline bool split_pays(int tiles, int split) { return tiles - (tiles + split - 1) / split >= 3; }
+
 struct AttnArgs {
   void* out;
   const int* pos_ptr;
   int tokens, heads, width, max_seq;
   float scale_log2;  // log2(e) / sqrt(head width)
+  int split;         // CTAs of a cluster that may share a (query tile, head)'s keys
   int* err;
 };
 
@@ -108,7 +127,7 @@ template <> __device__ __forceinline__ float2 unpack2<__nv_bfloat16>(uint32_t u)
   return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
 }
 
-template <typename T>
+template <typename T, bool SPLIT>
 __global__ void __launch_bounds__(kAThreads, 1)
     attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const AttnArgs p) {
@@ -161,40 +180,45 @@ __global__ void __launch_bounds__(kAThreads, 1)
   const int n_keys = max(0, min(pos0 + last_q + 1, p.max_seq));
   const int nkt = (n_keys + kAK - 1) / kAK;
   const int col0 = h * kAD;
-  auto load_kv = [&](int kt) {
-    const int s = kt & 1;
+  // this CTA's key tiles: z, z + parts, ...
+  const int z = SPLIT ? blockIdx.z : 0;
+  const int parts = SPLIT && split_pays(nkt, p.split) ? min(p.split, nkt) : 1;
+  const int nloc = z < parts ? (nkt - z + parts - 1) / parts : 0;
+  auto load_kv = [&](int i) {
+    const int s = i & 1, k0 = (z + i * parts) * kAK;
     mbar_arrive_expect_tx(kv_full(s), 2 * kTile);
     const uint32_t ks = smem_u32(smem + kOffK + s * kTile), vs = smem_u32(smem + kOffV + s * kTile);
-    tma_load_2d(ks, &tmK, kv_full(s), col0, kt * kAK);
-    tma_load_2d(ks + kHalf, &tmK, kv_full(s), col0 + 64, kt * kAK);
-    tma_load_2d(vs, &tmV, kv_full(s), col0, kt * kAK);
-    tma_load_2d(vs + kHalf, &tmV, kv_full(s), col0 + 64, kt * kAK);
+    tma_load_2d(ks, &tmK, kv_full(s), col0, k0);
+    tma_load_2d(ks + kHalf, &tmK, kv_full(s), col0 + 64, k0);
+    tma_load_2d(vs, &tmV, kv_full(s), col0, k0);
+    tma_load_2d(vs + kHalf, &tmV, kv_full(s), col0 + 64, k0);
   };
-  const int early = max(0, min(min(2, nkt), pos0 / kAK));  // whole tiles of older rows, one per buffer
+  // whole tiles of older rows, one per buffer
+  const int early = min(min(2, nloc), (max(pos0, 0) / kAK + parts - 1 - z) / parts);
   if (warp == 0 && elect_one())
-    for (int kt = 0; kt < early; ++kt) load_kv(kt);
+    for (int i = 0; i < early; ++i) load_kv(i);
   pdl_wait();
   pdl_launch_dependents();
 
   if (warp == 0) {
-    if (elect_one()) {
+    if (nloc > 0 && elect_one()) {
       // ---------------- TMA producer
       mbar_arrive_expect_tx(q_full, kTile);
       tma_load_2d(smem_u32(smem + kOffQ), &tmQ, q_full, col0, t0);
       tma_load_2d(smem_u32(smem + kOffQ + kHalf), &tmQ, q_full, col0 + 64, t0);
-      int kt = early;
-      for (; kt < nkt; ++kt) {
-        if (kt >= 2 && !mbar_wait_bounded(kv_empty(kt & 1), ((kt >> 1) - 1) & 1, abort_flag, p.err)) break;
-        load_kv(kt);
+      int i = early;
+      for (; i < nloc; ++i) {
+        if (i >= 2 && !mbar_wait_bounded(kv_empty(i & 1), ((i >> 1) - 1) & 1, abort_flag, p.err)) break;
+        load_kv(i);
       }
       // let every load issued land before the CTA can exit
       volatile int no_abort = 0;
       mbar_wait_bounded(q_full, 0, &no_abort, nullptr);
-      for (int j = (kt > 2 ? kt - 2 : 0); j < kt; ++j)
+      for (int j = (i > 2 ? i - 2 : 0); j < i; ++j)
         mbar_wait_bounded(kv_full(j & 1), (j >> 1) & 1, &no_abort, nullptr);
     }
   } else if (warp == 1) {
-    if (elect_one()) {
+    if (nloc > 0 && elect_one()) {
       // ---------------- MMA issuer
       constexpr int bf = std::is_same<T, __nv_bfloat16>::value ? 1 : 0;
       constexpr uint32_t idesc_s = idesc_f16(bf, kAQ, kAK);
@@ -202,8 +226,8 @@ __global__ void __launch_bounds__(kAThreads, 1)
       const uint64_t qd = smem_desc_sw128(smem_u32(smem + kOffQ)), kd = smem_desc_sw128(smem_u32(smem + kOffK));
       const uint64_t pd[2] = {smem_desc_sw128(smem_u32(smem + kOffPh)), smem_desc_sw128(smem_u32(smem + kOffPl))};
       const uint64_t vd = smem_desc_sw128_mn(smem_u32(smem + kOffV));
-      // scores of tile kt into TMEM buffer kt % 2 (read by the softmax of
-      // tile kt - 2, which has handed its P over by now)
+      // scores of the CTA's tile kt into TMEM buffer kt % 2 (read by the
+      // softmax of tile kt - 2, which has handed its P over by now)
       auto scores = [&](int kt) -> bool {
         const uint32_t b = (uint32_t)(kt & 1);
         if (!mbar_wait_bounded(kv_full(b), (kt >> 1) & 1, abort_flag, p.err)) return false;
@@ -218,9 +242,9 @@ __global__ void __launch_bounds__(kAThreads, 1)
         tc_commit(s_full(b));
         return true;
       };
-      bool ok = mbar_wait_bounded(q_full, 0, abort_flag, p.err) && nkt > 0 && scores(0);
-      for (int kt = 0; ok && kt < nkt; ++kt) {
-        if (kt + 1 < nkt && !scores(kt + 1)) break;
+      bool ok = mbar_wait_bounded(q_full, 0, abort_flag, p.err) && scores(0);
+      for (int kt = 0; ok && kt < nloc; ++kt) {
+        if (kt + 1 < nloc && !scores(kt + 1)) break;
         if (!mbar_wait_bounded(p_full, kt & 1, abort_flag, p.err)) break;
         tc_fence_after();
         const uint64_t vt = vd + (uint32_t)(kt & 1) * (uint32_t)(kTile >> 4);
@@ -277,8 +301,8 @@ __global__ void __launch_bounds__(kAThreads, 1)
         for (int i = 0; i < 16; ++i) o[c0 + i] = fmaf(o[c0 + i], alpha, __uint_as_float(r[i]));
       }
     };
-    for (int kt = 0; kt < nkt; ++kt) {
-      const int b = kt & 1, k0 = kt * kAK + half * 64;  // this thread's first key
+    for (int kt = 0; kt < nloc; ++kt) {
+      const int b = kt & 1, k0 = (z + kt * parts) * kAK + half * 64;  // this thread's first key
       ok = ok && mbar_wait_bounded(s_full(b), (kt >> 1) & 1, abort_flag, p.err);
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
@@ -301,11 +325,12 @@ __global__ void __launch_bounds__(kAThreads, 1)
       }
       xch[half * kAQ + row] = mx;
       pair_sync();
-      // key 0 is visible to every query: the maximum is finite from tile 0 on
+      // (key 0 is visible to every query; a row may see none of another CTA's tiles)
       mx = fmaxf(m, fmaxf(mx, xch[(half ^ 1) * kAQ + row]));
+      const float base = SPLIT && mx == -INFINITY ? 0.f : mx;
       pair_sync();  // read by both before either writes again
       if (kt > 0) add_tile(kt - 1);  // and P may be written again
-      alpha = exp2f((m - mx) * p.scale_log2);  // 0 on the first tile (m = -inf)
+      alpha = exp2f((m - base) * p.scale_log2);  // 0 on the first tile (m = -inf)
       m = mx;
       if (ok) {
         float lt = 0.f;
@@ -314,8 +339,8 @@ __global__ void __launch_bounds__(kAThreads, 1)
           uint32_t hi[4], lo[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const float p0 = exp2f((__uint_as_float(s[8 * c + 2 * i]) - mx) * p.scale_log2);
-            const float p1 = exp2f((__uint_as_float(s[8 * c + 2 * i + 1]) - mx) * p.scale_log2);
+            const float p0 = exp2f((__uint_as_float(s[8 * c + 2 * i]) - base) * p.scale_log2);
+            const float p1 = exp2f((__uint_as_float(s[8 * c + 2 * i + 1]) - base) * p.scale_log2);
             lt += p0;
             lt += p1;
             hi[i] = pack2<T>(p0, p1);
@@ -336,12 +361,21 @@ __global__ void __launch_bounds__(kAThreads, 1)
         mbar_arrive(p_full);
       }
     }
-    if (nkt > 0) {
-      add_tile(nkt - 1);
+    if (nloc > 0) {
+      add_tile(nloc - 1);
       xch[half * kAQ + row] = l;
       pair_sync();
       const float other = xch[(half ^ 1) * kAQ + row];
-      if (ok && tq < p.tokens) {
+      if (SPLIT && parts > 1) {
+        pair_sync();  // both have read
+        if (half == 0) {
+          xch[row] = m;
+          xch[kAQ + row] = l + other;
+        }
+        float4* mine = reinterpret_cast<float4*>(smem + kOffK) + row * (kORow / 4) + half * 16;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) mine[c] = make_float4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+      } else if (ok && tq < p.tokens) {
         const float inv = 1.0f / (half ? other + l : l + other);
         uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + (int64_t)tq * p.width + col0 + half * 64);
 #pragma unroll
@@ -359,6 +393,50 @@ __global__ void __launch_bounds__(kAThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (SPLIT && parts > 1) {
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    // a warp per row, four columns per lane: rows shared out over the CTAs
+    // (several rows at a time take registers that the tile loop needs)
+    const int rows = min(kAQ, p.tokens - t0);
+    if (z < parts && warp >= 2) {
+      float* x = reinterpret_cast<float*>(smem + kOffX);
+      float4* ov = reinterpret_cast<float4*>(smem + kOffK);
+      for (int row = (warp - 2) * parts + z; row < rows; row += parts * (kASoft / 32)) {
+        float mr[kAMaxSplit], lr[kAMaxSplit], M = -INFINITY;
+        float4 v[kAMaxSplit];
+#pragma unroll
+        for (int c = 0; c < kAMaxSplit; ++c) {
+          if (c < parts) {
+            const float* rx = cluster.map_shared_rank(x, c);
+            mr[c] = rx[row];
+            lr[c] = rx[kAQ + row];
+            v[c] = cluster.map_shared_rank(ov, c)[row * (kORow / 4) + lane];
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < kAMaxSplit; ++c)
+          if (c < parts) M = fmaxf(M, mr[c]);
+        float L = 0.f;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < kAMaxSplit; ++c) {
+          if (c < parts) {
+            const float w = exp2f((mr[c] - M) * p.scale_log2);  // 0 where no key of the CTA is visible
+            L = fmaf(lr[c], w, L);
+            a.x = fmaf(v[c].x, w, a.x);
+            a.y = fmaf(v[c].y, w, a.y);
+            a.z = fmaf(v[c].z, w, a.z);
+            a.w = fmaf(v[c].w, w, a.w);
+          }
+        }
+        const float inv = 1.0f / L;
+        *reinterpret_cast<uint2*>(static_cast<T*>(p.out) + (int64_t)(t0 + row) * p.width + col0 + lane * 4) =
+            make_uint2(pack2<T>(a.x * inv, a.y * inv), pack2<T>(a.z * inv, a.w * inv));
+      }
+    }
+    cluster.sync();  // every row has been read before any CTA exits
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
@@ -371,13 +449,42 @@ int done(cudaError_t e, const char* what) {
   return SWAPNET_OK;
 }
 
+// Clusters of c CTAs of this kernel that the device runs at once (cached per size and device).
+template <typename T> int active_clusters(int c) {
+  static std::atomic<int> cached[64][kAMaxSplit + 1];  // the count + 1, 0 until known
+  const int dev = device_index();
+  if (dev >= 0) {
+    const int v = cached[dev][c].load(std::memory_order_relaxed);
+    if (v > 0) return v - 1;
+  }
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(1, 1, c);
+  cfg.blockDim = dim3(kAThreads);
+  cfg.dynamicSmemBytes = kASmem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = c;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, attention_tc_kernel<T, true>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  if (dev >= 0) cached[dev][c].store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+
 template <typename T>
 int launch_t(const void* q, const void* kc, const void* vc, const int* pos_ptr, int tokens, int heads, int width,
              int max_seq, void* out, int* err, cudaStream_t s) {
   static std::atomic<uint64_t> attr_done{0};
-  auto kern = attention_tc_kernel<T>;
   if (attr_needed(attr_done)) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(attention_tc_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem) != cudaSuccess ||
+        cudaFuncSetAttribute(attention_tc_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem) != cudaSuccess)
       return done(cudaGetLastError(), "attention shared memory");
     attr_set(attr_done);
   }
@@ -399,16 +506,28 @@ int launch_t(const void* q, const void* kc, const void* vc, const int* pos_ptr, 
   a.err = err;
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((tokens + kAQ - 1) / kAQ, heads);
+  // the widest split of a cache's key tiles whose clusters all run at once;
+  // not two: 64 clusters of two cost 2 us more on a short prefix (32 heads,
+  // 256 tokens on 200 keys of a 1500-key cache 13.8 us unsplit, 15.9) and
+  // save 3.8 on 900 keys
+  const int tiles = (max_seq + kAK - 1) / kAK, ctas = (tokens + kAQ - 1) / kAQ * heads;
+  a.split = std::min(tiles, kAMaxSplit);
+  while (a.split > 1 && ctas > active_clusters<T>(a.split)) --a.split;
+  if (a.split < 3 || !split_pays(tiles, a.split)) a.split = 1;
+  cfg.gridDim = dim3((tokens + kAQ - 1) / kAQ, heads, a.split);
   cfg.blockDim = dim3(kAThreads);
   cfg.dynamicSmemBytes = kASmem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = a.split;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return done(cudaLaunchKernelEx(&cfg, kern, tq, tk, tv, a), "tensor-core attention launch");
+  cfg.numAttrs = a.split > 1 ? 2 : 1;
+  return done(cudaLaunchKernelEx(&cfg, a.split > 1 ? attention_tc_kernel<T, true> : attention_tc_kernel<T, false>, tq, tk, tv, a), "tensor-core attention launch");
 }
 
 }  // namespace
