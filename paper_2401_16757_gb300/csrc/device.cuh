@@ -242,6 +242,18 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
   return d;
 }
 
+// The same for a 64-byte-swizzled tile: rows of 64 bytes, 8-row groups 512
+// bytes apart, swizzle mode 4 (64B).
+__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
 // Instruction descriptor, kind::f16: fp32 accumulator, A/B both fp16 (0)
 // or both bf16 (1), both K-major, shape M x N.
 __host__ __device__ constexpr uint32_t idesc_f16(int ab_bf16, int M, int N) {

@@ -495,11 +495,11 @@ int make_tmap_conv4d(CUtensorMap* m, int dtype, const void* base, int n, int h, 
     SN_FAIL(SWAPNET_ERR_MISALIGNED, "TMA conv operand must be 16-byte aligned");
   const cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
   const cuuint64_t strides[3] = {(cuuint64_t)c * 2, (cuuint64_t)w * c * 2, (cuuint64_t)h * w * c * 2};
-  const cuuint32_t box[4] = {(cuuint32_t)kBK, (cuuint32_t)(wt * stride), (cuuint32_t)(ht * stride), 1};
+  const cuuint32_t box[4] = {(cuuint32_t)(c == kTap2C ? kTap2C : kBK), (cuuint32_t)(wt * stride), (cuuint32_t)(ht * stride), 1};
   const cuuint32_t estr[4] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1};
   const CUresult r = fn(m, dtype == SWAPNET_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
                         4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        c == kTap2C ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS)
     SN_FAIL(SWAPNET_ERR_CUDA, "cuTensorMapEncodeTiled (conv) failed (" + std::to_string((int)r) + ")");
@@ -722,12 +722,13 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
   int wt = 0, ht = 0;
   int64_t patches = 0;
   bool tap = false, tap_persist = false;
-  if (g.conv && g.C % kBK == 0) {
+  const bool pair_taps = g.conv && g.C == kTap2C && Nd <= 128;  // two taps per k-block
+  if (g.conv && (g.C % kBK == 0 || pair_taps)) {
     const double util = conv_patch(g.Ho, g.Wo, g.stride, &wt, &ht);
     if (wt > 0)
       patches = (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * ((g.Wo + wt - 1) / wt) * ((g.Ho + ht - 1) / ht);
     tap_persist = wt > 0 && util >= 0.75;
-    tap = tap_persist || (wt > 0 && patches <= mt);
+    tap = !pair_taps && (tap_persist || (wt > 0 && patches <= mt));
   }
   const bool gather = g.conv && !tap;
   const int nseg = std::max(1, g.nseg);
@@ -761,19 +762,25 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
     if (pbn == 256 && mt_pers * ((Nd + 255) / 256) * 2 <= sms) pbn = 128;  // twice the CTAs
     // N tiles of 64 with A by TMA: four (else two) 128-row sub-tiles per
     // tile share each weight stage when that still leaves a tile per SM
+    // and is not slower for the tiles' last round (3x3 64 -> 64 at batch 8,
+    // 112x112: 16.5 us with four, 12.1 so; batch 16, 224x224: 84.3, 69.7)
     int msub = 1;
+    auto us_of = [&](int ms) { return persist_us(pbn, ms, (mt_pers + ms - 1) / ms * ((Nd + pbn - 1) / pbn), KB, sms); };
+    double one = us_of(1);
     if (pbn == 64 && (!g.conv || tap_persist)) {
-      if ((mt_pers + 3) / 4 * ((Nd + 63) / 64) >= sms) msub = 4;
-      else if ((mt_pers + 1) / 2 * ((Nd + 63) / 64) >= sms) msub = 2;
+      for (int ms : {2, 4}) {
+        if ((mt_pers + ms - 1) / ms * ((Nd + 63) / 64) < sms || us_of(ms) > one) continue;
+        msub = ms;
+        one = us_of(ms);
+      }
     }
-    const double one = persist_us(pbn, msub, (mt_pers + msub - 1) / msub * ((Nd + pbn - 1) / pbn), KB, sms);
     if (one < best && nseg == 1) {
       best = one;
       p->persist = 1;
       p->bn = pbn;
       p->msub = msub;
     }
-    if (mt_pers > 1 && (!g.conv || tap_persist)) {
+    if (mt_pers > 1 && (!g.conv || (tap_persist && !pair_taps))) {
       double two = 0.0;
       const int bn2 = pair_tile(mt_pers, Nd, nseg, KB, sms, &two);
       if (two < best) {

@@ -19,7 +19,11 @@
 // gather), kATap (convolution A by one 4-D TMA per k-block: the 64 channels
 // of one filter tap at a wt x ht patch of output pixels, the image border
 // and the stride handled by the copy engine's zero fill and element stride;
-// the output tile is then that patch, rows >= wt * ht unused).
+// the output tile is then that patch, rows >= wt * ht unused), kATap2 (the
+// same for 32 channels: a k-block is two taps, each a 64-byte-swizzled half
+// of the A tile; past the last tap the channel coordinate is out of range,
+// zero fill: 3x3 32 -> 64 at 208x208 13.1 -> 7.0 us against the gather, whose
+// address work and 16-byte copies bound it, batch 16 at 112x112 46.0 -> 19.4).
 // A ring of shared-memory stages (full / empty mbarriers) feeds the MMAs,
 // continuous across tiles.  The accumulator is double-buffered in TMEM
 // (2 x BN columns, tfull / tempty mbarriers): the MMAs of the next tile run
@@ -64,7 +68,8 @@ template <int BN, int MS> struct PCfg {
   static_assert(2 * MS * BN <= 512, "TMEM holds 512 fp32 columns");
 };
 
-constexpr int kAT2d = 0, kAGather = 1, kATap = 2;
+constexpr int kAT2d = 0, kAGather = 1, kATap = 2, kATap2 = 3;
+constexpr int kPAHalf = kPA / 2;
 
 template <int BN, int AMODE, int MS> constexpr int persist_threads() {
   return 64 + 32 * PCfg<BN, MS>::kEpiWarps + (AMODE == kAGather ? 128 : 0);
@@ -74,7 +79,7 @@ template <typename T, int BN, int AMODE, int MS>
 __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
     tc_persist_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const TcArgs p) {
-  constexpr bool GATHER = AMODE == kAGather;
+  constexpr bool GATHER = AMODE == kAGather, TAP2 = AMODE == kATap2, TAP = AMODE == kATap || TAP2;
   static_assert(MS == 1 || !GATHER, "the gather threads cover one 128-row sub-tile");
   using Cfg = PCfg<BN, MS>;
   constexpr int kStages = Cfg::kStages;
@@ -98,9 +103,9 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
   // m-tiles: 128-row blocks of the output matrix, or pixel patches (kATap)
   const int hw = p.Ho * p.Wo;
   const int patches = p.tiles_w * p.tiles_h;
-  const int mt = AMODE == kATap ? (p.M / hw) * patches : (p.M + kPBM - 1) / kPBM;
+  const int mt = TAP ? (p.M / hw) * patches : (p.M + kPBM - 1) / kPBM;
   const int nt = (p.N + BN - 1) / BN;
-  const uint32_t a_bytes = AMODE == kATap ? (uint32_t)(p.wt * p.ht * 128) : (AMODE == kAT2d ? kPA : 0);
+  const uint32_t a_bytes = TAP ? (uint32_t)(p.wt * p.ht * 128) : (AMODE == kAT2d ? kPA : 0);
   const int mtp = (mt + MS - 1) / MS;  // tiles along M (MS sub-tiles each)
   const int tiles = mtp * nt;
   const int KB = (p.K + kPBK - 1) / kPBK;
@@ -146,6 +151,13 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
         *m0 = (tile % mtp) * MS * kPBM;
         *n0 = (tile / mtp) * BN;
       };
+      auto tap_pair = [&](uint32_t dst, uint32_t bar, int kb, int x, int y, int img) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int tap = 2 * kb + h, ry = tap / p.kw, rx = tap - ry * p.kw;
+          tma_load_4d(dst + h * kPAHalf, &tmA, bar, ry < p.kh ? 0 : p.C, x + rx, y + ry, img);
+        }
+      };
       auto load_a = [&](int s, int g) {
         const int tile = tile_of(g / KB);
         const int k0 = (g % KB) * kPBK;
@@ -156,6 +168,10 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
           const uint32_t dst = smem_u32(sA + s * Cfg::kSA + sub * kPA);
           if (AMODE == kAT2d) {
             tma_load_2d(dst, &tmA, full_bar(s), k0, idx * kPBM);
+          } else if (TAP2) {
+            const int img = idx / patches, rem = idx - img * patches;
+            const int th = rem / p.tiles_w, tw = rem - th * p.tiles_w;
+            tap_pair(dst, full_bar(s), k0 / kPBK, tw * p.wt * p.stride - p.pad, th * p.ht * p.stride - p.pad, img);
           } else if (AMODE == kATap) {
             const int img = idx / patches, rem = idx - img * patches;
             const int th = rem / p.tiles_w, tw = rem - th * p.tiles_w;
@@ -190,7 +206,7 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
 #pragma unroll
           for (int sub = 0; sub < MS; ++sub) {
             const int idx = (tile % mtp) * MS + sub;
-            if (AMODE == kATap) {
+            if (TAP) {
               const int img = idx / patches, rem = idx - img * patches;
               const int th = rem / p.tiles_w, tw = rem - th * p.tiles_w;
               ay[sub] = tw * p.wt * p.stride - p.pad;
@@ -218,6 +234,7 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
             for (int sub = 0; sub < MS; ++sub) {
               const uint32_t dst = smem_u32(sA + s * Cfg::kSA + sub * kPA);
               if (AMODE == kAT2d) tma_load_2d(dst, &tmA, full_bar(s), kb * kPBK, ay[sub]);
+              else if (TAP2) tap_pair(dst, full_bar(s), kb, ay[sub], az[sub], aw[sub]);
               else tma_load_4d(dst, &tmA, full_bar(s), c0, ay[sub] + rx, az[sub] + ry, aw[sub]);
             }
           }
@@ -249,7 +266,7 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
     if (elect_one()) {
       // ---------------- MMA issuer
       constexpr uint32_t idesc = idesc_f16(std::is_same<T, __nv_bfloat16>::value ? 1 : 0, kPBM, BN);
-      const uint64_t ad0 = smem_desc_sw128(smem_u32(sA)), bd0 = smem_desc_sw128(smem_u32(sB));
+      const uint64_t ad0 = TAP2 ? smem_desc_sw64(smem_u32(sA)) : smem_desc_sw128(smem_u32(sA)), bd0 = smem_desc_sw128(smem_u32(sB));
       uint32_t s = 0, par = 0;
       bool ok = true;
       for (int lt = 0; lt < my_tiles && ok; ++lt) {
@@ -269,7 +286,8 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
           for (int sub = 0; sub < MS; ++sub) {
 #pragma unroll
             for (int k = 0; k < kPBK / 16; ++k)
-              tc_mma_f16(d + (uint32_t)(sub * BN), ad + (uint64_t)(sub * (kPA >> 4)) + 2ull * k, bd + 2ull * k, idesc,
+              tc_mma_f16(d + (uint32_t)(sub * BN), ad + (uint64_t)(sub * (kPA >> 4) + (TAP2 ? (k >> 1) * (kPAHalf >> 4) + 2 * (k & 1) : 2 * k)),
+                         bd + 2ull * k, idesc,
                          (kb | k) != 0);
           }
           tc_commit(empty_bar(s));
@@ -307,7 +325,7 @@ __global__ void __launch_bounds__(persist_threads<BN, AMODE, MS>(), 1)
         const int idx = (tile % mtp) * MS + sub;  // m-tile (or pixel patch) of this sub-tile
         int m = -1;
         if (idx < mt) {
-          if (AMODE == kATap) {
+          if (TAP) {
             const int img = idx / patches, rem = idx - img * patches;
             const int th = rem / p.tiles_w, tw = rem - th * p.tiles_w;
             if (row < p.wt * p.ht) {
@@ -447,7 +465,7 @@ int launch_persist_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_
   a.kh = g.kh; a.kw = g.kw; a.stride = g.stride; a.pad = g.pad;
   a.e = g.e; a.y = g.y; a.ldy = g.ldy; a.err = err;
   a.wt = pl.wt; a.ht = pl.ht; a.tiles_w = pl.tiles_w; a.tiles_h = pl.tiles_h;
-  const int64_t mt = AMODE == kATap ? (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * pl.tiles_w * pl.tiles_h
+  const int64_t mt = AMODE == kATap || AMODE == kATap2 ? (int64_t)g.M / ((int64_t)g.Ho * g.Wo) * pl.tiles_w * pl.tiles_h
                                     : (g.M + kPBM - 1) / kPBM;
   const int64_t tiles = (mt + MS - 1) / MS * ((g.N + BN - 1) / BN);
   const int sms = g.num_sms > 0 ? g.num_sms : 148;
@@ -469,7 +487,13 @@ int launch_persist_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_
 
 template <typename T, int BN>
 int launch_persist_bn(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
+  const bool taps32 = pl.tma_conv && g.C == kTap2C;
+  if constexpr (BN <= 128) {
+    if (taps32 && pl.msub == 1) return launch_persist_inst<T, BN, kATap2, 1>(g, pl, err, s);
+  }
   if constexpr (BN == 64) {  // sub-tiles only with N tiles of 64
+    if (taps32 && pl.msub == 2) return launch_persist_inst<T, BN, kATap2, 2>(g, pl, err, s);
+    if (taps32 && pl.msub == 4) return launch_persist_inst<T, BN, kATap2, 4>(g, pl, err, s);
     if (pl.msub == 4) {
       if (!g.conv) return launch_persist_inst<T, BN, kAT2d, 4>(g, pl, err, s);
       if (pl.tma_conv) return launch_persist_inst<T, BN, kATap, 4>(g, pl, err, s);
@@ -481,6 +505,7 @@ int launch_persist_bn(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t 
       SN_FAIL(SWAPNET_ERR_INVALID_ARG, "persistent GEMM: two sub-tiles need A by TMA");
     }
   }
+  if (taps32) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "persistent GEMM: two taps per k-block need N tiles of 64 or 128");
   if (pl.msub != 1) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "persistent GEMM: sub-tiles need N tiles of 64");
   if (!g.conv) return launch_persist_inst<T, BN, kAT2d, 1>(g, pl, err, s);
   if (pl.tma_conv) return launch_persist_inst<T, BN, kATap, 1>(g, pl, err, s);

@@ -155,6 +155,8 @@ struct TcGemm {
                         // bias may come from the kernel just before set this.
 };
 // Pre-encoded descriptors of one GEMM (built once per layer at load time).
+constexpr int kTap2C = 32;  // channels of a convolution whose k-blocks are two taps (persistent kernel)
+
 struct TcPlan {
   CUtensorMap tmA;  // valid when conv == 0
   CUtensorMap tmB[kTcMaxSeg];

@@ -83,6 +83,21 @@ def test_paired_gemm(dtype, act, res_post, rows, k, n):
     _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
 
 
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("k,stride,cout,hw,batch", [
+    (3, 1, 64, 161, 2),   # an odd number of taps, ragged patches
+    (3, 2, 40, 301, 2),
+    (4, 2, 128, 320, 3),  # an even number, N tiles of 128
+    (5, 1, 64, 104, 32),  # four sub-tiles
+])
+def test_two_taps_per_k_block(dtype, k, stride, cout, hw, batch):
+    """Convolutions of 32 channels on the persistent kernel, A by 4-D TMA."""
+    conv = dict(op="conv", src=[-1], cin=32, cout=cout, kh=k, kw=k, stride=stride, pad=k // 2, act="leaky", res=None,
+                res_post=False)
+    rs = _check([conv, dict(conv, res=0, res_post=True)], (batch, hw, hw, 32), dtype)
+    assert all(t["persistent"] and t["tap_tma"] for t in rs.engine.unit_tiling())
+
+
 @pytest.mark.parametrize("stride,cin,cout,hw,batch", [(1, 64, 256, 52, 3), (2, 128, 160, 75, 5), (1, 64, 96, 57, 4)])
 def test_paired_conv(stride, cin, cout, hw, batch):
     """Convolutions by 4-D TMA on pairs of SMs: patches past the last one, strides, ragged patch edges."""
