@@ -536,13 +536,14 @@ int launch_t(const void* q, const void* kc, const void* vc, const int* pos_ptr, 
 // query and head), whose time grows with queries x heads x keys while this
 // one's is about 6 us and 1.5 us per 128 keys of the cache's filled part
 // (which only the device knows).  Measured, split-key against this, RoPE
-// included: 128 (query, head) pairs on a cache of 100 keys 6.2-10.7 against
-// 6.6 us, of 900 keys 24 against 18.8 us; 1024 pairs 52 against 8.8 and 339
-// against 19 us; caches of at most 128 keys 6.3 against 6.7 us at 256 pairs,
-// 9.9 against 6.8 us at 512.
+// included: 128 (query, head) pairs on 150 keys 7.5-8.1 against 7.7-8.0 us, on
+// 300 keys 11.4 against 9.8, on 1000 23 against 8-11; caches of at most 128
+// keys 4.9-8.0 against 6.3 us at 256 pairs, 7.7-11.2 against 6.3 at 384.
+// (64 pairs on more than 1000 keys, 12.6 against 7.9-10.7, would pay 2 us in
+// a cache that is still nearly empty.)
 bool attention_tc_supported(int dtype, int tokens, int heads, int width, int max_seq) {
   return (dtype == SWAPNET_F16 || dtype == SWAPNET_BF16) && heads > 0 && width == heads * kAD &&
-         (int64_t)tokens * heads >= (max_seq > kAK ? 128 : 512);
+         (int64_t)tokens * heads >= (max_seq > kAK ? 128 : 384);
 }
 
 int launch_attention_tc(int dtype, const void* q, const void* kc, const void* vc, const int* pos_ptr, int tokens,

@@ -162,7 +162,8 @@ def test_swiglu_extreme_gates(rows):
     (1, 8, 0, 40), (1, 8, 299, 300),                    # one query: the split-key kernel, first and last position
     (3, 4, 62, 200), (5, 2, 510, 4096), (127, 1, 130, 1030),  # the run's own keys across chunks and load passes
     (15, 8, 200, 400), (16, 8, 200, 400),               # either side of 128 (query, head) pairs
-    (63, 8, 20, 128), (64, 8, 64, 128),                 # a cache of one key tile: either side of 512 pairs
+    (63, 8, 20, 128), (64, 8, 64, 128),                 # a cache of one key tile
+    (47, 8, 81, 128), (48, 8, 20, 128),                 # the same, either side of 384 pairs
     (128, 2, 200, 400), (40, 4, 1000, 1100), (300, 3, 250, 2000),  # key tiles shared by a cluster: rows that see
     (64, 2, 100, 4000), (513, 8, 300, 900),             # nothing of a CTA's, uneven shares, caches barely filled
     (128, 1, 0, 129), (129, 1, 127, 256), (130, 2, 126, 1000),  # query and key tiles full, one over
