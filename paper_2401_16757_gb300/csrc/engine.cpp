@@ -952,6 +952,30 @@ static bool whole_tc(const swapnet_engine* e, int u) {
          X.tc.splits == 1 && !U.host && U.row0 == 0 && U.rows == L.d.cout && L.d.res == SWAPNET_SRC_NONE;
 }
 
+// Whether the output of layer a and the tensor of layer b (its output) share
+// memory: outputs of the model lie in the output buffer, the rest in the
+// workspace, where a tensor's space is given away after its last reader.
+static bool outputs_overlap(const Model& m, int a, int b) {
+  const Layer &A = m.L[a], &B = m.L[b];
+  if ((A.out_off >= 0) != (B.out_off >= 0)) return false;
+  const int64_t oa = A.out_off >= 0 ? A.out_off : A.ws_off, ob = B.out_off >= 0 ? B.out_off : B.ws_off;
+  return oa < ob + (int64_t)B.out_bytes && ob < oa + (int64_t)A.out_bytes;
+}
+
+// A shared launch of units u .. v writes v's output when unit u runs, earlier
+// than the workspace's lifetimes say, so its space may not yet be given away:
+// neither by an output of the launch that nobody reads (dead at once) nor by
+// a residual whose last reader is in the launch.
+static bool may_join(const swapnet_engine* e, int u, int v) {
+  const Model& m = e->plan.model;
+  const int lv = e->plan.units[v].layer;
+  for (int w = u; w < v; ++w) {
+    const int lw = e->plan.units[w].layer, r = m.L[lw].d.res;
+    if (outputs_overlap(m, lv, lw) || (r != SWAPNET_SRC_NONE && outputs_overlap(m, lv, r))) return false;
+  }
+  return true;
+}
+
 // Merged launches (option merge): inside one block, consecutive whole
 // GEMV layers that read the same input with the same K and rows run as one
 // launch: up to kSkMaxSeg siblings none of which reads another's output
@@ -975,7 +999,8 @@ static void plan_merges(swapnet_engine* e) {
         int k = 1;
         for (; k < kTcMaxSeg && u + k < B.u1 && whole_tc(e, u + k); ++k) {
           const Layer& L = m.L[p.units[u + k].layer];
-          if (L.d.src0 != L0.d.src0 || L.d.cin != L0.d.cin || L.n != L0.n || L.d.cout != L0.d.cout || L.d.act != L0.d.act)
+          if (L.d.src0 != L0.d.src0 || L.d.cin != L0.d.cin || L.n != L0.n || L.d.cout != L0.d.cout ||
+              L.d.act != L0.d.act || !may_join(e, u, u + k))
             break;
         }
         if (k == 1) continue;
@@ -991,7 +1016,7 @@ static void plan_merges(swapnet_engine* e) {
       };
       if (same_input(u + 1)) {
         const Layer& L1 = m.L[p.units[u + 1].layer];
-        if (L1.d.res == p.units[u].layer && L1.d.cout == L0.d.cout) {
+        if (L1.d.res == p.units[u].layer && L1.d.cout == L0.d.cout && may_join(e, u, u + 1)) {
           e->merge_n[u] = 1;
           e->merge_pair[u] = 1;
           e->merged_into[u + 1] = 1;
@@ -1007,7 +1032,7 @@ static void plan_merges(swapnet_engine* e) {
           const int li = p.units[u + i].layer;
           reads_group = reads_group || L.d.res == li || L.d.src0 == li;
         }
-        if (reads_group) break;
+        if (reads_group || !may_join(e, u, u + k)) break;
       }
       if (k == 1) continue;
       e->merge_n[u] = k - 1;

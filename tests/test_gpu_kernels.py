@@ -227,6 +227,30 @@ def test_sibling_linears_share_a_launch(dtype, rows, k, n, count):
     check_close(m, runs[0].decode(got), oracle_outputs(m, w, x))
 
 
+@pytest.mark.parametrize("dtype,rows", [("f16", 2), ("bf16", 200), ("bf16", 1), ("f32", 1)])
+@pytest.mark.parametrize("residual", [False, True])
+def test_siblings_whose_buffers_overlap_run_one_by_one(dtype, rows, residual):
+    """A sibling that would write, in a shared launch, where another one's unread output or its residual lies: the
+    workspace gives both layers one buffer, so they run one after the other."""
+    if residual:
+        layers = [_linear(-1, 256, 256), _linear(0, 256, 256), _linear(-1, 256, 256, "relu", res=1),
+                  _linear(-1, 256, 256), _linear(2, 256, 256, res=3)]
+        early, late = 1, 3
+    else:
+        layers = [_linear(-1, 256, 256), _linear(-1, 256, 256), _linear(1, 256, 256)]
+        early, late = 0, 1
+    m = dict(name="yolov3", model_id=49, dtype=dtype, input=(rows, 1, 1, 256), layers=layers, outputs=[len(layers) - 1])
+    offs = OP.workspace(m)[1]
+    assert offs[early] == offs[late]
+    w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
+    host = capi.HostWeights(w)
+    runs = [Runner(m, w, capi.Plan.resident(d, capi.options(merge=g)), host) for g in (1, 0)]
+    got, sep = (r.run(x) for r in runs)
+    assert [r.engine.stats()["kernel_launches"] for r in runs] == [len(layers)] * 2
+    assert all(a.tobytes() == b.tobytes() for a, b in zip(got, sep))
+    check_close(m, runs[0].decode(got), oracle_outputs(m, w, x))
+
+
 @pytest.mark.parametrize("rows", [2, 4, 5, 8, 9, 16])
 @pytest.mark.parametrize("k,n", [(4, 1), (128, 9), (1020, 40), (1024, 64), (1028, 7), (3000, 130)])
 def test_few_row_fp32_linear(rows, k, n):
