@@ -157,6 +157,44 @@ def test_swiglu_extreme_gates(rows):
     assert torch.all((out - ref).abs() <= ref.abs() * 2.0 ** -8 * 1.01 + 1e-33)
 
 
+_QUOTIENT_SWEEP = r"""
+#include <cstdio>
+#include "tc_epi.cuh"
+using namespace swapnet;
+template <typename T> __device__ float value(unsigned i) {
+  const unsigned short b = (unsigned short)i;
+  return to_f<T>(*reinterpret_cast<const T*>(&b));
+}
+template <> __device__ float value<float>(unsigned i) { return ((int)i - (1 << 25)) * (110.0f / (1 << 25)); }
+template <typename T> __global__ void sweep(unsigned* differ) {
+  const float r = value<T>(blockIdx.x * 256u + threadIdx.x), d = 1.0f + expf(-r);
+  const float a = r / d, b = gate_quotient(r, d);
+  if (__float_as_uint(a) != __float_as_uint(b) && !(isnan(a) && isnan(b))) atomicAdd(differ, 1u);
+}
+int main() {
+  unsigned *n, h;
+  if (cudaMalloc(&n, 4) != cudaSuccess || cudaMemset(n, 0, 4) != cudaSuccess) return 2;
+  sweep<__half><<<256, 256>>>(n);
+  sweep<__nv_bfloat16><<<256, 256>>>(n);
+  sweep<float><<<1 << 18, 256>>>(n);
+  if (cudaMemcpy(&h, n, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return 2;
+  std::printf("%u\n", h);
+  return 0;
+}
+"""
+
+
+def test_gate_quotient_is_the_division(tmp_path):
+    """The SwiGLU epilogue's quotient, bit for bit against the division: every fp16 and bf16 gate, and 2^26 fp32 gates
+    over the range of expf."""
+    import subprocess
+    from paper_2401_16757_gb300 import build
+    src, exe = tmp_path / "sweep.cu", tmp_path / "sweep"
+    src.write_text(_QUOTIENT_SWEEP)
+    subprocess.run([build._nvcc()] + build.ARCH + build.FLAGS + ["-I" + build.CSRC, "-o", str(exe), str(src)], check=True)
+    assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split() == ["0"]
+
+
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("tokens,heads,pos,max_seq", [
     (1, 8, 0, 40), (1, 8, 299, 300),                    # one query: the split-key kernel, first and last position
