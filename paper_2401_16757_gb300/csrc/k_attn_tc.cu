@@ -17,7 +17,8 @@
 //               m (the halves exchange theirs through shared memory) and
 //               denominator l, p = e^(s - m) written to shared memory as two
 //               bf16/fp16 parts p_hi + p_lo (p_lo = round(p - p_hi)), so the
-//               product with V keeps about 16 significant bits of p, not 8
+//               product with V keeps about 16 significant bits of p, not 8;
+//               runs of fewer than 64 queries keep all 24 (SHORT)
 //   O_t = P V   tcgen05.mma, M 128 x N 128 x K 16 steps for each part; V
 //               is the value tile as loaded by TMA (two 64-dim boxes),
 //               [keys][dims] with the dims contiguous, i.e. the B operand in
@@ -63,16 +64,32 @@ constexpr int kASoft = 256;      // softmax threads: two per query
 constexpr int kAThreads = 64 + kASoft;  // warp 0 TMA, warp 1 MMA, warps 2..9 softmax
 constexpr int kHalf = 128 * 64 * 2;  // one 128-row x 64-column swizzled half tile (16 KB)
 constexpr int kTile = 2 * kHalf;     // 128 x 128 elements
-// shared memory: Q | K stage 0, 1 | V stage 0, 1 | P_hi | P_lo | exchange | barriers
+// shared memory: Q | K stage 0, 1 | V stage 0, 1 | P (its parts) | exchange | barriers
 constexpr int kOffQ = 0;
 constexpr int kOffK = kOffQ + kTile;
 constexpr int kOffV = kOffK + 2 * kTile;
-constexpr int kOffPh = kOffV + 2 * kTile;
-constexpr int kOffPl = kOffPh + kTile;
-constexpr int kOffX = kOffPl + kTile;  // [half][query] floats
+constexpr int kOffP = kOffV + 2 * kTile;
+constexpr int kOffX = kOffP + 2 * kTile;  // [half][query] floats
 constexpr int kOffBar = kOffX + 2 * kAQ * 4;
 constexpr int kASmem = kOffBar + 128 + 1024;  // + barriers, TMEM slot, flags; + alignment slack
 static_assert(kASmem <= 232448, "attention tile set exceeds the shared memory of a CTA");
+// SHORT: runs of fewer than 64 queries use half of the MMA's rows, so the room
+// of two parts of P holds three of 64 rows (the MMA's other rows read whatever
+// lies behind them, results nobody uses): p = p_hi + p_mid + p_lo, all of its
+// 24 bits, as the split-key kernel has them for fewer (query, head) pairs.
+// Outputs that are not the rounded float64 result, 63 queries of 8 heads on 900
+// keys, bf16: 2.1e-4 there, 2.2e-3 with two parts, 4.5e-4 so (the rest is the
+// sums of the tensor cores).  The third part costs 0.2-0.6 us per key tile of
+// a CTA (63 x 8 on 900 keys 9.6 -> 9.7 us, 17 x 16 on 3000 14.1 -> 15.9).
+// fp16 parts carry p * 2^15, so that their exponent range takes the small ones.
+constexpr int kShortRows = 64;
+template <bool SHORT> struct PCfg {
+  static constexpr int kParts = SHORT ? 3 : 2;
+  static constexpr int kHalfBytes = SHORT ? kHalf / 2 : kHalf;  // 64 columns of a part
+  static constexpr int kPartBytes = 2 * kHalfBytes;
+  static constexpr int kWriters = SHORT ? kASoft / 2 : kASoft;  // threads that own a row
+  static_assert((kParts - 1) * kPartBytes + kHalfBytes + kHalf <= 2 * kTile, "the parts and the rows behind them");
+};
 constexpr int kAMaxSplit = 8;   // portable cluster size
 constexpr int kORow = kAD + 4;  // floats of an output row handed to the cluster (over the key and value tiles)
 static_assert(kAQ * kORow * 4 <= 4 * kTile, "the output rows overlay the key and value tiles");
@@ -127,10 +144,12 @@ template <> __device__ __forceinline__ float2 unpack2<__nv_bfloat16>(uint32_t u)
   return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
 }
 
-template <typename T, bool SPLIT>
+template <typename T, bool SPLIT, bool SHORT>
 __global__ void __launch_bounds__(kAThreads, 1)
     attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const AttnArgs p) {
+  using P = PCfg<SHORT>;
+  constexpr float kPScale = SHORT && std::is_same<T, __half>::value ? 32768.0f : 1.0f;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
@@ -154,7 +173,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
     }
     mbar_init(s_full(0), 1);
     mbar_init(s_full(1), 1);
-    mbar_init(p_full, kASoft);
+    mbar_init(p_full, P::kWriters);
     mbar_init(o_full, 1);
     mbar_init(done_bar, 1);
     *abort_flag = 0;
@@ -224,7 +243,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
       constexpr uint32_t idesc_s = idesc_f16(bf, kAQ, kAK);
       constexpr uint32_t idesc_pv = idesc_f16(bf, kAQ, kAD) | (1u << 16);  // B (values) MN-major, N = 128
       const uint64_t qd = smem_desc_sw128(smem_u32(smem + kOffQ)), kd = smem_desc_sw128(smem_u32(smem + kOffK));
-      const uint64_t pd[2] = {smem_desc_sw128(smem_u32(smem + kOffPh)), smem_desc_sw128(smem_u32(smem + kOffPl))};
+      const uint64_t pd = smem_desc_sw128(smem_u32(smem + kOffP));
       const uint64_t vd = smem_desc_sw128_mn(smem_u32(smem + kOffV));
       // scores of the CTA's tile kt into TMEM buffer kt % 2 (read by the
       // softmax of tile kt - 2, which has handed its P over by now)
@@ -249,11 +268,11 @@ __global__ void __launch_bounds__(kAThreads, 1)
         tc_fence_after();
         const uint64_t vt = vd + (uint32_t)(kt & 1) * (uint32_t)(kTile >> 4);
 #pragma unroll
-        for (int part = 0; part < 2; ++part) {
+        for (int part = 0; part < P::kParts; ++part) {
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)  // 16 keys per step, all 128 head dims (both 64-wide halves)
-            tc_mma_f16(tO, pd[part] + (uint64_t)((ks >> 2) * (kHalf >> 4) + 2 * (ks & 3)), vt + (uint64_t)(ks * (2048 >> 4)),
-                       idesc_pv, (part | ks) != 0);
+            tc_mma_f16(tO, pd + (uint64_t)((part * P::kPartBytes + (ks >> 2) * P::kHalfBytes) / 16 + 2 * (ks & 3)),
+                       vt + (uint64_t)(ks * (2048 >> 4)), idesc_pv, (part | ks) != 0);
         }
         tc_commit(o_full);
         tc_commit(kv_empty(kt & 1));
@@ -264,7 +283,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
       volatile int no_abort = 0;
       mbar_wait_bounded(done_bar, 0, &no_abort, nullptr);
     }
-  } else {
+  } else if (!SHORT || (warp & 3) < kShortRows / 32) {
     // ---------------- softmax and output: warps 2..9, half a query row per thread
     const int q4 = warp & 3, half = (warp - 2) >> 2;
     const int row = q4 * 32 + lane;
@@ -275,7 +294,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
     // horizon of the warp's first row: keys up to it are visible to all 32
     const int qpos_min = min(pos0 + min(t0 + q4 * 32, p.tokens - 1), p.max_seq - 1);
     const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-    const uint32_t prow = (uint32_t)half * kHalf + (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
+    const uint32_t prow = (uint32_t)half * P::kHalfBytes + (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
     const uint32_t psw = (uint32_t)(row & 7);
     float* xch = reinterpret_cast<float*>(smem + kOffX);
     // the two warps of a row quarter meet here; both take part in every
@@ -336,24 +355,27 @@ __global__ void __launch_bounds__(kAThreads, 1)
         float lt = 0.f;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {  // 8 keys: one 16-byte chunk of each part
-          uint32_t hi[4], lo[4];
+          uint32_t part[P::kParts][4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const float p0 = exp2f((__uint_as_float(s[8 * c + 2 * i]) - base) * p.scale_log2);
             const float p1 = exp2f((__uint_as_float(s[8 * c + 2 * i + 1]) - base) * p.scale_log2);
             lt += p0;
             lt += p1;
-            hi[i] = pack2<T>(p0, p1);
-            const float2 h = unpack2<T>(hi[i]);
-            lo[i] = pack2<T>(p0 - h.x, p1 - h.y);
+            float2 rest = make_float2(p0 * kPScale, p1 * kPScale);
+#pragma unroll
+            for (int j = 0; j < P::kParts; ++j) {
+              part[j][i] = pack2<T>(rest.x, rest.y);
+              const float2 h = unpack2<T>(part[j][i]);
+              rest = make_float2(rest.x - h.x, rest.y - h.y);
+            }
           }
           const uint32_t off = prow + (((uint32_t)c ^ psw) << 4);
-          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(smem_u32(smem + kOffPh) + off), "r"(hi[0]), "r"(hi[1]),
-                       "r"(hi[2]), "r"(hi[3])
-                       : "memory");
-          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(smem_u32(smem + kOffPl) + off), "r"(lo[0]), "r"(lo[1]),
-                       "r"(lo[2]), "r"(lo[3])
-                       : "memory");
+#pragma unroll
+          for (int j = 0; j < P::kParts; ++j)
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(smem_u32(smem + kOffP + j * P::kPartBytes) + off), "r"(part[j][0]),
+                         "r"(part[j][1]), "r"(part[j][2]), "r"(part[j][3])
+                         : "memory");
         }
         l = l * alpha + lt;
         fence_proxy_async_smem();  // P is read by the tensor cores (async proxy)
@@ -376,7 +398,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
 #pragma unroll
         for (int c = 0; c < 16; ++c) mine[c] = make_float4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
       } else if (ok && tq < p.tokens) {
-        const float inv = 1.0f / (half ? other + l : l + other);
+        const float inv = 1.0f / (kPScale * (half ? other + l : l + other));
         uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.out) + (int64_t)tq * p.width + col0 + half * 64);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -430,7 +452,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
             a.w = fmaf(v[c].w, w, a.w);
           }
         }
-        const float inv = 1.0f / L;
+        const float inv = 1.0f / (kPScale * L);
         *reinterpret_cast<uint2*>(static_cast<T*>(p.out) + (int64_t)(t0 + row) * p.width + col0 + lane * 4) =
             make_uint2(pack2<T>(a.x * inv, a.y * inv), pack2<T>(a.z * inv, a.w * inv));
       }
@@ -470,7 +492,7 @@ template <typename T> int active_clusters(int c) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, attention_tc_kernel<T, true>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, attention_tc_kernel<T, true, false>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
@@ -483,9 +505,10 @@ int launch_t(const void* q, const void* kc, const void* vc, const int* pos_ptr, 
              int max_seq, void* out, int* err, cudaStream_t s) {
   static std::atomic<uint64_t> attr_done{0};
   if (attr_needed(attr_done)) {
-    if (cudaFuncSetAttribute(attention_tc_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem) != cudaSuccess ||
-        cudaFuncSetAttribute(attention_tc_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem) != cudaSuccess)
-      return done(cudaGetLastError(), "attention shared memory");
+    for (auto kern : {attention_tc_kernel<T, false, false>, attention_tc_kernel<T, true, false>,
+                      attention_tc_kernel<T, false, true>, attention_tc_kernel<T, true, true>})
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem) != cudaSuccess)
+        return done(cudaGetLastError(), "attention shared memory");
     attr_set(attr_done);
   }
   const int dt = std::is_same<T, __nv_bfloat16>::value ? SWAPNET_BF16 : SWAPNET_F16;
@@ -527,20 +550,23 @@ int launch_t(const void* q, const void* kc, const void* vc, const int* pos_ptr, 
   attr[1].val.clusterDim.z = a.split;
   cfg.attrs = attr;
   cfg.numAttrs = a.split > 1 ? 2 : 1;
-  return done(cudaLaunchKernelEx(&cfg, a.split > 1 ? attention_tc_kernel<T, true> : attention_tc_kernel<T, false>, tq, tk, tv, a), "tensor-core attention launch");
+  const auto kern = tokens < kShortRows
+                        ? (a.split > 1 ? attention_tc_kernel<T, true, true> : attention_tc_kernel<T, false, true>)
+                        : (a.split > 1 ? attention_tc_kernel<T, true, false> : attention_tc_kernel<T, false, false>);
+  return done(cudaLaunchKernelEx(&cfg, kern, tq, tk, tv, a), "tensor-core attention launch");
 }
 
 }  // namespace
 
 // Where this kernel takes over from the split-key one (a cluster of CTAs per
 // query and head), whose time grows with queries x heads x keys while this
-// one's is about 6 us and 1.5 us per 128 keys of the cache's filled part
-// (which only the device knows).  Measured, split-key against this, RoPE
-// included: 128 (query, head) pairs on 150 keys 7.5-8.1 against 7.7-8.0 us, on
-// 300 keys 11.4 against 9.8, on 1000 23 against 8-11; caches of at most 128
-// keys 4.9-8.0 against 6.3 us at 256 pairs, 7.7-11.2 against 6.3 at 384.
-// (64 pairs on more than 1000 keys, 12.6 against 7.9-10.7, would pay 2 us in
-// a cache that is still nearly empty.)
+// one's is about 6.6 us and 2 us per 128 keys of the cache's filled part
+// (which only the device knows) on one CTA.  Measured, split-key against this,
+// RoPE included: 128 (query, head) pairs in a cache of 160 7.1-7.6 against
+// 6.5-8.9 us, of 340 10.6-11.5 against 6.5-11.4, of 1030 13.3-22.9 against
+// 6.8-11.8; caches of at most 128 keys 4.9-8.0 against 6.9 us at 256 pairs,
+// 10.9-11.4 against 6.8 at 384.  (64 pairs on more than 1000 keys, 12.6
+// against 8.5-11, would pay 2 us in a cache that is still nearly empty.)
 bool attention_tc_supported(int dtype, int tokens, int heads, int width, int max_seq) {
   return (dtype == SWAPNET_F16 || dtype == SWAPNET_BF16) && heads > 0 && width == heads * kAD &&
          (int64_t)tokens * heads >= (max_seq > kAK ? 128 : 384);
