@@ -136,6 +136,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
 // the previous kernel in the stream is still running; they must wait here
 // before touching anything that kernel writes.  Every CTA calls it, so a
 // grid never completes before the grids it depends on.
+// What that kernel may write is read by plain loads after the wait: read-only
+// ones (__ldg, `const T* __restrict__` parameters) ask for memory that no one
+// writes while this kernel runs, and the compiler may move them across the
+// wait.  They are for weights alone.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -44,7 +44,7 @@ int done(cudaError_t e, const char* what) {
 // Row t of the output is row ids[t] of the table, read straight from the
 // page-locked host table (device alias) with 16-byte loads.
 template <typename T>
-__global__ void __launch_bounds__(256) embed_kernel(const T* __restrict__ table, const int* __restrict__ ids,
+__global__ void __launch_bounds__(256) embed_kernel(const T* __restrict__ table, const int* ids,
                                                     int vocab, int d, T* __restrict__ out, int* err) {
   pdl_wait();
   pdl_launch_dependents();
@@ -83,7 +83,7 @@ template <typename T> struct Chunk8 {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const T* __restrict__ x, const T* __restrict__ g,
+__global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const T* x, const T* __restrict__ g,
                                                                int d, float eps, T* __restrict__ y, int vec) {
   __shared__ float wsum[kNormThreads / 32];
   pdl_wait();
@@ -162,9 +162,9 @@ template <> struct RopeVec<1> { using type = uint32_t; };
 template <> struct RopeVec<4> { using type = uint4; };
 
 template <typename T, int HPT, int NP>
-__global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, const T* __restrict__ k,
-                                                          const T* __restrict__ v, T* __restrict__ kc,
-                                                          T* __restrict__ vc, const int* __restrict__ pos_ptr,
+__global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, const T* k,
+                                                          const T* v, T* __restrict__ kc,
+                                                          T* __restrict__ vc, const int* pos_ptr,
                                                           int heads, int dh, float theta, int max_seq, int* err) {
   using Vec = typename RopeVec<NP>::type;
   const int t = blockIdx.y;
@@ -294,7 +294,6 @@ constexpr int kSpFixed = kSpPart + kSpAcc + 2 * kSpMaxSplit + kSpWarps;
 
 size_t attention_split_smem_bytes(int chunk) { return sizeof(float) * (kSpFixed + (size_t)chunk); }
 
-// (kc and vc are written by the launch that this one overlaps: no read-only loads)
 template <typename T>
 __global__ void __launch_bounds__(kSpThreads, 2)
     attention_split_kernel(const T* q, const T* kc, const T* vc, const int* pos_ptr, int width, int max_seq, int chunk,
@@ -472,7 +471,7 @@ __device__ __forceinline__ void arg_take(float& best, int& bi, float ov, int oi)
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kArgThreads) argmax_kernel(const T* __restrict__ x, int n, int* __restrict__ out,
+__global__ void __launch_bounds__(kArgThreads) argmax_kernel(const T* x, int n, int* __restrict__ out,
                                                              int vec) {
   __shared__ float sv[kArgThreads / 32];
   __shared__ int si[kArgThreads / 32];

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kGvWarps * 32, MT <= 2 ? 2 : 1) gemv_kernel(co
     const int k = k0 + p * kPass;
 #pragma unroll
     for (int m = 0; m < MT; ++m)
-      b.x[m] = m < j.M && k < K ? __ldg(reinterpret_cast<const uint4*>(x + (int64_t)m * K + k)) : make_uint4(0u, 0u, 0u, 0u);
+      b.x[m] = m < j.M && k < K ? *reinterpret_cast<const uint4*>(x + (int64_t)m * K + k) : make_uint4(0u, 0u, 0u, 0u);
   };
   auto next_load = [&]() {
     if (++lp == passes) {
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kGvWarps * 32, MT <= 2 ? 2 : 1) gemv_kernel(co
 constexpr int kRwWarps = 8;
 
 template <int MT, int FT>
-__global__ void __launch_bounds__(kRwWarps * 32, 2) linear_rows_kernel(const float* __restrict__ x, int M, int K,
+__global__ void __launch_bounds__(kRwWarps * 32, 2) linear_rows_kernel(const float* x, int M, int K,
                                                                        const float* __restrict__ W, int N, Epi e,
                                                                        float* __restrict__ y, int64_t ldy) {
   constexpr int NV = MT * FT;  // sums per lane, a power of two of at least 32
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kRwWarps * 32, 2) linear_rows_kernel(const flo
     float4 xv[MT];
 #pragma unroll
     for (int m = 0; m < MT; ++m)
-      xv[m] = m < M && k < K ? __ldg(reinterpret_cast<const float4*>(x + (int64_t)m * K + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      xv[m] = m < M && k < K ? *reinterpret_cast<const float4*>(x + (int64_t)m * K + k) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -457,7 +457,7 @@ __device__ __forceinline__ void tl_load4(uint32_t dst, const T* base, int r, int
 }
 
 template <typename T, int TM, int TN, int RM, int RN, int BK>
-__global__ void __launch_bounds__(kTlThreads, 2) linear_tiled_kernel(const T* __restrict__ x, int M, int K,
+__global__ void __launch_bounds__(kTlThreads, 2) linear_tiled_kernel(const T* x, int M, int K,
                                                                      const T* __restrict__ W, int N, Epi e,
                                                                      T* __restrict__ y, int64_t ldy, int vec) {
   using C = TlCfg<TM, TN, RM, RN, BK>;
@@ -581,7 +581,7 @@ int tiled_launch(const T* x, int M, int K, const T* W, int N, const Epi& e, T* y
 constexpr int kDcCo = 16;
 
 template <typename T>
-__global__ void __launch_bounds__(128) conv_direct_kernel(const T* __restrict__ x, int n, int h, int w, int cin,
+__global__ void __launch_bounds__(128) conv_direct_kernel(const T* x, int n, int h, int w, int cin,
                                                           const T* __restrict__ W, int cout, int kh, int kw,
                                                           int stride, int pad, int oh, int ow, Epi e,
                                                           T* __restrict__ y) {
@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(128) conv_direct_kernel(const T* __restrict__ 
 
 // ------------------------------------------------------------ pooling etc.
 template <typename T>
-__global__ void maxpool_kernel(const T* __restrict__ x, int n, int h, int w, int c, int kh, int kw, int stride,
+__global__ void maxpool_kernel(const T* x, int n, int h, int w, int c, int kh, int kw, int stride,
                                int pad, int oh, int ow, T* __restrict__ y) {
   pdl_wait();
   pdl_launch_dependents();
@@ -667,7 +667,7 @@ __global__ void maxpool_kernel(const T* __restrict__ x, int n, int h, int w, int
 }
 
 template <typename T>
-__global__ void gap_kernel(const T* __restrict__ x, int n, int hw, int c, T* __restrict__ y) {
+__global__ void gap_kernel(const T* x, int n, int hw, int c, T* __restrict__ y) {
   pdl_wait();
   pdl_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -680,7 +680,7 @@ __global__ void gap_kernel(const T* __restrict__ x, int n, int hw, int c, T* __r
 }
 
 template <typename T>
-__global__ void upsample2x_kernel(const T* __restrict__ x, int n, int h, int w, int c, T* __restrict__ y) {
+__global__ void upsample2x_kernel(const T* x, int n, int h, int w, int c, T* __restrict__ y) {
   pdl_wait();
   pdl_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -695,7 +695,7 @@ __global__ void upsample2x_kernel(const T* __restrict__ x, int n, int h, int w, 
 }
 
 template <typename T>
-__global__ void concat_kernel(const T* __restrict__ a, int ca, const T* __restrict__ b, int cb, int64_t pixels,
+__global__ void concat_kernel(const T* a, int ca, const T* b, int cb, int64_t pixels,
                               T* __restrict__ y) {
   pdl_wait();
   pdl_launch_dependents();
@@ -711,7 +711,7 @@ __global__ void concat_kernel(const T* __restrict__ a, int ca, const T* __restri
 // multiple of the vector width, rows 16-byte aligned).  Max is exact, so
 // the result equals the scalar kernels'.
 template <typename T>
-__global__ void maxpool_vec_kernel(const uint4* __restrict__ x, int n, int h, int w, int cv, int kh, int kw,
+__global__ void maxpool_vec_kernel(const uint4* x, int n, int h, int w, int cv, int kh, int kw,
                                    int stride, int pad, int oh, int ow, uint4* __restrict__ y) {
   constexpr int V = Vec16<T>::N;
   pdl_wait();
@@ -728,14 +728,27 @@ __global__ void maxpool_vec_kernel(const uint4* __restrict__ x, int n, int h, in
   float m[V];
 #pragma unroll
   for (int i = 0; i < V; ++i) m[i] = -INFINITY;
-  for (int r = 0; r < kh; ++r) {
-    const int iy = oy * stride + r - pad;
-    if (iy < 0 || iy >= h) continue;
-    for (int s = 0; s < kw; ++s) {
-      const int ix = ox * stride + s - pad;
-      if (ix < 0 || ix >= w) continue;
+  // four taps' loads in flight at a time
+  const int taps = kh * kw;
+  int r = 0, t = 0;
+  for (int k = 0; k < taps; k += 4) {
+    uint4 v[4];
+    bool ok[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int iy = oy * stride + r - pad, ix = ox * stride + t - pad;
+      ok[u] = k + u < taps && (unsigned)iy < (unsigned)h && (unsigned)ix < (unsigned)w;
+      if (ok[u]) v[u] = x[(((int64_t)img * h + iy) * w + ix) * cv + ch];
+      if (++t == kw) {
+        t = 0;
+        ++r;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (!ok[u]) continue;
       float f[V];
-      unpack16<T>(__ldg(x + (((int64_t)img * h + iy) * w + ix) * cv + ch), f);
+      unpack16<T>(v[u], f);
 #pragma unroll
       for (int i = 0; i < V; ++i) m[i] = fmaxf(m[i], f[i]);
     }
@@ -743,7 +756,7 @@ __global__ void maxpool_vec_kernel(const uint4* __restrict__ x, int n, int h, in
   y[idx] = pack16<T>(m);
 }
 
-__global__ void upsample2x_vec_kernel(const uint4* __restrict__ x, int n, int h, int w, int cv,
+__global__ void upsample2x_vec_kernel(const uint4* x, int n, int h, int w, int cv,
                                       uint4* __restrict__ y) {
   pdl_wait();
   pdl_launch_dependents();
@@ -759,7 +772,7 @@ __global__ void upsample2x_vec_kernel(const uint4* __restrict__ x, int n, int h,
   y[idx] = x[(((int64_t)img * h + oy / 2) * w + ox / 2) * cv + ch];
 }
 
-__global__ void concat_vec_kernel(const uint4* __restrict__ a, int ca, const uint4* __restrict__ b, int cb,
+__global__ void concat_vec_kernel(const uint4* a, int ca, const uint4* b, int cb,
                                   int64_t pixels, uint4* __restrict__ y) {
   pdl_wait();
   pdl_launch_dependents();

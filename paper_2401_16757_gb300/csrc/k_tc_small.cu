@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) tc_conv_small_kernel(const Smal
               const int2 t = tab[kb * 64 + h + u];
               const int iy = iy0 + (t.y >> 16), ix = ix0 + (t.y & 0xffff);
               const bool valid = mv && (unsigned)iy < (unsigned)p.H && (unsigned)ix < (unsigned)p.Wd;
-              e[u] = valid ? __ldg(xw + t.x) : zero;
+              e[u] = valid ? xw[t.x] : zero;
             }
             e2[h >> 1] = bits2<T>(e[0], e[1]);
           }
