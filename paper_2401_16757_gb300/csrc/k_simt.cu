@@ -44,6 +44,15 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
   return r;
 }
 
+// 16 bytes of the launch before's output: a plain load, kept behind the wait
+// (both are volatile) but free to pass this kernel's own stores, none of which
+// writes there.
+__device__ __forceinline__ uint4 ld_input16(const void* p) {
+  uint4 r;
+  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+  return r;
+}
+
 template <typename T> __device__ __forceinline__ void unpack16(const uint4& v, float* f) {
   const T* e = reinterpret_cast<const T*>(&v);
 #pragma unroll
@@ -157,7 +166,7 @@ __global__ void __launch_bounds__(kGvWarps * 32, MT <= 2 ? 2 : 1) gemv_kernel(co
     const int k = k0 + p * kPass;
 #pragma unroll
     for (int m = 0; m < MT; ++m)
-      b.x[m] = m < j.M && k < K ? *reinterpret_cast<const uint4*>(x + (int64_t)m * K + k) : make_uint4(0u, 0u, 0u, 0u);
+      b.x[m] = m < j.M && k < K ? ld_input16(x + (int64_t)m * K + k) : make_uint4(0u, 0u, 0u, 0u);
   };
   auto next_load = [&]() {
     if (++lp == passes) {
