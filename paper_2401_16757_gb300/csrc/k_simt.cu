@@ -69,8 +69,8 @@ template <typename T> __device__ __forceinline__ uint4 pack16(const float* f) {
 
 // ------------------------------------------------------------ GEMV
 // Linear layers of 1 to 4 rows of 16-bit values, or one row of fp32: the time
-// is streaming the weights.  Persistent CTAs (two per SM) take groups of eight
-// weight rows; K is walked in passes, of which a lane takes one 16-byte chunk
+// is streaming the weights.  Persistent CTAs (as many as are resident: two per
+// SM, one with sums for 3 or 4 rows) take groups of eight weight rows; K is walked in passes, of which a lane takes one 16-byte chunk
 // of every row (chunk 32 w + l of the pass for lane l of warp w), so a loaded
 // chunk of x meets eight rows.  The loads of two passes are in flight ahead of
 // the one being summed, across groups, so that a group's reductions and
@@ -91,11 +91,16 @@ template <typename T> __device__ __forceinline__ uint4 pack16(const float* f) {
 // none while it sums, whose last wave of CTAs leaves the chip part empty:
 // 11008 x 4096 bf16 19.0 -> 13.7 us (6.6 TB/s, launch included), 4096 x 11008
 // 19.1 -> 15.0, 4096 x 4096 (from L2) 6.1 -> 4.4, 32000 x 4096 40.2 -> 36.7.
+// Four rows of 4096 x 4096 14.5 -> 9.0 (FMAs and conversions; 9.6 with twice the
+// CTAs that fit).
 constexpr int kGvWarps = 8;
 constexpr int kGvRows = 8;  // weight rows per group
+// CTAs of an instance on an SM: 118-124 registers a thread with sums for one
+// or two rows of x, 206 with four.
+constexpr int gv_ctas(int mt) { return mt <= 2 ? 2 : 1; }
 
 template <typename T, int MT>
-__global__ void __launch_bounds__(kGvWarps * 32, MT <= 2 ? 2 : 1) gemv_kernel(const SkJob j, const int groups) {
+__global__ void __launch_bounds__(kGvWarps * 32, gv_ctas(MT)) gemv_kernel(const SkJob j, const int groups) {
   constexpr int V = Vec16<T>::N;
   constexpr int NV = MT * kGvRows;
   constexpr int kPass = kGvWarps * 32 * V;  // k per pass
@@ -375,6 +380,12 @@ cudaError_t rows_launch(const SkJob& j, cudaStream_t s) {
                     static_cast<float*>(g.y), g.ldy);
 }
 
+template <typename T, int MT> int gemv_launch(const SkJob& j, int groups, cudaStream_t s) {
+  const int grid = std::max(1, std::min(groups, gv_ctas(MT) * std::max(1, j.num_sms)));
+  const cudaError_t e = launch_pdl(gemv_kernel<T, MT>, dim3(grid), dim3(kGvWarps * 32), 0, s, j, groups);
+  return e == cudaSuccess ? SWAPNET_OK : SWAPNET_ERR_CUDA;
+}
+
 template <typename T> int skinny_dispatch(const SkJob& j, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
     if (skinny_rows_kernel(SWAPNET_F32, j.M)) {
@@ -387,14 +398,13 @@ template <typename T> int skinny_dispatch(const SkJob& j, cudaStream_t s) {
   int groups = (j.seg[0].N + per - 1) / per;
   if (!j.pair)
     for (int i = 1; i < j.nseg; ++i) groups += (j.seg[i].N + per - 1) / per;
-  const dim3 grid(std::max(1, std::min(groups, 2 * std::max(1, j.num_sms)))), block(kGvWarps * 32);
-  cudaError_t e;
-  if (j.M <= 1) e = launch_pdl(gemv_kernel<T, 1>, grid, block, 0, s, j, groups);
-  else if (j.M <= 2) e = launch_pdl(gemv_kernel<T, 2>, grid, block, 0, s, j, groups);
-  else if (j.M <= 4) e = launch_pdl(gemv_kernel<T, 4>, grid, block, 0, s, j, groups);
-  else SN_FAIL(SWAPNET_ERR_UNSUPPORTED, "skinny linear: more rows than the GEMV takes");  // 16-bit layers of 5 rows and
-                                                                                          // more run on the tensor cores
-  return e == cudaSuccess ? SWAPNET_OK : SWAPNET_ERR_CUDA;
+  if (j.M <= 1) return gemv_launch<T, 1>(j, groups, s);
+  if constexpr (sizeof(T) == 2) {  // (fp32 layers of more rows have been launched above)
+    if (j.M <= 2) return gemv_launch<T, 2>(j, groups, s);
+    if (j.M <= 4) return gemv_launch<T, 4>(j, groups, s);
+  }
+  // 16-bit layers of 5 rows and more run on the tensor cores
+  SN_FAIL(SWAPNET_ERR_UNSUPPORTED, "skinny linear: more rows than the GEMV takes");
 }
 
 // ------------------------------------------------------------ tiled linear
