@@ -218,10 +218,15 @@ typedef struct swapnet_options {
                                      together.  Objective 0, two slots, no resident
                                      prefix.  Consecutive inferences of one engine must
                                      be issued on one stream (as for any engine). */
-  int32_t merge;                 /* 1 (default): linear layers of one block that read
-                                     the same input (e.g. q, k, v; a SwiGLU gate and
-                                     up projection) run as one launch; 0: one launch
-                                     per layer.  Results are identical either way;
+  int32_t merge;                 /* 1 (default): consecutive whole linear layers of one
+                                     block that read the same input run as one launch:
+                                     up to three (e.g. q, k, v), or a SwiGLU gate and
+                                     its up projection, of up to 4 rows (fp32: 16);
+                                     with more rows on the tensor cores up to three of
+                                     equal width and activation without a residual
+                                     whose K is not split.  Layers whose buffers
+                                     overlap stay apart.  0: one launch per layer.
+                                     Results are identical either way;
                                      profiling gives every layer of a merged launch
                                      that launch's start and end. */
   int32_t pageable;              /* 0 (default): the host weights are page-locked

@@ -933,13 +933,12 @@ static bool small_conv_ok(const Model& m, const Layer& L) {
 
 static int plan_side(swapnet_engine* e);
 
-// A whole (unsplit) linear layer on the GEMV kernel, its weights in the arena
-// or read in place.
+// A whole (unsplit) linear layer on the GEMV or few-row fp32 kernel, its
+// weights in the arena or read in place.
 static bool whole_skinny(const swapnet_engine* e, int u) {
   const Unit& U = e->plan.units[u];
   const Layer& L = e->plan.model.L[U.layer];
-  return e->unit_kind[u] == SWAPNET_KERNEL_SKINNY && !skinny_rows_kernel(e->plan.model.dtype, L.n) && !U.host &&
-         U.row0 == 0 && U.rows == L.d.cout;
+  return e->unit_kind[u] == SWAPNET_KERNEL_SKINNY && !U.host && U.row0 == 0 && U.rows == L.d.cout;
 }
 
 // A whole linear layer on the tensor-core kernels, without residual and
@@ -976,9 +975,9 @@ static bool may_join(const swapnet_engine* e, int u, int v) {
   return true;
 }
 
-// Merged launches (option merge): inside one block, consecutive whole
-// GEMV layers that read the same input with the same K and rows run as one
-// launch: up to kSkMaxSeg siblings none of which reads another's output
+// Merged launches (option merge): inside one block, consecutive whole GEMV
+// (or few-row fp32) layers that read the same input with the same K and rows
+// run as one launch: up to kSkMaxSeg siblings none of which reads another's output
 // (e.g. the q, k, v projections), or a pair whose second layer takes the
 // first's output as its residual and nothing else of it (e.g. gate and up
 // of a SwiGLU feed-forward).  Siblings of equal width and activation on the
@@ -1075,8 +1074,8 @@ static int run_group(swapnet_engine* e, int u, const void* din, void* dout, cuda
     const Layer& L = m.L[p.units[v].layer];
     const UnitExec& X = e->ux[v];
     const char* r = L.d.res == SWAPNET_SRC_NONE ? nullptr : act_ptr(e, L.d.res, din, dout);
-    j.seg[i] = SkSeg{X.w, Epi{X.b, r, L.d.cout, L.d.act, L.d.res_post}, L.d.cout,
-                     out_ptr(e, p.units[v].layer, dout), L.d.cout};
+    j.seg[i] = SkSeg{X.w, L.d.cout, Epi{X.b, r, L.d.cout, L.d.act, L.d.res_post}, out_ptr(e, p.units[v].layer, dout),
+                     L.d.cout};
   }
   j.num_sms = e->num_sms;
   return launch_linear_skinny_job(m.dtype, j, s);

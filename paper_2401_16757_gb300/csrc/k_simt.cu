@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kGvWarps * 32, gv_ctas(MT)) gemv_kernel(const 
 }
 
 // ------------------------------------------------------------ few-row fp32 linear
-// fp32 layers of kRowsMin to 16 rows: one CTA per FT output features, K walked
+// fp32 layers of 2 to 16 rows: one CTA per FT output features, K walked
 // in chunks of 1024, of which warp w takes the k 128 w .. + 127 and lane l four
 // of them.  Weights and x come straight from global memory, 16 bytes per lane
 // and row, every load of a chunk in flight at once (the first chunk's weights
@@ -299,25 +299,49 @@ __global__ void __launch_bounds__(kGvWarps * 32, gv_ctas(MT)) gemv_kernel(const 
 // L1 once per feature and warp: 8 x 1024 x 1024, weights in L2, 6.3 us
 // in a chain of layers, 2.3 with this; 8 x 4096 x 4096 79 -> 13 us; 16 x 2048 x
 // 2048 26 -> 7.8. One row alone is left to the GEMV (1024 x 1024 1.8 against 1.9).
+// Six blocks of three siblings, a SwiGLU pair and a layer, width 256, 8 rows:
+// 41.0 us with shared launches, 59.5 with one each (1024: 112.6, 122.8).
 constexpr int kRwWarps = 8;
 
-template <int MT, int FT>
-__global__ void __launch_bounds__(kRwWarps * 32, 2) linear_rows_kernel(const float* x, int M, int K,
-                                                                       const float* __restrict__ W, int N, Epi e,
-                                                                       float* __restrict__ y, int64_t ldy) {
+// One launch may serve several layers that read the same x, as the GEMV's: the
+// CTAs are dealt to the segments in order, or (pair) a CTA takes FT / 2 features
+// of the gate and of its paired layer.  NS: layers that a launch may hold (1 or
+// kSkMaxSeg; a layer alone does not carry the parameters of three).
+template <int NS> struct RowsJob {
+  const float* x;
+  int M, K, nseg, pair;
+  SkSeg seg[NS];
+};
+
+template <int MT, int FT, int NS>
+__global__ void __launch_bounds__(kRwWarps * 32, 2) linear_rows_kernel(const RowsJob<NS> j) {
+  constexpr bool MULTI = NS > 1;
   constexpr int NV = MT * FT;  // sums per lane, a power of two of at least 32
   static_assert(NV >= 32 && (NV & (NV - 1)) == 0 && NV <= kRwWarps * 32, "halving reduction");
   __shared__ float red[kRwWarps][NV];
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int o0 = blockIdx.x * FT;
+  const int M = j.M, K = j.K;
+  const float* x = j.x;
+  const bool pair = MULTI && j.pair;
+  const int per = pair ? FT / 2 : FT;  // features of a layer per CTA
+  int cta = blockIdx.x, si = 0;
+  if (MULTI && !pair)
+    while (si + 1 < j.nseg && cta >= (j.seg[si].N + FT - 1) / FT) cta -= (j.seg[si++].N + FT - 1) / FT;
+  SkSeg S = j.seg[0];
+#pragma unroll
+  for (int i = 1; i < NS; ++i)
+    if (i == si) S = j.seg[i];
+  const int o0 = cta * per;
   const int k0 = warp * 128 + lane * 4;
   float4 w[FT];
   auto load_w = [&](int k) {
 #pragma unroll
     for (int f = 0; f < FT; ++f) {
+      const bool up = pair && f >= FT / 2;  // the paired layer's half
+      const int o = o0 + (up ? f - FT / 2 : f);
       w[f] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (o0 + f < N && k < K) {
-        const uint4 u = ld_stream16(W + (int64_t)(o0 + f) * K + k);
+      if (o < S.N && k < K) {
+        const uint4 u = ld_stream16(static_cast<const float*>(up ? j.seg[NS > 1].W : S.W) + (int64_t)o * K + k);
         w[f] = make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w));
       }
     }
@@ -360,24 +384,37 @@ __global__ void __launch_bounds__(kRwWarps * 32, 2) linear_rows_kernel(const flo
 #pragma unroll
   for (int i = 0; i < NV / 32; ++i) red[warp][lane * (NV / 32) + i] = v[i];
   __syncthreads();
-  const int i = threadIdx.x, m = i / FT, o = o0 + i % FT;
-  if (i < NV && m < M && o < N) {
+  const int m = threadIdx.x / per, f = threadIdx.x % per, o = o0 + f;
+  if (m >= M || o >= S.N) return;
+  auto total = [&](int i) {
     float s = red[0][i];
 #pragma unroll
     for (int h = 1; h < kRwWarps; ++h) s += red[h][i];
-    const float* bias = static_cast<const float*>(e.bias);
-    const float* res = static_cast<const float*>(e.res);
-    y[(int64_t)m * ldy + o] = epilogue(s, bias ? bias[o] : 0.f, res ? res[(int64_t)m * e.ldr + o] : 0.f, res != nullptr, e.act,
-                                       e.res_post);
-  }
+    return s;
+  };
+  auto emit = [&](const SkSeg& q, float s, float r, bool has_r) {
+    const float* bias = static_cast<const float*>(q.e.bias);
+    const float out = epilogue(s, bias ? bias[o] : 0.f, r, has_r, q.e.act, q.e.res_post);
+    static_cast<float*>(q.y)[(int64_t)m * q.ldy + o] = out;
+    return out;
+  };
+  const float* res = static_cast<const float*>(S.e.res);
+  const float gate = emit(S, total(m * FT + f), res ? res[(int64_t)m * S.e.ldr + o] : 0.f, res != nullptr);
+  if (pair) emit(j.seg[NS > 1], total(m * FT + f + FT / 2), gate, true);
 }
 
-template <int MT, int FT>
-cudaError_t rows_launch(const SkJob& j, cudaStream_t s) {
-  const SkSeg& g = j.seg[0];
-  return launch_pdl(linear_rows_kernel<MT, FT>, dim3((g.N + FT - 1) / FT), dim3(kRwWarps * 32), 0, s,
-                    static_cast<const float*>(j.x), j.M, j.K, static_cast<const float*>(g.W), g.N, g.e,
-                    static_cast<float*>(g.y), g.ldy);
+template <int MT, int FT, int NS>
+int rows_launch_ns(const SkJob& j, cudaStream_t s) {
+  RowsJob<NS> r{static_cast<const float*>(j.x), j.M, j.K, j.nseg, j.pair, {}};
+  for (int i = 0; i < NS; ++i) r.seg[i] = j.seg[i];
+  const int per = j.pair ? FT / 2 : FT;
+  int ctas = (j.seg[0].N + per - 1) / per;
+  for (int i = 1; i < j.nseg && !j.pair; ++i) ctas += (j.seg[i].N + per - 1) / per;
+  const cudaError_t e = launch_pdl(linear_rows_kernel<MT, FT, NS>, dim3(ctas), dim3(kRwWarps * 32), 0, s, r);
+  return e == cudaSuccess ? SWAPNET_OK : SWAPNET_ERR_CUDA;
+}
+template <int MT, int FT> int rows_launch(const SkJob& j, cudaStream_t s) {
+  return j.nseg > 1 ? rows_launch_ns<MT, FT, kSkMaxSeg>(j, s) : rows_launch_ns<MT, FT, 1>(j, s);
 }
 
 template <typename T, int MT> int gemv_launch(const SkJob& j, int groups, cudaStream_t s) {
@@ -388,11 +425,7 @@ template <typename T, int MT> int gemv_launch(const SkJob& j, int groups, cudaSt
 
 template <typename T> int skinny_dispatch(const SkJob& j, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (skinny_rows_kernel(SWAPNET_F32, j.M)) {
-      if (j.nseg != 1) SN_FAIL(SWAPNET_ERR_UNSUPPORTED, "few-row fp32 linear: one layer per launch");
-      const cudaError_t e = j.M <= 4 ? rows_launch<4, 8>(j, s) : (j.M <= 8 ? rows_launch<8, 8>(j, s) : rows_launch<16, 4>(j, s));
-      return e == cudaSuccess ? SWAPNET_OK : SWAPNET_ERR_CUDA;
-    }
+    if (j.M > 1) return j.M <= 4 ? rows_launch<4, 8>(j, s) : (j.M <= 8 ? rows_launch<8, 8>(j, s) : rows_launch<16, 4>(j, s));
   }
   const int per = j.pair ? kGvRows / 2 : kGvRows;
   int groups = (j.seg[0].N + per - 1) / per;
@@ -826,8 +859,6 @@ static int last_launch() {
   return SWAPNET_OK;
 }
 
-bool skinny_rows_kernel(int dtype, int M) { return dtype == SWAPNET_F32 && M >= kRowsMin; }
-
 int launch_linear_skinny_job(int dtype, const SkJob& j, cudaStream_t s) {
   const int es = dtype_size(dtype);
   if (j.M < 1 || j.M > 16 || j.K < 1 || j.nseg < 1 || j.nseg > kSkMaxSeg || (j.pair && j.nseg != 2))
@@ -849,7 +880,7 @@ int launch_linear_skinny(int dtype, const void* x, int M, int K, const void* W, 
   j.M = M;
   j.K = K;
   j.nseg = 1;
-  j.seg[0] = SkSeg{W, e, N, y, ldy};
+  j.seg[0] = SkSeg{W, N, e, y, ldy};
   j.num_sms = num_sms;
   return launch_linear_skinny_job(dtype, j, s);
 }

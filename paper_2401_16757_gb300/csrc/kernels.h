@@ -48,12 +48,10 @@ struct Epi {
 };
 
 // y[m, col0 + o] (row stride ldy) = epi(sum_k x[m,k] W[o,k]) for o < N,
-// M <= 16.  fp32 / fp16 / bf16; fixed-order reduction (deterministic).
+// fp32 of M <= 16 rows, fp16 / bf16 of M <= 4; fixed-order reduction
+// (deterministic).
 int launch_linear_skinny(int dtype, const void* x, int M, int K, const void* W, int N, const Epi& e, void* y,
                          int64_t ldy, int num_sms, cudaStream_t s);
-// fp32 layers of this many rows run the few-row kernel, one layer per launch.
-constexpr int kRowsMin = 2;
-bool skinny_rows_kernel(int dtype, int M);
 
 // Several skinny linear layers reading the same x (M rows, K columns) in one
 // launch: segment i computes y_i[m, o] = epi_i(sum_k x[m,k] W_i[o,k]) for
@@ -63,8 +61,8 @@ bool skinny_rows_kernel(int dtype, int M);
 constexpr int kSkMaxSeg = 3;
 struct SkSeg {
   const void* W;
+  int N;  // (beside W: what a kernel reads first shares a line of its parameters)
   Epi e;
-  int N;
   void* y;
   int64_t ldy;
 };

@@ -320,6 +320,22 @@ def test_few_row_fp32_linear(rows, k, n):
     assert set(rs.engine.unit_kernels()) == {"skinny_linear"}
 
 
+@pytest.mark.parametrize("rows", [2, 3, 5, 8, 16])
+def test_few_row_fp32_siblings_share_a_launch(rows):
+    """fp32 siblings of ragged widths in one launch, one with a residual, and a gate with its SwiGLU layer in another:
+    the bits of one launch each, and the oracle."""
+    layers = [_linear(-1, 1300, 260), _linear(0, 260, 13), _linear(0, 260, 260, "relu", res=0), _linear(0, 260, 9, bias=False),
+              _linear(2, 260, 36), _linear(2, 260, 36, "swiglu", res=4)]
+    m = dict(name="yolov3", model_id=50, dtype="f32", input=(rows, 1, 1, 1300), layers=layers, outputs=[1, 2, 3, 5])
+    w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
+    host = capi.HostWeights(w)
+    a, b = (Runner(m, w, capi.Plan.resident(d, capi.options(merge=g)), host) for g in (1, 0))
+    got = a.run(x)
+    assert all(p.tobytes() == q.tobytes() for p, q in zip(got, b.run(x)))
+    assert a.engine.stats()["kernel_launches"] == 3 and b.engine.stats()["kernel_launches"] == 6
+    check_close(m, a.decode(got), oracle_outputs(m, w, x))
+
+
 @pytest.mark.parametrize("dtype,rows", [("f16", 1), ("bf16", 1), ("f16", 2), ("bf16", 3), ("f16", 4), ("f32", 1)])
 @pytest.mark.parametrize("k,n", [(8, 1), (2048, 9), (2056, 40), (4104, 300), (11008, 21), (1024, 5000)])
 def test_gemv(dtype, rows, k, n):
