@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
   // The launch before rotates q and appends the run's own cache rows; it let
   // this one start only after every launch before it had completed, so the
   // position and the key and value tiles of earlier runs are read already.
-  const int pos0 = *p.pos_ptr;
+  const int pos0 = min(*p.pos_ptr, p.max_seq);  // (a position outside the cache is reported by the rotation)
   const int last_q = min(t0 + kAQ, p.tokens) - 1;
   const int n_keys = max(0, min(pos0 + last_q + 1, p.max_seq));
   const int nkt = (n_keys + kAK - 1) / kAK;

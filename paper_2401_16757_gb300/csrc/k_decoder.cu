@@ -177,11 +177,12 @@ __global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, con
   pdl_wait();
   pdl_launch_dependents();  // after the wait: attention_split_kernel reads older cache rows before its own
   if (h0 >= heads) return;
-  const int pos = *pos_ptr + t;
-  if (pos >= max_seq) {
+  const int pos0 = *pos_ptr;
+  if (pos0 < 0 || pos0 >= max_seq - t) {  // (no sum that could overflow)
     if (id == 0) atomicExch(err, kDevErrBounds);
     return;
   }
+  const int pos = pos0 + t;
   const int width = heads * dh;
   Vec qv[HPT], kv[HPT], vv[HPT];
 #pragma unroll
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(kSpThreads, 2)
   const int c = (int)cluster.block_rank();
   const int split = (int)cluster.num_blocks();
   const int h = blockIdx.y, t = blockIdx.z;
-  const int pos0 = *pos_ptr;
+  const int pos0 = min(*pos_ptr, max_seq);  // (a position outside the cache is reported by the rotation)
   const int n = min(pos0 + t + 1, max_seq);
   const int j0 = c * chunk, j1 = min(j0 + chunk, n);
   const int jo = min(j1, pos0);  // keys from pos0 on belong to this run

@@ -267,6 +267,43 @@ def test_attention_of_short_runs_keeps_fp32_probabilities(tokens, heads, pos, ma
     assert float((out != ref.to(torch.bfloat16).double()).double().mean()) <= 2.0 ** -10
 
 
+@pytest.mark.parametrize("tokens,heads", [(1, 8), (3, 2), (64, 8), (130, 32)])
+@pytest.mark.parametrize("pos", ["full", -1, -100, 2 ** 31 - 1, -2 ** 31])
+def test_positions_outside_the_cache_are_refused(tokens, heads, pos):
+    """A cache position that leaves no room for the run, or none at all (negative, or so large that adding the run
+    overflows): reported by the next sync, nothing written around the cache, and the engine usable afterwards."""
+    import torch
+    d, max_seq, guard = heads * 128, 160, 1 << 20
+    if pos == "full":
+        pos = max_seq - tokens + 1
+    m = dict(name="llm", model_id=51, dtype="bf16", input=(tokens, 1, 1, d), outputs=[3],
+             layers=[_linear(-1, d, d, bias=False), _linear(-1, d, d, bias=False), _linear(-1, d, d, bias=False),
+                     dict(op="attention", src=[0, 1, 2], heads=heads, max_seq=max_seq, theta=10000.0)])
+    w, x = synth.gen.model_weights(m), synth.gen.model_input(m)
+    r = Runner(m, w, capi.Plan.resident(capi.Desc(m)))
+    size = r.info["state_bytes"]
+    memory = torch.full((2 * guard + size,), 0x3c, dtype=torch.uint8, device="cuda")
+    state = memory[guard:guard + size]
+    r.engine.bind_state(state.data_ptr(), size)
+    state[:4].view(torch.int32).fill_(0)
+    good = r.run(x)
+    state.fill_(0x3c)
+    state[:4].view(torch.int32).fill_(pos)
+    with pytest.raises(capi.SwapnetError) as ei:
+        r.run(x)
+    assert ei.value.code == capi.ERR_INVALID_ARG
+    torch.cuda.synchronize()
+    room = max(0, max_seq - pos) if pos > 0 else 0  # rows of the run that still had a place
+    rows = memory.clone()
+    rows[guard:guard + 4] = 0x3c
+    cache = rows[guard + 256:guard + size].view(2, max_seq, d * 2)
+    if room:
+        cache[:, pos:] = 0x3c
+    assert torch.all(rows == 0x3c)
+    state.zero_()
+    assert all(a.tobytes() == b.tobytes() for a, b in zip(r.run(x), good))
+
+
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("rows,k,n,count", [
     (40, 200, 130, 2), (200, 256, 255, 3),      # per tile, ragged columns
