@@ -1477,7 +1477,6 @@ int swapnet_engine_adapt(swapnet_engine* e, const swapnet_plan* plan) {
 
 namespace swapnet {
 
-// Enqueue one inference: swaps on the copy stream, layers on `s`.
 // Enqueue one inference: swaps on the copy stream, layers on `s`.  Each
 // inference is self-contained: the copy stream forks from `s` (so swaps
 // start after everything already queued on `s`, which also orders them
@@ -1488,7 +1487,8 @@ namespace swapnet {
 // Units that may run on the side stream: a whole-layer conv / linear unit
 // whose layer may start early (Layer::start < layer), whose last producer's
 // unit is on the main stream in the same block, and whose consumers are all
-// in that block (they wait for it; the block's slot is released after them).
+// in that block (they wait for it; the block's slot is released after them),
+// while nothing that runs until then is written over its inputs.
 static int plan_side(swapnet_engine* e) {
   const swapnet_plan& p = e->plan;
   const Model& m = p.model;
@@ -1528,6 +1528,13 @@ static int plan_side(swapnet_engine* e) {
         cons.push_back(v);
       }
     if (!ok || cons.empty()) continue;
+    // The workspace keeps what the unit reads until its place in the layer
+    // order; beside the main stream it may run until its first consumer, so
+    // no unit in between may be given that space.
+    for (int v = u + 1; v < cons[0] && ok; ++v)
+      for (int s : {L.d.src0, L.d.src1, L.d.res})
+        if (s >= 0 && outputs_overlap(m, p.units[v].layer, s)) ok = false;
+    if (!ok) continue;
     e->is_side[u] = 1;
     e->side_after[du].push_back(u);
     for (int v : cons) e->side_wait[v].push_back(u);

@@ -267,6 +267,24 @@ def test_attention_of_short_runs_keeps_fp32_probabilities(tokens, heads, pos, ma
     assert float((out != ref.to(torch.bfloat16).double()).double().mean()) <= 2.0 ** -10
 
 
+def test_side_branch_whose_input_is_overwritten_before_its_consumer():
+    """A long convolution that may run beside three short ones, the last of which is given the space of its input:
+    the bits of one stream, many times over."""
+    conv = lambda src, k, res=None: dict(op="conv", src=[src], cin=64, cout=64, kh=k, kw=k, stride=1, pad=k // 2, act="relu",
+                                         res=res, res_post=False)
+    layers = [conv(-1, 1), conv(0, 1), conv(0, 11), conv(1, 1), conv(3, 1), conv(4, 1, res=2)]
+    m = dict(name="yolov3", model_id=52, dtype="f16", input=(2, 40, 40, 64), layers=layers, outputs=[5])
+    offs = OP.workspace(m)[1]
+    assert offs[4] == offs[0]
+    w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
+    host = capi.HostWeights(w)
+    one, both = (Runner(m, w, capi.Plan.resident(d, capi.options(branches=b)), host) for b in (0, 1))
+    ref = one.run(x)
+    check_close(m, one.decode(ref), oracle_outputs(m, w, x))
+    for _ in range(20):
+        assert both.run(x)[0].tobytes() == ref[0].tobytes()
+
+
 @pytest.mark.parametrize("tokens,heads", [(1, 8), (3, 2), (64, 8), (130, 32)])
 @pytest.mark.parametrize("pos", ["full", -1, -100, 2 ** 31 - 1, -2 ** 31])
 def test_positions_outside_the_cache_are_refused(tokens, heads, pos):
