@@ -527,10 +527,12 @@ int swapnet_engine_unit_kernels(const swapnet_engine* eng, int32_t* kinds, uint3
  * per output tile), splits (K splits; 1 = none), cluster (1: the splits of a
  * tile reduce through a thread-block cluster), persistent (1: one CTA per SM
  * loops over the tiles), tap_tma (1: convolution A loaded by one 4-D TMA per
- * filter tap).  Units off the tensor cores get all zeros.  Same count
- * protocol as swapnet_engine_unit_kernels. */
+ * filter tap), pair (1: persistent on pairs of SMs), sub_tiles (128-row parts
+ * of a tile), shared (1: one launch with its siblings, whose tiling this is).
+ * Units off the tensor cores get all zeros.  Same count protocol as
+ * swapnet_engine_unit_kernels. */
 typedef struct swapnet_unit_tiling {
-  int32_t n_tile, splits, cluster, persistent, tap_tma, reserved[3];
+  int32_t n_tile, splits, cluster, persistent, tap_tma, pair, sub_tiles, shared;
 } swapnet_unit_tiling;
 int swapnet_engine_unit_tiling(const swapnet_engine* eng, swapnet_unit_tiling* tiling, uint32_t cap,
                                uint32_t* n);

@@ -84,7 +84,7 @@ KERNEL_KIND = {1: "tc_gemm", 2: "tc_conv", 3: "skinny_linear", 4: "direct_conv",
 
 class UnitTiling(C.Structure):
     _fields_ = [("n_tile", C.c_int32), ("splits", C.c_int32), ("cluster", C.c_int32), ("persistent", C.c_int32),
-                ("tap_tma", C.c_int32), ("reserved", C.c_int32 * 3)]
+                ("tap_tma", C.c_int32), ("pair", C.c_int32), ("sub_tiles", C.c_int32), ("shared", C.c_int32)]
 
 
 class EngineBlock(C.Structure):
@@ -544,7 +544,7 @@ class Engine:
         check(lib().swapnet_engine_unit_tiling(self.h, None, 0, C.byref(n)), "swapnet_engine_unit_tiling")
         arr = (UnitTiling * max(1, n.value))()
         check(lib().swapnet_engine_unit_tiling(self.h, arr, n.value, None), "swapnet_engine_unit_tiling")
-        return [{f: getattr(u, f) for f, _ in UnitTiling._fields_ if f != "reserved"} for u in arr[:n.value]]
+        return [{f: getattr(u, f) for f, _ in UnitTiling._fields_} for u in arr[:n.value]]
 
     def set_profiling(self, enable):
         check(lib().swapnet_engine_set_profiling(self.h, 1 if enable else 0), "swapnet_engine_set_profiling")

@@ -1041,6 +1041,17 @@ static void plan_merges(swapnet_engine* e) {
   }
 }
 
+// The shared tensor-core launch of unit u and the merge_n[u] units after it,
+// without outputs (the plan of a launch does not depend on them).
+static void group_gemm(const swapnet_engine* e, int u, const char* x, TcGemm* g) {
+  unit_gemm(e, e->plan.units[u], e->ux[u], x, nullptr, nullptr, g);
+  g->nseg = 1 + e->merge_n[u];
+  for (int i = 1; i < g->nseg; ++i) {
+    g->Wx[i - 1] = e->ux[u + i].w;
+    g->bx[i - 1] = e->ux[u + i].b;
+  }
+}
+
 // Launch unit u with the merge_n[u] units after it as one launch.
 static int run_group(swapnet_engine* e, int u, const void* din, void* dout, cudaStream_t s) {
   const swapnet_plan& p = e->plan;
@@ -1049,14 +1060,10 @@ static int run_group(swapnet_engine* e, int u, const void* din, void* dout, cuda
   if (e->unit_kind[u] == SWAPNET_KERNEL_TC_GEMM) {
     UnitExec& X = e->ux[u];
     TcGemm g;
-    unit_gemm(e, p.units[u], X, act_ptr(e, L0.d.src0, din, dout), nullptr, out_ptr(e, p.units[u].layer, dout), &g);
-    g.nseg = 1 + e->merge_n[u];
-    for (int i = 1; i < g.nseg; ++i) {
-      g.Wx[i - 1] = e->ux[u + i].w;
-      g.bx[i - 1] = e->ux[u + i].b;
-      g.yx[i - 1] = out_ptr(e, p.units[u + i].layer, dout);
-    }
-    if (!X.tc_group.ready || X.group_for != g.A) {
+    group_gemm(e, u, act_ptr(e, L0.d.src0, din, dout), &g);
+    g.y = out_ptr(e, p.units[u].layer, dout);
+    for (int i = 1; i < g.nseg; ++i) g.yx[i - 1] = out_ptr(e, p.units[u + i].layer, dout);
+    if (X.group_for != g.A) {
       const int rc = tc_prepare(g, &X.tc_group);
       if (rc) return rc;
       X.group_for = g.A;
@@ -1148,6 +1155,15 @@ static int prepare_units(swapnet_engine* e) {
     }
   }
   plan_merges(e);
+  for (size_t u = 0; u < p.units.size(); ++u) {
+    if (!e->merge_n[u] || e->unit_kind[u] != SWAPNET_KERNEL_TC_GEMM) continue;
+    UnitExec& X = e->ux[u];
+    TcGemm g;
+    group_gemm(e, (int)u, static_cast<const char*>(X.tmA_for), &g);
+    const int rc = tc_prepare(g, &X.tc_group);
+    if (rc) return rc;
+    X.group_for = g.A;
+  }
   return SWAPNET_OK;
 }
 
@@ -1934,15 +1950,21 @@ int swapnet_engine_unit_tiling(const swapnet_engine* e, swapnet_unit_tiling* t, 
     if (!e) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "null engine");
     if (n) *n = (uint32_t)e->ux.size();
     for (uint32_t i = 0; t && i < cap && i < e->ux.size(); ++i) {
-      const UnitExec& X = e->ux[i];
+      uint32_t first = i;  // of the units that share its launch
+      while (e->merged_into[first]) --first;
+      const bool shared = first != i || e->merge_n[i];
+      const TcPlan& tc = shared ? e->ux[first].tc_group : e->ux[i].tc;
       swapnet_unit_tiling r;
       std::memset(&r, 0, sizeof(r));
-      if (X.use_tc) {
-        r.n_tile = X.tc.bn;
-        r.splits = X.tc.splits;
-        r.cluster = X.tc.splits > 1;
-        r.persistent = X.tc.persist;
-        r.tap_tma = X.tc.tma_conv;
+      if (e->ux[i].use_tc) {
+        r.n_tile = tc.bn;
+        r.splits = tc.splits;
+        r.cluster = tc.splits > 1;
+        r.persistent = tc.persist;
+        r.tap_tma = tc.tma_conv;
+        r.pair = tc.pair;
+        r.sub_tiles = tc.pair ? 2 : std::max(1, tc.msub);
+        r.shared = shared;
       }
       t[i] = r;
     }

@@ -338,6 +338,8 @@ def test_sibling_linears_share_a_launch(dtype, rows, k, n, count):
     runs = [Runner(m, w, capi.Plan.resident(d, capi.options(merge=g)), host) for g in (1, 0)]
     got, sep = (r.run(x) for r in runs)
     launches = [r.engine.stats()["kernel_launches"] for r in runs]
+    tiling, alone = (r.engine.unit_tiling()[1:] for r in runs)
+    assert all(t == tiling[0] and t["shared"] for t in tiling[:3]) and not any(t["shared"] for t in tiling[3:] + alone)
     assert launches[1] - launches[0] == (count - 1 if count <= 3 else count - 2)
     assert all(a.tobytes() == b.tobytes() for a, b in zip(got, sep))
     check_close(m, runs[0].decode(got), oracle_outputs(m, w, x))
