@@ -29,21 +29,32 @@ def _check(layers, inp, dtype, budget=None):
     return rs
 
 
+def _routes(rs):
+    """Per unit on the tensor cores: which kernel, its N tile, the splits of K and, persistent, the 128-row parts of a
+    tile.  A test of a kernel's edges asserts them, so that a change of the choice does not empty it."""
+    return [("pair" if t["pair"] else "persist" if t["persistent"] else "tile", t["n_tile"], t["splits"], t["sub_tiles"])
+            for t in rs.engine.unit_tiling()]
+
+
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("act,res_post", [("relu", False), ("leaky", True), ("swiglu", False)])
-@pytest.mark.parametrize("rows,k,n", [
-    (200, 256, 40),     # one tile per CTA, one 32-column piece and a quarter
-    (200, 256, 255),    # odd width: 2-byte moves
-    (40, 2048, 130),    # K split over a cluster, rows shared out, odd multiple of 2
-    (129, 1024, 264),   # the same, second M tile of one row
-    (12, 2048, 520),    # few rows: columns shared out
-    (16, 2048, 333),
-    (2600, 128, 264),   # persistent
-    (2600, 128, 255),
-    (5000, 64, 48),
+@pytest.mark.parametrize("rows,k,n,route", [
+    (200, 256, 40, ("tile", 64, 1, 1)),       # one 32-column piece and a quarter
+    (200, 256, 255, ("tile", 64, 1, 1)),      # odd width: 2-byte moves
+    (1000, 200, 1000, ("tile", 64, 1, 1)),    # ragged k-block, ragged last columns
+    (897, 64, 1501, ("tile", 128, 1, 1)),     # one k-block
+    (40, 2048, 130, ("tile", 64, 7, 1)),      # K split over a cluster, rows shared out, odd multiple of 2
+    (129, 4096, 264, ("tile", 64, 8, 1)),     # the same, second M tile of one row
+    (12, 2048, 520, ("tile", 64, 8, 1)),      # few rows: columns shared out
+    (16, 2048, 333, ("tile", 64, 8, 1)),
+    (1095, 3928, 1975, ("persist", 128, 1, 1)),
+    (2377, 2552, 1935, ("persist", 256, 1, 1)),
+    (97601, 328, 33, ("persist", 64, 1, 1)),  # one row in the last tile
+    (97700, 456, 47, ("persist", 64, 1, 2)),
 ])
-def test_tile_epilogue(dtype, act, res_post, rows, k, n):
-    _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
+def test_tile_epilogue(dtype, act, res_post, rows, k, n, route):
+    rs = _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
+    assert _routes(rs) == [route] * 2
 
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
@@ -63,24 +74,34 @@ def test_few_row_gemm(dtype, rows, k, n, n_tile, splits):
     assert (t["n_tile"], t["splits"], t["persistent"]) == (n_tile, splits, 0)
 
 
-@pytest.mark.parametrize("hw", [160, 220])
-def test_sub_tiles_with_a_residual(hw):
-    """Two and four 128-row sub-tiles per tile, the residual of the next
-    sub-tile requested during the one before."""
-    conv = dict(op="conv", src=[-1], cin=64, cout=48, kh=1, kw=1, stride=1, pad=0, act="none", res=None, res_post=False)
-    _check([conv, dict(conv, act="leaky", res=0, res_post=True)], (2, hw, hw, 64), "f16")
+@pytest.mark.parametrize("k,cin,cout,hw,batch,route", [
+    (1, 456, 40, 222, 2, ("persist", 64, 1, 2)),  # A by 2-D TMA
+    (3, 64, 48, 161, 6, ("persist", 64, 1, 2)),   # by 4-D TMA
+    (3, 64, 48, 203, 4, ("persist", 64, 1, 1)),
+    (1, 64, 48, 160, 2, ("pair", 64, 1, 2)),
+])
+def test_sub_tiles_with_a_residual(k, cin, cout, hw, batch, route):
+    """Two 128-row sub-tiles per tile, the residual of the next sub-tile
+    requested during the one before; one, and a pair of SMs, beside it."""
+    conv = dict(op="conv", src=[-1], cin=cin, cout=cout, kh=k, kw=k, stride=1, pad=k // 2, act="none", res=None,
+                res_post=False)
+    rs = _check([conv, dict(conv, act="leaky", res=0, res_post=True)], (batch, hw, hw, cin), "f16")
+    assert _routes(rs) == [route] * 2
 
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("act,res_post", [("none", False), ("swiglu", False)])
-@pytest.mark.parametrize("rows,k,n", [
-    (1000, 200, 1000),   # 4 x 256-row tiles, last one half empty; ragged k-block, ragged last columns
-    (897, 64, 1501),     # one k-block, odd width, an odd number of 128-row blocks
-    (385, 1088, 4160),   # several tiles per pair
-    (2049, 576, 288),    # one row in the last tile
+@pytest.mark.parametrize("rows,k,n,n_tile", [
+    (1000, 520, 4000, 128),   # ragged last rows, k-block and columns
+    (1793, 520, 1501, 192),   # odd width; an odd number of 128-row blocks, one row in the last, the other CTA's empty
+    (1025, 264, 5003, 64),
+    (5001, 40, 1001, 64),     # one k-block
+    (2049, 1032, 3104, 128),  # three rounds of tiles
+    (897, 1032, 9001, 256),   # two
 ])
-def test_paired_gemm(dtype, act, res_post, rows, k, n):
-    _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
+def test_paired_gemm(dtype, act, res_post, rows, k, n, n_tile):
+    rs = _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
+    assert _routes(rs) == [("pair", n_tile, 1, 2)] * 2
 
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
@@ -88,22 +109,31 @@ def test_paired_gemm(dtype, act, res_post, rows, k, n):
     (3, 1, 64, 161, 2),   # an odd number of taps, ragged patches
     (3, 2, 40, 301, 2),
     (4, 2, 128, 320, 3),  # an even number, N tiles of 128
-    (5, 1, 64, 104, 32),  # four sub-tiles
+    (5, 1, 64, 104, 32),  # two sub-tiles
 ])
 def test_two_taps_per_k_block(dtype, k, stride, cout, hw, batch):
     """Convolutions of 32 channels on the persistent kernel, A by 4-D TMA."""
     conv = dict(op="conv", src=[-1], cin=32, cout=cout, kh=k, kw=k, stride=stride, pad=k // 2, act="leaky", res=None,
                 res_post=False)
     rs = _check([conv, dict(conv, res=0, res_post=True)], (batch, hw, hw, 32), dtype)
-    assert all(t["persistent"] and t["tap_tma"] for t in rs.engine.unit_tiling())
+    assert _routes(rs) == [("persist", 128 if cout > 64 else 64, 1, 2 if batch == 32 else 1)] * 2
+    assert all(t["tap_tma"] for t in rs.engine.unit_tiling())
 
 
-@pytest.mark.parametrize("stride,cin,cout,hw,batch", [(1, 64, 256, 52, 3), (2, 128, 160, 75, 5), (1, 64, 96, 57, 4)])
-def test_paired_conv(stride, cin, cout, hw, batch):
+@pytest.mark.parametrize("stride,cin,cout,hw,batch,route", [
+    (1, 64, 256, 52, 3, ("pair", 96, 1, 2)),
+    (2, 128, 160, 101, 8, ("pair", 160, 1, 2)),
+    (1, 128, 416, 57, 4, ("pair", 224, 1, 2)),
+    (2, 256, 320, 75, 5, ("pair", 160, 1, 2)),   # an odd number of patches
+    (2, 128, 160, 75, 5, ("tile", 128, 1, 1)),   # 4-D TMA per tile
+    (1, 64, 96, 57, 4, ("tile", 128, 1, 1)),
+])
+def test_paired_conv(stride, cin, cout, hw, batch, route):
     """Convolutions by 4-D TMA on pairs of SMs: patches past the last one, strides, ragged patch edges."""
     conv = dict(op="conv", src=[-1], cin=cin, cout=cout, kh=3, kw=3, stride=stride, pad=1, act="leaky", res=None,
                 res_post=False)
-    _check([conv, dict(conv, res=0, res_post=True)], (batch, hw, hw, cin), "f16")
+    rs = _check([conv, dict(conv, res=0, res_post=True)], (batch, hw, hw, cin), "f16")
+    assert _routes(rs) == [route] * 2 and all(t["tap_tma"] for t in rs.engine.unit_tiling())
 
 
 @pytest.mark.parametrize("dtype,rows,k,n", [
@@ -323,12 +353,14 @@ def test_positions_outside_the_cache_are_refused(tokens, heads, pos):
 
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
-@pytest.mark.parametrize("rows,k,n,count", [
-    (40, 200, 130, 2), (200, 256, 255, 3),      # per tile, ragged columns
-    (600, 320, 1000, 3), (513, 64, 2056, 3),    # pairs of SMs: ragged last tile of every layer, one row in the last row tile
-    (2600, 128, 96, 4),                         # more siblings than one launch takes
+@pytest.mark.parametrize("rows,k,n,count,route", [
+    (40, 200, 130, 2, ("tile", 64, 1, 1)), (200, 256, 255, 3, ("tile", 64, 1, 1)),   # ragged columns
+    (600, 320, 1000, 3, ("tile", 128, 1, 1)), (513, 64, 2056, 3, ("tile", 128, 1, 1)),
+    # pairs of SMs: ragged last tile of every layer, one row in the last row tile
+    (513, 520, 3001, 3, ("pair", 192, 1, 2)), (1025, 264, 1001, 3, ("pair", 64, 1, 2)), (897, 520, 1501, 2, ("pair", 192, 1, 2)),
+    (2600, 128, 96, 4, ("tile", 64, 1, 1)),     # more siblings than one launch takes
 ])
-def test_sibling_linears_share_a_launch(dtype, rows, k, n, count):
+def test_sibling_linears_share_a_launch(dtype, rows, k, n, count, route):
     """Tensor-core linear layers that read the same input in one launch: the bits of one launch each, and the oracle."""
     layers = [_linear(-1, k, k, "relu")] + [_linear(0, k, n, "leaky", bias=i != 1) for i in range(count)]
     m = dict(name="yolov3", model_id=47, dtype=dtype, input=(rows, 1, 1, k), layers=layers,
@@ -339,6 +371,7 @@ def test_sibling_linears_share_a_launch(dtype, rows, k, n, count):
     got, sep = (r.run(x) for r in runs)
     launches = [r.engine.stats()["kernel_launches"] for r in runs]
     tiling, alone = (r.engine.unit_tiling()[1:] for r in runs)
+    assert _routes(runs[0])[1] == route
     assert all(t == tiling[0] and t["shared"] for t in tiling[:3]) and not any(t["shared"] for t in tiling[3:] + alone)
     assert launches[1] - launches[0] == (count - 1 if count <= 3 else count - 2)
     assert all(a.tobytes() == b.tobytes() for a, b in zip(got, sep))
