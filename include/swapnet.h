@@ -198,7 +198,8 @@ typedef struct swapnet_options {
                                      bytes.  Objective 0 only. */
   int32_t split_cap;             /* 0 (default): the kernels choose how many ways to
                                      split K for layers with fewer output tiles than
-                                     SMs; n > 0: at most n (1 = never split).  A
+                                     SMs, at most 8; n > 0: at most n (1 = never
+                                     split; above 8 as 8).  A
                                      tuning knob; results differ in the last bits
                                      between split counts (each count is
                                      deterministic). */
@@ -649,8 +650,9 @@ void swapnet_engine_free(swapnet_engine* eng);
  * output tiles leave idle (128 x 64 tiles, 128 x 128 where those give every
  * SM one; at most 32 ways, two 64-deep k-blocks each), counted as if they
  * were kept in one array with 64 KiB beside them, exceed
- * SWAPNET_NOALLOC_SCRATCH_BYTES.  Calls share nothing: they may overlap on
- * different streams and threads.
+ * SWAPNET_NOALLOC_SCRATCH_BYTES.  The kernels need no such array; the limit
+ * stands so that what the call refuses does not change.  Calls share nothing:
+ * they may overlap on different streams and threads.
  *
  * Ordering: the kernel starts only after the work queued before it on
  * `stream` has completed (no programmatic early start), so A, W and bias may

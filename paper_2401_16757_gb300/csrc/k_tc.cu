@@ -66,10 +66,10 @@ template <int BN, int AMODE> struct Cfg {
   static constexpr int kARegion = kStages * kAStage + kABytes - kAStage;  // the last stage's MMA reads 128 rows too
   static constexpr int kBBytes = BN * kBK * 2;
   static constexpr int kStageBytes = kARegion + kStages * kBBytes;
-  // cluster split-K receive buffer.  Row owners: up to 16 splits x
+  // cluster split-K receive buffer.  Row owners: up to kTcMaxSplit splits x
   // ceil(128/splits) rows.  Few rows (column owners): splits x kFewRows rows x
   // (columns per owner, a multiple of 8, + 4): 2 to 8 splits of up to BN + 76 floats.
-  static constexpr int kRecvBytes = kFew ? kFewRows * (BN + 76) * 4 : (kBM + 15) * (BN + 4) * 4;
+  static constexpr int kRecvBytes = kFew ? kFewRows * (BN + 76) * 4 : (kBM + kTcMaxSplit - 1) * (BN + 4) * 4;
   static constexpr int kBiasBytes = BN * 4;
   static constexpr int kSmem = kStageBytes + kRecvBytes + kBiasBytes + 512 + 1024;
   static_assert(kSmem <= 232448, "dynamic shared memory above the 227 KB per-CTA limit");
@@ -548,14 +548,6 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
                                         : (g.M + kBM - 1) / kBM;
   const dim3 grid((unsigned)mtiles, (g.N + BN - 1) / BN * std::max(1, g.nseg), pl.splits);
   const bool csplit = pl.splits > 1;
-  if (csplit) {
-    static std::atomic<uint64_t> np_done{0};  // per instantiation, one bit per device
-    if (attr_needed(np_done)) {
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-        SN_FAIL(SWAPNET_ERR_CUDA, "non-portable cluster attribute failed");
-      attr_set(np_done);
-    }
-  }
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = grid;
@@ -584,13 +576,13 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
 }
 
 
-// Clusters of c CTAs (2 to 8, along the split dimension) of this kernel
+// Clusters of c CTAs (2 to kTcMaxSplit, along the split dimension) of this kernel
 // instance that the device runs at once (cudaOccupancyMaxActiveClusters;
 // cached per instance, size and device).
 template <typename T, int BN, int AMODE>
 int active_clusters_inst(int c) {
-  static std::atomic<int> cached[64][9];  // the count + 1, 0 until known
-  if (c < 2 || c > 8) return 0;
+  static std::atomic<int> cached[64][kTcMaxSplit + 1];  // the count + 1, 0 until known
+  if (c < 2 || c > kTcMaxSplit) return 0;
   const int dev = device_index();
   if (dev >= 0) {
     const int v = cached[dev][c].load(std::memory_order_relaxed);
@@ -736,7 +728,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
   const int64_t mt_tile = tap ? patches : mt, mt_pers = tap_persist ? patches : mt;
   double best = 0.0;
   // ---- per tile, K split over clusters
-  const int cap = std::max(1, std::min(std::min(8, g.cluster_max), KB));
+  const int cap = std::max(1, std::min(std::min(kTcMaxSplit, g.cluster_max), KB));
   auto consider = [&](int bn, int splits, double us) {
     if (best > 0.0 && us >= best) return;
     best = us;
@@ -760,19 +752,17 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
   if (g.allow_persist && !few) {
     int pbn = Nd <= 64 ? 64 : (Nd <= 128 ? 128 : 256);
     if (pbn == 256 && mt_pers * ((Nd + 255) / 256) * 2 <= sms) pbn = 128;  // twice the CTAs
-    // N tiles of 64 with A by TMA: four (else two) 128-row sub-tiles per
-    // tile share each weight stage when that still leaves a tile per SM
-    // and is not slower for the tiles' last round (3x3 64 -> 64 at batch 8,
-    // 112x112: 16.5 us with four, 12.1 so; batch 16, 224x224: 84.3, 69.7)
+    // N tiles of 64 with A by TMA: two 128-row sub-tiles per tile share each
+    // weight stage where that still leaves a tile per SM and the tiles' last
+    // round does not cost more.  (Four: never the least, their epilogue is
+    // twice as long and the stages shallower; 3x3 64 -> 64 at batch 8, 112x112
+    // 16.5 us with four, 12.1 so; batch 16, 224x224: 84.3, 69.7.)
     int msub = 1;
     auto us_of = [&](int ms) { return persist_us(pbn, ms, (mt_pers + ms - 1) / ms * ((Nd + pbn - 1) / pbn), KB, sms); };
     double one = us_of(1);
-    if (pbn == 64 && (!g.conv || tap_persist)) {
-      for (int ms : {2, 4}) {
-        if ((mt_pers + ms - 1) / ms * ((Nd + 63) / 64) < sms || us_of(ms) > one) continue;
-        msub = ms;
-        one = us_of(ms);
-      }
+    if (pbn == 64 && (!g.conv || tap_persist) && (mt_pers + 1) / 2 >= sms && us_of(2) <= one) {
+      msub = 2;
+      one = us_of(2);
     }
     if (one < best && nseg == 1) {
       best = one;
@@ -949,7 +939,7 @@ extern "C" int swapnet_gemm_noalloc(int32_t dtype, const void* A, const void* W,
     g.e.bias = bias; g.e.res = nullptr; g.e.ldr = N; g.e.act = act; g.e.res_post = 0;
     g.y = Y; g.ldy = N;
     g.num_sms = d.sms;
-    g.cluster_max = 16;
+    g.cluster_max = kTcMaxSplit;
     g.allow_persist = 1;
     // W and bias are caller memory that the previous work on the stream (an
     // earlier call, say) may have written: no early start before it completes

@@ -11,8 +11,7 @@
 //   warp 1       TMEM owner and MMA issuer (one elected lane)
 //   warps 2..9   epilogue: TMEM -> registers -> bias / residual / activation
 //                -> shared memory -> global, warp w reading TMEM lanes
-//                32 * (w % 4) .. + 31 of one half of the tile's columns (four
-//                warps and all columns where the stages leave no room for eight)
+//                32 * (w % 4) .. + 31 of one half of the tile's columns
 //   then 4 warps (convolutions without whole-tap TMA) implicit im2col gather of
 //                A with cp.async
 // A-operand modes: kAT2d (row-major A by 2-D TMA), kAGather (cp.async im2col
@@ -49,18 +48,18 @@ constexpr int kPBM = 128;
 constexpr int kPBK = 64;  // one 128-byte swizzle row of 16-bit elements
 constexpr int kPA = kPBM * kPBK * 2;
 
-// MS: 128-row sub-tiles per tile sharing each weight stage (1, or 2 or 4
-// for N tiles of 64, where one 128x64 MMA chain per k16 step is too little
-// work per stage): a tile is then MS*128 x BN, MS accumulators side by side
-// in TMEM (2 x MS x BN columns with the double buffer: 512 for MS = 4).
+// MS: 128-row sub-tiles per tile sharing each weight stage (1, or 2 for N
+// tiles of 64, where one 128x64 MMA chain per k16 step is too little work per
+// stage): a tile is then MS*128 x BN, MS accumulators side by side in TMEM
+// (2 x MS x BN columns with the double buffer).
 template <int BN, int MS> struct PCfg {
-  static constexpr int kStages = BN == 256 ? 4 : (BN == 128 ? 6 : (MS == 4 ? 3 : (MS == 2 ? 5 : 8)));
+  static constexpr int kStages = BN == 256 ? 4 : (BN == 128 ? 6 : (MS == 2 ? 5 : 8));
   static constexpr int kLag = kStages - 2;  // gather: cp.async groups in flight per thread
   static constexpr int kB = BN * kPBK * 2;
   static constexpr int kSA = MS * kPA;      // A bytes per stage
   static constexpr int kStageBytes = kStages * (kSA + kB);
-  static constexpr int kEpiWarps = MS == 4 ? 4 : 8;
-  static constexpr int kCols = BN / (kEpiWarps / 4);      // columns per epilogue warp
+  static constexpr int kEpiWarps = 8;
+  static constexpr int kCols = BN / 2;                    // columns per epilogue warp
   static constexpr int kBias = kEpiWarps * kCols * 4;     // [epilogue warp][its columns] fp32
   static constexpr int kStaging = kEpiWarps * kEpiStage;  // a 32 x 32 output piece per warp
   static constexpr int kSmem = kStageBytes + kBias + kStaging + 256 + 1024;
@@ -493,12 +492,6 @@ int launch_persist_bn(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t 
   }
   if constexpr (BN == 64) {  // sub-tiles only with N tiles of 64
     if (taps32 && pl.msub == 2) return launch_persist_inst<T, BN, kATap2, 2>(g, pl, err, s);
-    if (taps32 && pl.msub == 4) return launch_persist_inst<T, BN, kATap2, 4>(g, pl, err, s);
-    if (pl.msub == 4) {
-      if (!g.conv) return launch_persist_inst<T, BN, kAT2d, 4>(g, pl, err, s);
-      if (pl.tma_conv) return launch_persist_inst<T, BN, kATap, 4>(g, pl, err, s);
-      SN_FAIL(SWAPNET_ERR_INVALID_ARG, "persistent GEMM: four sub-tiles need A by TMA");
-    }
     if (pl.msub == 2) {
       if (!g.conv) return launch_persist_inst<T, BN, kAT2d, 2>(g, pl, err, s);
       if (pl.tma_conv) return launch_persist_inst<T, BN, kATap, 2>(g, pl, err, s);

@@ -120,6 +120,7 @@ int launch_zerocopy(const ZcSeg* segs, int nseg, int ctas, cudaStream_t s);
 // and no residual (e.g. the q, k, v projections) may share a launch: nseg of
 // them, segment i > 0 with weights, bias and output in Wx / bx / yx[i - 1].
 constexpr int kTcMaxSeg = 3;
+constexpr int kTcMaxSplit = 8;  // K splits of a tile: the portable cluster size
 struct TcGemm {
   int nseg;           // 0 or 1: one layer
   const void* Wx[kTcMaxSeg - 1];
@@ -144,7 +145,7 @@ struct TcGemm {
                         // of; tiling and split-K follow it, so every piece sums
                         // each output in the same order as the unsplit layer
   int cluster_max;      // K is split across a thread-block cluster of at most
-                        // this many CTAs (DSMEM reduction)
+                        // this many CTAs and kTcMaxSplit (DSMEM reduction)
   int no_pdl;           // 1: launch without programmatic dependent launch.  The
                         // kernel reads its bias and issues its first weight
                         // loads before waiting on the previous kernel, which
