@@ -119,6 +119,45 @@ def test_noalloc_chained_calls_against_oracle(dtype):
     assert rel_l2(got2, ref2) <= 2e-3, rel_l2(got2, ref2)
 
 
+@pytest.mark.parametrize("entry", ["gemm_noalloc", "infer"])
+def test_first_cuda_call_of_a_thread(entry):
+    """A thread that has made no CUDA call yet, and so has no context: the allocation-free call, and an eager inference
+    whose first layer needs a new tensor map, run there as in any other thread."""
+    import threading
+    import torch
+    M, K, N, dtype = 64, 512, 128, "f16"
+    m = _layer_model(M, K, N, dtype)
+    w, x = synth.gen.model_weights(m), synth.gen.model_input(m)
+    ref = _oracle_linear(x.reshape(M, K), w[0][0], w[0][1], dtype)
+    dev = [torch.from_numpy(np.ascontiguousarray(t).view(np.uint8).reshape(-1).copy()).cuda() for t in (x, w[0][0], w[0][1])]
+    outs = [torch.full((M * N * 2,), 0xFF, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    other = dev[0].clone()
+    eng = capi.Engine(capi.Plan.resident(capi.Desc(m), capi.options(graphs=0)), capi.HostWeights(w))
+    stream = torch.cuda.current_stream().cuda_stream
+    torch.cuda.synchronize()
+    errors = []
+
+    def call(src, out):
+        try:
+            if entry == "infer":
+                eng.infer(src.data_ptr(), out.data_ptr(), stream)
+            else:
+                capi.gemm_noalloc(capi.DTYPE[dtype], src.data_ptr(), dev[1].data_ptr(), dev[2].data_ptr(), out.data_ptr(), M, N,
+                                  K, act=capi.ACT["relu"], stream=stream)
+        except capi.SwapnetError as e:
+            errors.append(e)
+
+    call(dev[0], outs[0])
+    t = threading.Thread(target=call, args=(other, outs[1]))
+    t.start()
+    t.join()
+    eng.sync()
+    assert not errors
+    for out in outs:
+        assert rel_l2(F.decode(out.cpu().numpy().view(np.float16), dtype).reshape(M, N), ref) <= 2e-3
+    eng.free()
+
+
 def test_noalloc_gemm_rejects_oversize_scratch():
     import torch
     # M=128, N=4864, K=4096 splits K in two: 2 x 128 x 4864 fp32 partials
