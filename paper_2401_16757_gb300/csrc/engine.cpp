@@ -1241,7 +1241,7 @@ static int run_unit(swapnet_engine* e, int u, const void* din, void* dout, cudaS
 
 // Everything an engine derives from its plan: arena (allocated when the
 // engine owns it), copy segments, unit pointers and TMA descriptors, side
-// branches, split-K scratch, the resident upload or prefix upload, and the
+// branches, the resident upload or prefix upload, and the
 // swap variants.  Used by swapnet_load and again by swapnet_engine_adapt.
 static bool prefetch_on(const swapnet_engine* e);
 

@@ -175,7 +175,10 @@ __global__ void __launch_bounds__(128) rope_append_kernel(T* __restrict__ q, con
 #pragma unroll
   for (int u = 0; u < NP; ++u) inv[u] = powf(theta, -2.0f * (float)(ch * NP + u) / (float)dh);
   pdl_wait();
-  pdl_launch_dependents();  // after the wait: attention_split_kernel reads older cache rows before its own
+  // After the wait, in every CTA: both attention kernels (each launched right
+  // behind this one) read the position and the cache rows of earlier runs
+  // before their own wait, which only ends with this launch.
+  pdl_launch_dependents();
   if (h0 >= heads) return;
   const int pos0 = *pos_ptr;
   if (pos0 < 0 || pos0 >= max_seq - t) {  // (no sum that could overflow)

@@ -454,13 +454,19 @@ template <typename T> int skinny_dispatch(const SkJob& j, cudaStream_t s) {
 //
 // What bounds it: for the batches it serves (17 to a few hundred rows) the
 // parallelism, hence two tiles: 32 x 32 with K split 8 ways inside the CTA
-// while 64 x 64 tiles would not fill the SMs, 64 x 64 (K split in two) from
-// there on.  100 x 1000 x 1000 fp32:
-// 91 us with 64 x 64 tiles of 16 k per step, loaded and waited for element by
-// element; 13.9 us now.
+// for up to 127 tiles of 64 x 64, 64 x 64 (K split in two) from there on.
+// 100 x 1000 x 1000 fp32: 91 us with 64 x 64 tiles of 16 k per step, loaded and
+// waited for element by element; 12.4 us now (40.3 with the wide tiles).  By
+// count, its reads of shared memory, 12 of 16 bytes per 64 packed FMAs of a
+// thread, take about 6 of them.
 constexpr int kTlStages = 4;
 constexpr int kTlThreads = 256;
-constexpr int kTlWideTiles = 128;  // 64 x 64 tiles from which they are taken
+// 64 x 64 tiles from which they are taken: wide against narrow 39.0 and 29.7 us
+// at 112 tiles (256 x 1024 x 1792), 38.9 and 38.5 at 128 (256 x 1024 x 2048),
+// 20.7 and 21.1 (64 x 512 x 8192), 52.3 and 55.3 at 132 (700 x 1023 x 768), 12.8
+// and 14.5 at 136 (512 x 260 x 1029).  (With a second round of wide tiles, from
+// 153 on, the narrow ones are faster again at first: 53.6 and 39.5 at 160.)
+constexpr int kTlWideTiles = 128;
 
 template <int TM, int TN, int RM, int RN, int BK> struct TlCfg {
   static constexpr int kCols = TM / RM;                     // threads along M in a group
@@ -890,7 +896,7 @@ int launch_linear_tiled(int dtype, const void* x, int M, int K, const void* W, i
   if (M < 1 || K < 1 || N < 1) SN_FAIL(SWAPNET_ERR_INVALID_ARG, "tiled linear: empty shape");
   // 16-byte copies need 16-byte aligned fp32 rows
   const int vec = dtype == SWAPNET_F32 && K % 4 == 0 && (((uintptr_t)x | (uintptr_t)W) & 15) == 0;
-  // 64 x 64 tiles once they give every SM one.  The two tiles share K out
+  // 64 x 64 tiles once they give most SMs one.  The two tiles share K out
   // differently, so the choice follows the whole layer's width: a column
   // piece of a layer sums each output as the whole layer would
   const int64_t tiles = (int64_t)((M + 63) / 64) * ((N_layer + 63) / 64);

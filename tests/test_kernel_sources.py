@@ -28,3 +28,16 @@ def test_outputs_of_an_overlapped_launch_are_not_read_as_read_only():
         params = re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", head)
         assert set(params) <= WEIGHTS, (name, params)
     assert seen >= 18
+
+
+def test_rotation_releases_the_attention_after_its_wait():
+    """The attention kernels read the position and older cache rows before their own wait: what they overlap, the
+    rotation launched right before them, lets them start only once everything ahead of it has ended."""
+    bodies = [body for _, head, body in _kernels() if "rope_append_kernel" in head]
+    assert len(bodies) == 1
+    assert 0 <= bodies[0].index("pdl_wait()") < bodies[0].index("pdl_launch_dependents()")
+    assert not re.search(r"\breturn\b", bodies[0][:bodies[0].index("pdl_launch_dependents()")])
+    text = open(os.path.join(CSRC, "k_decoder.cu")).read()
+    launch = text[text.index("int launch_attention("):]
+    between = launch[launch.index("rope_append_kernel<T, 1, 1>"):launch.index("attention_split_kernel<T>, static_cast")]
+    assert between.count("launch_pdl(") == 0 and between.count("launch_attention_tc(") == 1
