@@ -7,9 +7,12 @@ decoder (13.5 GB of weights) through a 4e9-byte weight arena, one step =
 the prefill of 512 token ids plus 32 greedy decode passes; every other
 workload (the MLP, ResNet-50, VGG-16 at batch 1 and 16, YOLOv3, the
 multi-DNN mix) is measured after it in the same call and reported under
-the line's `configs` key (--configs none skips them).
+the `configs` key (--configs none skips them).
 
-Reported (one JSON line, rank 0):
+Standard output gets one JSON line (rank 0) of at most 2400 characters, which
+a log that keeps only the last few kilobytes still holds whole; everything that
+was measured goes to standard error as a second JSON line, {"details": ...}.
+Reported:
   value        whole-job inferences/s (device-timed, inputs resident in HBM)
   ms_per_step  swapped latency; dinf_ms the all-resident latency with the
                same kernels; ratio = swapped / DInf
@@ -681,8 +684,9 @@ def run_llm(args, rank, world, group):
         "metric": METRIC, "value": world * 1000.0 / step_ms, "unit": unit,
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": step_ms,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
-        "config": {"workload": text, "budget_bytes": budget, "weight_bytes": ip["weight_bytes"],
-                   "prefill_blocks": ip["n_blocks"], "decode_blocks": idd["n_blocks"],
+        "config": {"workload": text, "model": "LLaMA-7B-shaped decoder", "global_batch": world, "seq_len": 512,
+                   "parallelism": "replicas" if world > 1 else "1 GPU", "budget_bytes": budget,
+                   "weight_bytes": ip["weight_bytes"], "prefill_blocks": ip["n_blocks"], "decode_blocks": idd["n_blocks"],
                    "plans_exact": [ip["exact"], idd["exact"]], "l2": "inputs (13.2 GB of weights) larger than L2",
                    "swap_variant": args.variant, "swap_variants_prefill": var_p, "swap_variants_decode": var_d,
                    "merged_gemv_launches": args.merge, "state_bytes": ip["state_bytes"]},
@@ -1378,8 +1382,53 @@ def main():
             torch.cuda.synchronize()
             torch.cuda.empty_cache()
     if rank == 0:
-        print(json.dumps(line))
+        print(json.dumps({"details": line}), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)))
     group.close()
+
+
+HEADLINE_CHARS = 2400
+
+
+def headline(line):
+    """The line of standard output: the contract's keys as measured, and of the rest the few numbers that sum it up
+    (floats rounded), per other workload swapped ms, resident ms and link bound / swapped.  Optional keys are left out,
+    the last first, should it come out longer than HEADLINE_CHARS."""
+    def rounded(x):
+        if isinstance(x, float):
+            return float("%.5g" % x)
+        if isinstance(x, dict):
+            return {k: rounded(v) for k, v in x.items()}
+        return [rounded(v) for v in x] if isinstance(x, list) else x
+
+    def part(key, keys):
+        d = line.get(key)
+        return {k: d[k] for k in keys if k in d} if isinstance(d, dict) else None
+
+    out = {k: line[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+                                "scaling", "vs_baseline", "dtype", "data", "gpu_launches") if k in line}
+    config = part("config", ("model", "workload", "global_batch", "seq_len", "parallelism", "budget_bytes", "weight_bytes",
+                             "n_blocks", "prefill_blocks", "decode_blocks", "l2"))
+    for key, d in (("config", config), ("e2e", part("e2e", ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"))),
+                   ("clocks", part("clocks", ("sm_mhz", "sm_max_mhz", "reasons")))):
+        if d is not None:
+            out[key] = d
+    optional = {"ratio": rounded(line.get("ratio")), "dinf_ms": rounded(line.get("dinf_ms")),
+                "roofline": rounded(part("roofline", ("bound", "kernel", "achieved", "peak", "unit", "frac"))),
+                "step_roofline": rounded(part("step_roofline", ("bound", "bound_ms", "frac"))),
+                "link": rounded(part("link", ("achieved_gbs", "peak_gbs"))),
+                "cpu_baseline": rounded(part("cpu_baseline", ("value", "unit", "cores", "kind")))}
+    if isinstance(line.get("configs"), dict):
+        optional["configs"] = {
+            c: r if "error" in r else rounded([r.get("ms_per_step"), r.get("dinf_ms", r.get("dinf_ms_per_step")),
+                                               r.get("step_roofline", {}).get("frac")])
+            for c, r in line["configs"].items()}
+        optional["configs_are"] = ["swapped ms", "DInf ms", "link bound / swapped"]
+    optional["details"] = "the JSON line of standard error"
+    kept = [k for k, v in optional.items() if v is not None]
+    while len(json.dumps(dict(out, **{k: optional[k] for k in kept}))) > HEADLINE_CHARS and kept:
+        kept.pop()
+    return dict(out, **{k: optional[k] for k in kept})
 
 
 def compact_line(r):

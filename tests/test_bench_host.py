@@ -57,6 +57,35 @@ def test_reference_arm_prints_one_oracle_line():
     assert line["value"] > 0 and line["unit"] == line["e2e"]["unit"]
 
 
+def test_headline_is_short_and_keeps_the_contract():
+    """The line of standard output holds every key of the contract unchanged in at most HEADLINE_CHARS characters,
+    whatever was measured beside it (logs that keep only the end of standard output lost the line otherwise)."""
+    f = 0.12345678901234567
+    big = {"k%d" % i: [f] * 40 for i in range(50)}
+    contract = {"metric": bench.METRIC, "value": f, "unit": "inferences/s (prefill 512 + 32 decode)", "n_gpus": 1, "steps": 20,
+                "warmup": 5, "ms_per_step": 2070.866057395935, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+                "dtype": "bf16", "data": "synthetic", "gpu_launches": 180160}
+    e2e = {"value": f, "unit": contract["unit"], "h2d_bytes_per_step": 2176, "d2h_bytes_per_step": 34826240}
+    clocks = {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"]}
+    config = dict(big, workload="w" * 170, model="m" * 60, global_batch=1, seq_len=512, parallelism="1 GPU",
+                  budget_bytes=4000000000, weight_bytes=13476831232, l2="l" * 80)
+    sub = dict(big, ms_per_step=f, dinf_ms=f, step_roofline={"frac": f, "bound_ms": f})
+    line = dict(contract, e2e=dict(e2e, **big), clocks=dict(clocks, samples=108), config=config, ratio=f, dinf_ms=f,
+                roofline=dict(big, bound="host_link", kernel="zerocopy_kernel", achieved=f, peak=f, unit="GB/s", frac=f),
+                step_roofline={"bound": "host link", "bound_ms": f, "frac": f}, link=dict(big, achieved_gbs=f, peak_gbs=f),
+                cpu_baseline=dict(value=f, unit="u", cores=16, kind="oracle", sample="s" * 3000), per_step=big, ablation=big,
+                configs={c: sub for c in ("mlp6", "resnet50", "vgg16_b1", "vgg16_b16", "yolov3", "multi")})
+    got = bench.headline(line)
+    assert len(json.dumps(got)) <= bench.HEADLINE_CHARS
+    assert {k: got[k] for k in contract} == contract and got["e2e"] == e2e and got["clocks"] == clocks
+    assert got["config"]["workload"] == config["workload"] and got["roofline"]["kernel"] == "zerocopy_kernel"
+    assert got["configs"]["multi"] == [0.12346] * 3
+    line["configs"] = {"c%d" % i: {"error": "e" * 500} for i in range(6)}
+    short = bench.headline(line)
+    assert len(json.dumps(short)) <= bench.HEADLINE_CHARS and "configs" not in short and short["value"] == f
+    assert bench.headline(contract) == dict(contract, details="the JSON line of standard error")
+
+
 def _rank_group_worker(rank, port, out_dir):
     os.environ.update(MASTER_ADDR="127.0.0.1", MASTER_PORT=str(port), RANK=str(rank), WORLD_SIZE="2")
     sys.path.insert(0, ROOT)
