@@ -466,7 +466,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// A tiled map of 16-bit elements with zero fill.  The driver's call needs a
+// A tiled map of 16-bit elements with zero fill.  The CUDA driver's call needs a
 // current context, which a thread whose first CUDA call leads here does not
 // have yet (the runtime binds one at its own calls): bind that of the thread's
 // device and ask again.
