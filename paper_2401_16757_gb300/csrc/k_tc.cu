@@ -55,6 +55,8 @@ constexpr int kABytes = kBM * kBK * 2;
 // 16 KB of A per stage and 4-6 stages before: 1024 -> 1024 4.2 to 3.4 us, 1024 <-> 2752 5.8
 // to 3.9, 2048 <-> 8192 12.9 to 8.4, 4096 -> 4096 9.4 to 8.7, 8192 -> 8192
 // 26.2 to 24.3 (5.5 TB/s); 25088 -> 4096 alone 37.9 to 33.2.
+// Siblings share a launch of it: twelve layers 2048 -> 11008 of 8 rows 131.0
+// us one by one, 102.6 three to a launch.
 constexpr int kA2d = 0, kAGather = 1, kATap = 2, kAFew = 3;
 constexpr int kFewRows = 16;
 
@@ -585,6 +587,11 @@ int launch_inst(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
   return SWAPNET_OK;
 }
 
+template <typename T, int NS> int launch_few(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) {
+  if (pl.bn == 64) return launch_inst<T, 64, kAFew, NS>(g, pl, err, s);
+  if (pl.bn == 128) return launch_inst<T, 128, kAFew, NS>(g, pl, err, s);
+  return launch_inst<T, 256, kAFew, NS>(g, pl, err, s);
+}
 
 // Clusters of c CTAs (2 to kTcMaxSplit, along the split dimension) of this kernel
 // instance that the device runs at once (cudaOccupancyMaxActiveClusters;
@@ -749,7 +756,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
     p->bn = bn;
     p->splits = splits;
   };
-  const bool few = !g.conv && g.M <= kFewRows && nseg == 1;
+  const bool few = !g.conv && g.M <= kFewRows;
   for (int bn : {64, 128, 256}) {
     if ((bn == 128 && Nd <= 64) || (bn == 256 && (!few || KB < 16))) continue;
     const int64_t tiles = mt_tile * ((Nd + bn - 1) / bn) * nseg;
@@ -759,7 +766,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
       if (used != c) continue;
       // every cluster at once: a second wave of them costs more than a split saves
       if (c > 1 && tiles > active_clusters(g.dtype, bn, gather, few, c)) continue;
-      consider(bn, c, few ? few_us(bn, tiles, c, KB, Nd, sms) : tile_us(bn, tiles, c, KB, tap, sms));
+      consider(bn, c, few ? few_us(bn, tiles, c, KB, (int64_t)Nd * nseg, sms) : tile_us(bn, tiles, c, KB, tap, sms));
     }
   }
   // ---- persistent, no split
@@ -831,11 +838,9 @@ int launch_tc_gemm(const TcGemm& g, const TcPlan& pl, int* err, cudaStream_t s) 
   if (pl.pair) return launch_tc_pair(g, pl, err, s);
   if (pl.persist) return launch_tc_persist(g, pl, err, s);
   const bool bf = g.dtype == SWAPNET_BF16;
-  if (pl.few) {
-    if (pl.bn == 64) return bf ? launch_inst<__nv_bfloat16, 64, kAFew>(g, pl, err, s) : launch_inst<__half, 64, kAFew>(g, pl, err, s);
-    if (pl.bn == 128) return bf ? launch_inst<__nv_bfloat16, 128, kAFew>(g, pl, err, s) : launch_inst<__half, 128, kAFew>(g, pl, err, s);
-    return bf ? launch_inst<__nv_bfloat16, 256, kAFew>(g, pl, err, s) : launch_inst<__half, 256, kAFew>(g, pl, err, s);
-  }
+  if (pl.few)
+    return g.nseg > 1 ? (bf ? launch_few<__nv_bfloat16, kTcMaxSeg>(g, pl, err, s) : launch_few<__half, kTcMaxSeg>(g, pl, err, s))
+                      : (bf ? launch_few<__nv_bfloat16, 1>(g, pl, err, s) : launch_few<__half, 1>(g, pl, err, s));
   if (g.nseg > 1) {
     if (pl.bn == 64)
       return bf ? launch_inst<__nv_bfloat16, 64, kA2d, kTcMaxSeg>(g, pl, err, s) : launch_inst<__half, 64, kA2d, kTcMaxSeg>(g, pl, err, s);

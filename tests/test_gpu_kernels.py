@@ -354,6 +354,8 @@ def test_positions_outside_the_cache_are_refused(tokens, heads, pos):
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("rows,k,n,count,route", [
+    # at most 16 rows, loaded in 16-row boxes like a layer alone: every N tile, ragged columns
+    (16, 72, 1001, 3, ("tile", 64, 1, 1)), (13, 64, 9793, 2, ("tile", 128, 1, 1)), (5, 1992, 11001, 3, ("tile", 256, 1, 1)),
     (40, 200, 130, 2, ("tile", 64, 1, 1)), (200, 256, 255, 3, ("tile", 64, 1, 1)),   # ragged columns
     (600, 320, 1000, 3, ("tile", 128, 1, 1)), (513, 64, 2056, 3, ("tile", 128, 1, 1)),
     # pairs of SMs: ragged last tile of every layer, one row in the last row tile
