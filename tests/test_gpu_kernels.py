@@ -429,7 +429,8 @@ def test_few_row_fp32_siblings_share_a_launch(rows):
 
 
 @pytest.mark.parametrize("dtype,rows", [("f16", 1), ("bf16", 1), ("f16", 2), ("bf16", 3), ("f16", 4), ("f32", 1)])
-@pytest.mark.parametrize("k,n", [(8, 1), (2048, 9), (2056, 40), (4104, 300), (11008, 21), (1024, 5000)])
+@pytest.mark.parametrize("k,n", [(8, 1), (2048, 9), (2056, 40), (4104, 300), (11008, 21), (1024, 5000),
+                                 (96, 1301), (200, 1304), (504, 2501), (1016, 2600)])  # one, two, four warps to a row
 def test_gemv(dtype, rows, k, n):
     """The GEMV at the edges of its passes (2048 or 1024 k), weight-row groups (8) and one group per CTA; a residual,
     and a gate with its SwiGLU layer in one launch."""
@@ -438,10 +439,11 @@ def test_gemv(dtype, rows, k, n):
     assert set(rs.engine.unit_kernels()) == {"skinny_linear"}
 
 
-def test_gemv_segments_of_ragged_widths():
+@pytest.mark.parametrize("k,n", [(520, 700), (520, 1301), (264, 4003)])
+def test_gemv_segments_of_ragged_widths(k, n):
     """Three siblings of widths that are no multiple of a group in one launch: the bits of one launch each."""
-    layers = [_linear(-1, 520, 13), _linear(-1, 520, 700, "relu"), _linear(-1, 520, 8)]
-    m = dict(name="yolov3", model_id=48, dtype="bf16", input=(1, 1, 1, 520), layers=layers, outputs=[0, 1, 2])
+    layers = [_linear(-1, k, 13), _linear(-1, k, n, "relu"), _linear(-1, k, 8)]
+    m = dict(name="yolov3", model_id=48, dtype="bf16", input=(1, 1, 1, k), layers=layers, outputs=[0, 1, 2])
     w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
     host = capi.HostWeights(w)
     a, b = (Runner(m, w, capi.Plan.resident(d, capi.options(merge=g)), host) for g in (1, 0))
