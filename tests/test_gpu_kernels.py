@@ -405,7 +405,9 @@ def test_siblings_whose_buffers_overlap_run_one_by_one(dtype, rows, residual):
 
 
 @pytest.mark.parametrize("rows", [2, 4, 5, 8, 9, 16])
-@pytest.mark.parametrize("k,n", [(4, 1), (128, 9), (1020, 40), (1024, 64), (1028, 7), (3000, 130)])
+@pytest.mark.parametrize("k,n", [(4, 1), (128, 9), (1020, 40), (1024, 64), (1028, 7), (3000, 130),
+                                 (100, 5003), (200, 4999), (512, 5001),  # one, two, four warps to a row
+                                 (1032, 5001)])                          # two rows: 16 features per CTA
 def test_few_row_fp32_linear(rows, k, n):
     """The few-row kernel at the edges of its k chunks (1024), features per CTA and rows; with a residual."""
     rs = _check([_linear(-1, k, n, "leaky"), _linear(-1, k, n, "relu", res=0)], (rows, 1, 1, k), "f32")
@@ -413,11 +415,12 @@ def test_few_row_fp32_linear(rows, k, n):
 
 
 @pytest.mark.parametrize("rows", [2, 3, 5, 8, 16])
-def test_few_row_fp32_siblings_share_a_launch(rows):
+@pytest.mark.parametrize("wide", [9, 5003])  # (5003: teams of warps)
+def test_few_row_fp32_siblings_share_a_launch(rows, wide):
     """fp32 siblings of ragged widths in one launch, one with a residual, and a gate with its SwiGLU layer in another:
     the bits of one launch each, and the oracle."""
-    layers = [_linear(-1, 1300, 260), _linear(0, 260, 13), _linear(0, 260, 260, "relu", res=0), _linear(0, 260, 9, bias=False),
-              _linear(2, 260, 36), _linear(2, 260, 36, "swiglu", res=4)]
+    layers = [_linear(-1, 1300, 260), _linear(0, 260, 13), _linear(0, 260, 260, "relu", res=0), _linear(0, 260, wide, bias=False),
+              _linear(2, 260, 4 * wide), _linear(2, 260, 4 * wide, "swiglu", res=4)]
     m = dict(name="yolov3", model_id=50, dtype="f32", input=(rows, 1, 1, 1300), layers=layers, outputs=[1, 2, 3, 5])
     w, x, d = synth.gen.model_weights(m), synth.gen.model_input(m), capi.Desc(m)
     host = capi.HostWeights(w)
