@@ -468,12 +468,14 @@ template <typename T, int MT, bool TEAMS> int gemv_launch_as(const SkJob& j, int
   const cudaError_t e = launch_pdl(gemv_kernel<T, MT, TEAMS>, dim3(grid), dim3(kGvWarps * 32), 0, s, j, groups, wk);
   return e == cudaSuccess ? SWAPNET_OK : SWAPNET_ERR_CUDA;
 }
-// Teams pay from more groups than SMs on: 1 row of 512 bf16, 2432 features (304
-// groups) 2.11 us without, 1.86 with; 1024 (128 groups) 1.70 and 1.84.
+// Teams pay from more groups than SMs on, of fp32 from twice as many: 1 row of
+// 512 bf16, 2432 features (304 groups) 2.11 us without, 1.86 with; 1024 (128
+// groups) 1.70 and 1.84; 1 row of 308 fp32, 2093 features 1.75 and 1.95, of 256,
+// 3648 features 2.19 and 1.96.
 template <typename T, int MT> int gemv_launch(const SkJob& j, int groups, cudaStream_t s) {
   int wk = 1;  // warps that a row needs
   while (wk < kGvWarps && wk * 32 * Vec16<T>::N < j.K) wk *= 2;
-  return wk < kGvWarps && groups > j.num_sms ? gemv_launch_as<T, MT, true>(j, groups, wk, s)
+  return wk < kGvWarps && groups > (sizeof(T) == 4 ? 2 : 1) * j.num_sms ? gemv_launch_as<T, MT, true>(j, groups, wk, s)
                                              : gemv_launch_as<T, MT, false>(j, groups, kGvWarps, s);
 }
 
