@@ -644,27 +644,37 @@ int active_clusters(int dtype, int bn, bool gather, bool few, int c) {
 
 // ---- which kernel, N tile and split of K: the least of the times below, in
 // us per launch inside a chain of dependent launches.  The constants are fits
-// to sweeps on the GB300 (every N tile and split of the layers of ResNet-50
-// and YOLOv3 at batch 1 and of linear layers of 8 to 2048 rows).  Against the
-// measured times of 45 such layers the fitted one of the choice taken is 13 %
-// off at most; of four 3x3 convolutions at batch 16, 0.66 to 1.05 of it.  What
-// counts is the ranking: of 4 to 23 choices the fastest or one within 2 % was
-// taken for 46 of the 49 (the others: 200 x 4096 x 4096 12.0 us, 9.9 per tile;
-// 1x1 64 -> 32 at 208 x 208 6.0, 3.7 on single SMs; 1x1 1024 -> 2048 stride 2 at
-// 14 x 14 4.3, 3.9 without a split).
+// to sweeps on the GB300 over every N tile, sub-tile count and split of linear
+// layers of 40 to 100000 rows and of 1x1 to 7x7 convolutions at batch 1 to 16
+// (4 to 25 choices each; mean error 8 %).  What counts is the ranking: of 94
+// layers 91 got the fastest choice or one within 2 %, the others lost 0.2-0.5 us.
+// (The fits before, of deep layers alone, took pairs of SMs with N tiles of 64
+// for wide layers of short K, 20000 x 256 x 256 11.4 us against 7.8 on single SMs,
+// and no split of a gathered operand, see tile_us.)  Not in them: an odd width's
+// 2-byte stores, which cost a pair of SMs less (3x3 64 -> 71 at 217 x 217, batch
+// 16, 211 us, 160 on pairs).
 
 // Per-tile kernel: `base` from the previous kernel's end to the last store
 // without a k-block, the k-blocks of one CTA (a split below five hides
 // nothing of the fill), and the exchange of a split.  More tiles than SMs
-// repeat everything but the launch.
-double tile_us(int bn, int64_t tiles, int splits, int KB, bool tap, int sms) {
+// repeat everything but the launch.  A gathered operand costs several times a
+// TMA one, more as more CTAs gather (3x3 96 -> 96 at 9 x 9, 14 k-blocks: 9.4 us
+// unsplit, 4.9 seven ways).  Ragged rows (K odd in units of 16 values, so that
+// a row starts in the middle of a 32-byte sector) load at about half the rate
+// (512 x 2752 x 2040 13.9 us, x 2048 8.5).  thin: a convolution of so few
+// features that all CTAs fetch the same few weight rows at once (3x3 256 -> 12 at
+// 182 x 182: 32.8 us on single SMs, 16.7 on pairs, half of which fetch none).
+double tile_us(int bn, int64_t tiles, int splits, int KB, bool tap, bool gather, bool ragged, bool thin, int sms) {
   const int kb = (KB + splits - 1) / splits;
-  // (long K: the weights come from HBM at the pace the stages allow)
-  const double per_kb = bn == 64 ? (tap ? 0.14 : 0.125) + 0.0002 * kb : 0.16 + 0.0008 * kb;
-  const double base = bn == 64 ? 2.1 : 2.9;
-  const int64_t waves = (tiles * splits + sms - 1) / sms;
+  const int64_t ctas = tiles * splits, waves = (ctas + sms - 1) / sms;
   const double split = splits > 1 ? (bn == 64 ? 1.5 : 2.8) + 0.02 * splits : 0.0;
-  return base + split + waves * per_kb * (splits > 1 ? std::max(kb, 5) : kb) + (waves - 1) * 2.2;
+  // (long K: the weights come from HBM at the pace the stages allow)
+  const double per_kb = gather ? (bn == 64 ? 0.5 : 0.6) + 0.002 * std::min<int64_t>(ctas, sms)
+                        : ragged ? (bn == 64 ? 0.235 : 0.345)
+                               : (bn == 64 ? (tap ? 0.14 : 0.125) + 0.0002 * kb : 0.16 + 0.0008 * kb) +
+                                     (thin ? 0.0011 * std::min<int64_t>(ctas, sms) : 0.0);
+  return (bn == 64 ? 2.1 : 2.9) + split + waves * std::max(per_kb * kb, splits > 1 && !gather ? (bn == 64 ? (tap ? 0.7 : 0.63) : 0.82) : 0.0) +
+         (waves - 1) * (bn == 64 ? 2.2 : 2.9);
 }
 
 // The per-tile kernel on at most kFewRows rows: streaming the weights is the
@@ -685,27 +695,57 @@ double few_us(int bn, int64_t tiles, int splits, int KB, int64_t N, int sms) {
          (waves - 1) * 2.5;
 }
 
-// Persistent kernel, one CTA per tile of msub x 128 rows: a tile's epilogue
-// overlaps the next tile's MMAs.
-double persist_us(int bn, int msub, int64_t tiles, int KB, int sms) {
-  const double per_kb = bn == 64 ? (msub > 1 ? 0.11 * msub : 0.125) : (bn == 128 ? 0.18 : 0.36);
-  const double epi = 0.7 * (msub > 1 ? msub : std::max(1, bn / 64));
-  return 3.2 + (double)((tiles + sms - 1) / sms) * std::max(KB * per_kb, epi) + epi;
+// Persistent kernel, one CTA per tile of msub x 128 rows: the fill, then per
+// tile the longer of its epilogue (which the next tile's MMAs overlap, not
+// wholly while they are short) and its k-blocks, at the pace of the loads (A: a
+// matrix by TMA, or one of ragged rows; 4-D TMA per filter tap; two taps per
+// k-block; gathered).
+enum class AFrom { kMatrix, kRagged, kTap, kTapPair, kGather };
+double persist_us(int bn, int msub, int64_t tiles, int KB, AFrom a, bool thin, int sms) {
+  const int64_t rounds = (tiles + sms - 1) / sms;
+  if (a == AFrom::kGather)
+    return (bn == 64 ? 2.3 : (bn == 128 ? 3.0 : 4.8)) +
+           rounds * KB * ((bn == 256 ? 0.6 : 0.5) + 0.002 * std::min<int64_t>(tiles, sms));
+  double fill, tile, tap;
+  if (bn == 64 && msub == 1) {
+    fill = 1.4 + std::min(0.1 * KB, 1.3);
+    tile = std::max({1.05, 0.75 + 0.075 * KB, 0.125 * KB});
+    tap = std::max(0.9 + 0.13 * KB, 0.173 * KB);
+  } else if (bn == 64) {
+    fill = 1.7 + std::min(0.06 * KB, 0.6);
+    tile = std::max(1.7, 0.95 + 0.22 * KB);
+    tap = std::max(0.95 + 0.25 * KB, 0.287 * KB);
+  } else if (bn == 128) {
+    fill = 1.7 + std::min(0.14 * KB, 1.2);
+    tile = std::max({1.8, 1.0 + 0.135 * KB, 0.25 + 0.18 * KB});
+    tap = std::max(0.9 + 0.155 * KB, 0.178 * KB);
+  } else {
+    fill = 2.15 + std::min(0.12 * KB, 1.7);
+    tile = std::max({3.15, 2.5 + 0.16 * KB, 0.295 * KB});
+    tap = 1.0 + 0.275 * KB;
+  }
+  if (a == AFrom::kTap) tile = std::max(tile, tap + (thin ? (msub > 1 ? 0.002 : 0.0009) * std::min<int64_t>(tiles, sms) * KB : 0.0));
+  if (a == AFrom::kTapPair) tile = std::max(tile, (msub > 1 ? 0.42 : 0.257) * KB);
+  if (a == AFrom::kRagged) tile = std::max(tile, (msub > 1 ? 0.5 : 0.17 + 0.0015 * bn) * KB);
+  return fill + rounds * tile;
 }
 
-// Persistent kernel on pairs of SMs, tiles of 256 x bn.
-double pair_us(int bn, int64_t tiles, int KB, int sms) {
-  const double epi = 0.7 * ((bn / 32 + 1) / 2);
-  const int64_t slots = sms / 2;
-  return 2.5 + (double)((tiles + slots - 1) / slots) * std::max(KB * (0.06 + 0.00085 * bn) + 0.2, epi) + epi;
+// Persistent kernel on pairs of SMs, tiles of 256 x bn: the same, a tile's
+// hand-over between the two SMs costs more than on one.
+double pair_us(int bn, int64_t tiles, int KB, bool tap, bool ragged, int sms) {
+  const int64_t slots = sms / 2, rounds = (tiles + slots - 1) / slots;
+  const double fill = 1.6 + 0.0042 * bn + std::min(KB, 16) * (0.03 + 0.0005 * bn);
+  const double loads = std::max((ragged ? 0.17 : 0.06) + 0.00085 * bn, 0.14);
+  return fill + rounds * std::max({1.1 + 0.01 * bn + (KB - 1) * (0.055 + 0.00005 * bn), 0.2 + KB * loads,
+                                   tap ? 1.0 + 0.15 * KB : 0.0});
 }
 
 // N tile of the paired kernel with the least pair_us (ties: the widest) for
 // mt 128-row blocks and nseg segments of N columns.
-int pair_tile(int64_t mt, int64_t N, int nseg, int KB, int sms, double* us) {
+int pair_tile(int64_t mt, int64_t N, int nseg, int KB, bool tap, bool ragged, int sms, double* us) {
   int best_bn = 0;
   for (int bn = 256; bn >= 64; bn -= 32) {
-    const double t = pair_us(bn, (mt + 1) / 2 * ((N + bn - 1) / bn) * nseg, KB, sms);
+    const double t = pair_us(bn, (mt + 1) / 2 * ((N + bn - 1) / bn) * nseg, KB, tap, ragged, sms);
     if (!best_bn || t < *us) {
       best_bn = bn;
       *us = t;
@@ -756,7 +796,7 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
     p->bn = bn;
     p->splits = splits;
   };
-  const bool few = !g.conv && g.M <= kFewRows;
+  const bool few = !g.conv && g.M <= kFewRows, ragged = !g.conv && g.K % 16, thin = tap && Nd <= 24;
   for (int bn : {64, 128, 256}) {
     if ((bn == 128 && Nd <= 64) || (bn == 256 && (!few || KB < 16))) continue;
     const int64_t tiles = mt_tile * ((Nd + bn - 1) / bn) * nseg;
@@ -766,34 +806,35 @@ int tc_prepare(const TcGemm& g, TcPlan* p) {
       if (used != c) continue;
       // every cluster at once: a second wave of them costs more than a split saves
       if (c > 1 && tiles > active_clusters(g.dtype, bn, gather, few, c)) continue;
-      consider(bn, c, few ? few_us(bn, tiles, c, KB, (int64_t)Nd * nseg, sms) : tile_us(bn, tiles, c, KB, tap, sms));
+      consider(bn, c, few ? few_us(bn, tiles, c, KB, (int64_t)Nd * nseg, sms) : tile_us(bn, tiles, c, KB, tap, gather, ragged, thin, sms));
     }
   }
   // ---- persistent, no split
   if (g.allow_persist && !few) {
-    int pbn = Nd <= 64 ? 64 : (Nd <= 128 ? 128 : 256);
-    if (pbn == 256 && mt_pers * ((Nd + 255) / 256) * 2 <= sms) pbn = 128;  // twice the CTAs
-    // N tiles of 64 with A by TMA: two 128-row sub-tiles per tile share each
-    // weight stage where that still leaves a tile per SM and the tiles' last
-    // round does not cost more.  (Four: never the least, their epilogue is
-    // twice as long and the stages shallower; 3x3 64 -> 64 at batch 8, 112x112
-    // 16.5 us with four, 12.1 so; batch 16, 224x224: 84.3, 69.7.)
-    int msub = 1;
-    auto us_of = [&](int ms) { return persist_us(pbn, ms, (mt_pers + ms - 1) / ms * ((Nd + pbn - 1) / pbn), KB, sms); };
-    double one = us_of(1);
-    if (pbn == 64 && (!g.conv || tap_persist) && (mt_pers + 1) / 2 >= sms && us_of(2) <= one) {
-      msub = 2;
-      one = us_of(2);
-    }
-    if (one < best && nseg == 1) {
-      best = one;
+    // N tiles of 64, 128 or 256 as the width needs, and 128 where 256 leaves SMs
+    // idle.  N tiles of 64 with A by TMA: two 128-row sub-tiles per tile share
+    // each weight stage where that still leaves a tile per SM.  (Four: their
+    // epilogue is twice as long and the stages shallower; 3x3 64 -> 64 at batch
+    // 8, 112x112 16.5 us with four, 12.1 so; batch 16, 224x224: 84.3, 69.7.)
+    const AFrom a = !g.conv ? (ragged ? AFrom::kRagged : AFrom::kMatrix)
+                            : (!tap_persist ? AFrom::kGather : (pair_taps ? AFrom::kTapPair : AFrom::kTap));
+    auto persist = [&](int bn, int ms) {
+      const double us = persist_us(bn, ms, (mt_pers + ms - 1) / ms * ((Nd + bn - 1) / bn), KB, a, thin, sms);
+      if (us >= best) return;
+      best = us;
       p->persist = 1;
-      p->bn = pbn;
-      p->msub = msub;
+      p->bn = bn;
+      p->msub = ms;
+    };
+    if (nseg == 1) {
+      if (Nd > 128) persist(256, 1);
+      if (Nd > 64) persist(128, 1);
+      else persist(64, 1);
+      if (Nd <= 64 && a != AFrom::kGather && (mt_pers + 1) / 2 >= sms) persist(64, 2);
     }
     if (mt_pers > 1 && (!g.conv || (tap_persist && !pair_taps))) {
       double two = 0.0;
-      const int bn2 = pair_tile(mt_pers, Nd, nseg, KB, sms, &two);
+      const int bn2 = pair_tile(mt_pers, Nd, nseg, KB, tap_persist, ragged, sms, &two);
       if (two < best) {
         p->persist = p->pair = 1;
         p->bn = bn2;

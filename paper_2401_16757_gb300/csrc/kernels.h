@@ -140,7 +140,7 @@ struct TcGemm {
   void* y;
   int64_t ldy;
   int num_sms;          // used by tc_prepare to size the grid
-  int allow_persist;    // 1: problems with a tile per SM take the persistent kernel
+  int allow_persist;    // 1: the persistent kernels may be chosen
   int N_layer;          // > 0: N of the whole layer this GEMM is a column piece
                         // of; tiling and split-K follow it, so every piece sums
                         // each output in the same order as the unsplit layer

@@ -47,9 +47,9 @@ def _routes(rs):
     (129, 4096, 264, ("tile", 64, 8, 1)),     # the same, second M tile of one row
     (12, 2048, 520, ("tile", 64, 8, 1)),      # few rows: columns shared out
     (16, 2048, 333, ("tile", 64, 8, 1)),
-    (1095, 3928, 1975, ("persist", 128, 1, 1)),
+    (1101, 264, 1975, ("persist", 128, 1, 1)),
     (2377, 2552, 1935, ("persist", 256, 1, 1)),
-    (97601, 328, 33, ("persist", 64, 1, 1)),  # one row in the last tile
+    (20001, 72, 33, ("persist", 64, 1, 1)),
     (97700, 456, 47, ("persist", 64, 1, 2)),
 ])
 def test_tile_epilogue(dtype, act, res_post, rows, k, n, route):
@@ -74,11 +74,35 @@ def test_few_row_gemm(dtype, rows, k, n, n_tile, splits):
     assert (t["n_tile"], t["splits"], t["persistent"]) == (n_tile, splits, 0)
 
 
+@pytest.mark.parametrize("layer,route", [
+    ((20000, 256, 256), ("persist", 128, 1, 1)),        # wide and short: 7.8 us, 11.4 on pairs with N tiles of 64
+    ((628, 144, 6272), ("persist", 256, 1, 1)),         # 6.0, 11.0
+    ((200, 4096, 4096), ("tile", 64, 1, 1)),            # 9.8, 12.0
+    ((100, 1016, 64), ("tile", 64, 8, 1)),              # ragged rows: 4.0 split, 5.3 not
+    ((100, 1024, 64), ("tile", 64, 1, 1)),              # 3.8, 3.9 split
+    ((3, 96, 96, 9), ("tile", 64, 7, 1)),               # gathered: 4.9 split, 9.4 not
+    ((3, 256, 12, 182), ("pair", 64, 1, 2)),            # few features: 16.7, 32.8 on single SMs
+])
+def test_choice_of_kernel(layer, route):
+    """Layers whose second-best choice costs much more (us measured on the GB300)."""
+    if len(layer) == 3:
+        rows, k, n = layer
+        lay, inp = _linear(-1, k, n), (rows, 1, 1, k)
+    else:
+        k, cin, cout, hw = layer
+        lay = dict(op="conv", src=[-1], cin=cin, cout=cout, kh=k, kw=k, stride=1, pad=k // 2, act="none", res=None, res_post=False)
+        inp = (1, hw, hw, cin)
+    m = dict(name="yolov3", model_id=53, dtype="f16", input=inp, layers=[lay], outputs=[0])
+    rs = Runner(m, synth.gen.model_weights(m), capi.Plan.resident(capi.Desc(m)))
+    assert _routes(rs) == [route]
+
+
 @pytest.mark.parametrize("k,cin,cout,hw,batch,route", [
     (1, 456, 40, 222, 2, ("persist", 64, 1, 2)),  # A by 2-D TMA
     (3, 64, 48, 161, 6, ("persist", 64, 1, 2)),   # by 4-D TMA
-    (3, 64, 48, 203, 4, ("persist", 64, 1, 1)),
-    (1, 64, 48, 160, 2, ("pair", 64, 1, 2)),
+    (3, 64, 40, 91, 3, ("persist", 64, 1, 1)),
+    (1, 64, 48, 160, 2, ("persist", 64, 1, 1)),
+    (5, 128, 17, 93, 4, ("pair", 64, 1, 2)),      # few features
 ])
 def test_sub_tiles_with_a_residual(k, cin, cout, hw, batch, route):
     """Two 128-row sub-tiles per tile, the residual of the next sub-tile
@@ -92,12 +116,12 @@ def test_sub_tiles_with_a_residual(k, cin, cout, hw, batch, route):
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("act,res_post", [("none", False), ("swiglu", False)])
 @pytest.mark.parametrize("rows,k,n,n_tile", [
-    (1000, 520, 4000, 128),   # ragged last rows, k-block and columns
+    (1000, 520, 4000, 224),   # ragged last rows, k-block and columns
     (1793, 520, 1501, 192),   # odd width; an odd number of 128-row blocks, one row in the last, the other CTA's empty
-    (1025, 264, 5003, 64),
-    (5001, 40, 1001, 64),     # one k-block
-    (2049, 1032, 3104, 128),  # three rounds of tiles
-    (897, 1032, 9001, 256),   # two
+    (5001, 1032, 1001, 160),
+    (4097, 1032, 500, 128),
+    (2049, 1032, 3104, 224),  # two rounds of tiles
+    (897, 1032, 9001, 256),
 ])
 def test_paired_gemm(dtype, act, res_post, rows, k, n, n_tile):
     rs = _check([_linear(-1, k, n), _linear(-1, k, n, act, res=0, res_post=res_post)], (rows, 1, 1, k), dtype)
@@ -105,23 +129,23 @@ def test_paired_gemm(dtype, act, res_post, rows, k, n, n_tile):
 
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
-@pytest.mark.parametrize("k,stride,cout,hw,batch", [
-    (3, 1, 64, 161, 2),   # an odd number of taps, ragged patches
-    (3, 2, 40, 301, 2),
-    (4, 2, 128, 320, 3),  # an even number, N tiles of 128
-    (5, 1, 64, 104, 32),  # two sub-tiles
+@pytest.mark.parametrize("k,stride,cout,hw,batch,sub_tiles", [
+    (3, 1, 64, 161, 2, 2),   # an odd number of taps, ragged patches
+    (3, 2, 40, 301, 2, 1),
+    (4, 2, 128, 320, 3, 1),  # an even number, N tiles of 128
+    (5, 1, 64, 104, 32, 2),
 ])
-def test_two_taps_per_k_block(dtype, k, stride, cout, hw, batch):
+def test_two_taps_per_k_block(dtype, k, stride, cout, hw, batch, sub_tiles):
     """Convolutions of 32 channels on the persistent kernel, A by 4-D TMA."""
     conv = dict(op="conv", src=[-1], cin=32, cout=cout, kh=k, kw=k, stride=stride, pad=k // 2, act="leaky", res=None,
                 res_post=False)
     rs = _check([conv, dict(conv, res=0, res_post=True)], (batch, hw, hw, 32), dtype)
-    assert _routes(rs) == [("persist", 128 if cout > 64 else 64, 1, 2 if batch == 32 else 1)] * 2
+    assert _routes(rs) == [("persist", 128 if cout > 64 else 64, 1, sub_tiles)] * 2
     assert all(t["tap_tma"] for t in rs.engine.unit_tiling())
 
 
 @pytest.mark.parametrize("stride,cin,cout,hw,batch,route", [
-    (1, 64, 256, 52, 3, ("pair", 96, 1, 2)),
+    (1, 64, 256, 52, 3, ("persist", 256, 1, 1)),  # 4-D TMA on single SMs
     (2, 128, 160, 101, 8, ("pair", 160, 1, 2)),
     (1, 128, 416, 57, 4, ("pair", 224, 1, 2)),
     (2, 256, 320, 75, 5, ("pair", 160, 1, 2)),   # an odd number of patches
@@ -359,7 +383,7 @@ def test_positions_outside_the_cache_are_refused(tokens, heads, pos):
     (40, 200, 130, 2, ("tile", 64, 1, 1)), (200, 256, 255, 3, ("tile", 64, 1, 1)),   # ragged columns
     (600, 320, 1000, 3, ("tile", 128, 1, 1)), (513, 64, 2056, 3, ("tile", 128, 1, 1)),
     # pairs of SMs: ragged last tile of every layer, one row in the last row tile
-    (513, 520, 3001, 3, ("pair", 192, 1, 2)), (1025, 264, 1001, 3, ("pair", 64, 1, 2)), (897, 520, 1501, 2, ("pair", 192, 1, 2)),
+    (513, 520, 3001, 3, ("pair", 192, 1, 2)), (1025, 264, 1001, 3, ("pair", 224, 1, 2)), (897, 520, 1501, 2, ("pair", 192, 1, 2)),
     (2600, 128, 96, 4, ("tile", 64, 1, 1)),     # more siblings than one launch takes
 ])
 def test_sibling_linears_share_a_launch(dtype, rows, k, n, count, route):

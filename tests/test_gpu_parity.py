@@ -60,14 +60,14 @@ def _check_model(m, budget_frac=0.5, slots=2, variant=capi.SWAP_AUTO):
     (5, 1, 4, 32, 21),      # Cin=4, K=100 (2 k-blocks)
     (3, 1, 3, 32, 224),     # 784 tiles: more tiles than resident CTAs (persistent loop)
     (7, 1, 5, 40, 15),      # K=245 beyond the small-channel kernel: SIMT direct conv
-    (3, 1, 64, 64, 112),    # pairs of SMs, N tile 64, A by 4-D TMA
-    (3, 1, 32, 128, 112),   # N tile 128, gather with k-blocks straddling taps
-    (1, 1, 64, 300, 112),   # pairs of SMs, N tile 64 (ragged), A by 2-D TMA
-    (3, 2, 64, 256, 224),   # pairs of SMs, N tile 128, strided
+    (3, 1, 64, 64, 112),    # persistent, N tile 64, A by 4-D TMA
+    (3, 1, 32, 128, 112),   # persistent, N tile 128, two taps per k-block
+    (1, 1, 64, 300, 112),   # persistent, N tile 128 (ragged), A by 2-D TMA
+    (3, 2, 64, 256, 224),   # persistent, N tile 128, 4-D TMA, strided
     (3, 1, 64, 64, 224),    # persistent, N tile 64, two 128-row patches per tile (784 patches)
-    (1, 1, 64, 48, 220),    # pairs of SMs, 2-D TMA, ragged m-tile count, N 48
-    (1, 1, 64, 48, 160),    # pairs of SMs, 2-D TMA (400 m-tiles)
-    (3, 1, 64, 64, 150),    # pairs of SMs, 4-D TMA over 32 x 4 patches (380 patches, ragged edge)
+    (1, 1, 64, 48, 220),    # persistent 2-D TMA, ragged m-tile count, N 48
+    (1, 1, 64, 48, 160),    # persistent 2-D TMA (400 m-tiles)
+    (3, 1, 64, 64, 150),    # persistent 4-D TMA over 32 x 4 patches (380 patches, ragged edge)
     (3, 1, 256, 256, 7),    # deep K, one M tile: gather with a cluster split of K
     (3, 1, 64, 24, 9),      # N below one 32-column chunk
     (3, 1, 64, 128, 14),    # few tiles, taps of 64 channels: A by 4-D TMA over 14 x 9 pixel patches

@@ -142,8 +142,8 @@ def _decoded(out, M, N, dtype):
 @pytest.mark.parametrize("M,K,N", [
     (1, 8, 1), (9, 8192, 130), (16, 2048, 1000),   # at most 16 rows, K split and not
     (200, 256, 255), (129, 4096, 264),             # one tile per CTA, K split and not
-    (1000, 520, 4000), (1025, 264, 5003),          # pairs of SMs
-    (1095, 3928, 1975), (97700, 456, 47),          # persistent
+    (1000, 520, 4000), (1025, 1032, 5003),         # pairs of SMs
+    (1101, 264, 1975), (97700, 456, 47),           # persistent
 ])
 def test_noalloc_gemm_over_its_kernels(dtype, M, K, N):
     import torch
