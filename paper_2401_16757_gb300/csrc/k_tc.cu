@@ -645,14 +645,15 @@ int active_clusters(int dtype, int bn, bool gather, bool few, int c) {
 // ---- which kernel, N tile and split of K: the least of the times below, in
 // us per launch inside a chain of dependent launches.  The constants are fits
 // to sweeps on the GB300 over every N tile, sub-tile count and split of linear
-// layers of 40 to 100000 rows and of 1x1 to 7x7 convolutions at batch 1 to 16
-// (4 to 25 choices each; mean error 8 %).  What counts is the ranking: of 94
-// layers 91 got the fastest choice or one within 2 %, the others lost 0.2-0.5 us.
+// layers of 40 to 100000 rows and of 1x1 to 7x7 convolutions at batch 1 to 32
+// (3 to 25 choices each; mean error 8 %).  What counts is the ranking: of 137
+// layers 130 got the fastest choice or one within 2 %.  The others lost 0.1-0.5 us,
+// but for two odd widths, whose 2-byte stores are not in the fits: 3x3 64 -> 71
+// at 48 x 48, batch 8, 8.4 us, 7.3 on pairs; 3x3 128 -> 255 at 52 x 52, batch 16,
+// 27.1 on pairs, 25.8 on single SMs.
 // (The fits before, of deep layers alone, took pairs of SMs with N tiles of 64
 // for wide layers of short K, 20000 x 256 x 256 11.4 us against 7.8 on single SMs,
-// and no split of a gathered operand, see tile_us.)  Not in them: an odd width's
-// 2-byte stores, which cost a pair of SMs less (3x3 64 -> 71 at 217 x 217, batch
-// 16, 211 us, 160 on pairs).
+// and no split of a gathered operand, see tile_us.)
 
 // Per-tile kernel: `base` from the previous kernel's end to the last store
 // without a k-block, the k-blocks of one CTA (a split below five hides
@@ -663,7 +664,9 @@ int active_clusters(int dtype, int bn, bool gather, bool few, int c) {
 // a row starts in the middle of a 32-byte sector) load at about half the rate
 // (512 x 2752 x 2040 13.9 us, x 2048 8.5).  thin: a convolution of so few
 // features that all CTAs fetch the same few weight rows at once (3x3 256 -> 12 at
-// 182 x 182: 32.8 us on single SMs, 16.7 on pairs, half of which fetch none).
+// 182 x 182: 32.8 us on single SMs, 16.7 on pairs, half of which fetch none).  Filter
+// taps on N tiles of 128 slow down as more CTAs load them (3x3, 36 k-blocks: 8.4 us
+// on 24 CTAs, 9.4 on 112).
 double tile_us(int bn, int64_t tiles, int splits, int KB, bool tap, bool gather, bool ragged, bool thin, int sms) {
   const int kb = (KB + splits - 1) / splits;
   const int64_t ctas = tiles * splits, waves = (ctas + sms - 1) / sms;
@@ -671,7 +674,9 @@ double tile_us(int bn, int64_t tiles, int splits, int KB, bool tap, bool gather,
   // (long K: the weights come from HBM at the pace the stages allow)
   const double per_kb = gather ? (bn == 64 ? 0.5 : 0.6) + 0.002 * std::min<int64_t>(ctas, sms)
                         : ragged ? (bn == 64 ? 0.235 : 0.345)
-                               : (bn == 64 ? (tap ? 0.14 : 0.125) + 0.0002 * kb : 0.16 + 0.0008 * kb) +
+                               : (bn == 64 ? (tap ? 0.14 : 0.125) + 0.0002 * kb
+                                : tap    ? 0.155 + 0.0003 * std::min<int64_t>(ctas, sms)
+                                         : 0.16 + 0.0008 * kb) +
                                      (thin ? 0.0011 * std::min<int64_t>(ctas, sms) : 0.0);
   return (bn == 64 ? 2.1 : 2.9) + split + waves * std::max(per_kb * kb, splits > 1 && !gather ? (bn == 64 ? (tap ? 0.7 : 0.63) : 0.82) : 0.0) +
          (waves - 1) * (bn == 64 ? 2.2 : 2.9);
@@ -718,7 +723,10 @@ double persist_us(int bn, int msub, int64_t tiles, int KB, AFrom a, bool thin, i
   } else if (bn == 128) {
     fill = 1.7 + std::min(0.14 * KB, 1.2);
     tile = std::max({1.8, 1.0 + 0.135 * KB, 0.25 + 0.18 * KB});
-    tap = std::max(0.9 + 0.155 * KB, 0.178 * KB);
+    // (all SMs at once; without the last term 256 -> 512 at 26 x 26, batch 4, came
+    // here at 10.2 us, 9.4 per tile, and 64 -> 71 at 217 x 217, batch 16, at 210 us,
+    // 160 on pairs)
+    tap = std::max(0.9 + 0.155 * KB, 0.178 * KB) + 0.03 * KB * std::min<int64_t>(tiles, sms) / sms;
   } else {
     fill = 2.15 + std::min(0.12 * KB, 1.7);
     tile = std::max({3.15, 2.5 + 0.16 * KB, 0.295 * KB});

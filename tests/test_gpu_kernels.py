@@ -82,6 +82,8 @@ def test_few_row_gemm(dtype, rows, k, n, n_tile, splits):
     ((100, 1024, 64), ("tile", 64, 1, 1)),              # 3.8, 3.9 split
     ((3, 96, 96, 9), ("tile", 64, 7, 1)),               # gathered: 4.9 split, 9.4 not
     ((3, 256, 12, 182), ("pair", 64, 1, 2)),            # few features: 16.7, 32.8 on single SMs
+    ((3, 256, 512, 26, 4), ("tile", 128, 1, 1)),        # one wave of taps: 9.4, 10.2 persistent
+    ((3, 64, 71, 217, 16), ("pair", 96, 1, 2)),         # many waves of them: 160, 210 on single SMs
 ])
 def test_choice_of_kernel(layer, route):
     """Layers whose second-best choice costs much more (us measured on the GB300)."""
@@ -89,9 +91,9 @@ def test_choice_of_kernel(layer, route):
         rows, k, n = layer
         lay, inp = _linear(-1, k, n), (rows, 1, 1, k)
     else:
-        k, cin, cout, hw = layer
+        k, cin, cout, hw, batch = layer + (1,) * (5 - len(layer))
         lay = dict(op="conv", src=[-1], cin=cin, cout=cout, kh=k, kw=k, stride=1, pad=k // 2, act="none", res=None, res_post=False)
-        inp = (1, hw, hw, cin)
+        inp = (batch, hw, hw, cin)
     m = dict(name="yolov3", model_id=53, dtype="f16", input=inp, layers=[lay], outputs=[0])
     rs = Runner(m, synth.gen.model_weights(m), capi.Plan.resident(capi.Desc(m)))
     assert _routes(rs) == [route]
